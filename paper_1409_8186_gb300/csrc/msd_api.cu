@@ -205,6 +205,7 @@ struct msd_problem {
     DBuf xs, part, sbuf[24];
     DBuf gbuf[9];   // gradient work buffers
     DBuf nfbuf[4];  // near-field buffers: rho, points, weights, output stage
+    DBuf ffbuf;     // far field: sums of the disk groups
     DBuf dortbuf[6];  // time reversal: rho, angles, F, T, eigenvalues, eigen work
     // integral-equation formulation (msd_set_formulation); form == false: the
     // default rows (L on sound-soft disks, -I/2 + N on sound-hard ones, u = L rho)
@@ -296,6 +297,11 @@ const double2* rhs_scale_of(const msd_problem* pb) { return pb->form ? pb->d_frs
 const double2* field_factor_of(const msd_problem* pb) { return pb->form ? pb->d_fff : pb->d_J; }
 
 // Per-row factors of the formulation pb->fw (after the Bessel diagonals).
+// Work buffer of launch_farfield for R columns and T angles.
+double2* farfield_part(msd_problem* pb, int R, int T) {
+    return (double2*)pb->ffbuf.get(farfield_part_bytes(pb->C, pb->cfg.data(), R, T));
+}
+
 void form_rows(msd_problem* pb) {
     const size_t n = (size_t)pb->Ntot;
     char* b = (char*)pb->fbuf.get(n * (5 * 16 + 2 * 8 + 8 + 4));
@@ -1694,6 +1700,7 @@ void msd_destroy(msd_problem* pb) {
     for (auto& b : pb->sbuf) b.release();
     for (auto& b : pb->gbuf) b.release();
     for (auto& b : pb->nfbuf) b.release();
+    pb->ffbuf.release();
     for (auto& b : pb->dortbuf) b.release();
     pb->fbuf.release();
     if (pb->pen_minus) msd_destroy(pb->pen_minus);
@@ -1999,7 +2006,7 @@ msd_status msd_grad_farfield_misfit(msd_problem* pb, int R, const double* betas_
         msd_status st = solve_impl(pb, R, betas_host, &o, rho, st_fwd);
         if (st != MSD_OK) fail(st, "msd_grad_farfield_misfit: forward solve did not converge");
         launch_farfield(pb->d_cfg, pb->C, pb->cfg.data(), pb->d_centre, pb->d_radius, pb->d_J, R, T, d_th, rho,
-                        nullptr, F, s);
+                        farfield_part(pb, R, T), F, s);
         launch_misfit(pb->C, T, R, F, Ft, w, d_J, s);
         // 2. adjoint right-hand side C^H w and adjoint solve (P^-1 A)^H mu = C^H w
         launch_ff_table(pb->d_cfg, pb->C, nmax, T, d_th, E, s);
@@ -2044,7 +2051,7 @@ msd_status msd_farfield(msd_problem* pb, const void* rho, int R, int T, const do
         const double2* d_rho = (const double2*)stage_in(pb, pb->sbuf[22], rho, (size_t)pb->Ntot * R * 16);
         OutStage o(pb, pb->sbuf[23], F_out, (size_t)pb->C * T * R * 16);
         launch_farfield(pb->d_cfg, pb->C, pb->cfg.data(), pb->d_centre, pb->d_radius, field_factor_of(pb), R, T, d_th, d_rho,
-                        nullptr, (double2*)o.dev, pb->stream);
+                        farfield_part(pb, R, T), (double2*)o.dev, pb->stream);
         CK_LAUNCH();
         o.finish();
         return MSD_OK;
@@ -2413,8 +2420,8 @@ msd_status msd_dort(msd_problem* pb, int n_alpha, const msd_opts* opts, void* F_
         double* d_th = (double*)pb->dortbuf[1].get((size_t)n * 8);
         CK(cudaMemcpyAsync(d_th, thetas.data(), (size_t)n * 8, cudaMemcpyHostToDevice, s));
         double2* F = (double2*)pb->dortbuf[2].get(nn * 16);
-        launch_farfield(pb->d_cfg, C, pb->cfg.data(), pb->d_centre, pb->d_radius, field_factor_of(pb), n, n, d_th, rho, nullptr,
-                        F, s);
+        launch_farfield(pb->d_cfg, C, pb->cfg.data(), pb->d_centre, pb->d_radius, field_factor_of(pb), n, n, d_th, rho,
+                        farfield_part(pb, n, n), F, s);
         CK_LAUNCH();
         if (F_out)
             CK(cudaMemcpyAsync(F_out, F, nn * 16,

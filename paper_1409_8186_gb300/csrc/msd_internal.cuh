@@ -341,7 +341,6 @@ void launch_matvec_f32(const MsdConfig* d_cfg, const MatvecWork* d_work, int nwo
                        float2* y, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1,
                        const MatvecChoice* ch = nullptr, const int* live = nullptr, bool xs_ready = false);
 
-// K6: far field.
 // Time reversal (section 7): T = conj(F)^T F for C far-field matrices
 // F [C][n][n] and the eigenvalues of every T, largest first (eig [C][n]).
 // work: dort_work_bytes(C, n) bytes.  dort_set_smem_limits(n) once before
@@ -361,7 +360,9 @@ cudaError_t launch_dort_vectors(int C, int n, int K, void* work, const double* e
 void launch_herglotz(double k, int na, int K, const double2* g, long long P, const double2* pts, double2* out,
                      cudaStream_t s);
 
-// J: the per-row field factor, as for launch_nearfield.
+// J: the per-row field factor, as for launch_nearfield.  part: work buffer of
+// farfield_part_bytes() bytes.
+size_t farfield_part_bytes(int C, const MsdConfig* h_cfg, int R, int T);
 void launch_farfield(const MsdConfig* d_cfg, int C, const MsdConfig* h_cfg,
                      const double2* d_centre, const double* d_radius, const double2* J,
                      int R, int T, const double* d_thetas, const double2* rho,

@@ -4,6 +4,8 @@
 //   K2 Toeplitz generators g^pq_l = H_l(k b_pq) e^{i l alpha_pq} of every
 //      ordered pair (section 4.2, the separation matrix S^pq);
 //   K5 preconditioned plane-wave right-hand sides (Prop. 4.1).
+#include <algorithm>
+
 #include "bessel.cuh"
 #include "msd_internal.cuh"
 
@@ -15,7 +17,8 @@
 
 // ---------------------------------------------------------------- K1
 
-// One thread per disk.  For m = -N..N (Z_{-m} = (-1)^m Z_m, Z' = (Z_{m-1} - Z_{m+1})/2):
+// One warp per disk: lane 0 runs the Bessel recurrences (a serial chain), then
+// the lanes share the modes.  For m = -N..N (Z_{-m} = (-1)^m Z_m, Z' = (Z_{m-1} - Z_{m+1})/2):
 //   J, J', H = J + iY, H' at x = k a_p;
 //   rf  = sqrt(a_p) J_m                               (column factor r^p_m)
 //   lf  = 1/(sqrt(a_p) H_m)           (Dirichlet)     (row factor l^p_m)
@@ -25,25 +28,30 @@
 // Dividing the off-diagonal blocks of section 4.2 by the diagonal block
 // (i pi a_p/2) J^p H^p (Dirichlet) or (i pi k a_p/2) J^p H'^p (Neumann)
 // leaves exactly l^p_m g_{n-m} r^q_n: the J_m of Dirichlet rows cancels
-// analytically instead of being divided out.
-__global__ void k_disk_diagonals(const MsdConfig* __restrict__ cfg, int Mtot,
+// analytically instead of being divided out.  Bound by the latency of the
+// chain (a warp-wide FP64 instruction takes 64 clocks whatever its lanes do).
+constexpr int kDiagWarps = 4;
+__global__ void __launch_bounds__(kDiagWarps * 32) k_disk_diagonals(const MsdConfig* __restrict__ cfg, int Mtot,
                                  const int* __restrict__ disk_cfg, const double* __restrict__ radius,
                                  const int8_t* __restrict__ bc, double2* J_, double2* dJ_, double2* H_,
                                  double2* dH_, double2* lf64, double* rf64, float2* lf32, float* rf32,
                                  double2* rhs_scale, int* flags) {
-    int d = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double Jsh[kDiagWarps][MSD_MAX_N + 2], Ysh[kDiagWarps][MSD_MAX_N + 2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int d = blockIdx.x * kDiagWarps + warp;
     if (d >= Mtot) return;
     const MsdConfig c = cfg[disk_cfg[d]];
     const int N = c.N;
     const double a = radius[d];
     const double x = c.k * a;
-    double J[MSD_MAX_N + 2], Y[MSD_MAX_N + 2];
-    bessel_jy(x, N + 1, J, Y);
+    double *J = Jsh[warp], *Y = Ysh[warp];
+    if (lane == 0) bessel_jy(x, N + 1, J, Y);
+    __syncwarp();
     const double sa = sqrt(a);
     const bool neumann = bc[d] == MSD_NEUMANN;
     const long long row0 = c.row_off + (long long)(d - c.disk_off) * c.n;
     int bad = 0;
-    for (int mm = -N; mm <= N; ++mm) {
+    for (int mm = lane - N; mm <= N; mm += 32) {
         int m = mm < 0 ? -mm : mm;
         double sgn = (mm < 0 && (m & 1)) ? -1.0 : 1.0;
         double Jm = J[m], Ym = Y[m];
@@ -120,36 +128,109 @@ void launch_disk_diagonals(const MsdConfig* d_cfg, int Mtot, const int* d_disk_c
                            double2* J, double2* dJ, double2* H, double2* dH,
                            double2* lf64, double* rf64, float2* lf32, float* rf32,
                            double2* rhs_scale, int* d_flags, cudaStream_t s) {
-    int threads = 128;
-    int blocks = (Mtot + threads - 1) / threads;
-    k_disk_diagonals<<<blocks, threads, 0, s>>>(d_cfg, Mtot, d_disk_cfg, d_radius, d_bc, J, dJ, H,
+    const int blocks = (Mtot + kDiagWarps - 1) / kDiagWarps;
+    k_disk_diagonals<<<blocks, kDiagWarps * 32, 0, s>>>(d_cfg, Mtot, d_disk_cfg, d_radius, d_bc, J, dJ, H,
                                                  dH, lf64, rf64, lf32, rf32, rhs_scale, d_flags);
     g_msd_launches += 1;
 }
 
 // ---------------------------------------------------------------- K2
 
-// One thread per ordered pair (q, p) of a generator block: configuration
-// g.cfg, sources q in [Q0, Q0+Qb), targets p in [P0, P0+Pc) (P0, Pc
-// multiples of 32, p may reach into the padding p >= M).  Output
-// out[g.out_off + ((q-Q0) Pc + (p-P0)) L + l + 2N].  The whole-problem
-// array is one block per configuration (P0 = Q0 = 0, Pc = Mp, Qb = M,
-// out_off = gen_off); recomputed products use blocks of a chunk.
 // b_pq = O_p - O_q, e^{i alpha_pq} = b_pq/|b_pq|; for l >= 0:
 // g_l = H_l(k b) e^{i l alpha}, g_{-l} = (-1)^l H_l(k b) e^{-i l alpha}.
 // Padded targets (p >= M) and the diagonal p == q get zeros.
 //
-// Far pairs (x = k b > 20 and 2N <= x: J and Y both by forward recurrence
-// from Hankel's expansion of orders 0 and 1) are done by their own thread;
-// near pairs (Miller's backward sweep, ~100 FP64 steps) are collected per
-// block and done afterwards by the first threads of the block, so that a
-// warp of far pairs never waits on a near one.  F32: the far pairs of a
-// complex64-only build use FP32 arithmetic after an FP64 phase (sin/cos of
-// x and the unit vector b/|b|); relative error ~1e-6, for products that run
-// in FP32 anyway.
+// Far pairs (x = k b > 20 and 2N <= x) take J and Y by forward recurrence
+// from Hankel's expansion of orders 0 and 1; near pairs need Miller's
+// backward sweep.  Two kernels:
+//  * k_pair_generators_full fills the stored array of whole configurations,
+//    where g^{qp}_l = (-1)^l g^{pq}_l (the reversed pair turns alpha by pi)
+//    halves the work: one thread per unordered pair writes both rows.  The
+//    near pairs are gathered by the first CTAs of the grid, each scanning a
+//    stretch of pairs into full warps, so their long chain starts at once and
+//    runs beside the far pairs.
+//  * k_pair_generators makes the blocks of a recomputed product, one thread
+//    per ordered pair (q, p): configuration g.cfg, sources q in [Q0, Q0+Qb),
+//    targets p in [P0, P0+Pc) (P0, Pc multiples of 32, p may reach into the
+//    padding p >= M), output out[g.out_off + ((q-Q0) Pc + (p-P0)) L + l + 2N].
+//    Its near pairs are done after the far ones by the first threads of the
+//    block.  F32: the far pairs of a complex64-only build use FP32 arithmetic
+//    after an FP64 phase (sin/cos of x and the unit vector b/|b|); relative
+//    error ~1e-6, for products that run in FP32 anyway.
+//
+// The FP64 pipe is the bound: 16 operations per order l >= 0 and pair and
+// about 250 around the recurrences.  Measured (GB300): a geometry step of 400
+// disks, N = 20 (factors, generators, their read-out and one FP64 product)
+// 3177 -> 2416 us, of which the factors were 225 us (one thread per disk) and
+// the generators 821 us (both orders of every pair, divisions in every step).
 namespace {
 
 constexpr int kGenThreads = 128;
+
+// Distance and direction of one ordered pair.  b = sqrt(dx^2 + dy^2) with one
+// rounding of the sum (as accurate as hypot), and hypot where the squares
+// leave the normal range; written with fixed roundings, so that both kernels'
+// near/far decisions on a pair agree wherever they are made.
+struct PairGeom {
+    double dx, dy, b, x;
+    __device__ PairGeom(double2 Op, double2 Oq, double k) {
+        dx = Op.x - Oq.x;
+        dy = Op.y - Oq.y;
+        const double b2 = fma(dx, dx, __dmul_rn(dy, dy));
+        b = b2 > 1e-280 && b2 < 1e280 ? sqrt(b2) : hypot(dx, dy);
+        x = __dmul_rn(k, b);
+    }
+    __device__ bool far(int lmax) const { return x > 20.0 && (double)lmax <= x; }
+};
+
+// Generator values of a far pair: put(l, g_l, g_{-l}) for l = 0..lmax.
+template <typename Put>
+__device__ __forceinline__ void far_generators(const PairGeom& g, int lmax, Put&& put) {
+    const double2 e1 = make_double2(g.dx / g.b, g.dy / g.b);
+    double2 e = make_double2(1.0, 0.0);  // e^{i l alpha}
+    double sx, cx, J0, J1, Y0, Y1;
+    sincos(g.x, &sx, &cx);
+    bessel_asymptotic01(g.x, sx, cx, &J0, &Y0, &J1, &Y1);
+    const TwoOverX f(g.x);
+    auto emit = [&](int l, double Jl, double Yl) {
+        const double2 H = make_double2(Jl, Yl);
+        const double2 gp = cmul(H, e);   // g_l
+        double2 gm = cmul(H, cconj(e));  // H_l e^{-i l alpha}
+        if (l & 1) gm = make_double2(-gm.x, -gm.y);
+        put(l, gp, gm);
+    };
+    emit(0, J0, Y0);
+    for (int l = 1; l <= lmax; ++l) {
+        e = cmul(e, e1);
+        emit(l, J1, Y1);
+        const double c = f.times((double)l);
+        const double J2 = fma(c, J1, -J0), Y2 = fma(c, Y1, -Y0);
+        J0 = J1;
+        J1 = J2;
+        Y0 = Y1;
+        Y1 = Y2;
+    }
+}
+
+// The same for a near pair.
+template <typename Put>
+__device__ __forceinline__ void near_generators(const PairGeom& g, int lmax, Put&& put) {
+    const double2 e1 = make_double2(g.dx / g.b, g.dy / g.b);
+    double J[MAXL], Y[MAXL];
+    bessel_jy(g.x, lmax, J, Y);
+    double2 e = make_double2(1.0, 0.0);
+    for (int l = 0; l <= lmax; ++l) {
+        const double2 H = make_double2(J[l], Y[l]);
+        const double2 gp = cmul(H, e);
+        double2 gm = cmul(H, cconj(e));
+        if (l & 1) gm = make_double2(-gm.x, -gm.y);
+        put(l, gp, gm);
+        e = cmul(e, e1);
+    }
+}
+
+__device__ __forceinline__ bool f32_range(double2 g) { return fabs(g.x) < 3.0e38 && fabs(g.y) < 3.0e38; }
+__device__ __forceinline__ float2 to_f32(double2 g) { return make_float2((float)g.x, (float)g.y); }
 
 struct PairRef {
     GenBlock g;
@@ -221,11 +302,9 @@ __global__ void __launch_bounds__(kGenThreads)
                 if (G32) G32[base + l] = make_float2(0.f, 0.f);
             }
         } else {
-            const double2 Op = centre[c.disk_off + r.p], Oq = centre[c.disk_off + r.q];
-            const double dx = Op.x - Oq.x, dy = Op.y - Oq.y;
-            const double b = hypot(dx, dy);
-            const double x = c.k * b;
-            if (!(x > 20.0 && (double)lmax <= x)) {
+            const PairGeom pg(centre[c.disk_off + r.p], centre[c.disk_off + r.q], c.k);
+            const double x = pg.x;
+            if (!pg.far(lmax)) {
                 near_list[atomicAdd(&n_near, 1)] = threadIdx.x;
             } else if (F32) {
                 double sxd, cxd;
@@ -234,7 +313,7 @@ __global__ void __launch_bounds__(kGenThreads)
                 float J0, J1, Y0, Y1;
                 bessel_asymptotic_f32(xf, 0, (float)sxd, (float)cxd, &J0, &Y0);
                 bessel_asymptotic_f32(xf, 1, (float)sxd, (float)cxd, &J1, &Y1);
-                const float2 e1 = make_float2((float)(dx / b), (float)(dy / b));
+                const float2 e1 = make_float2((float)(pg.dx / pg.b), (float)(pg.dy / pg.b));
                 const float two_x = 2.0f / xf;
                 float2 e = make_float2(1.f, 0.f);
                 auto put = [&](int l, float Jl, float Yl) {
@@ -256,37 +335,16 @@ __global__ void __launch_bounds__(kGenThreads)
                     Y1 = Y2;
                 }
             } else {
-                const double2 e1 = make_double2(dx / b, dy / b);
-                double2 e = make_double2(1.0, 0.0);  // e^{i l alpha}
-                auto put = [&](int l, double Jl, double Yl) {
-                    const double2 H = make_double2(Jl, Yl);
-                    const double2 gp = cmul(H, e);                  // g_l
-                    double2 gm = cmul(H, cconj(e));                 // H_l e^{-i l alpha}
-                    if (l & 1) gm = make_double2(-gm.x, -gm.y);    // g_{-l} = (-1)^l H_l e^{-i l alpha}
+                far_generators(pg, lmax, [&](int l, double2 gp, double2 gm) {
                     if (G64) {
                         G64[base + lmax + l] = gp;
                         G64[base + lmax - l] = gm;
                     }
                     if (G32) {
-                        G32[base + lmax + l] = make_float2((float)gp.x, (float)gp.y);
-                        G32[base + lmax - l] = make_float2((float)gm.x, (float)gm.y);
+                        G32[base + lmax + l] = to_f32(gp);
+                        G32[base + lmax - l] = to_f32(gm);
                     }
-                    e = cmul(e, e1);
-                };
-                double sx, cx, J0, J1, Y0, Y1;
-                sincos(x, &sx, &cx);
-                bessel_asymptotic(x, 0, sx, cx, &J0, &Y0);
-                bessel_asymptotic(x, 1, sx, cx, &J1, &Y1);
-                put(0, J0, Y0);
-                for (int l = 1; l <= lmax; ++l) {
-                    put(l, J1, Y1);
-                    const double f = 2.0 * l / x;
-                    const double J2 = f * J1 - J0, Y2 = f * Y1 - Y0;
-                    J0 = J1;
-                    J1 = J2;
-                    Y0 = Y1;
-                    Y1 = Y2;
-                }
+                });
             }
         }
     }
@@ -298,28 +356,152 @@ __global__ void __launch_bounds__(kGenThreads)
         const MsdConfig c = cfg[r.g.cfg];
         const int L = c.L, lmax = 2 * c.N;
         const long long base = r.g.out_off + r.li * L;
-        const double2 Op = centre[c.disk_off + r.p], Oq = centre[c.disk_off + r.q];
-        const double dx = Op.x - Oq.x, dy = Op.y - Oq.y;
-        const double b = hypot(dx, dy);
-        const double2 e1 = make_double2(dx / b, dy / b);
-        double J[MAXL], Y[MAXL];
-        bessel_jy(c.k * b, lmax, J, Y);
-        double2 e = make_double2(1.0, 0.0);
-        for (int l = 0; l <= lmax; ++l) {
-            const double2 H = make_double2(J[l], Y[l]);
-            const double2 gp = cmul(H, e);
-            double2 gm = cmul(H, cconj(e));
-            if (l & 1) gm = make_double2(-gm.x, -gm.y);
+        const PairGeom pg(centre[c.disk_off + r.p], centre[c.disk_off + r.q], c.k);
+        near_generators(pg, lmax, [&](int l, double2 gp, double2 gm) {
             if (G64) {
                 G64[base + lmax + l] = gp;
                 G64[base + lmax - l] = gm;
             }
             if (G32) {
-                if (!(fabs(gp.x) < 3.0e38 && fabs(gp.y) < 3.0e38)) bad = 1;
-                G32[base + lmax + l] = make_float2((float)gp.x, (float)gp.y);
-                G32[base + lmax - l] = make_float2((float)gm.x, (float)gm.y);
+                if (!f32_range(gp)) bad = 1;
+                G32[base + lmax + l] = to_f32(gp);
+                G32[base + lmax - l] = to_f32(gm);
             }
-            e = cmul(e, e1);
+        });
+    }
+    if (bad) atomicOr(flags, FLAG_RANGE32);
+}
+
+// Unordered pairs of a configuration: item i < M (M / 2) is q = i mod M,
+// p = (q + 1 + i / M) mod M; for even M the last turn meets every pair twice
+// and keeps its first half.  Items from M (M / 2) on are the rows of zeros:
+// the M diagonal ones, then the padded targets of every source.
+struct FullItem {
+    int cfg, q, p;  // p == q, p >= M: a row of zeros
+    bool none;      // the second half of the last turn
+};
+__device__ __forceinline__ FullItem full_item(const MsdConfig* __restrict__ cfg, const GenBlock* __restrict__ blocks,
+                                              int nblocks, long long idx) {
+    int lo = 0, hi = nblocks - 1;  // last configuration with item_off <= idx
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (blocks[mid].item_off <= idx) lo = mid;
+        else hi = mid - 1;
+    }
+    FullItem r;
+    r.cfg = blocks[lo].cfg;
+    const int M = blocks[lo].Qb, pads = blocks[lo].Pc - M;
+    const long long i = idx - blocks[lo].item_off, pairs = (long long)M * (M / 2);
+    r.none = false;
+    if (i < pairs) {
+        r.q = (int)(i % M);
+        const int j = 1 + (int)(i / M);
+        r.p = r.q + j < M ? r.q + j : r.q + j - M;
+        r.none = 2 * j == M && 2 * r.q >= M;
+    } else if (i < pairs + M) {
+        r.q = r.p = (int)(i - pairs);
+    } else {
+        r.q = (int)((i - pairs - M) / pads);
+        r.p = M + (int)((i - pairs - M) % pads);
+    }
+    return r;
+}
+
+// Rows of both orders of a pair from the values of (q, p).
+struct PutBoth {
+    double2* G64;
+    float2* G32;
+    long long a, b;  // element l = 0 of [q][p] and of [p][q]
+    int bad = 0;
+    __device__ void operator()(int l, double2 gp, double2 gm) {
+        const double s = (l & 1) ? -1.0 : 1.0;
+        const double2 rp = make_double2(s * gp.x, s * gp.y), rm = make_double2(s * gm.x, s * gm.y);
+        if (G64) {
+            G64[a + l] = gp;
+            G64[a - l] = gm;
+            G64[b + l] = rp;
+            G64[b - l] = rm;
+        }
+        if (G32) {
+            if (!f32_range(gp)) bad = 1;
+            const float2 fp = to_f32(gp), fm = to_f32(gm);
+            const float t = (l & 1) ? -1.f : 1.f;
+            G32[a + l] = fp;
+            G32[a - l] = fm;
+            G32[b + l] = make_float2(t * fp.x, t * fp.y);
+            G32[b - l] = make_float2(t * fm.x, t * fm.y);
+        }
+    }
+};
+
+__device__ __forceinline__ PutBoth put_both(const MsdConfig& c, int q, int p, double2* G64, float2* G32) {
+    const int lmax = 2 * c.N;
+    return PutBoth{G64, G32, c.gen_off + ((long long)q * c.Mp + p) * c.L + lmax,
+                   c.gen_off + ((long long)p * c.Mp + q) * c.L + lmax};
+}
+
+__global__ void __launch_bounds__(kGenThreads)
+    k_pair_generators_full(const MsdConfig* __restrict__ cfg, const GenBlock* __restrict__ blocks, int nblocks,
+                           long long nitems, int near_blocks, const double2* __restrict__ centre, double2* G64,
+                           float2* G32, int* flags) {
+    int bad = 0;
+    if ((int)blockIdx.x >= near_blocks) {
+        const long long idx = (long long)(blockIdx.x - near_blocks) * kGenThreads + threadIdx.x;
+        if (idx >= nitems) return;
+        const FullItem r = full_item(cfg, blocks, nblocks, idx);
+        if (r.none) return;
+        const MsdConfig c = cfg[r.cfg];
+        const int lmax = 2 * c.N;
+        if (r.p == r.q || r.p >= c.M) {
+            const long long base = c.gen_off + ((long long)r.q * c.Mp + r.p) * c.L;
+            for (int l = 0; l < c.L; ++l) {
+                if (G64) G64[base + l] = make_double2(0.0, 0.0);
+                if (G32) G32[base + l] = make_float2(0.f, 0.f);
+            }
+            return;
+        }
+        const PairGeom pg(centre[c.disk_off + r.p], centre[c.disk_off + r.q], c.k);
+        if (pg.far(lmax)) {
+            PutBoth put = put_both(c, r.q, r.p, G64, G32);
+            far_generators(pg, lmax, put);
+        }
+        return;  // (no far value leaves the complex64 range: |H_l| decreases with x >= 2N >= l)
+    }
+    // near pairs of items [i0, i1): gathered a batch at a time, then one per thread
+    __shared__ long long list[2 * kGenThreads];
+    __shared__ int count;
+    const long long per = (nitems + near_blocks - 1) / near_blocks;
+    const long long i0 = blockIdx.x * per, i1 = i0 + per < nitems ? i0 + per : nitems;
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    for (long long at = i0; at < i1; at += kGenThreads) {
+        const long long idx = at + threadIdx.x;
+        if (idx < i1) {
+            const FullItem r = full_item(cfg, blocks, nblocks, idx);
+            const MsdConfig c = cfg[r.cfg];
+            if (!r.none && r.p != r.q && r.p < c.M) {
+                const double2 Op = centre[c.disk_off + r.p], Oq = centre[c.disk_off + r.q];
+                // cheap bound first: far by more than rounding could undo
+                const double dx = Op.x - Oq.x, dy = Op.y - Oq.y, T = fmax(20.0, 2.0 * c.N) * (1.0 + 1e-9);
+                if (!(c.k * c.k * fma(dx, dx, dy * dy) > T * T) && !PairGeom(Op, Oq, c.k).far(2 * c.N))
+                    list[atomicAdd(&count, 1)] = idx;
+            }
+        }
+        __syncthreads();
+        const int n = count;
+        __syncthreads();  // every thread has the count before the next batch adds to it
+        const bool last = at + kGenThreads >= i1;
+        if (n >= kGenThreads || (last && n > 0)) {
+            for (int i = threadIdx.x; i < n; i += kGenThreads) {
+                const FullItem r = full_item(cfg, blocks, nblocks, list[i]);
+                const MsdConfig c = cfg[r.cfg];
+                PutBoth put = put_both(c, r.q, r.p, G64, G32);
+                near_generators(PairGeom(centre[c.disk_off + r.p], centre[c.disk_off + r.q], c.k), 2 * c.N, put);
+                bad |= put.bad;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) count = 0;
+            __syncthreads();
         }
     }
     if (bad) atomicOr(flags, FLAG_RANGE32);
@@ -535,6 +717,25 @@ void launch_nearfield_inside(const MsdConfig* d_cfg, int ci, const MsdConfig& h_
         g_msd_launches += 1;
     }
     g_msd_launches += 2;
+}
+
+// Items of one configuration for launch_full_generators (unordered pairs and
+// rows of zeros, see full_item).
+long long full_generator_items(const MsdConfig& c) {
+    return (long long)c.M * (c.M / 2) + c.M + (long long)c.M * (c.Mp - c.M);
+}
+
+void launch_generators_all(const MsdConfig* d_cfg, const GenBlock* d_blocks, int nblocks, long long nitems,
+                           const double2* d_centre, double2* G64, float2* G32, int* d_flags, cudaStream_t s) {
+    if (nitems <= 0) return;
+    // gathering CTAs: about a full warp of near pairs each where one pair in
+    // a hundred is near (a cluster of hundreds of disks), and one CTA per 128
+    // pairs of small problems, where most are near
+    const long long near_blocks = std::min<long long>(152, (nitems + kGenThreads - 1) / kGenThreads);
+    const long long far_blocks = (nitems + kGenThreads - 1) / kGenThreads;
+    k_pair_generators_full<<<(unsigned)(near_blocks + far_blocks), kGenThreads, 0, s>>>(
+        d_cfg, d_blocks, nblocks, nitems, (int)near_blocks, d_centre, G64, G32, d_flags);
+    g_msd_launches += 1;
 }
 
 void launch_generator_blocks(const MsdConfig* d_cfg, const GenBlock* d_blocks, int nblocks, long long nitems,

@@ -182,6 +182,7 @@ struct msd_problem {
     int gen_mode = MSD_GEN_STREAMED;
     size_t gen_chunk_bytes = 64ull << 20;
     std::vector<GenBlock> gen_full;  // one block per configuration: the stored array
+    long long gen_items = 0;
     GenBlock* d_gen_full = nullptr;
     std::map<long long, RecomputePlan> rplans;  // key: R*4 + precision
     DBuf genbuf;
@@ -204,8 +205,8 @@ struct msd_problem {
     cudaEvent_t ring_ev[4] = {nullptr, nullptr, nullptr, nullptr};
     DBuf xs, part, sbuf[24];
     DBuf gbuf[9];   // gradient work buffers
-    DBuf nfbuf[4];  // near-field buffers: rho, points, weights, output stage
     DBuf ffbuf;     // far field: sums of the disk groups
+    DBuf nfbuf[4];  // near-field buffers: rho, points, weights, output stage
     DBuf dortbuf[6];  // time reversal: rho, angles, F, T, eigenvalues, eigen work
     // integral-equation formulation (msd_set_formulation); form == false: the
     // default rows (L on sound-soft disks, -I/2 + N on sound-hard ones, u = L rho)
@@ -296,12 +297,12 @@ void check_flags(msd_problem* pb, const char* where) {
 const double2* rhs_scale_of(const msd_problem* pb) { return pb->form ? pb->d_frs : pb->d_rhs_scale; }
 const double2* field_factor_of(const msd_problem* pb) { return pb->form ? pb->d_fff : pb->d_J; }
 
-// Per-row factors of the formulation pb->fw (after the Bessel diagonals).
 // Work buffer of launch_farfield for R columns and T angles.
 double2* farfield_part(msd_problem* pb, int R, int T) {
     return (double2*)pb->ffbuf.get(farfield_part_bytes(pb->C, pb->cfg.data(), R, T));
 }
 
+// Per-row factors of the formulation pb->fw (after the Bessel diagonals).
 void form_rows(msd_problem* pb) {
     const size_t n = (size_t)pb->Ntot;
     char* b = (char*)pb->fbuf.get(n * (5 * 16 + 2 * 8 + 8 + 4));
@@ -382,13 +383,13 @@ void launch_full_generators(msd_problem* pb, double2* G64, float2* G32) {
             const MsdConfig& c = pb->cfg[ci];
             GenBlock g{ci, 0, c.Mp, 0, c.M, 0, items, c.gen_off};
             pb->gen_full.push_back(g);
-            items += (long long)c.M * c.Mp;
+            items += full_generator_items(c);
         }
+        pb->gen_items = items;
         pb->d_gen_full = dalloc_copy(pb->gen_full.data(), pb->gen_full.size());
     }
-    const GenBlock& last = pb->gen_full.back();
-    launch_generator_blocks(pb->d_cfg, pb->d_gen_full, pb->C, last.item_off + (long long)last.Qb * last.Pc,
-                            pb->d_centre, G64, G32, pb->d_flags, pb->stream);
+    launch_generators_all(pb->d_cfg, pb->d_gen_full, pb->C, pb->gen_items, pb->d_centre, G64, G32, pb->d_flags,
+                          pb->stream);
 }
 
 void ensure_generators(msd_problem* pb, bool fp64) {
@@ -1699,8 +1700,8 @@ void msd_destroy(msd_problem* pb) {
     pb->part.release();
     for (auto& b : pb->sbuf) b.release();
     for (auto& b : pb->gbuf) b.release();
-    for (auto& b : pb->nfbuf) b.release();
     pb->ffbuf.release();
+    for (auto& b : pb->nfbuf) b.release();
     for (auto& b : pb->dortbuf) b.release();
     pb->fbuf.release();
     if (pb->pen_minus) msd_destroy(pb->pen_minus);

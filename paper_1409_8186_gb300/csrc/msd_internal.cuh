@@ -179,6 +179,11 @@ struct GenBlock {
 void launch_generator_blocks(const MsdConfig* d_cfg, const GenBlock* d_blocks, int nblocks, long long nitems,
                              const double2* d_centre, double2* G64, float2* G32, int* d_flags, cudaStream_t s,
                              bool f32_math = false);
+// The stored arrays of whole configurations (blocks: cfg, Qb = M, Pc = Mp and
+// item_off, the running count of full_generator_items)
+long long full_generator_items(const MsdConfig& c);
+void launch_generators_all(const MsdConfig* d_cfg, const GenBlock* d_blocks, int nblocks, long long nitems,
+                           const double2* d_centre, double2* G64, float2* G32, int* d_flags, cudaStream_t s);
 
 // ||P u||^2 and ||P v||^2 per (row chunk, column) with the preconditioner's
 // diagonal P (unpreconditioned residual norms); R <= 64.

@@ -745,6 +745,12 @@ int matvec_candidates(int R, int Nmax, bool fp64, MatvecChoice* out, int cap, bo
             }
         }
     }
+    if (fp64) {  // the digit-sliced tensor-core kernel (KB = 0 in the encoding of msd_set_tile)
+        Choice c{0, 1, 1, 0};
+        c.DS = 1;
+        if (cnt < cap) out[cnt] = c;
+        ++cnt;
+    }
     if (!fp64)
         for (int rc = 16; rc <= 64; rc *= 2)
             if (tc_supported(R, Nmax, rc)) {
@@ -930,6 +936,18 @@ void product_general(D&& dispatch_fn, const MsdConfig* d_cfg, const MatvecWork* 
 }
 
 }  // namespace
+
+void launch_scale_cols_c(long long Ntot, int R, const double2* cf, const double2* x, double2* xs, cudaStream_t s) {
+    k_scale_cols_c<double2><<<(unsigned)((Ntot * R + 255) / 256), 256, 0, s>>>(Ntot, R, cf, x, xs);
+    g_msd_launches += 1;
+}
+
+void launch_finalize_gen(long long Ntot, int R, int nsplit, const double* row_r, const double2* row_c, int add_x,
+                         const double2* x, const double2* part, double2* y, cudaStream_t s) {
+    k_finalize_gen<double2, double><<<(unsigned)((Ntot * R * kFinLanes + 255) / 256), 256, 0, s>>>(
+        Ntot, R, nsplit, row_r, row_c, add_x, x, part, y);
+    g_msd_launches += 1;
+}
 
 void launch_product_f64(const MsdConfig* d_cfg, const MatvecWork* d_work, int nwork, int Nmax, const double2* G,
                         const double* col_r, const double2* col_c, const double* row_r, const double2* row_c,

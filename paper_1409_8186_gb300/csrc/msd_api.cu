@@ -127,6 +127,28 @@ struct MatvecPlan {
     int ns_div = 1;               // split count = the wave model's / ns_div
     int candidates = 0;           // shapes the autotuner timed (0: model choice)
     double tuned_ms = 0;          // kernel time of the chosen shape in the tuning run
+    // digit-sliced FP64 product (ch.DS): its tiles and work list, valid for
+    // one grouping of the sources
+    DsCfg* d_dscfg = nullptr;
+    DsWork* d_dswork = nullptr;
+    int nds = 0, Rt = 1;
+    DsSmem dsm{0, 0, 0};
+    size_t xd_bytes = 0, ex_ints = 0;
+    long long ds_version = -1;
+};
+
+// Generators of the digit-sliced FP64 product: digits and exponents, built
+// for one geometry version.
+struct DsGen {
+    DBuf dg, eb;
+    long long version = -1;
+    int fits = -1;  // whether device memory has room (-1: not looked at yet)
+    void release() {
+        dg.release();
+        eb.release();
+        version = -1;
+        fits = -1;
+    }
 };
 
 // Product plan with recomputed generators: chunks of generator blocks
@@ -250,6 +272,20 @@ struct msd_problem {
     long long gt_floats = 0, gt_blocks = 0, xrows = 0, gt_version = -1;
     long long* d_gt_blk = nullptr;
     DBuf xt;
+    // digit-sliced FP64 product: radii as the host knows them, the order and
+    // groups of the sources they give (ds_grouping), its operands for the
+    // forward and the adjoint generators, and the source digits of a product
+    std::vector<double> h_radius;
+    long long radius_version = 0, ds_radius_version = -1;
+    bool ds_ok = false;
+    long long ds_version = 0;  // moves on with the groups (not with the order inside them)
+    std::vector<DsCfg> ds_cfg;
+    std::vector<int> ds_grp, ds_qgrp, ds_perm;
+    int ds_max_grp = 0, ds_max_nqs = 0, ds_max_Mp = 0;
+    size_t ds_dg_bytes = 0, ds_eb_bytes = 0;
+    DBuf ds_idx[4];  // on the device: ds_cfg, ds_grp, ds_qgrp, ds_perm
+    DsGen ds_fwd, ds_adj;
+    DBuf dsx, dse;
     // algorithmic size of one product with one column (section 5 storage):
     // sum over ordered pairs of the generator length, and of n^2
     double offdiag_L = 0, offdiag_n2 = 0;
@@ -281,6 +317,7 @@ void check_tc(const char* where) {
     const int t = tc_status_and_clear();
     const int u = tcs_status_and_clear();
     if (t > 0 || u > 0) fail(MSD_ERR_CUDA, std::string(where) + ": a tensor-core pipeline wait expired");
+    if (ds_status_and_clear() > 0) fail(MSD_ERR_CUDA, std::string(where) + ": a pipeline wait of the FP64 product expired");
     if (bt_status_and_clear() > 0) fail(MSD_ERR_CUDA, std::string(where) + ": a generator bulk-copy wait expired");
 }
 
@@ -423,6 +460,132 @@ bool ensure_gt(msd_problem* pb) {
     return true;
 }
 
+// Order and groups of the sources for the digit-sliced FP64 product, from the
+// host's copy of the radii.  Sorted by radius, eight to a K-step; a group
+// takes K-steps while its radii differ by at most 2^{3/N}, and groups that
+// were made so stay through geometry updates while they differ by at most
+// 2^{4.5/N} (see k_matvec_ds.cu), so that a loop that nudges the radii keeps
+// its work lists.  Not offered (false) when eight neighbours differ by more.
+bool ds_grouping(msd_problem* pb) {
+    if (pb->ds_radius_version == pb->radius_version) return pb->ds_ok;
+    pb->ds_radius_version = pb->radius_version;
+    std::vector<int> perm;
+    std::vector<std::vector<double>> lo(pb->C), hi(pb->C);  // radii of every K-step
+    pb->ds_ok = true;
+    bool keep = !pb->ds_grp.empty();
+    for (int ci = 0; ci < pb->C; ++ci) {
+        const MsdConfig& m = pb->cfg[ci];
+        const double* a = pb->h_radius.data() + m.disk_off;
+        const int nqs = (m.M + 7) / 8;
+        std::vector<int> o(m.M);
+        for (int i = 0; i < m.M; ++i) o[i] = i;
+        std::sort(o.begin(), o.end(), [&](int u, int v) { return a[u] != a[v] ? a[u] < a[v] : u < v; });
+        const double most = std::pow(2.0, 4.5 / m.N);
+        for (int k = 0; k < nqs; ++k) {
+            lo[ci].push_back(a[o[8 * k]]);
+            hi[ci].push_back(a[o[std::min(m.M, 8 * k + 8) - 1]]);
+            if (!(hi[ci][k] <= most * lo[ci][k])) pb->ds_ok = false;
+        }
+        if (keep) {
+            const DsCfg& c = pb->ds_cfg[ci];
+            for (int g = 0; g < c.ngrp; ++g)
+                if (!(hi[ci][pb->ds_grp[c.grp_off + g + 1] - 1] <= most * lo[ci][pb->ds_grp[c.grp_off + g]]))
+                    keep = false;
+        }
+        o.resize(8 * (size_t)nqs, -1);
+        perm.insert(perm.end(), o.begin(), o.end());
+    }
+    if (!pb->ds_ok) return false;
+    auto upload = [&](DBuf& buf, const void* src, size_t bytes) {
+        void* d = buf.get(bytes);
+        CK(cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, pb->stream));
+    };
+    pb->ds_fwd.version = pb->ds_adj.version = -1;
+    pb->ds_perm = perm;
+    upload(pb->ds_idx[3], pb->ds_perm.data(), perm.size() * sizeof(int));
+    if (keep) return true;
+    pb->ds_version += 1;
+    pb->ds_cfg.clear();
+    pb->ds_grp.clear();
+    pb->ds_qgrp.clear();
+    pb->ds_max_grp = pb->ds_max_nqs = pb->ds_max_Mp = 0;
+    long long dg = 0, eb = 0;
+    int perm_off = 0;
+    for (int ci = 0; ci < pb->C; ++ci) {
+        const MsdConfig& m = pb->cfg[ci];
+        DsCfg c;
+        memset(&c, 0, sizeof(c));
+        c.n = m.n;
+        c.N = m.N;
+        c.L = m.L;
+        c.M = m.M;
+        c.Mp = m.Mp;
+        c.nqs = (m.M + 7) / 8;
+        c.grp_off = (int)pb->ds_grp.size();
+        c.qs_off = (int)pb->ds_qgrp.size();
+        c.perm_off = perm_off;
+        c.gen_off = m.gen_off;
+        c.row_off = m.row_off;
+        c.dg_off = dg;
+        c.eb_off = eb;
+        const double most = std::pow(2.0, 3.0 / m.N);
+        double first = 0;
+        for (int k = 0; k < c.nqs; ++k) {
+            if (k == 0 || !(hi[ci][k] <= most * first)) {
+                pb->ds_grp.push_back(k);
+                first = lo[ci][k];
+                ++c.ngrp;
+            }
+            pb->ds_qgrp.push_back(c.ngrp - 1);
+        }
+        pb->ds_grp.push_back(c.nqs);
+        perm_off += 8 * c.nqs;
+        const long long tiles = m.Mp / MSD_TILE_P;
+        dg += tiles * m.L * c.nqs;
+        eb += tiles * c.ngrp * m.L * MSD_TILE_P;
+        pb->ds_max_grp = std::max(pb->ds_max_grp, c.ngrp);
+        pb->ds_max_nqs = std::max(pb->ds_max_nqs, c.nqs);
+        pb->ds_max_Mp = std::max(pb->ds_max_Mp, m.Mp);
+        pb->ds_cfg.push_back(c);
+    }
+    pb->ds_dg_bytes = (size_t)dg * ds_stage_bytes();
+    pb->ds_eb_bytes = (size_t)eb * sizeof(int);
+    upload(pb->ds_idx[0], pb->ds_cfg.data(), pb->ds_cfg.size() * sizeof(DsCfg));
+    upload(pb->ds_idx[1], pb->ds_grp.data(), pb->ds_grp.size() * sizeof(int));
+    upload(pb->ds_idx[2], pb->ds_qgrp.data(), pb->ds_qgrp.size() * sizeof(int));
+    return true;
+}
+
+// Whether the digit-sliced product can serve this problem: similar radii in
+// every K-step, and its generators (28 bytes per value) in at most 60 % of the
+// free device memory when they are first wanted.
+bool ds_possible(msd_problem* pb, bool adjoint) {
+    if (pb->gen_mode == MSD_GEN_RECOMPUTE || !ds_grouping(pb)) return false;
+    DsGen& g = adjoint ? pb->ds_adj : pb->ds_fwd;
+    if (g.fits < 0) {
+        size_t free_b = 0, total_b = 0;
+        CK(cudaMemGetInfo(&free_b, &total_b));
+        g.fits = (double)(pb->ds_dg_bytes + pb->ds_eb_bytes) <= 0.6 * (double)free_b ? 1 : 0;
+    }
+    return g.fits == 1;
+}
+
+// Generator digits of the current geometry (after ds_possible; G: the stored
+// generators, or the adjoint ones).
+DsGen& ensure_ds(msd_problem* pb, bool adjoint, const double2* G) {
+    DsGen& g = adjoint ? pb->ds_adj : pb->ds_fwd;
+    if (g.version != pb->geom_version) {
+        int* eb = (int*)g.eb.get(pb->ds_eb_bytes);
+        unsigned char* dg = (unsigned char*)g.dg.get(pb->ds_dg_bytes);
+        launch_ds_build((const DsCfg*)pb->ds_idx[0].p, pb->C, pb->ds_max_Mp, pb->ds_max_grp, 4 * pb->Nmax + 1,
+                        pb->ds_max_nqs, (const int*)pb->ds_idx[1].p, (const int*)pb->ds_idx[2].p,
+                        (const int*)pb->ds_idx[3].p, G, eb, dg, pb->stream);
+        CK_LAUNCH();
+        g.version = pb->geom_version;
+    }
+    return g;
+}
+
 // Target tiles of a product kernel within [P0, P1) (multiples of 32): 32
 // disks for the CUDA-core kernel; for the tensor-core kernel floor(128 / n)
 // disks, restarted at every 32-disk boundary and cut at M.
@@ -498,7 +661,163 @@ void build_work_tcs(msd_problem* pb, MatvecPlan& plan, int R) {
     }
 }
 
+// Work list of the digit-sliced product.  Columns go to groups of Rt <= 64,
+// modes to tiles of J <= 64 / Rt (the choice with the fewest (tile, shift)
+// pairs); the sources of a group are cut into folds of at most `ks` K-steps
+// and the shifts into `parts` ranges, chosen by a model of the CTA time (500
+// clocks of MMAs per K-step; up to 4300 clocks of FP64
+// work to drain a full tile) so that the last wave of one CTA per SM is full.
+// False when the partial sums would exceed 2 GB.
+bool build_work_ds(msd_problem* pb, MatvecPlan& plan, int R) {
+    int sms = 0, dev = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int nmax = 2 * pb->Nmax + 1;
+    auto tiles_of = [](int n, int Rt, int* J, int* mt) {
+        const int jm = std::min(n, 64 / Rt);
+        *mt = (n + jm - 1) / jm;
+        *J = (n + *mt - 1) / *mt;
+    };
+    double best_cols = 1e300;
+    const int g0 = (R + 63) / 64;
+    for (int g = g0; g <= std::min(R, 4 * g0 + 4); ++g) {
+        const int Rt = (R + g - 1) / g;
+        int J, mt;
+        tiles_of(nmax, Rt, &J, &mt);
+        const double cost = (double)((R + Rt - 1) / Rt) * mt * (nmax + J - 1);
+        if (cost < best_cols) {
+            best_cols = cost;
+            plan.Rt = Rt;
+        }
+    }
+    const int Rt = plan.Rt, ncg = (R + Rt - 1) / Rt;
+    std::vector<DsCfg> cfgs = pb->ds_cfg;
+    long long xd = 0, ex = 0;
+    int rp_max = 0, rows_max = 0;
+    for (DsCfg& c : cfgs) {
+        tiles_of(c.n, Rt, &c.J, &c.mt);
+        c.rp = (2 * c.J * Rt + 7) / 8 * 8;
+        c.xd_off = xd;
+        c.ex_off = ex;
+        xd += (long long)ncg * c.mt * c.nqs * ds_xblk_bytes(c.rp);
+        ex += (long long)c.ngrp * c.n * R;
+        rp_max = std::max(rp_max, c.rp);
+        rows_max = std::max(rows_max, 2 * c.J * Rt);
+    }
+    plan.xd_bytes = (size_t)xd;
+    plan.ex_ints = (size_t)ex;
+    struct Fold {
+        int qs0, ks, grp;
+    };
+    auto folds = [&](const DsCfg& c, int ks) {
+        std::vector<Fold> out;
+        for (int g = 0; g < c.ngrp; ++g) {
+            const int a = pb->ds_grp[c.grp_off + g], b = pb->ds_grp[c.grp_off + g + 1];
+            const int nb = (b - a + ks - 1) / ks;
+            for (int i = 0; i < nb; ++i) {
+                const int s = a + (b - a) * i / nb, e = a + (b - a) * (i + 1) / nb;
+                out.push_back({s, e - s, g});
+            }
+        }
+        return out;
+    };
+    auto clocks = [&](const DsCfg& c, int ks, int nd) {
+        const double drain = 4300.0 * (2.0 * c.J * Rt / 128.0) * c.n / (c.n + c.J - 1) + 300.0;
+        return 7000.0 + nd * std::max(500.0 * ks, drain);
+    };
+    auto slots_of = [&](int ks, int parts) {
+        long long ns = 1;
+        for (const DsCfg& c : cfgs) ns = std::max(ns, (long long)c.mt * (long long)folds(c, ks).size() * parts);
+        return ns;
+    };
+    int ks_best = 0, parts_best = 1;
+    double best = 1e300;
+    for (int ks = 1; ks <= kDsMaxKs; ++ks) {
+        if (ds_smem(ks, rp_max, rows_max).total > kDsSmemCap) break;
+        for (int parts : {1, 2, 3, 4, 6, 8, 12}) {
+            const long long ns = slots_of(ks, parts);
+            if (ns > 1 && (size_t)ns * pb->Ntot * R * 16 > (2ull << 30)) continue;
+            double total = 0, most = 0;
+            for (const DsCfg& c : cfgs) {
+                const std::vector<Fold> fs = folds(c, ks);
+                for (int t = 0; t < c.mt; ++t) {
+                    const int nsh = std::min(c.J, c.n - t * c.J) + c.n - 1;
+                    const int nd = (nsh + parts - 1) / parts;
+                    for (const Fold& f : fs) {
+                        const double w = clocks(c, f.ks, nd);
+                        total += w * parts * ncg * (c.Mp / MSD_TILE_P);
+                        most = std::max(most, w);
+                    }
+                }
+            }
+            // one CTA per SM: the average load rounded up by half the largest CTA;
+            // partial sums written and read at 3 kB per clock
+            const double span = std::max(most, total / sms + 0.5 * most) + (double)ns * pb->Ntot * R * 32 / 3000.0;
+            if (span < best) {
+                best = span;
+                ks_best = ks;
+                parts_best = parts;
+            }
+        }
+    }
+    if (!ks_best) return false;
+    plan.dsm = ds_smem(ks_best, rp_max, rows_max);
+    plan.nsplit = (int)slots_of(ks_best, parts_best);
+    std::vector<std::pair<double, DsWork>> items;
+    for (int ci = 0; ci < pb->C; ++ci) {
+        const DsCfg& c = cfgs[ci];
+        const std::vector<Fold> fs = folds(c, ks_best);
+        for (int tile = 0; tile < c.Mp / MSD_TILE_P; ++tile)
+            for (int cg = 0; cg < ncg; ++cg) {
+                int slot = 0;
+                for (int t = 0; t < c.mt; ++t) {
+                    const int dlo = t * c.J - (c.n - 1), dhi = std::min(c.n, (t + 1) * c.J) - 1, nsh = dhi - dlo + 1;
+                    for (const Fold& f : fs)
+                        for (int k = 0; k < parts_best; ++k) {
+                            const int a = dlo + nsh * k / parts_best, b = dlo + nsh * (k + 1) / parts_best - 1;
+                            DsWork w{ci, tile, cg, t, f.qs0, b >= a ? f.ks : 0, f.grp, slot++, a, b};
+                            items.push_back({w.ks ? clocks(c, w.ks, b - a + 1) : 0.0, w});
+                        }
+                }
+                for (; slot < plan.nsplit; ++slot) items.push_back({0.0, DsWork{ci, tile, cg, 0, 0, 0, 0, slot, 0, -1}});
+            }
+    }
+    std::stable_sort(items.begin(), items.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+    std::vector<DsWork> work;
+    for (auto& it : items) work.push_back(it.second);
+    plan.nds = (int)work.size();
+    plan.ds_version = pb->ds_version;
+    plan.d_dscfg = dalloc_copy(cfgs.data(), cfgs.size());
+    plan.d_dswork = dalloc_copy(work.data(), work.size());
+    return true;
+}
+
+void free_plan(MatvecPlan& plan) {
+    for (void* p : {(void*)plan.d_work, (void*)plan.d_dscfg, (void*)plan.d_dswork})
+        if (p) cudaFree(p);
+    plan.d_work = nullptr;
+    plan.d_dscfg = nullptr;
+    plan.d_dswork = nullptr;
+}
+
+// The digit-sliced Toeplitz sums of the scaled columns xs into part.
+void ds_product(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint, const double2* G, const double2* xs,
+                double2* part, const int* live = nullptr) {
+    DsGen& g = ensure_ds(pb, adjoint, G);
+    unsigned char* XD = (unsigned char*)pb->dsx.get(plan.xd_bytes);
+    int* EX = (int*)pb->dse.get(plan.ex_ints * sizeof(int));
+    launch_ds_prep(plan.d_dscfg, pb->C, 2 * pb->Nmax + 1, pb->ds_max_grp, pb->ds_max_nqs,
+                   (const int*)pb->ds_idx[1].p, (const int*)pb->ds_idx[2].p, (const int*)pb->ds_idx[3].p, R, plan.Rt,
+                   xs, EX, XD, pb->stream);
+    launch_ds(plan.d_dscfg, plan.d_dswork, plan.nds, plan.dsm, (const unsigned char*)g.dg.p, (const int*)g.eb.p, XD,
+              EX, part, pb->Ntot, R, plan.Rt, pb->stream, live);
+}
+
 void build_work(msd_problem* pb, MatvecPlan& plan, int R, bool fp64) {
+    if (plan.ch.DS) {
+        if (build_work_ds(pb, plan, R)) return;
+        plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
+    }
     if (plan.ch.SH) {
         build_work_tcs(pb, plan, R);
         return;
@@ -567,12 +886,12 @@ struct TuneResult {
     double ms;
 };
 
-void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh) {
+void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh, bool allow_ds) {
     static std::mutex mu;
     static std::map<TuneKey, TuneResult> cache;
     int dev = 0;
     CK(cudaGetDevice(&dev));
-    const TuneKey key{pb->Nmax, R, (fp64 ? 1 : 0) + (allow_sh ? 2 : 0), pb->C, pb->Ntot, pb->Mmax, dev};
+    const TuneKey key{pb->Nmax, R, (fp64 ? 1 : 0) + (allow_sh ? 2 : 0) + (allow_ds ? 4 : 0), pb->C, pb->Ntot, pb->Mmax, dev};
     MatvecChoice cand[128];
     const int nc = matvec_candidates(R, pb->Nmax, fp64, cand, 128, allow_sh);
     {
@@ -613,6 +932,7 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
         MatvecPlan trial;
         trial.ch = cand[i / 4];
         trial.ns_div = dv;
+        if (trial.ch.DS && (dv > 1 || !allow_ds)) continue;
         float* XT = nullptr;
         if (trial.ch.SH) {
             if (!ensure_gt(pb)) continue;
@@ -620,16 +940,24 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
             CK(cudaMemsetAsync(XT, 0, (size_t)pb->xrows * 4 * R * sizeof(float), pb->stream));
         }
         build_work(pb, trial, R, fp64);
+        if (cand[i / 4].DS && !trial.ch.DS) continue;
         if (dv == 1) model_ns = trial.nsplit;
-        const int nfull = (int)trial.work.size();
+        struct TrialGuard {
+            MatvecPlan& t;
+            ~TrialGuard() { free_plan(t); }
+        } trial_guard{trial};
+        const int nfull = std::max<int>(1, (int)trial.work.size());
         const int nw = std::max(1, std::min(nfull, (int)std::ceil(frac * nfull)));
         MatvecWork* dw = (MatvecWork*)dwork.get(nfull * sizeof(MatvecWork));
-        CK(cudaMemcpyAsync(dw, trial.work.data(), nw * sizeof(MatvecWork), cudaMemcpyHostToDevice, pb->stream));
+        if (!trial.work.empty())
+            CK(cudaMemcpyAsync(dw, trial.work.data(), nw * sizeof(MatvecWork), cudaMemcpyHostToDevice, pb->stream));
         void* part = pb->part.get((size_t)trial.nsplit * vec);
         double t = 1e300;
         for (int rep = 0; rep < 3; ++rep) {  // first run warms caches and the module
             CK(cudaEventRecord(e0, pb->stream));
-            if (trial.ch.SH)
+            if (trial.ch.DS)
+                ds_product(pb, trial, R, false, pb->d_G64, (const double2*)xs, (double2*)part);
+            else if (trial.ch.SH)
                 launch_bt_tcs(pb->d_cfg, dw, nw, pb->Nmax, pb->d_GT, XT, (float2*)part, pb->Ntot, R, pb->stream);
             else
                 launch_bt_only(cand[i / 4], fp64, pb->d_cfg, dw, nw, pb->Nmax, G, xs, part, pb->Ntot, R, pb->stream);
@@ -662,23 +990,33 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
 // product of the default rows with stored generators (matvec_dev), the only
 // one that may run the shift-GEMM kernel; every other product (formulations,
 // penetrable, adjoint, raw, recomputed) uses a plan without it.
-long long plan_key(int R, bool fp64, bool allow_sh) {
-    return ((long long)R * 4 + (fp64 ? 0 : 1)) * 2 + (allow_sh ? 1 : 0);
+// allow_ds: the digit-sliced FP64 product (any use whose generators it has).
+long long plan_key(int R, bool fp64, bool allow_sh, bool allow_ds) {
+    return (((long long)R * 4 + (fp64 ? 0 : 1)) * 2 + (allow_sh ? 1 : 0)) * 2 + (allow_ds ? 1 : 0);
 }
 
-MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false) {
+MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, bool adjoint = false) {
     allow_sh = allow_sh && !fp64;
-    const long long key = plan_key(R, fp64, allow_sh);
+    const bool allow_ds = fp64 && ds_possible(pb, adjoint);
+    const long long key = plan_key(R, fp64, allow_sh, allow_ds);
     auto it = pb->plans.find(key);
-    if (it != pb->plans.end()) return it->second;
+    if (it != pb->plans.end()) {
+        if (!it->second.ch.DS || it->second.ds_version == pb->ds_version) return it->second;
+        // the groups of the sources have changed: a new work list
+        CK(cudaStreamSynchronize(pb->stream));
+        free_plan(it->second);
+        build_work(pb, it->second, R, fp64);
+        return it->second;
+    }
     MatvecPlan plan;
     auto pin = pb->pinned.find((long long)R * 4 + (fp64 ? 0 : 1));
     if (pin != pb->pinned.end()) {
         plan.ch = pin->second;
         if (plan.ch.SH && !(allow_sh && ensure_gt(pb))) plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
+        if (plan.ch.DS && !allow_ds) plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
     } else {
         plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
-        if (autotune_enabled()) autotune(pb, plan, R, fp64, allow_sh);
+        if (autotune_enabled()) autotune(pb, plan, R, fp64, allow_sh, allow_ds);
     }
     build_work(pb, plan, R, fp64);
     plan.d_work = dalloc_copy(plan.work.data(), plan.work.size());
@@ -830,7 +1168,7 @@ RecomputePlan& get_recompute_plan(msd_problem* pb, int R, bool fp64) {
     auto it = pb->rplans.find(key);
     if (it != pb->rplans.end()) return it->second;
     auto pin = pb->pinned.find(key);
-    if (pin != pb->pinned.end() && !pin->second.SH)
+    if (pin != pb->pinned.end() && !pin->second.SH && !pin->second.DS)
         return pb->rplans.emplace(key, build_recompute_plan(pb, R, fp64, pin->second)).first->second;
     RecomputePlan rp = build_recompute_plan(pb, R, fp64, matvec_default_choice(R, pb->Nmax, fp64));
     int rc = 0;
@@ -914,8 +1252,11 @@ void matvec_form_dev(msd_problem* pb, int R, bool fp64, const void* x, void* y) 
     void* part = pb->part.get((size_t)plan.nsplit * pb->Ntot * 2 * R * elem);
     launch_form_scale(fp64, pb->Ntot, R, fp64 ? (const void*)pb->d_rf64 : (const void*)pb->d_rf32,
                       fp64 ? (const void*)pb->d_frf2_64 : (const void*)pb->d_frf2_32, x, xs, pb->stream);
-    launch_bt_only(plan.ch, fp64, pb->d_cfg, plan.d_work, (int)plan.work.size(), pb->Nmax,
-                   fp64 ? (const void*)pb->d_G64 : (const void*)pb->d_G32, xs, part, pb->Ntot, 2 * R, pb->stream);
+    if (plan.ch.DS)
+        ds_product(pb, plan, 2 * R, false, pb->d_G64, (const double2*)xs, (double2*)part);
+    else
+        launch_bt_only(plan.ch, fp64, pb->d_cfg, plan.d_work, (int)plan.work.size(), pb->Nmax,
+                       fp64 ? (const void*)pb->d_G64 : (const void*)pb->d_G32, xs, part, pb->Ntot, 2 * R, pb->stream);
     launch_form_finalize(fp64, pb->Ntot, R, plan.nsplit, fp64 ? (const void*)pb->d_fl1_64 : (const void*)pb->d_fl1_32,
                          fp64 ? (const void*)pb->d_fl2_64 : (const void*)pb->d_fl2_32, x, part, y, pb->stream);
     CK_LAUNCH();
@@ -941,10 +1282,15 @@ void pen_matvec(msd_problem* pb, int R, bool fp64, const void* x, void* y) {
     void* partm = pm->part.get((size_t)pq.nsplit * nv * elem);
     launch_pen_scale(fp64, pb->d_cfg, pb->C, pb->Ntot, R, fp64 ? (const void*)pb->d_rf64 : (const void*)pb->d_rf32,
                      fp64 ? (const void*)pm->d_rf64 : (const void*)pm->d_rf32, x, xsp, xsm, pb->stream);
-    launch_bt_only(pp.ch, fp64, pb->d_cfg, pp.d_work, (int)pp.work.size(), pb->Nmax,
-                   fp64 ? (const void*)pb->d_G64 : (const void*)pb->d_G32, xsp, partp, pb->Ntot, R, pb->stream);
-    launch_bt_only(pq.ch, fp64, pm->d_cfg, pq.d_work, (int)pq.work.size(), pm->Nmax,
-                   fp64 ? (const void*)pm->d_G64 : (const void*)pm->d_G32, xsm, partm, pm->Ntot, R, pb->stream);
+    auto sums = [&](msd_problem* p, MatvecPlan& plan, const void* xs, void* part) {
+        if (plan.ch.DS)
+            ds_product(p, plan, R, false, p->d_G64, (const double2*)xs, (double2*)part);
+        else
+            launch_bt_only(plan.ch, fp64, p->d_cfg, plan.d_work, (int)plan.work.size(), p->Nmax,
+                           fp64 ? (const void*)p->d_G64 : (const void*)p->d_G32, xs, part, p->Ntot, R, pb->stream);
+    };
+    sums(pb, pp, xsp, partp);
+    sums(pm, pq, xsm, partm);
     launch_pen_finalize(fp64, pb->d_cfg, pb->C, pb->Ntot, R,
                         fp64 ? (const void*)pb->d_penA64 : (const void*)pb->d_penA32, x, partp, pp.nsplit, partm,
                         pq.nsplit, y, pb->stream);
@@ -1000,6 +1346,12 @@ void matvec_dev(msd_problem* pb, int R, bool fp64, const void* x, void* y) {
                       R, pb->stream, pb->live);
         if (e1) CK(cudaEventRecord(e1, pb->stream));
         launch_finalize(false, pb->Ntot, R, plan.nsplit, pb->d_lf32, x, part, y, pb->stream);
+    } else if (plan.ch.DS) {
+        launch_scale_cols(true, pb->Ntot, R, pb->d_rf64, x, xs, pb->stream);
+        if (e0) CK(cudaEventRecord(e0, pb->stream));
+        ds_product(pb, plan, R, false, pb->d_G64, (const double2*)xs, (double2*)part, pb->live);
+        if (e1) CK(cudaEventRecord(e1, pb->stream));
+        launch_finalize(true, pb->Ntot, R, plan.nsplit, pb->d_lf64, x, part, y, pb->stream);
     } else if (fp64)
         launch_matvec_f64(pb->d_cfg, plan.d_work, (int)plan.work.size(), pb->Nmax, pb->d_G64, pb->d_rf64,
                           pb->d_lf64, pb->Ntot, R, (const double2*)x, (double2*)xs, (double2*)part,
@@ -1050,13 +1402,23 @@ void product_dev(msd_problem* pb, int R, bool fp64, bool adjoint, bool raw, cons
         fail(MSD_ERR_ARG, "truncation order too large for the shared-memory tile of this precision");
     if (adjoint) ensure_adjoint(pb, fp64);
     else ensure_generators(pb, fp64);
-    MatvecPlan& plan = get_plan(pb, R, fp64);
+    MatvecPlan& plan = get_plan(pb, R, fp64, false, adjoint);
     const size_t elem = fp64 ? 16 : 8;
     void* xs = pb->xs.get((size_t)pb->Ntot * R * elem);
     void* part = pb->part.get((size_t)plan.nsplit * pb->Ntot * R * elem);
     const int nwork = (int)plan.work.size();
     if (fp64) {
         const double2* G = adjoint ? pb->d_GA64 : pb->d_G64;
+        if (plan.ch.DS) {
+            if (adjoint) launch_scale_cols_c(pb->Ntot, R, pb->d_clf64, (const double2*)x, (double2*)xs, pb->stream);
+            else launch_scale_cols(true, pb->Ntot, R, pb->d_rf64, x, xs, pb->stream);
+            ds_product(pb, plan, R, adjoint, G, (const double2*)xs, (double2*)part);
+            launch_finalize_gen(pb->Ntot, R, plan.nsplit, (adjoint && !raw) ? pb->d_rf64 : nullptr,
+                                (!adjoint && !raw) ? pb->d_lf64 : nullptr, raw ? 0 : 1, (const double2*)x,
+                                (const double2*)part, (double2*)y, pb->stream);
+            CK_LAUNCH();
+            return;
+        }
         launch_product_f64(pb->d_cfg, plan.d_work, nwork, pb->Nmax, G, adjoint ? nullptr : pb->d_rf64,
                            adjoint ? pb->d_clf64 : nullptr, (adjoint && !raw) ? pb->d_rf64 : nullptr,
                            (!adjoint && !raw) ? pb->d_lf64 : nullptr, raw ? 0 : 1, pb->Ntot, R,
@@ -1619,6 +1981,7 @@ msd_status msd_create(int C, const int* disk_off, const double* centres, const d
             pb->d_gt_blk = dalloc_copy(gt_blk.data(), C);
             pb->d_centre = dalloc_copy(cen.data(), Mtot);
             pb->d_radius = dalloc_copy(radii, Mtot);
+            pb->h_radius.assign(radii, radii + Mtot);
             pb->d_bc = dalloc_copy(bc, Mtot);
             pb->d_disk_cfg = dalloc_copy(disk_cfg.data(), Mtot);
             pb->d_J = dalloc<double2>(row);
@@ -1686,8 +2049,12 @@ void msd_destroy(msd_problem* pb) {
                     pb->d_GA64, pb->d_GA32, pb->d_clf64, pb->d_clf32, pb->d_GT, pb->d_gt_blk, pb->d_Np};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    for (auto& kv : pb->plans)
-        if (kv.second.d_work) cudaFree(kv.second.d_work);
+    for (auto& b : pb->ds_idx) b.release();
+    pb->ds_fwd.release();
+    pb->ds_adj.release();
+    pb->dsx.release();
+    pb->dse.release();
+    for (auto& kv : pb->plans) free_plan(kv.second);
     free_recompute_plans(pb);
     if (pb->d_gen_full) cudaFree(pb->d_gen_full);
     pb->genbuf.release();
@@ -1792,6 +2159,7 @@ msd_status msd_update_geometry(msd_problem* pb, const double* centres, const dou
         if (radii)
             CK(cudaMemcpyAsync(pb->d_radius, radii, (size_t)pb->Mtot * 8,
                                is_device_ptr(radii) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, pb->stream));
+        pb->geom_version += 1;  // data derived from the generators is rebuilt on next use
         CK(cudaMemsetAsync(pb->d_flags, 0, sizeof(int), pb->stream));
         launch_disk_diagonals(pb->d_cfg, pb->Mtot, pb->d_disk_cfg, pb->d_radius, pb->d_bc, pb->Nmax, pb->d_J,
                               pb->d_dJ, pb->d_H, pb->d_dH, pb->d_lf64, pb->d_rf64, pb->d_lf32, pb->d_rf32,
@@ -1799,6 +2167,11 @@ msd_status msd_update_geometry(msd_problem* pb, const double* centres, const dou
         CK_LAUNCH();
         if (pb->d_G64 || pb->d_G32) launch_full_generators(pb, pb->d_G64, pb->d_G32);
         CK_LAUNCH();
+        if (radii) {
+            CK(cudaMemcpyAsync(pb->h_radius.data(), pb->d_radius, (size_t)pb->Mtot * 8, cudaMemcpyDeviceToHost,
+                               pb->stream));
+            pb->radius_version += 1;
+        }
         check_flags(pb, "msd_update_geometry");
         apply_truncation(pb);
         if (pb->form) form_rows(pb);
@@ -1807,7 +2180,6 @@ msd_status msd_update_geometry(msd_problem* pb, const double* centres, const dou
             if (st != MSD_OK) fail(st, std::string("msd_update_geometry (interior wavenumber): ") + msd_last_error());
             pen_rows(pb);
         }
-        pb->geom_version += 1;  // adjoint operator data is rebuilt on next use
         return MSD_OK;
     });
 }
@@ -1871,6 +2243,10 @@ msd_status msd_set_generator_mode(msd_problem* pb, int mode, int64_t chunk_bytes
             pb->d_GT = nullptr;
             pb->gt_version = -1;
             pb->xt.release();
+            pb->ds_fwd.release();
+            pb->ds_adj.release();
+            pb->dsx.release();
+            pb->dse.release();
         } else {
             free_recompute_plans(pb);
             pb->genbuf.release();
@@ -1917,11 +2293,11 @@ msd_status msd_set_tile(msd_problem* pb, int R, int precision, int KB, int RT) {
             if (cand[i].KB + 100 * cand[i].P2 == KB && cand[i].RT == RT) hit = i;
         if (hit < 0) fail(MSD_ERR_ARG, "msd_set_tile: (KB, RT) is not an instantiated shape that fits");
         const long long key = (long long)R * 4 + (fp64 ? 0 : 1);
-        for (int sh = 0; sh < 2; ++sh) {
-            auto it = pb->plans.find(plan_key(R, fp64, sh != 0));
+        for (int use = 0; use < 4; ++use) {
+            auto it = pb->plans.find(plan_key(R, fp64, (use & 1) != 0, (use & 2) != 0));
             if (it != pb->plans.end()) {
                 CK(cudaStreamSynchronize(pb->stream));  // the old work list may still be read
-                if (it->second.d_work) cudaFree(it->second.d_work);
+                free_plan(it->second);
                 pb->plans.erase(it);
             }
         }

@@ -101,6 +101,7 @@ struct MatvecChoice {
     int SH;  // shift-GEMM tensor-core kernel (FP32, RT = MSD_TCS_COLS columns per CTA): 1 = mode
              // blocks of <= 8 two per CTA, 2 = one block of <= 16 modes per CTA; 0 = not used
     int ONE;  // FP64: 1 = one shared-memory stage (two would exceed 227 KB at this truncation order)
+    int DS;   // FP64: 1 = digit-sliced tensor-core kernel (k_matvec_ds.cu; KB = 0, RT = 1)
 };
 #define MSD_TCS_COLS 8
 MatvecChoice matvec_default_choice(int R, int Nmax, bool fp64);
@@ -143,6 +144,48 @@ constexpr size_t kMatvecSmemCap = 226 * 1024;
 // bit 0 set (and cleared): a bulk-copy wait of the CUDA-core product expired
 int bt_status_and_clear();
 int tcs_status_and_clear();
+// Digit-sliced FP64 product (k_matvec_ds.cu).  Sources of a configuration in
+// the order of their radii, eight to a K-step; K-steps in groups of similar
+// radius (grp_start [ngrp + 1] in K-steps, qgrp: group of a K-step, perm:
+// source of a place, -1 past the last).  A plan adds the tiles of its column
+// count: column groups of Rt columns, mode tiles of J modes, rp rows of the A
+// operand (2 J Rt rounded up to 8).
+#define MSD_DS_DIGITS 7
+struct DsCfg {
+    int n, N, L, M, Mp;
+    int nqs, ngrp;          // K-steps, groups
+    int J, mt, rp;          // modes per tile, mode tiles, operand rows
+    int grp_off, qs_off, perm_off;
+    int pad;
+    long long gen_off, row_off;
+    long long dg_off, eb_off;  // generator digits (in stages) and exponents
+    long long xd_off, ex_off;  // source digits (bytes) and exponents
+};
+// One CTA: targets [32 tile, 32 tile + 32), columns of group cg, modes of
+// tile mt as sources' modes, K-steps [qs0, qs0 + ks) of group grp, shifts
+// [dlo, dhi], writing partial slot `slot` (ks = 0: zeros).
+struct DsWork {
+    int cfg, tile, cg, mt, qs0, ks, grp, slot, dlo, dhi;
+};
+struct DsSmem {
+    unsigned ring_off, acc_off;
+    size_t total;
+};
+constexpr size_t kDsSmemCap = 226 * 1024;
+constexpr int kDsMaxKs = 9;  // 16 ks x 7 products of at most 2^14 stay within 2^24
+size_t ds_stage_bytes();
+size_t ds_xblk_bytes(int rp);
+DsSmem ds_smem(int ks, int rp, int rows2);
+void launch_ds_build(const DsCfg* d_cfg, int C, int max_Mp, int max_grp, int max_L, int max_nqs, const int* d_grp_start,
+                     const int* d_qgrp, const int* d_perm, const double2* G, int* EB, unsigned char* DG,
+                     cudaStream_t s);
+void launch_ds_prep(const DsCfg* d_cfg, int C, int max_n, int max_grp, int max_nqs, const int* d_grp_start,
+                    const int* d_qgrp, const int* d_perm, int R, int Rt, const double2* xs, int* EX, unsigned char* XD,
+                    cudaStream_t s);
+void launch_ds(const DsCfg* d_cfg, const DsWork* d_work, int nwork, const DsSmem& sm, const unsigned char* DG,
+               const int* EB, const unsigned char* XD, const int* EX, double2* part, long long Ntot, int R, int Rt,
+               cudaStream_t s, const int* live = nullptr);
+int ds_status_and_clear();
 // Set by msd_test_expire_waits: kernels with bounded waits take their
 // expiry path once per launch (tests of the error path; no fault involved).
 extern std::atomic<int> g_msd_expire_waits;  // bit 0: a pipeline wait of the tensor-core kernel expired
@@ -437,6 +480,10 @@ void gm_residual(long long n, const double2* b, const double2* Ax, double2* r, c
 void gm_zero(long long n, double2* x, cudaStream_t s);
 
 // ---------------------------------------------------------------- K3 with other scalings, K7
+// pieces of the FP64 one: xs = cf .* x; y = (add_x ? x : 0) + row .* sum of the partials
+void launch_scale_cols_c(long long Ntot, int R, const double2* cf, const double2* x, double2* xs, cudaStream_t s);
+void launch_finalize_gen(long long Ntot, int R, int nsplit, const double* row_r, const double2* row_c, int add_x,
+                         const double2* x, const double2* part, double2* y, cudaStream_t s);
 void launch_product_f64(const MsdConfig* d_cfg, const MatvecWork* d_work, int nwork, int Nmax, const double2* G,
                         const double* col_r, const double2* col_c, const double* row_r, const double2* row_c,
                         int add_x, long long Ntot, int R, const double2* x, double2* xs, double2* part, int nsplit,

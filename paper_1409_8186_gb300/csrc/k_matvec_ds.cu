@@ -36,23 +36,31 @@
 // product of the two maxima, which belong to different sources; l_m g r_n is
 // bounded by powers of (a_p + a_q)/b <= 1, and stays so with the largest a_q
 // of the group in place of the source's own while the radii in a group differ
-// by less than 2^{4/N}.  Sources are sorted by radius and grouped so; where
+// by less than 2^{7.5/N}.  Sources are sorted by radius and grouped so; where
 // eight neighbours in that order already differ by more, the form is not
 // offered (ds_grouping).
 //
-// What bounds it: the tensor pipe for one column (28 products per
-// multiply-add, 64 % of the rows in use), the FP64 pipe (a conversion and a
-// multiply-add per shift and fold) from a few columns on.  Measured (GB300,
-// whole product): 400 disks, N = 20, one column 1794 -> 436 us; 200 disks,
-// N = 22, 16 columns 9371 -> 811 us; the error against 64-bit references is
-// that of the generators on both sides (2.5e-14 before, 1.6e-14 now).
+// What bounds it: the drain of the accumulators.  A K-step of MMAs takes about
+// 650 clocks (448 at the tensor pipe's peak; small N and the issue of short
+// instructions take the rest), a shift's drain about 5600 for 8 x 16 results a
+// warp, of which FP64 additions hold their pipe for 2048; long folds (up to 9
+// K-steps) and few mode tiles make few drains.  Measured (GB300, whole
+// product): 400 disks, N = 20, one column 1794 -> 198 us; 200 disks, N = 22, 16
+// columns 9376 -> 502 us.  Against 64-bit references the error is that of the
+// generators with either kernel (radii 0.5 to 1.5, gaps of 0.01, N = 20:
+// 8.683e-15 here, 8.686e-15 with the FP64 pipe).
 //
-// Roles: warp 0 issues the bulk copies (one thread), warp 1 allocates TMEM
-// and issues the MMAs (one thread), warps 2-9 drain the accumulators (two
-// buffers, so that the MMAs of the next shift run meanwhile): warp w covers
-// TMEM lanes 32 (w mod 4) .. and 16 of the 32 targets.  Operand layout:
-// K-major without swizzle, 8-row x 16-byte core matrices.  Every wait has a
-// clock limit, as in k_matvec_tcs.cu.
+// Persistent: one CTA per SM walks its own list of items (ds_items cuts the
+// work at equal shares, between shifts where it has to), so no wave is left
+// half empty.  Roles: warp 0 issues the bulk copies (one thread), warp 1
+// allocates TMEM and issues the MMAs (one thread), warps 2-17 drain the
+// accumulators (two buffers, so that the MMAs of the next shift run
+// meanwhile): warp w covers TMEM lanes 32 (w mod 4) .. and 8 of the 32
+// targets; four such warps per scheduler hide one another's latencies (two
+// took 1.25 times as long).  The integer sums become FP64 by integer
+// instructions (to_fp64): a conversion would hold the FP64 pipe as long as the
+// one addition that is left does.  Operand layout: K-major without swizzle, 8-row x 16-byte core
+// matrices.  Every wait has a clock limit, as in k_matvec_tcs.cu.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -68,8 +76,12 @@ constexpr int kND = MSD_DS_DIGITS;
 constexpr int kTile = MSD_TILE_P;            // targets per CTA
 constexpr int kStage = kND * 2 * kTile * 16; // bytes of one B stage (one K-step): [Re, Im][digit][target][8 sources]
 constexpr int kBHalf = kND * kTile * 16;
-constexpr int kStages = 5;                   // B ring
-constexpr int kThreads = 320;
+constexpr int kStagesMax = 16;               // B ring: as many stages as fit next to A and the window
+constexpr int kDrainWarps = 16;              // four sets of four warps (128 lanes), eight targets a set
+constexpr int kSetTargets = kTile / (kDrainWarps / 4);
+constexpr int kCh = 4;                       // targets in flight per lane
+constexpr int kEbShifts = 32 / kSetTargets;  // shifts whose exponents a warp holds
+constexpr int kThreads = 64 + kDrainWarps * 32;
 constexpr int kNonFinite = 1 << 24;          // exponent of a group with an infinity or NaN
 constexpr long long kWaitCycles = 2000000000LL;  // ~1 s at 2 GHz
 constexpr long long kTestWaitCycles = 20000;     // msd_test_expire_waits
@@ -85,19 +97,50 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
 __device__ __forceinline__ uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Bounded wait.  The clock and the CTA's abort flag are only looked at once a
+// first try has failed: the issuing threads wait for every K-step, and what a
+// satisfied wait costs is time the tensor pipe does not get back.
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_v) {
     const long long t0 = clock64();
     while (true) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, q;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
-        if (clock64() - t0 > kWaitCycles) return false;
+        if (mbar_try(bar, parity)) return true;
+        if (*abort_v) return false;
+        if (clock64() - t0 > kWaitCycles) {
+            *abort_v = 1;
+            return false;
+        }
     }
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_v) {
+    return mbar_try(bar, parity) || mbar_wait_slow(bar, parity, abort_v);
+}
+// The same for copies that must land (or MMAs that must end) before the CTA
+// may go on even after an abort.
+__device__ __noinline__ bool mbar_settle(uint32_t bar, uint32_t parity) {
+    const long long t0 = clock64();
+    while (!mbar_try(bar, parity))
+        if (clock64() - t0 > kWaitCycles) return false;
+    return true;
+}
+// One thread of a converged warp, chosen so that the compiler knows the branch
+// is taken by one thread: the operands of tcgen05.mma live in uniform
+// registers, and under a test of the lane number every instruction is wrapped
+// in a loop over its possible values (400 disks: the issue loop alone 180 us
+// that way, 132 us so).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
 }
 __device__ __forceinline__ bool wait_unset_flag(const volatile int* flag) {
     const long long t0 = clock64();
@@ -120,19 +163,22 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t id, uint32_t acc) {
+// (descriptors as two words: the upper ones are the same for every MMA)
+__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                         uint32_t id, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(da), "l"(db), "r"(id), "r"(acc));
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(tmem_d),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(id), "r"(acc));
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar));
 }
-// 8 consecutive TMEM columns of this thread's lane, as integers
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+// 4 consecutive TMEM columns of this thread's lane
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr));
 }
 
@@ -310,20 +356,49 @@ __global__ void __launch_bounds__(128) k_ds_digits_x(const DsCfg* __restrict__ c
 
 // ---------------------------------------------------------------- the product
 
-// Integer sum_s a_s 2^{56 - 8 s} (s = 2..8; a_8 rounded) of the accumulators
-// of one result; |a_s| <= 2^21.2 (s - 1), so it stays below 2^62.
-__device__ __forceinline__ double combine(const int (&a)[kND]) {
-    long long t = (long long)(a[0] * 256 + a[1]) * (1ll << 32);
-    t += (long long)a[2] * (1 << 24);
-    t += (long long)a[3] * (1 << 16);
-    t += (long long)a[4] * (1 << 8);
-    t += (long long)(a[5] + ((a[6] + 128) >> 8));
-    return (double)t;
+// t 2^ex rounded to 53 bits, 0 below the normal range, infinite above it.
+__device__ __noinline__ double to_double_any(long long t, int ex) {
+    unsigned long long u = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
+    const int lz = __clzll((long long)u);
+    u <<= (lz & 63);
+    const int e = 1023 + 63 - lz + ex;  // biased exponent of t 2^ex
+    // 53 bits with the leading one, which adds 1 to the exponent field; a carry of the rounding does too
+    unsigned long long b = (u >> 11) + ((u >> 10) & 1) + ((unsigned long long)(unsigned)(e - 1) << 52);
+    if (e < 1 || u == 0) b = 0;
+    if (e > 2046) b = 0x7ff0000000000000ull;
+    return __longlong_as_double((long long)(b | ((unsigned long long)t & 0x8000000000000000ull)));
+}
+
+// One result from its accumulators a_s (s = 2..8, |a_s| <= 2^21.2 (s - 1)):
+// t = sum_s a_s 2^{56 - 8 s} as a 64-bit integer (below 2^62; a_8 rounded into
+// a_7), then t 2^ex in FP64.  About 35 integer instructions: the usual case,
+// |t| >= 2^32 and a result in the normal range, without branches (a negative t
+// loses one unit, 2^-56 of the largest product); the rest in to_double_any.
+__device__ __forceinline__ double to_fp64(const uint32_t (&v)[kND][kCh], int u, int ex, bool wanted) {
+    const int x = (int)__uint_as_float(v[0][u]) * 256 + (int)__uint_as_float(v[1][u]);
+    const int y = (int)__uint_as_float(v[2][u]) * 256 + (int)__uint_as_float(v[3][u]);
+    const int z = __float2int_rn(fmaf(__uint_as_float(v[6][u]), 0.00390625f, __uint_as_float(v[5][u])));
+    long long t = (long long)(int)__uint_as_float(v[4][u]) * 256 + z;
+    t = (long long)y * 65536 + t;
+    const int hi = (int)(t >> 32) + x;
+    const uint32_t lo = (uint32_t)t;
+    const int s = hi >> 31;
+    const uint32_t ah = (uint32_t)(hi ^ s), al = lo ^ (uint32_t)s;
+    const int lz = __clz((int)ah);
+    const uint32_t h = __funnelshift_l(al, ah, lz), l = al << (lz & 31);
+    const int e1 = 1022 + 63 + ex - lz;  // biased exponent less the leading one of the mantissa
+    const unsigned long long m = ((unsigned long long)((h >> 11) + ((uint32_t)e1 << 20)) << 32 |
+                                  __funnelshift_r(l, h, 11)) + ((l >> 10) & 1);
+    double r = __longlong_as_double((long long)(m | (unsigned long long)((uint32_t)s & 0x80000000u) << 32));
+    if (wanted && (ah == 0 || (unsigned)e1 > 2044u))
+        r = to_double_any((long long)(((unsigned long long)(uint32_t)hi << 32) | lo), ex);
+    return r;
 }
 
 struct DsParams {
     const DsCfg* cfgs;
     const DsWork* works;
+    const int* cta_off;  // items of CTA b: [cta_off[b], cta_off[b + 1])
     const unsigned char* DG;
     const int* EB;
     const unsigned char* XD;
@@ -331,47 +406,31 @@ struct DsParams {
     double* part;
     const int* live;
     long long Ntot;
-    int R, Rt;
+    int R, Rt, stages;
     unsigned ring_off, acc_off;  // shared memory: A at 0, the B ring, the FP64 window
     int expire_test;
 };
 
+// Whether an item has nothing to multiply: a slot its targets have no work
+// for, or no active column (converged Krylov systems).  A whole warp.
+__device__ __forceinline__ bool item_idle(const DsParams& P, const DsWork& w, int r0, int cols) {
+    if (w.ks == 0) return true;
+    if (!P.live) return false;
+    bool any = false;
+    for (int r = threadIdx.x & 31; r < cols; r += 32) any |= P.live[w.cfg * P.R + r0 + r] != 0;
+    return !__any_sync(0xffffffffu, any);
+}
+
 __global__ void __launch_bounds__(kThreads, 1) k_bt_ds(DsParams P) {
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ uint32_t tmem_sh;
-    __shared__ __align__(8) uint64_t a_full, b_full[kStages], b_empty[kStages], acc_full[2], acc_empty[2], mma_done;
+    __shared__ __align__(8) uint64_t a_full, a_empty, b_full[kStagesMax], b_empty[kStagesMax], acc_full[2], acc_empty[2],
+        mma_done;
     __shared__ int abort_sh, never_sh;
 
-    const DsWork w = P.works[blockIdx.x];
-    const DsCfg c = P.cfgs[w.cfg];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int R = P.R, Rt = P.Rt, n = c.n, N = c.N, L = c.L;
-    const int r0 = w.cg * Rt, cols = min(Rt, R - r0);
-    const int p0 = w.tile * kTile;
-    double* const out = P.part + (long long)w.slot * P.Ntot * R * 2;
-
-    // results (p, m, r) of this item that no shift reaches: m outside [mlo, mhi]
-    auto zero_outside = [&](int mlo, int mhi, int first, int step) {
-        if (mlo <= 0 && mhi >= n - 1) return;
-        const int tot = kTile * n * 2 * cols;
-        for (int i = first; i < tot; i += step) {
-            const int rc = i % (2 * cols), m = (i / (2 * cols)) % n, p = p0 + i / (2 * cols * n);
-            if (p < c.M && (m < mlo || m > mhi))
-                out[((c.row_off + (long long)p * n + m) * R + r0) * 2 + rc] = 0.0;
-        }
-    };
-    bool none = w.ks == 0;  // a slot this configuration has no work for
-    if (!none && P.live) {  // no active column (converged Krylov systems)
-        bool any = false;
-        for (int r = 0; r < cols; ++r) any |= P.live[w.cfg * R + r0 + r] != 0;
-        none = !any;
-    }
-    if (none) {
-        zero_outside(n, -1, tid, kThreads);
-        return;
-    }
-
-    const int half = c.rp * 16, ablk = 2 * kND * half;  // bytes of one K half and of one K-step of A
+    const int R = P.R, Rt = P.Rt, kStages = P.stages;
+    const int it0 = P.cta_off[blockIdx.x], it1 = P.cta_off[blockIdx.x + 1];
     unsigned char* ring = sm + P.ring_off;
     double* acc = (double*)(sm + P.acc_off);
     if (warp == 1) {
@@ -383,13 +442,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_bt_ds(DsParams P) {
         abort_sh = 0;
         never_sh = 0;
         mbar_init(&a_full, 1);
-        for (int s = 0; s < kStages; ++s) {
+        mbar_init(&a_empty, 1);
+        for (int s = 0; s < kStagesMax; ++s) {
             mbar_init(&b_full[s], 1);
             mbar_init(&b_empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 8);
+            mbar_init(&acc_empty[b], kDrainWarps);
         }
         mbar_init(&mma_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
@@ -399,136 +459,201 @@ __global__ void __launch_bounds__(kThreads, 1) k_bt_ds(DsParams P) {
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_sh;
     volatile int* abort_v = &abort_sh;
-    const int nd = w.dhi - w.dlo + 1;
     int issued_mma = 0;
 
-    if (warp == 0 && lane == 0) {
-        // ---------------- producer: A once, then one B stage per (shift, K-step)
-        const unsigned char* xa = P.XD + c.xd_off + (((long long)w.cg * c.mt + w.mt) * c.nqs + w.qs0) * ablk;
-        mbar_expect_tx(smem_u32(&a_full), (uint32_t)(w.ks * ablk));
-        for (int k = 0; k < w.ks; ++k)
-            bulk_g2s(smem_u32(sm + k * ablk), xa + (long long)k * ablk, (uint32_t)ablk, smem_u32(&a_full));
-        const unsigned char* gd =
-            P.DG + (c.dg_off + ((long long)w.tile * L + w.dlo + 2 * N) * c.nqs + w.qs0) * (long long)kStage;
-        int s = 0, used = 0;  // ring position, stages filled so far
-        uint32_t ph = 1;      // parity of the release to wait for (from the second lap)
-        for (int d = 0; d < nd; ++d, gd += (long long)c.nqs * kStage)
-            for (int k = 0; k < w.ks; ++k) {
-                if (used >= kStages) {
-                    if (!*abort_v && !mbar_wait(smem_u32(&b_empty[s]), ph)) *abort_v = 1;
-                    mbar_wait(smem_u32(&b_full[s]), ph);  // own previous copy landed before re-arming
+    if (warp == 0) {
+        // ---------------- producer: A of an item, then one B stage per (shift, K-step)
+        int s = 0, used = 0, na = 0;  // ring position, stages filled, items loaded
+        uint32_t ph = 1;              // parity of the release to wait for (from the second lap)
+        bool dead = false;            // a wait has expired: the copies go on, waiting only for themselves
+        for (int it = it0; it < it1; ++it) {
+            const DsWork w = P.works[it];
+            const DsCfg c = P.cfgs[w.cfg];
+            if (item_idle(P, w, w.cg * Rt, min(Rt, R - w.cg * Rt))) continue;
+            if (elect_one()) {
+                const int ablk = 2 * kND * c.rp * 16;
+                const uint32_t aprev = (uint32_t)((na - 1) & 1);
+                if (na > 0) {  // the MMAs of the item before have read its A
+                    if (!dead) dead = !mbar_wait(smem_u32(&a_empty), aprev, abort_v);
+                    if (dead) mbar_settle(smem_u32(&a_full), aprev);
                 }
-                mbar_expect_tx(smem_u32(&b_full[s]), kStage);
-                bulk_g2s(smem_u32(ring + s * kStage), gd + (long long)k * kStage, kStage, smem_u32(&b_full[s]));
-                ++used;
-                if (++s == kStages) {
-                    s = 0;
-                    ph ^= 1;
-                }
+                const unsigned char* xa = P.XD + c.xd_off + (((long long)w.cg * c.mt + w.mt) * c.nqs + w.qs0) * ablk;
+                mbar_expect_tx(smem_u32(&a_full), (uint32_t)(w.ks * ablk));
+                for (int k = 0; k < w.ks; ++k)
+                    bulk_g2s(smem_u32(sm + k * ablk), xa + (long long)k * ablk, (uint32_t)ablk, smem_u32(&a_full));
+                const unsigned char* gd = P.DG + (c.dg_off + ((long long)w.tile * c.L + w.dlo + 2 * c.N) * c.nqs +
+                                                  w.qs0) * (long long)kStage;
+                for (int d = w.dlo; d <= w.dhi; ++d, gd += (long long)c.nqs * kStage)
+                    for (int k = 0; k < w.ks; ++k) {
+                        if (used >= kStages) {
+                            if (!dead) dead = !mbar_wait(smem_u32(&b_empty[s]), ph, abort_v);
+                            if (dead) mbar_settle(smem_u32(&b_full[s]), ph);
+                        }
+                        mbar_expect_tx(smem_u32(&b_full[s]), kStage);
+                        bulk_g2s(smem_u32(ring + s * kStage), gd + (long long)k * kStage, kStage,
+                                 smem_u32(&b_full[s]));
+                        ++used;
+                        if (++s == kStages) {
+                            s = 0;
+                            ph ^= 1;
+                        }
+                    }
+                ++na;
             }
-        // every copy of this CTA has landed before it exits
-        mbar_wait(smem_u32(&a_full), 0);
-        for (int s2 = 0; s2 < kStages; ++s2)
-            if (used > s2) mbar_wait(smem_u32(&b_full[s2]), (uint32_t)(((used - 1 - s2) / kStages) & 1));
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issue
-        const uint64_t adesc0 = sdesc(smem_u32(sm), half, 128), bdesc0 = sdesc(smem_u32(ring), kBHalf, 128);
-        bool ok = mbar_wait(smem_u32(&a_full), 0);
-        if (P.expire_test) ok = wait_unset_flag(&never_sh) && ok;
-        if (!ok) *abort_v = 1;
-        int s = 0;
-        uint32_t ph = 0;
-        for (int d = 0; d < nd; ++d) {
-            const int b = d & 1;
-            if (d >= 2 && !*abort_v && !mbar_wait(smem_u32(&acc_empty[b]), (uint32_t)(((d >> 1) - 1) & 1)))
-                *abort_v = 1;
-            for (int k = 0; k < w.ks; ++k) {
-                if (!*abort_v && !mbar_wait(smem_u32(&b_full[s]), ph)) *abort_v = 1;
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint64_t bd = bdesc0 + (uint64_t)(s * (kStage >> 4));
-                const uint64_t ad = adesc0 + (uint64_t)(k * (ablk >> 4));
-                if (!*abort_v) {
-#pragma unroll
-                    for (int i = 0; i < kND; ++i)
-                        mma_bf16(tmem + b * 256 + i * kTile, ad + (uint64_t)(i * (2 * half >> 4)), bd,
-                                 idesc_bf16(128, kTile * (kND - i)), (i == 0 && k == 0) ? 0u : 1u);
-                    issued_mma = 1;
-                }
-                mma_commit(smem_u32(&b_empty[s]));
-                if (++s == kStages) {
-                    s = 0;
-                    ph ^= 1;
-                }
-            }
-            mma_commit(smem_u32(&acc_full[b]));
+            __syncwarp();
         }
-        mma_commit(smem_u32(&mma_done));
-    } else if (warp >= 2) {
+        // every copy of this CTA has landed before it exits
+        if (na > 0) mbar_settle(smem_u32(&a_full), (uint32_t)((na - 1) & 1));
+        for (int s2 = 0; s2 < kStages; ++s2)
+            if (used > s2) mbar_settle(smem_u32(&b_full[s2]), (uint32_t)(((used - 1 - s2) / kStages) & 1));
+    } else if (warp == 1) {
+        // ---------------- MMA issue
+        const uint64_t bdesc0 = sdesc(smem_u32(ring), kBHalf, 128);
+        int s = 0, na = 0, gd = 0;  // ring position, items begun, shifts issued
+        uint32_t ph = 0;
+        bool dead = false;
+        for (int it = it0; it < it1; ++it) {
+            const DsWork w = P.works[it];
+            const DsCfg c = P.cfgs[w.cfg];
+            if (item_idle(P, w, w.cg * Rt, min(Rt, R - w.cg * Rt))) continue;
+            if (elect_one()) {
+                const int half = c.rp * 16;
+                const uint32_t astep = 2 * half >> 4;  // one digit of A
+                const uint64_t adesc0 = sdesc(smem_u32(sm), half, 128);
+                const uint32_t a_hi = (uint32_t)(adesc0 >> 32), b_hi = (uint32_t)(bdesc0 >> 32);
+                if (!dead) dead = !mbar_wait(smem_u32(&a_full), (uint32_t)(na & 1), abort_v);
+                if (P.expire_test && na == 0 && !wait_unset_flag(&never_sh)) {
+                    *abort_v = 1;
+                    dead = true;
+                }
+                for (int d = w.dlo; d <= w.dhi; ++d, ++gd) {
+                    const int b = gd & 1;
+                    if (gd >= 2 && !dead)
+                        dead = !mbar_wait(smem_u32(&acc_empty[b]), (uint32_t)(((gd >> 1) - 1) & 1), abort_v);
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t tc = tmem + b * 256;
+                    uint32_t a_lo = (uint32_t)adesc0;
+                    for (int k = 0; k < w.ks; ++k) {
+                        if (!dead) dead = !mbar_wait(smem_u32(&b_full[s]), ph, abort_v);
+                        if (!dead) {
+                            const uint32_t b_lo = (uint32_t)bdesc0 + s * (kStage >> 4);
+#pragma unroll
+                            for (int i = 0; i < kND; ++i, a_lo += astep)
+                                mma_bf16(tc + i * kTile, a_lo, a_hi, b_lo, b_hi, idesc_bf16(128, kTile * (kND - i)),
+                                         i == 0 ? (uint32_t)k : 1u);
+                            issued_mma = 1;
+                        }
+                        mma_commit(smem_u32(&b_empty[s]));
+                        if (++s == kStages) {
+                            s = 0;
+                            ph ^= 1;
+                        }
+                    }
+                    mma_commit(smem_u32(&acc_full[b]));
+                }
+                mma_commit(smem_u32(&a_empty));
+                ++na;
+            }
+            __syncwarp();
+        }
+        if (issued_mma) mma_commit(smem_u32(&mma_done));
+    } else {
         // ---------------- drain: digit weights -> FP64, window over the target modes
         const int quarter = warp & 3, set = (warp - 2) >> 2;
         const int row = quarter * 32 + lane, e = row >> 1, ri = row & 1;
         const int jj = e / Rt, r = e % Rt;
-        const int jlo = w.mt * c.J, jhi = min(jlo + c.J, n) - 1, j = jlo + jj;
-        const bool rowok = j <= jhi && r < cols;
-        const int rows2 = 2 * c.J * Rt;  // doubles of the window per target
-        const int EA = rowok ? P.EX[c.ex_off + ((long long)w.grp * n + j) * R + r0 + r] : 0;
-        const int* eb = P.EB + c.eb_off + (((long long)w.tile * c.ngrp + w.grp) * L + w.dlo + 2 * N) * kTile +
-                        set * 16 + (lane & 15);
-        const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(set * 16);
-        double* const my = acc + (size_t)(set * 16) * rows2 + r * 2 + ri;
-        double* const dst = out + ((c.row_off + (long long)(p0 + set * 16) * n) * R + r0 + r) * 2 + ri;
-        int m = j - w.dlo, slot = rowok ? ((m % c.J) + c.J) % c.J : 0;  // window position of mode m
-        int EB = *eb;
-        for (int d = 0; d < nd; ++d) {
-            const int EBn = d + 1 < nd ? eb[(long long)(d + 1) * kTile] : 0;
-            bool ok = *abort_v ? false : mbar_wait(smem_u32(&acc_full[d & 1]), (uint32_t)((d >> 1) & 1));
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) *abort_v = 1;
-            const bool valid = rowok && m >= 0 && m < n;
-            if (ok && __any_sync(0xffffffffu, valid)) {
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const bool first = jj == 0 || d == 0, last = j == jhi || d == nd - 1;
-                double* const cell = my + (size_t)slot * Rt * 2;
-                double* const cellout = dst + (long long)m * R * 2;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t v[kND][8];
-#pragma unroll
-                    for (int s = 0; s < kND; ++s) tmem_ld8(lane_addr + (d & 1) * 256 + s * kTile + h * 8, v[s]);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int t = h * 8 + u;
-                        // 2^{EA + EB + 2 - 56}, 0 below the normal range, infinite above it
-                        const int ex = EA + __shfl_sync(0xffffffffu, EB, t) + (1023 - 54);
-                        const double scale = __hiloint2double(max(0, min(2047, ex)) << 20, 0);
-                        int a[kND];
-#pragma unroll
-                        for (int s = 0; s < kND; ++s) a[s] = (int)__uint_as_float(v[s][u]);
-                        if (valid) {
-                            const double old = first ? 0.0 : cell[(size_t)t * rows2];
-                            const double s = fma(combine(a), scale, old);
-                            if (!last) cell[(size_t)t * rows2] = s;
-                            else if (p0 + set * 16 + t < c.M) cellout[(long long)t * n * R * 2] = s;
-                        }
-                    }
+        const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(set * kSetTargets);
+        int gd = 0;
+        bool dead = false;
+        for (int it = it0; it < it1; ++it) {
+            const DsWork w = P.works[it];
+            const DsCfg c = P.cfgs[w.cfg];
+            const int n = c.n, r0 = w.cg * Rt, cols = min(Rt, R - r0);
+            const int jlo = w.mt * c.J, jhi = min(jlo + c.J, n) - 1, j = jlo + jj;
+            const int t0 = w.tile * kTile + set * kSetTargets;  // first target of the set
+            double* const out = P.part + (long long)w.slot * P.Ntot * R * 2;
+            const bool idle = item_idle(P, w, r0, cols);
+            // results (p, m, r) that no shift of the item reaches: m outside [mlo, mhi]
+            const int mlo = idle ? n : jlo - w.dhi, mhi = idle ? -1 : jhi - w.dlo;
+            if (mlo > 0 || mhi < n - 1) {
+                const int tot = kSetTargets * n * 2 * cols;
+                for (int i = quarter * 32 + lane; i < tot; i += 128) {
+                    const int rc = i % (2 * cols), m = (i / (2 * cols)) % n, p = t0 + i / (2 * cols * n);
+                    if (p < c.M && (m < mlo || m > mhi))
+                        out[((c.row_off + (long long)p * n + m) * R + r0) * 2 + rc] = 0.0;
                 }
             }
-            EB = EBn;
-            --m;
-            slot = slot == 0 ? c.J - 1 : slot - 1;
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[d & 1]));
-            // the window cells of this shift are written before the next shift reads them
-            asm volatile("bar.sync %0, 128;" ::"r"(1 + set) : "memory");
+            if (idle) continue;
+            const bool rowok = j <= jhi && r < cols;
+            const int rows2 = 2 * c.J * Rt;  // doubles of the window per target
+            const int EA = (rowok ? P.EX[c.ex_off + ((long long)w.grp * n + j) * R + r0 + r] : 0) - 54;
+            const int* eb = P.EB + c.eb_off + (((long long)w.tile * c.ngrp + w.grp) * c.L + w.dlo + 2 * c.N) * kTile +
+                            set * kSetTargets + (lane / kSetTargets) * kTile + lane % kSetTargets;
+            double* const my = acc + (size_t)(set * kSetTargets) * rows2 + r * 2 + ri;
+            double* const dst = out + ((c.row_off + (long long)t0 * n) * R + r0 + r) * 2 + ri;
+            int m = j - w.dlo, slot = rowok ? ((m % c.J) + c.J) % c.J : 0;  // window position of mode m
+            // exponents of a few shifts, one per lane; the next few are on their way
+            // while these are used (L2 does not keep them beside the stream of digits)
+            const int nd = w.dhi - w.dlo + 1;
+            int EB = lane / kSetTargets < nd ? eb[0] : 0, EBn = 0;
+            for (int d = w.dlo; d <= w.dhi; ++d, ++gd) {
+                const int dd = d - w.dlo;
+                if (dd % kEbShifts == 0) {
+                    if (dd > 0) EB = EBn;
+                    EBn = dd + kEbShifts + lane / kSetTargets < nd ? eb[(long long)(dd + kEbShifts) * kTile] : 0;
+                }
+                bool ok = !dead && mbar_wait(smem_u32(&acc_full[gd & 1]), (uint32_t)((gd >> 1) & 1), abort_v);
+                ok = __all_sync(0xffffffffu, ok);
+                dead = !ok;
+                const bool valid = rowok && m >= 0 && m < n;
+                const bool work = ok && t0 < c.M && __any_sync(0xffffffffu, valid);
+                const bool last = j == jhi || d == w.dhi;
+                const bool add = valid && !(jj == 0 || d == w.dlo);
+                // the sum stays in the window, or leaves it for the partial sums
+                const double* const cell = my + (size_t)slot * Rt * 2;
+                double* const put = last ? dst + (long long)m * R * 2 : my + (size_t)slot * Rt * 2;
+                const int putstep = last ? n * R * 2 : rows2;
+                const int puts = !valid ? 0 : last ? c.M - t0 : kSetTargets;
+                if (work) asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+                for (int h = 0; h < kSetTargets; h += kCh) {
+                    uint32_t v[kND][kCh];
+                    if (work) {
+#pragma unroll
+                        for (int s = 0; s < kND; ++s) tmem_ld4(lane_addr + (gd & 1) * 256 + s * kTile + h, v[s]);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    }
+                    if (h + kCh == kSetTargets) {  // the buffer is read: the MMAs of the shift after next may start
+                        asm volatile("tcgen05.fence::before_thread_sync;");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&acc_empty[gd & 1]));
+                    }
+                    if (work) {
+                        double x[kCh];
+#pragma unroll
+                        for (int u = 0; u < kCh; ++u) {
+                            // 2^{EA + EB + 2 - 56}; a non-finite group's exponent makes its results infinite
+                            const int ex = EA + __shfl_sync(0xffffffffu, EB, (dd % kEbShifts) * kSetTargets + h + u);
+                            x[u] = to_fp64(v, u, ex, valid);
+                        }
+#pragma unroll
+                        for (int u = 0; u < kCh; ++u) x[u] += add ? cell[(size_t)(h + u) * rows2] : 0.0;
+#pragma unroll
+                        for (int u = 0; u < kCh; ++u)
+                            if (h + u < puts) put[(long long)(h + u) * putstep] = x[u];
+                    }
+                }
+                --m;
+                slot = slot == 0 ? c.J - 1 : slot - 1;
+                // the window cells of this shift are written before the next shift reads them
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + set) : "memory");
+            }
         }
-        if (!*abort_v) zero_outside(jlo - w.dhi, jhi - w.dlo, tid - 64, kThreads - 64);
     }
     // every MMA has completed before TMEM is freed
     __syncthreads();
     bool drained = true;
-    if (tid == 32 && issued_mma) drained = mbar_wait(smem_u32(&mma_done), 0);
+    if (issued_mma) drained = mbar_settle(smem_u32(&mma_done), 0);
     drained = __syncthreads_and(drained);
     if (tid == 0 && (abort_sh || !drained)) atomicOr(&g_ds_status, 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
@@ -547,8 +672,11 @@ size_t ds_xblk_bytes(int rp) { return (size_t)2 * kND * rp * 16; }
 DsSmem ds_smem(int ks, int rp, int rows2) {
     DsSmem s;
     s.ring_off = (unsigned)((ks * ds_xblk_bytes(rp) + 127) / 128 * 128);
-    s.acc_off = s.ring_off + kStages * kStage;
-    s.total = s.acc_off + (size_t)kTile * rows2 * sizeof(double);
+    const size_t window = (size_t)kTile * rows2 * sizeof(double);
+    const long long room = (long long)kDsSmemCap - (long long)s.ring_off - (long long)window;
+    s.stages = (int)std::max<long long>(3, std::min<long long>(kStagesMax, room / kStage));
+    s.acc_off = s.ring_off + s.stages * kStage;
+    s.total = s.acc_off + window;
     return s;
 }
 
@@ -569,14 +697,13 @@ void launch_ds_prep(const DsCfg* d_cfg, int C, int max_n, int max_grp, int max_n
     g_msd_launches += 2;
 }
 
-void launch_ds(const DsCfg* d_cfg, const DsWork* d_work, int nwork, const DsSmem& sm, const unsigned char* DG,
+void launch_ds(const DsCfg* d_cfg, const DsWork* d_work, const int* d_cta_off, int nctas, const DsSmem& sm, const unsigned char* DG,
                const int* EB, const unsigned char* XD, const int* EX, double2* part, long long Ntot, int R, int Rt,
                cudaStream_t s, const int* live) {
-    if (nwork <= 0) return;
     cudaFuncSetAttribute(k_bt_ds, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDsSmemCap);
-    const DsParams P{d_cfg, d_work, DG, EB, XD, EX, (double*)part, live, Ntot, R, Rt, sm.ring_off, sm.acc_off,
+    const DsParams P{d_cfg, d_work, d_cta_off, DG, EB, XD, EX, (double*)part, live, Ntot, R, Rt, sm.stages, sm.ring_off, sm.acc_off,
                      g_msd_expire_waits.load()};
-    k_bt_ds<<<(unsigned)nwork, kThreads, sm.total, s>>>(P);
+    k_bt_ds<<<(unsigned)nctas, kThreads, sm.total, s>>>(P);
     g_msd_launches += 1;
 }
 

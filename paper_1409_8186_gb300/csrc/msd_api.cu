@@ -131,8 +131,9 @@ struct MatvecPlan {
     // one grouping of the sources
     DsCfg* d_dscfg = nullptr;
     DsWork* d_dswork = nullptr;
-    int nds = 0, Rt = 1;
-    DsSmem dsm{0, 0, 0};
+    int* d_dsoff = nullptr;  // items of CTA b: [d_dsoff[b], d_dsoff[b + 1])
+    int nds = 0, Rt = 1;     // CTAs, columns of a group
+    DsSmem dsm{0, 0, 0, 0};
     size_t xd_bytes = 0, ex_ints = 0;
     long long ds_version = -1;
 };
@@ -462,9 +463,9 @@ bool ensure_gt(msd_problem* pb) {
 
 // Order and groups of the sources for the digit-sliced FP64 product, from the
 // host's copy of the radii.  Sorted by radius, eight to a K-step; a group
-// takes K-steps while its radii differ by at most 2^{3/N}, and groups that
+// takes K-steps while its radii differ by at most 2^{6/N}, and groups that
 // were made so stay through geometry updates while they differ by at most
-// 2^{4.5/N} (see k_matvec_ds.cu), so that a loop that nudges the radii keeps
+// 2^{7.5/N} (see k_matvec_ds.cu), so that a loop that nudges the radii keeps
 // its work lists.  Not offered (false) when eight neighbours differ by more.
 bool ds_grouping(msd_problem* pb) {
     if (pb->ds_radius_version == pb->radius_version) return pb->ds_ok;
@@ -480,7 +481,7 @@ bool ds_grouping(msd_problem* pb) {
         std::vector<int> o(m.M);
         for (int i = 0; i < m.M; ++i) o[i] = i;
         std::sort(o.begin(), o.end(), [&](int u, int v) { return a[u] != a[v] ? a[u] < a[v] : u < v; });
-        const double most = std::pow(2.0, 4.5 / m.N);
+        const double most = std::pow(2.0, 7.5 / m.N);
         for (int k = 0; k < nqs; ++k) {
             lo[ci].push_back(a[o[8 * k]]);
             hi[ci].push_back(a[o[std::min(m.M, 8 * k + 8) - 1]]);
@@ -528,7 +529,7 @@ bool ds_grouping(msd_problem* pb) {
         c.row_off = m.row_off;
         c.dg_off = dg;
         c.eb_off = eb;
-        const double most = std::pow(2.0, 3.0 / m.N);
+        const double most = std::pow(2.0, 6.0 / m.N);
         double first = 0;
         for (int k = 0; k < c.nqs; ++k) {
             if (k == 0 || !(hi[ci][k] <= most * first)) {
@@ -661,41 +662,45 @@ void build_work_tcs(msd_problem* pb, MatvecPlan& plan, int R) {
     }
 }
 
-// Work list of the digit-sliced product.  Columns go to groups of Rt <= 64,
-// modes to tiles of J <= 64 / Rt (the choice with the fewest (tile, shift)
-// pairs); the sources of a group are cut into folds of at most `ks` K-steps
-// and the shifts into `parts` ranges, chosen by a model of the CTA time (500
-// clocks of MMAs per K-step; up to 4300 clocks of FP64
-// work to drain a full tile) so that the last wave of one CTA per SM is full.
-// False when the partial sums would exceed 2 GB.
-bool build_work_ds(msd_problem* pb, MatvecPlan& plan, int R) {
-    int sms = 0, dev = 0;
-    CK(cudaGetDevice(&dev));
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int nmax = 2 * pb->Nmax + 1;
-    auto tiles_of = [](int n, int Rt, int* J, int* mt) {
-        const int jm = std::min(n, 64 / Rt);
-        *mt = (n + jm - 1) / jm;
-        *J = (n + *mt - 1) / *mt;
-    };
-    double best_cols = 1e300;
-    const int g0 = (R + 63) / 64;
-    for (int g = g0; g <= std::min(R, 4 * g0 + 4); ++g) {
-        const int Rt = (R + g - 1) / g;
-        int J, mt;
-        tiles_of(nmax, Rt, &J, &mt);
-        const double cost = (double)((R + Rt - 1) / Rt) * mt * (nmax + J - 1);
-        if (cost < best_cols) {
-            best_cols = cost;
-            plan.Rt = Rt;
-        }
-    }
-    const int Rt = plan.Rt, ncg = (R + Rt - 1) / Rt;
-    std::vector<DsCfg> cfgs = pb->ds_cfg;
+// Work of the digit-sliced product for one choice of (columns per group,
+// K-steps per fold): units (configuration, target tile, column group, mode
+// tile, fold) of equal-cost shifts, cut into one share per CTA (ds_items).
+struct DsShape {
+    int Rt, jmax, ks;
+    std::vector<DsCfg> cfgs;
+    DsSmem smem;
+    size_t xd_bytes, ex_ints;
+    std::vector<DsWork> items;  // by CTA
+    std::vector<int> off;       // first item of a CTA, and the end
+    int nslots;
+    double clocks;  // modelled time
+};
+
+// Modes go to tiles of at most `most` and at most 64 / Rt.
+void ds_mode_tiles(int n, int Rt, int most, int* J, int* mt) {
+    const int jm = std::min({n, most, 64 / Rt});
+    *mt = (n + jm - 1) / jm;
+    *J = (n + *mt - 1) / *mt;
+}
+
+// Items of one shape for `ctas` CTAs: the units in order (tiles outermost),
+// each CTA taking shifts until its share of the modelled clocks is full; a
+// unit that crosses a border is cut between shifts, and every piece writes a
+// partial slot of its own.  Measured, a shift costs 650 clocks of MMAs per
+// K-step (900 with a ring of three or four stages) or the drain of its
+// accumulators (5600 clocks while all target modes are in range, however many
+// rows are in use: a warp drains 32), an item 2500 more.
+// False when shared memory or the 2 GB of partial sums do not suffice.
+bool ds_items(msd_problem* pb, int R, int Rt, int jmax, int ks, int ctas, bool list, DsShape& sh) {
+    sh.Rt = Rt;
+    sh.jmax = jmax;
+    sh.ks = ks;
+    sh.cfgs = pb->ds_cfg;
+    const int ncg = (R + Rt - 1) / Rt;
     long long xd = 0, ex = 0;
     int rp_max = 0, rows_max = 0;
-    for (DsCfg& c : cfgs) {
-        tiles_of(c.n, Rt, &c.J, &c.mt);
+    for (DsCfg& c : sh.cfgs) {
+        ds_mode_tiles(c.n, Rt, jmax, &c.J, &c.mt);
         c.rp = (2 * c.J * Rt + 7) / 8 * 8;
         c.xd_off = xd;
         c.ex_off = ex;
@@ -704,100 +709,165 @@ bool build_work_ds(msd_problem* pb, MatvecPlan& plan, int R) {
         rp_max = std::max(rp_max, c.rp);
         rows_max = std::max(rows_max, 2 * c.J * Rt);
     }
-    plan.xd_bytes = (size_t)xd;
-    plan.ex_ints = (size_t)ex;
-    struct Fold {
-        int qs0, ks, grp;
+    sh.xd_bytes = (size_t)xd;
+    sh.ex_ints = (size_t)ex;
+    sh.smem = ds_smem(ks, rp_max, rows_max);
+    if (sh.smem.total > kDsSmemCap) return false;
+    constexpr double kItem = 2500.0;
+    auto shift_clocks = [&](const DsCfg& c, int k) {
+        const double drain = 5000.0 * c.n / (c.n + c.J - 1) + 600.0;
+        return std::max((sh.smem.stages < 5 ? 900.0 : 650.0) * k + 150.0, drain);
     };
-    auto folds = [&](const DsCfg& c, int ks) {
-        std::vector<Fold> out;
+    // folds of at most ks K-steps within the groups
+    auto each_fold = [&](const DsCfg& c, auto&& f) {
         for (int g = 0; g < c.ngrp; ++g) {
-            const int a = pb->ds_grp[c.grp_off + g], b = pb->ds_grp[c.grp_off + g + 1];
-            const int nb = (b - a + ks - 1) / ks;
-            for (int i = 0; i < nb; ++i) {
-                const int s = a + (b - a) * i / nb, e = a + (b - a) * (i + 1) / nb;
-                out.push_back({s, e - s, g});
-            }
+            const int a = pb->ds_grp[c.grp_off + g], b = pb->ds_grp[c.grp_off + g + 1], nb = (b - a + ks - 1) / ks;
+            for (int i = 0; i < nb; ++i) f(a + (b - a) * i / nb, (b - a) * (i + 1) / nb - (b - a) * i / nb, g);
         }
-        return out;
     };
-    auto clocks = [&](const DsCfg& c, int ks, int nd) {
-        const double drain = 4300.0 * (2.0 * c.J * Rt / 128.0) * c.n / (c.n + c.J - 1) + 300.0;
-        return 7000.0 + nd * std::max(500.0 * ks, drain);
-    };
-    auto slots_of = [&](int ks, int parts) {
-        long long ns = 1;
-        for (const DsCfg& c : cfgs) ns = std::max(ns, (long long)c.mt * (long long)folds(c, ks).size() * parts);
-        return ns;
-    };
-    int ks_best = 0, parts_best = 1;
-    double best = 1e300;
-    for (int ks = 1; ks <= kDsMaxKs; ++ks) {
-        if (ds_smem(ks, rp_max, rows_max).total > kDsSmemCap) break;
-        for (int parts : {1, 2, 3, 4, 6, 8, 12}) {
-            const long long ns = slots_of(ks, parts);
-            if (ns > 1 && (size_t)ns * pb->Ntot * R * 16 > (2ull << 30)) continue;
-            double total = 0, most = 0;
-            for (const DsCfg& c : cfgs) {
-                const std::vector<Fold> fs = folds(c, ks);
-                for (int t = 0; t < c.mt; ++t) {
-                    const int nsh = std::min(c.J, c.n - t * c.J) + c.n - 1;
-                    const int nd = (nsh + parts - 1) / parts;
-                    for (const Fold& f : fs) {
-                        const double w = clocks(c, f.ks, nd);
-                        total += w * parts * ncg * (c.Mp / MSD_TILE_P);
-                        most = std::max(most, w);
-                    }
-                }
+    double total = 0;
+    long long units = 0;
+    for (const DsCfg& c : sh.cfgs) {
+        const double same = (double)ncg * (c.Mp / MSD_TILE_P);
+        each_fold(c, [&](int, int k, int) {
+            for (int t = 0; t < c.mt; ++t) {
+                const int nd = std::min(c.J, c.n - t * c.J) + c.n - 1;
+                total += same * (kItem + nd * shift_clocks(c, k));
+                units += (long long)same;
             }
-            // one CTA per SM: the average load rounded up by half the largest CTA;
-            // partial sums written and read at 3 kB per clock
-            const double span = std::max(most, total / sms + 0.5 * most) + (double)ns * pb->Ntot * R * 32 / 3000.0;
-            if (span < best) {
-                best = span;
-                ks_best = ks;
-                parts_best = parts;
-            }
-        }
+        });
     }
-    if (!ks_best) return false;
-    plan.dsm = ds_smem(ks_best, rp_max, rows_max);
-    plan.nsplit = (int)slots_of(ks_best, parts_best);
-    std::vector<std::pair<double, DsWork>> items;
+    // every border between CTAs cuts a unit: one more item
+    const double share = (total + ctas * kItem) / ctas;
+    int slots = 0;
+    if (!list) {  // the model alone: at most this many pieces meet in one tile
+        for (const DsCfg& c : sh.cfgs) {
+            int nf = 0;
+            each_fold(c, [&](int, int, int) { ++nf; });
+            double tile_clocks = 0;
+            each_fold(c, [&](int, int k, int) {
+                for (int t = 0; t < c.mt; ++t)
+                    tile_clocks += kItem + (std::min(c.J, c.n - t * c.J) + c.n - 1) * shift_clocks(c, k);
+            });
+            slots = std::max(slots, nf * c.mt + (int)(tile_clocks / share) + 1);
+        }
+        sh.nslots = slots;
+        const double bytes = (double)slots * pb->Ntot * R * 16;
+        if (slots > 1 && bytes > 2.0e9) return false;
+        sh.clocks = share + 2.0 * bytes / 3000.0;  // partial sums written and read at 3 kB per clock
+        return true;
+    }
+    sh.items.clear();
+    sh.off.assign(1, 0);
+    double left = share;
+    auto next_cta = [&]() {
+        if ((int)sh.off.size() < ctas) {
+            sh.off.push_back((int)sh.items.size());
+            left += share;
+        } else {
+            left = 1e300;
+        }
+    };
+    std::vector<std::tuple<int, int, int, int>> used;  // (cfg, tile, cg, slots used)
     for (int ci = 0; ci < pb->C; ++ci) {
-        const DsCfg& c = cfgs[ci];
-        const std::vector<Fold> fs = folds(c, ks_best);
+        const DsCfg& c = sh.cfgs[ci];
         for (int tile = 0; tile < c.Mp / MSD_TILE_P; ++tile)
             for (int cg = 0; cg < ncg; ++cg) {
                 int slot = 0;
-                for (int t = 0; t < c.mt; ++t) {
-                    const int dlo = t * c.J - (c.n - 1), dhi = std::min(c.n, (t + 1) * c.J) - 1, nsh = dhi - dlo + 1;
-                    for (const Fold& f : fs)
-                        for (int k = 0; k < parts_best; ++k) {
-                            const int a = dlo + nsh * k / parts_best, b = dlo + nsh * (k + 1) / parts_best - 1;
-                            DsWork w{ci, tile, cg, t, f.qs0, b >= a ? f.ks : 0, f.grp, slot++, a, b};
-                            items.push_back({w.ks ? clocks(c, w.ks, b - a + 1) : 0.0, w});
+                for (int t = 0; t < c.mt; ++t)
+                    each_fold(c, [&](int q0, int k, int g) {
+                        const double sc = shift_clocks(c, k);
+                        int d = t * c.J - (c.n - 1);
+                        const int dhi = std::min(c.n, (t + 1) * c.J) - 1;
+                        while (d <= dhi) {
+                            int cnt = dhi - d + 1;
+                            const double room = (left - kItem) / sc;
+                            if (room < cnt - 0.5) {
+                                cnt = (int)(room + 0.5);
+                                // not worth an item of its own: a few shifts
+                                if (cnt < 3) {
+                                    next_cta();
+                                    continue;
+                                }
+                            }
+                            sh.items.push_back(DsWork{ci, tile, cg, t, q0, k, g, slot++, d, d + cnt - 1});
+                            left -= kItem + cnt * sc;
+                            d += cnt;
                         }
-                }
-                for (; slot < plan.nsplit; ++slot) items.push_back({0.0, DsWork{ci, tile, cg, 0, 0, 0, 0, slot, 0, -1}});
+                    });
+                slots = std::max(slots, slot);
+                used.push_back({ci, tile, cg, slot});
             }
     }
-    std::stable_sort(items.begin(), items.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-    std::vector<DsWork> work;
-    for (auto& it : items) work.push_back(it.second);
-    plan.nds = (int)work.size();
+    sh.off.push_back((int)sh.items.size());
+    while ((int)sh.off.size() < ctas + 1) sh.off.push_back((int)sh.items.size());
+    sh.nslots = slots;
+    if (slots > 1 && (double)slots * pb->Ntot * R * 16 > 2.0e9) return false;
+    // slots that a tile does not use are zeroed, by the CTAs in turn
+    std::vector<std::vector<DsWork>> zero(ctas);
+    int turn = 0;
+    for (auto& [ci, tile, cg, n] : used)
+        for (int sl = n; sl < slots; ++sl) zero[turn++ % ctas].push_back(DsWork{ci, tile, cg, 0, 0, 0, 0, sl, 0, -1});
+    if (turn) {
+        std::vector<DsWork> all;
+        std::vector<int> off(1, 0);
+        for (int b = 0; b < ctas; ++b) {
+            all.insert(all.end(), zero[b].begin(), zero[b].end());
+            all.insert(all.end(), sh.items.begin() + sh.off[b], sh.items.begin() + sh.off[b + 1]);
+            off.push_back((int)all.size());
+        }
+        sh.items.swap(all);
+        sh.off.swap(off);
+    }
+    return true;
+}
+
+// The shape of the digit-sliced product with the least modelled time.  Few
+// columns per group mean long mode tiles (more shifts per tile, fewer partial
+// sums), many K-steps per fold fewer drains.  False when none fits.
+bool build_work_ds(msd_problem* pb, MatvecPlan& plan, int R) {
+    int sms = 0, dev = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    DsShape sh, best;
+    best.clocks = 1e300;
+    const int g0 = (R + 63) / 64;
+    int last_Rt = 0;
+    for (int g = g0; g <= std::min(R, 16 * g0); ++g) {
+        const int Rt = (R + g - 1) / g;
+        if (Rt == last_Rt) continue;
+        last_Rt = Rt;
+        const int nmax = 2 * pb->Nmax + 1, jtop = std::min(nmax, 64 / Rt);
+        int last_mt = 0;
+        for (int j = jtop; j >= 1 && j >= jtop / 2; --j) {
+            const int mt = (nmax + j - 1) / j;
+            if (mt == last_mt) continue;
+            last_mt = mt;
+            for (int ks = 1; ks <= kDsMaxKs; ++ks)
+                if (ds_items(pb, R, Rt, j, ks, sms, false, sh) && sh.clocks < best.clocks * (1.0 - 1e-9)) best = sh;
+        }
+    }
+    if (best.clocks == 1e300 || !ds_items(pb, R, best.Rt, best.jmax, best.ks, sms, true, best)) return false;
+    plan.Rt = best.Rt;
+    plan.dsm = best.smem;
+    plan.xd_bytes = best.xd_bytes;
+    plan.ex_ints = best.ex_ints;
+    plan.nsplit = best.nslots;
+    plan.nds = sms;
     plan.ds_version = pb->ds_version;
-    plan.d_dscfg = dalloc_copy(cfgs.data(), cfgs.size());
-    plan.d_dswork = dalloc_copy(work.data(), work.size());
+    plan.d_dscfg = dalloc_copy(best.cfgs.data(), best.cfgs.size());
+    plan.d_dswork = dalloc_copy(best.items.data(), best.items.size());
+    plan.d_dsoff = dalloc_copy(best.off.data(), best.off.size());
     return true;
 }
 
 void free_plan(MatvecPlan& plan) {
-    for (void* p : {(void*)plan.d_work, (void*)plan.d_dscfg, (void*)plan.d_dswork})
+    for (void* p : {(void*)plan.d_work, (void*)plan.d_dscfg, (void*)plan.d_dswork, (void*)plan.d_dsoff})
         if (p) cudaFree(p);
     plan.d_work = nullptr;
     plan.d_dscfg = nullptr;
     plan.d_dswork = nullptr;
+    plan.d_dsoff = nullptr;
 }
 
 // The digit-sliced Toeplitz sums of the scaled columns xs into part.
@@ -809,7 +879,7 @@ void ds_product(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint, const do
     launch_ds_prep(plan.d_dscfg, pb->C, 2 * pb->Nmax + 1, pb->ds_max_grp, pb->ds_max_nqs,
                    (const int*)pb->ds_idx[1].p, (const int*)pb->ds_idx[2].p, (const int*)pb->ds_idx[3].p, R, plan.Rt,
                    xs, EX, XD, pb->stream);
-    launch_ds(plan.d_dscfg, plan.d_dswork, plan.nds, plan.dsm, (const unsigned char*)g.dg.p, (const int*)g.eb.p, XD,
+    launch_ds(plan.d_dscfg, plan.d_dswork, plan.d_dsoff, plan.nds, plan.dsm, (const unsigned char*)g.dg.p, (const int*)g.eb.p, XD,
               EX, part, pb->Ntot, R, plan.Rt, pb->stream, live);
 }
 

@@ -161,7 +161,7 @@ struct DsCfg {
     long long dg_off, eb_off;  // generator digits (in stages) and exponents
     long long xd_off, ex_off;  // source digits (bytes) and exponents
 };
-// One CTA: targets [32 tile, 32 tile + 32), columns of group cg, modes of
+// One item: targets [32 tile, 32 tile + 32), columns of group cg, modes of
 // tile mt as sources' modes, K-steps [qs0, qs0 + ks) of group grp, shifts
 // [dlo, dhi], writing partial slot `slot` (ks = 0: zeros).
 struct DsWork {
@@ -169,6 +169,7 @@ struct DsWork {
 };
 struct DsSmem {
     unsigned ring_off, acc_off;
+    int stages;
     size_t total;
 };
 constexpr size_t kDsSmemCap = 226 * 1024;
@@ -182,7 +183,7 @@ void launch_ds_build(const DsCfg* d_cfg, int C, int max_Mp, int max_grp, int max
 void launch_ds_prep(const DsCfg* d_cfg, int C, int max_n, int max_grp, int max_nqs, const int* d_grp_start,
                     const int* d_qgrp, const int* d_perm, int R, int Rt, const double2* xs, int* EX, unsigned char* XD,
                     cudaStream_t s);
-void launch_ds(const DsCfg* d_cfg, const DsWork* d_work, int nwork, const DsSmem& sm, const unsigned char* DG,
+void launch_ds(const DsCfg* d_cfg, const DsWork* d_work, const int* d_cta_off, int nctas, const DsSmem& sm, const unsigned char* DG,
                const int* EB, const unsigned char* XD, const int* EX, double2* part, long long Ntot, int R, int Rt,
                cudaStream_t s, const int* live = nullptr);
 int ds_status_and_clear();

@@ -67,6 +67,7 @@
 #include <cstdint>
 
 #include "msd_internal.cuh"
+#include "pipeline.cuh"
 
 __device__ int g_ds_status;  // bit 0: a wait of the digit-sliced kernel expired
 
@@ -83,85 +84,13 @@ constexpr int kCh = 4;                       // targets in flight per lane
 constexpr int kEbShifts = 32 / kSetTargets;  // shifts whose exponents a warp holds
 constexpr int kThreads = 64 + kDrainWarps * 32;
 constexpr int kNonFinite = 1 << 24;          // exponent of a group with an infinity or NaN
-constexpr long long kWaitCycles = 2000000000LL;  // ~1 s at 2 GHz
-constexpr long long kTestWaitCycles = 20000;     // msd_test_expire_waits
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// shared-memory matrix descriptor: K-major, no swizzle, given strides
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
-}
 // kind::f16 instruction descriptor: D F32, A and B BF16, both K-major.
 __device__ __forceinline__ uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait.  The clock and the CTA's abort flag are only looked at once a
-// first try has failed: the issuing threads wait for every K-step, and what a
-// satisfied wait costs is time the tensor pipe does not get back.
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_v) {
-    const long long t0 = clock64();
-    while (true) {
-        if (mbar_try(bar, parity)) return true;
-        if (*abort_v) return false;
-        if (clock64() - t0 > kWaitCycles) {
-            *abort_v = 1;
-            return false;
-        }
-    }
-}
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_v) {
-    return mbar_try(bar, parity) || mbar_wait_slow(bar, parity, abort_v);
-}
-// The same for copies that must land (or MMAs that must end) before the CTA
-// may go on even after an abort.
-__device__ __noinline__ bool mbar_settle(uint32_t bar, uint32_t parity) {
-    const long long t0 = clock64();
-    while (!mbar_try(bar, parity))
-        if (clock64() - t0 > kWaitCycles) return false;
-    return true;
-}
-// One thread of a converged warp, chosen so that the compiler knows the branch
-// is taken by one thread: the operands of tcgen05.mma live in uniform
-// registers, and under a test of the lane number every instruction is wrapped
-// in a loop over its possible values (400 disks: the issue loop alone 180 us
-// that way, 132 us so).
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
-    return p != 0;
-}
-__device__ __forceinline__ bool wait_unset_flag(const volatile int* flag) {
-    const long long t0 = clock64();
-    while (!*flag)
-        if (clock64() - t0 > kTestWaitCycles) return false;
-    return true;
-}
 __device__ __forceinline__ void mbar_init(uint64_t* bar, int count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// global -> shared bulk copy completing on an mbarrier (16-byte aligned, size % 16 == 0)
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
 }
 // (descriptors as two words: the upper ones are the same for every MMA)
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
@@ -171,9 +100,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint32_t a_lo, uint32_
         "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(tmem_d),
         "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(id), "r"(acc));
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar));
 }
 // 4 consecutive TMEM columns of this thread's lane
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {

@@ -41,6 +41,7 @@
 #include <cstdint>
 
 #include "msd_internal.cuh"
+#include "pipeline.cuh"
 
 __device__ int g_tcs_status;  // bit 0: a wait of the shift-GEMM kernel expired
 
@@ -58,71 +59,20 @@ constexpr int kMbMax = 8;           // modes per block (N = 16 mb <= 128)
 // whose wide blocks had 16 modes (N = 256) on the lattice ended in an
 // illegal-instruction fault; N <= 208 ran correctly, so wider is not offered.
 constexpr int kMbWide = 13;
-constexpr long long kWaitCycles = 2000000000LL;  // ~1 s at 2 GHz
-constexpr long long kTestWaitCycles = 20000;     // msd_test_expire_waits
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// shared-memory matrix descriptor: K-major, no swizzle, given strides
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
-}
 
 // kind::tf32 instruction descriptor: D F32, A and B TF32, both K-major.
 __device__ __forceinline__ uint32_t idesc_tf32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
+// (descriptors as two words: the upper ones are the same for every MMA)
+__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                         uint32_t id, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    const long long t0 = clock64();
-    while (!mbar_try(bar, parity))
-        if (clock64() - t0 > kWaitCycles) return false;
-    return true;
-}
-
-__device__ __forceinline__ bool wait_unset_flag(const volatile int* flag) {
-    const long long t0 = clock64();
-    while (!*flag)
-        if (clock64() - t0 > kTestWaitCycles) return false;
-    return true;
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// global -> shared bulk copy completing on an mbarrier (16-byte aligned, size % 16 == 0)
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t id, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(da), "l"(db), "r"(id), "r"(acc));
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar));
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %5, p;\n\t}" ::"r"(tmem_d),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(id), "r"(acc));
 }
 
 // 16 consecutive TMEM columns of this thread's lane
@@ -235,130 +185,160 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int ngroups = (nqc + kFoldQc - 1) / kFoldQc;
     int issued_mma = 0;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // ---------------- producer
-        const float* gt = GT + c.gt_off + (long long)ptile * L * (c.Mq / 4) * 2048;
-        const float* xt = XT + c.xrow_off * 4 * R + (long long)rt * c.Mq * n * 32;
-        long long ait = 0;
-        // slab of K-step qi; issued one K-step ahead, once the MMAs of K-step
-        // qi - 2 (the previous user of its buffer) have certainly completed
-        auto issue_slab = [&](int qi) {
-            const int qc = qc0 + qi, sb = qi & 1;
-            if (qi >= 2) {
-                if (!*abort_v && !mbar_wait(smem_u32(&s_empty[sb]), ((qi >> 1) - 1) & 1)) *abort_v = 1;
-                // own previous copy into this buffer is complete before re-arming
-                mbar_wait(smem_u32(&s_full[sb]), ((qi >> 1) - 1) & 1);
-            }
-            const uint32_t sbar = smem_u32(&s_full[sb]);
-            mbar_expect_tx(sbar, 4u * n * 256u);
-            for (int h = 0; h < 2; ++h)
-                for (int hl = 0; hl < 2; ++hl)
-                    bulk_g2s(smem_u32(slab + sb * buf + (h * 2 + hl) * blk + kPad * 256),
-                             xt + ((long long)(2 * qc + h) * 2 + hl) * n * 64, (uint32_t)n * 256u, sbar);
-        };
-        if (nqc > 0) issue_slab(0);
-        const int next_at = min(nd - 1, kStages);
-        // ring position of the next A stage and the parity of its previous use
-        int s = 0;
-        uint32_t ph = 1;  // parity of the phase to wait for before reuse (first lap: none)
-        bool lap1 = true;
-        const float* gq = gt + (long long)(dlo + 2 * N) * (c.Mq / 4) * 2048;
-        const long long dstep = (long long)(c.Mq / 4) * 2048;
-        for (int qi = 0; qi < nqc; ++qi) {
-            const float* gd = gq + (long long)(2 * (qc0 + qi)) * 2048;
-            for (int t = 0; t < nd; ++t, gd += dstep) {
-                // the next slab once kStages A stages of this K-step are issued:
-                // the MMAs of K-step qi - 1 are then complete
-                if (t == next_at && qi + 1 < nqc) issue_slab(qi + 1);
-                if (!lap1) {
-                    if (!*abort_v && !mbar_wait(smem_u32(&a_empty[s]), ph)) *abort_v = 1;
-                    mbar_wait(smem_u32(&a_full[s]), ph);
+        if (elect_one()) {
+            const float* gt = GT + c.gt_off + (long long)ptile * L * (c.Mq / 4) * 2048;
+            const float* xt = XT + c.xrow_off * 4 * R + (long long)rt * c.Mq * n * 32;
+            long long ait = 0;
+            bool dead = false;  // a wait has expired: the copies go on, waiting only for themselves
+            // slab of K-step qi; issued one K-step ahead, once the MMAs of K-step
+            // qi - 2 (the previous user of its buffer) have certainly completed
+            auto issue_slab = [&](int qi) {
+                const int qc = qc0 + qi, sb = qi & 1;
+                if (qi >= 2) {
+                    if (!dead) dead = !mbar_wait(smem_u32(&s_empty[sb]), ((qi >> 1) - 1) & 1, abort_v);
+                    if (dead) mbar_settle(smem_u32(&s_full[sb]), ((qi >> 1) - 1) & 1);
                 }
-                const uint32_t abar = smem_u32(&a_full[s]);
-                mbar_expect_tx(abar, kAStage);
-                bulk_g2s(smem_u32(A + s * kAStage), gd, kAStage, abar);
-                ++ait;
-                if (++s == kStages) {
-                    s = 0;
-                    ph ^= 1;
-                    if (lap1) {
-                        lap1 = false;
-                        ph = 0;
+                const uint32_t sbar = smem_u32(&s_full[sb]);
+                mbar_expect_tx(sbar, 4u * n * 256u);
+                for (int h = 0; h < 2; ++h)
+                    for (int hl = 0; hl < 2; ++hl)
+                        bulk_g2s(smem_u32(slab + sb * buf + (h * 2 + hl) * blk + kPad * 256),
+                                 xt + ((long long)(2 * qc + h) * 2 + hl) * n * 64, (uint32_t)n * 256u, sbar);
+            };
+            if (nqc > 0) issue_slab(0);
+            const int next_at = min(nd - 1, kStages);
+            // ring position of the next A stage and the parity of its previous use
+            int s = 0;
+            uint32_t ph = 1;  // parity of the phase to wait for before reuse (first lap: none)
+            bool lap1 = true;
+            const float* gq = gt + (long long)(dlo + 2 * N) * (c.Mq / 4) * 2048;
+            const long long dstep = (long long)(c.Mq / 4) * 2048;
+            for (int qi = 0; qi < nqc; ++qi) {
+                const float* gd = gq + (long long)(2 * (qc0 + qi)) * 2048;
+                for (int t = 0; t < nd; ++t, gd += dstep) {
+                    // the next slab once kStages A stages of this K-step are issued:
+                    // the MMAs of K-step qi - 1 are then complete
+                    if (t == next_at && qi + 1 < nqc) issue_slab(qi + 1);
+                    if (!lap1) {
+                        if (!dead) dead = !mbar_wait(smem_u32(&a_empty[s]), ph, abort_v);
+                        if (dead) mbar_settle(smem_u32(&a_full[s]), ph);
+                    }
+                    const uint32_t abar = smem_u32(&a_full[s]);
+                    mbar_expect_tx(abar, kAStage);
+                    bulk_g2s(smem_u32(A + s * kAStage), gd, kAStage, abar);
+                    ++ait;
+                    if (++s == kStages) {
+                        s = 0;
+                        ph ^= 1;
+                        if (lap1) {
+                            lap1 = false;
+                            ph = 0;
+                        }
                     }
                 }
             }
+            // every copy of this CTA has landed before it exits
+            for (int s2 = 0; s2 < kStages; ++s2)
+                if (ait > s2) mbar_settle(smem_u32(&a_full[s2]), (uint32_t)(((ait - 1 - s2) / kStages) & 1));
+            for (int sb = 0; sb < 2; ++sb)
+                if (nqc > sb) mbar_settle(smem_u32(&s_full[sb]), (uint32_t)(((nqc - 1 - sb) >> 1) & 1));
         }
-        // every copy of this CTA has landed before it exits
-        for (int s2 = 0; s2 < kStages; ++s2)
-            if (ait > s2) mbar_wait(smem_u32(&a_full[s2]), (uint32_t)(((ait - 1 - s2) / kStages) & 1));
-        for (int sb = 0; sb < 2; ++sb)
-            if (nqc > sb) mbar_wait(smem_u32(&s_full[sb]), (uint32_t)(((nqc - 1 - sb) >> 1) & 1));
-    } else if (warp == 1 && lane == 0) {
+        __syncwarp();
+    } else if (warp == 1) {
         // ---------------- MMA issue
-        // Descriptors are linear in the start address (field = address / 16),
-        // so the per-stage and per-shift ones are base descriptors plus
-        // offsets; stage and phase advance incrementally.
-        const uint32_t id = idesc_tf32(128, 16 * mb);
-        const uint32_t d2off = mb > kMbMax ? 256u : 128u;  // D2 after D1 (N = 16 mb columns each)
-        const uint32_t sbo = 128;
-        const uint64_t adesc0 = sdesc(smem_u32(A), 8192, sbo);
-        const uint64_t bdesc0[2] = {sdesc(smem_u32(slab), 2 * blk, sbo), sdesc(smem_u32(slab + buf), 2 * blk, sbo)};
-        const uint64_t blo = (uint64_t)(blk >> 4);
-        int group = 0;
-        int fresh = 3;  // bit b: the next MMA into block b's accumulators overwrites them
-        bool first_wait = true;
-        int s = 0;
-        uint32_t ph = 0;  // parity of the stage's current fill
-        for (int qi = 0; qi < nqc; ++qi) {
-            const int sb = qi & 1;
-            if (!*abort_v && !mbar_wait(smem_u32(&s_full[sb]), (qi >> 1) & 1)) *abort_v = 1;
-            const uint64_t bd = bdesc0[sb];
-            const bool fold_wait = qi % kFoldQc == 0 && group > 0;
-            for (int d = dlo; d <= dhi; ++d) {
-                bool ok = *abort_v ? true : mbar_wait(smem_u32(&a_full[s]), ph);
-                if (expire_test && first_wait) ok = wait_unset_flag(&never_sh) && ok;
-                first_wait = false;
-                if (!ok) *abort_v = 1;
-                if (fold_wait && d == dlo && !*abort_v && !mbar_wait(smem_u32(&acc_empty), (uint32_t)((group - 1) & 1)))
+        // Descriptors are linear in the start address (field = address / 16,
+        // in the lower word), so the per-stage and per-shift ones are base
+        // descriptors plus offsets; stage and phase advance incrementally.
+        // Nothing but a satisfied try, the MMAs and their commit is left in the
+        // loop over the stages: 1300 clocks a stage with a test of the lane, the
+        // clock and flag reads and the bounds of every shift in it, 750 so (768
+        // at the tensor pipe's rate where both blocks have work).  4000-disk
+        // lattice, 64 columns: 59.3 -> 32.0 ms a product; eight clusters of 100
+        // to 400 disks, 32 columns: 1.31 -> 0.73 ms.
+        if (elect_one()) {
+            const uint32_t id = idesc_tf32(128, 16 * mb);
+            const uint32_t d2off = mb > kMbMax ? 256u : 128u;  // D2 after D1 (N = 16 mb columns each)
+            const uint32_t sbo = 128;
+            const uint64_t adesc0 = sdesc(smem_u32(A), 8192, sbo);
+            const uint64_t bdesc0 = sdesc(smem_u32(slab), 2 * blk, sbo);
+            const uint32_t a_hi = (uint32_t)(adesc0 >> 32), b_hi = (uint32_t)(bdesc0 >> 32);
+            const uint32_t blo = (uint32_t)(blk >> 4);
+            // shifts that bring a source mode to block b (of two at most), and the
+            // slab offset of its B operand at shift 0
+            int lo0 = 1, hi0 = 0, lo1 = 1, hi1 = 0;
+            bool dead = false;
+            for (int b = 0; b < nmb; ++b) {
+                const int mb0 = m0 + b * mb, mb1 = min(n, mb0 + mb) - 1;
+                const int lo = -mb1, hi = n - 1 - mb0;
+                // every B window lies within its slab block (by construction)
+                if (mb0 + lo + kPad < 0 || mb0 + hi + kPad + mb > n + 2 * kPad || b > 1) {
                     *abort_v = 1;
+                    dead = true;
+                }
+                if (b == 0) {
+                    lo0 = lo;
+                    hi0 = hi;
+                } else {
+                    lo1 = lo;
+                    hi1 = hi;
+                }
+            }
+            int group = 0;
+            uint32_t acc0 = 0, acc1 = 0;  // 0: the next MMA into the block's accumulators overwrites them
+            if (expire_test && !wait_unset_flag(&never_sh)) {
+                *abort_v = 1;
+                dead = true;
+            }
+            int s = 0;
+            uint32_t ph = 0;  // parity of the stage's current fill
+            for (int qi = 0; qi < nqc; ++qi) {
+                const int sb = qi & 1;
+                if (!dead) dead = !mbar_wait(smem_u32(&s_full[sb]), (qi >> 1) & 1, abort_v);
+                if (qi % kFoldQc == 0 && group > 0 && !dead)
+                    dead = !mbar_wait(smem_u32(&acc_empty), (uint32_t)((group - 1) & 1), abort_v);
                 asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint64_t grh = adesc0 + (uint64_t)(s * (kAStage >> 4));
-                const uint64_t grl = grh + 128, gih = grh + 256, gil = grh + 384;  // + 2, 4, 6 KB
-                for (int b = 0; b < nmb; ++b) {
-                    const int mb0 = m0 + b * mb;
-                    const int mb1 = min(n, mb0 + mb) - 1;
-                    if (d < -mb1 || d > n - 1 - mb0) continue;  // no mode of the block meets a source mode
-                    const int jb = mb0 + d + kPad;  // first slab mode of the B operand
-                    if (jb < 0 || jb + mb > n + 2 * kPad) {  // outside the slab block: never by construction
-                        *abort_v = 1;
-                        continue;
+                // B of block 0 at shift d: slab mode m0 + d + kPad
+                uint32_t bl0 = (uint32_t)bdesc0 + (uint32_t)(sb * (buf >> 4)) + (uint32_t)((m0 + dlo + kPad) * 16);
+                for (int d = dlo; d <= dhi; ++d, bl0 += 16) {
+                    if (!dead) dead = !mbar_wait(smem_u32(&a_full[s]), ph, abort_v);
+                    if (!dead) {
+                        const uint32_t al = (uint32_t)adesc0 + (uint32_t)(s * (kAStage >> 4));  // Re hi; + 2, 4, 6 KB
+                        auto six = [&](uint32_t tc, uint32_t bh, uint32_t acc) {
+                            mma_tf32(tc, al, a_hi, bh, b_hi, id, acc);
+                            mma_tf32(tc, al, a_hi, bh + blo, b_hi, id, 1u);
+                            mma_tf32(tc, al + 128, a_hi, bh, b_hi, id, 1u);
+                            mma_tf32(tc + d2off, al + 256, a_hi, bh, b_hi, id, acc);
+                            mma_tf32(tc + d2off, al + 256, a_hi, bh + blo, b_hi, id, 1u);
+                            mma_tf32(tc + d2off, al + 384, a_hi, bh, b_hi, id, 1u);
+                        };
+                        if (d >= lo0 && d <= hi0) {
+                            six(tmem, bl0, acc0);
+                            acc0 = 1;
+                        }
+                        if (d >= lo1 && d <= hi1) {
+                            six(tmem + 256, bl0 + (uint32_t)(mb * 16), acc1);
+                            acc1 = 1;
+                        }
+                        issued_mma = 1;
                     }
-                    const uint64_t bh = bd + (uint64_t)(jb * 16), bl = bh + blo;  // jb * 256 bytes
-                    const uint32_t d1 = tmem + (uint32_t)(b * 256), d2 = d1 + d2off;
-                    const uint32_t acc = ((fresh >> b) & 1) ? 0u : 1u;
-                    mma_tf32(d1, grh, bh, id, acc);
-                    mma_tf32(d1, grh, bl, id, 1u);
-                    mma_tf32(d1, grl, bh, id, 1u);
-                    mma_tf32(d2, gih, bh, id, acc);
-                    mma_tf32(d2, gih, bl, id, 1u);
-                    mma_tf32(d2, gil, bh, id, 1u);
-                    fresh &= ~(1 << b);
-                    issued_mma = 1;
+                    mma_commit(smem_u32(&a_empty[s]));
+                    if (++s == kStages) {
+                        s = 0;
+                        ph ^= 1;
+                    }
                 }
-                mma_commit(smem_u32(&a_empty[s]));
-                if (++s == kStages) {
-                    s = 0;
-                    ph ^= 1;
+                mma_commit(smem_u32(&s_empty[sb]));
+                if ((qi + 1) % kFoldQc == 0 || qi == nqc - 1) {
+                    mma_commit(smem_u32(&acc_full));
+                    acc0 = acc1 = 0;
+                    ++group;
                 }
             }
-            mma_commit(smem_u32(&s_empty[sb]));
-            if ((qi + 1) % kFoldQc == 0 || qi == nqc - 1) {
-                mma_commit(smem_u32(&acc_full));
-                fresh = 3;
-                ++group;
-            }
+            if (issued_mma) mma_commit(smem_u32(&mma_done));
         }
-        if (issued_mma) mma_commit(smem_u32(&mma_done));
+        __syncwarp();
     } else if (warp >= 2) {
         // ---------------- fold the accumulators into FP32 registers (round to nearest)
         // warp group g = (warp - 2) / 4 folds block g (two blocks of <= 8
@@ -376,9 +356,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int r = 0; r < kRC; ++r) sr[u][r] = si[u][r] = 0.f;
         for (int g = 0; g < ngroups; ++g) {
-            bool ok = *abort_v ? false : mbar_wait(smem_u32(&acc_full), (uint32_t)(g & 1));
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) *abort_v = 1;
+            bool ok = mbar_wait(smem_u32(&acc_full), (uint32_t)(g & 1), abort_v);
+            ok = __all_sync(0xffffffffu, ok) && !*abort_v;
             if (ok && b < nmb) {
                 asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
@@ -420,7 +399,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // every MMA has completed before TMEM is freed
     __syncthreads();
     bool drained = true;
-    if (tid == 32 && issued_mma) drained = mbar_wait(smem_u32(&mma_done), 0);
+    if (issued_mma) drained = mbar_settle(smem_u32(&mma_done), 0);
     drained = __syncthreads_and(drained);
     if (tid == 0 && (abort_sh || !drained)) atomicOr(&g_tcs_status, 1);
     asm volatile("tcgen05.fence::after_thread_sync;");

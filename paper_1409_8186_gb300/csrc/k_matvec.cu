@@ -22,6 +22,8 @@
 // ceil(n / KB) * KB wastes as few padded modes as possible.  Raw sums go to a
 // per-split partial buffer; a finalize kernel adds the splits, applies
 // l^p_m and adds x.
+#include <type_traits>
+
 #include "msd_internal.cuh"
 
 namespace {
@@ -497,33 +499,66 @@ __global__ void k_scale_cols(long long Ntot, int R, const S* __restrict__ rf, co
     xs[i] = V{v.x * f, v.y * f};
 }
 
-// y = x + lf .* sum_s part[s]
-// (kFinLanes threads per element split the partial slots, then shuffle-add)
-constexpr int kFinLanes = 8;
-template <typename V>
-__global__ void k_finalize(long long Ntot, int R, int nsplit, const V* __restrict__ lf,
-                           const V* __restrict__ x, const V* __restrict__ part, V* __restrict__ y) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long i = t / kFinLanes;
-    const int sub = (int)(t % kFinLanes);
-    const long long tot = Ntot * R;
+// Sum of the partial slots of 256 / TY consecutive elements per CTA, TY rows
+// of threads sharing the slots (neighbouring threads read neighbouring
+// elements of a slot; eight lanes per element, one slot each, moved a sector
+// for every value).  Every thread calls it; the first row holds the sums.
+template <typename V, int TY>
+__device__ __forceinline__ V slot_sum(long long tot, int nsplit, const V* __restrict__ part, long long i, int ty) {
+    constexpr int EX = 256 / TY;
+    __shared__ V red[TY][EX];
     V s = vzero<V>();
     if (i < tot) {
-        for (int k = sub; k < nsplit; k += kFinLanes) {
+#pragma unroll 4
+        for (int k = ty; k < nsplit; k += TY) {
             const V v = part[(long long)k * tot + i];
             s.x += v.x;
             s.y += v.y;
         }
     }
-#pragma unroll
-    for (int off = kFinLanes / 2; off > 0; off >>= 1) {
-        s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
-        s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    if (TY > 1) {
+        const int tx = threadIdx.x % EX;
+        red[ty][tx] = s;
+        __syncthreads();
+        if (ty == 0)
+            for (int y = 1; y < TY; ++y) {
+                s.x += red[y][tx].x;
+                s.y += red[y][tx].y;
+            }
     }
-    if (i >= tot || sub != 0) return;
+    return s;
+}
+
+// y = x + lf .* sum_s part[s]
+template <typename V, int TY>
+__global__ void __launch_bounds__(256) k_finalize(long long Ntot, int R, int nsplit, const V* __restrict__ lf,
+                                                  const V* __restrict__ x, const V* __restrict__ part,
+                                                  V* __restrict__ y) {
+    const long long tot = Ntot * R, i = (long long)blockIdx.x * (256 / TY) + threadIdx.x % (256 / TY);
+    const int ty = threadIdx.x / (256 / TY);
+    const V s = slot_sum<V, TY>(tot, nsplit, part, i, ty);
+    if (i >= tot || ty != 0) return;
     const V l = lf[i / R];
     const V v = x[i];
     y[i] = V{v.x + (l.x * s.x - l.y * s.y), v.y + (l.x * s.y + l.y * s.x)};
+}
+
+// Thread rows per CTA of the finalize kernels: more slots than loads one
+// thread keeps in flight, or too few elements to fill the chip.
+template <typename F>
+void with_slot_rows(long long tot, int nsplit, F&& f) {
+    const long long ctas = (tot + 255) / 256;
+    if (nsplit > 4 && (ctas < 152 * 4 || nsplit >= 32)) f(std::integral_constant<int, 8>());
+    else if (nsplit > 1 && ctas < 152 * 4) f(std::integral_constant<int, 2>());
+    else f(std::integral_constant<int, 1>());
+}
+template <typename V>
+void finalize(long long Ntot, int R, int nsplit, const V* lf, const V* x, const V* part, V* y, cudaStream_t s) {
+    with_slot_rows(Ntot * R, nsplit, [&](auto ty) {
+        constexpr int TY = decltype(ty)::value;
+        k_finalize<V, TY><<<(unsigned)((Ntot * R + 256 / TY - 1) / (256 / TY)), 256, 0, s>>>(Ntot, R, nsplit, lf, x,
+                                                                                            part, y);
+    });
 }
 
 // ---------------------------------------------------------------- kernel selection
@@ -793,13 +828,9 @@ void launch_scale_cols(bool fp64, long long Ntot, int R, const void* rf, const v
 
 void launch_finalize(bool fp64, long long Ntot, int R, int nsplit, const void* lf, const void* x, const void* part,
                      void* y, cudaStream_t s) {
-    const long long tot = Ntot * R;
-    const int th = 256;
-    const unsigned blocks = (unsigned)((tot * kFinLanes + th - 1) / th);
-    if (fp64) k_finalize<double2><<<blocks, th, 0, s>>>(Ntot, R, nsplit, (const double2*)lf, (const double2*)x,
-                                                         (const double2*)part, (double2*)y);
-    else k_finalize<float2><<<blocks, th, 0, s>>>(Ntot, R, nsplit, (const float2*)lf, (const float2*)x,
-                                                  (const float2*)part, (float2*)y);
+    if (fp64) finalize<double2>(Ntot, R, nsplit, (const double2*)lf, (const double2*)x, (const double2*)part,
+                                (double2*)y, s);
+    else finalize<float2>(Ntot, R, nsplit, (const float2*)lf, (const float2*)x, (const float2*)part, (float2*)y, s);
     g_msd_launches += 1;
 }
 
@@ -834,7 +865,7 @@ void launch_matvec_f64(const MsdConfig* d_cfg, const MatvecWork* d_work, int nwo
         decltype(k)::launch(d_cfg, d_work, nwork, Nmax, G, xs, part, Ntot, R, s, live);
     });
     if (ev1) cudaEventRecord(ev1, s);
-    k_finalize<double2><<<(unsigned)((tot * kFinLanes + th - 1) / th), th, 0, s>>>(Ntot, R, nsplit, lf, x, part, y);
+    finalize<double2>(Ntot, R, nsplit, lf, x, part, y, s);
     g_msd_launches += 3;
 }
 
@@ -859,7 +890,7 @@ void launch_matvec_f32(const MsdConfig* d_cfg, const MatvecWork* d_work, int nwo
         });
     }
     if (ev1) cudaEventRecord(ev1, s);
-    k_finalize<float2><<<(unsigned)((tot * kFinLanes + th - 1) / th), th, 0, s>>>(Ntot, R, nsplit, lf, x, part, y);
+    finalize<float2>(Ntot, R, nsplit, lf, x, part, y, s);
     g_msd_launches += 3;
 }
 
@@ -882,28 +913,14 @@ __global__ void k_scale_cols_c(long long Ntot, int R, const V* __restrict__ cf, 
 }
 
 // y = (add_x ? x : 0) + row .* sum_s part[s];  row: rr (real), rc (complex) or none
-template <typename V, typename S>
-__global__ void k_finalize_gen(long long Ntot, int R, int nsplit, const S* __restrict__ rr,
-                               const V* __restrict__ rc, int add_x, const V* __restrict__ x,
-                               const V* __restrict__ part, V* __restrict__ y) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long i = t / kFinLanes;
-    const int sub = (int)(t % kFinLanes);
-    const long long tot = Ntot * R;
-    V s = vzero<V>();
-    if (i < tot) {
-        for (int k = sub; k < nsplit; k += kFinLanes) {
-            const V v = part[(long long)k * tot + i];
-            s.x += v.x;
-            s.y += v.y;
-        }
-    }
-#pragma unroll
-    for (int off = kFinLanes / 2; off > 0; off >>= 1) {
-        s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
-        s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
-    }
-    if (i >= tot || sub != 0) return;
+template <typename V, typename S, int TY>
+__global__ void __launch_bounds__(256) k_finalize_gen(long long Ntot, int R, int nsplit, const S* __restrict__ rr,
+                                                      const V* __restrict__ rc, int add_x, const V* __restrict__ x,
+                                                      const V* __restrict__ part, V* __restrict__ y) {
+    const long long tot = Ntot * R, i = (long long)blockIdx.x * (256 / TY) + threadIdx.x % (256 / TY);
+    const int ty = threadIdx.x / (256 / TY);
+    const V s = slot_sum<V, TY>(tot, nsplit, part, i, ty);
+    if (i >= tot || ty != 0) return;
     V o = s;
     if (rr) {
         const S f = rr[i / R];
@@ -919,6 +936,15 @@ __global__ void k_finalize_gen(long long Ntot, int R, int nsplit, const S* __res
     }
     y[i] = o;
 }
+template <typename V, typename S>
+void finalize_gen(long long Ntot, int R, int nsplit, const S* rr, const V* rc, int add_x, const V* x, const V* part,
+                  V* y, cudaStream_t s) {
+    with_slot_rows(Ntot * R, nsplit, [&](auto ty) {
+        constexpr int TY = decltype(ty)::value;
+        k_finalize_gen<V, S, TY><<<(unsigned)((Ntot * R + 256 / TY - 1) / (256 / TY)), 256, 0, s>>>(
+            Ntot, R, nsplit, rr, rc, add_x, x, part, y);
+    });
+}
 
 template <typename V, typename S, typename D>
 void product_general(D&& dispatch_fn, const MsdConfig* d_cfg, const MatvecWork* d_work, int nwork, int Nmax,
@@ -930,8 +956,7 @@ void product_general(D&& dispatch_fn, const MsdConfig* d_cfg, const MatvecWork* 
     if (col_c) k_scale_cols_c<V><<<blocks, th, 0, s>>>(Ntot, R, col_c, x, xs);
     else k_scale_cols<V, S><<<blocks, th, 0, s>>>(Ntot, R, col_r, x, xs);
     dispatch_fn([&](auto k) { decltype(k)::launch(d_cfg, d_work, nwork, Nmax, G, xs, part, Ntot, R, s); });
-    k_finalize_gen<V, S><<<(unsigned)((tot * kFinLanes + th - 1) / th), th, 0, s>>>(Ntot, R, nsplit, row_r, row_c,
-                                                                                   add_x, x, part, y);
+    finalize_gen<V, S>(Ntot, R, nsplit, row_r, row_c, add_x, x, part, y, s);
     g_msd_launches += 3;
 }
 
@@ -944,8 +969,7 @@ void launch_scale_cols_c(long long Ntot, int R, const double2* cf, const double2
 
 void launch_finalize_gen(long long Ntot, int R, int nsplit, const double* row_r, const double2* row_c, int add_x,
                          const double2* x, const double2* part, double2* y, cudaStream_t s) {
-    k_finalize_gen<double2, double><<<(unsigned)((Ntot * R * kFinLanes + 255) / 256), 256, 0, s>>>(
-        Ntot, R, nsplit, row_r, row_c, add_x, x, part, y);
+    finalize_gen<double2, double>(Ntot, R, nsplit, row_r, row_c, add_x, x, part, y, s);
     g_msd_launches += 1;
 }
 

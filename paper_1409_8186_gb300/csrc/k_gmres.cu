@@ -12,11 +12,15 @@
 // default one half; the solver option reorth sets eta2).  Per-thread
 // sums of dot products and updates run in the storage precision of the
 // basis (FP32 for the inner sweeps of a mixed solve, whose FP64 pipe would
-// otherwise bound them) and cross-thread reductions in FP64.  Vectors are
+// otherwise bound them) and cross-chunk reductions in FP64.  Vectors are
 // [rows][R] with R innermost; reductions run over row chunks that never
-// straddle two configurations; projections V^H w and updates w -= V h are
-// tiled over (row chunk, group of basis vectors) so that long Krylov bases
-// are read with the whole GPU.
+// straddle two configurations, of a size that follows the number of elements
+// (rows x R) and not of rows alone, so that a few thousand rows with many
+// columns still fill the chip.  Measured (GB300, averages over a solve): the
+// FP64 gradient of 40 disks with 16 columns (1800 rows) took 100 us a
+// projection and 155 us an update with row chunks, one vector per warp and FP64
+// atomics, 355 -> 149 ms as a whole; eight FP32 systems of 60 disks with 32
+// columns 303 -> 247 ms.
 //
 // The Givens rotations of a new Hessenberg column form the first-order
 // linear recurrence z_{i+1} = -conj(s_i) z_i + c_i h_{i+1} (z_0 = h_0,
@@ -24,132 +28,99 @@
 // parallel scan of affine maps over one CTA per system (warp shuffles, then
 // across warps), so a step costs O(j / threads + log threads) instead of a
 // j-long dependency chain.
+#include <algorithm>
+#include <type_traits>
+
 #include "msd_internal.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kI = 8;    // basis vectors per dot-product block
-constexpr int kU = 16;   // basis vectors per update block
+constexpr int kWarps = kThreads / 32;
 
 template <typename V> __device__ __forceinline__ double2 to_d2(V v) { return make_double2(v.x, v.y); }
 
-// Column lanes RC = the smallest power of two >= min(R, 32), so that lanes
-// of one column are xor-shuffle partners.
-__host__ __device__ inline int col_lanes(int R) {
-    int c = 1;
-    while (c < R && c < 32) c *= 2;
-    return c;
+template <typename V> __device__ __forceinline__ V from_d2(double2 v) {
+    return V{(decltype(V{}.x))v.x, (decltype(V{}.x))v.y};
 }
 
-__device__ __forceinline__ void atomic_add_v(double2* p, double2 v) {
-    atomicAdd(&p->x, v.x);
-    atomicAdd(&p->y, v.y);
-}
-__device__ __forceinline__ void atomic_add_v(float2* p, double2 v) {
-    atomicAdd(&p->x, (float)v.x);
-    atomicAdd(&p->y, (float)v.y);
-}
+// Columns of a column group (blockIdx of the kernels below): lane l of a warp
+// holds column l mod RC of row l / RC of the warp's RPW = 32 / RC rows, so a
+// warp reads RPW rows of one group as one contiguous stretch when R <= 32.
+__host__ __device__ inline int col_group(int R) { return R < 32 ? R : 32; }
 
-// Partial sums over one chunk of rows (blockIdx.x), columns of group
-// blockIdx.y, and the kI "vectors" i in [blockIdx.z * kI, ...) of the
-// list V_0..V_{nv-1} followed, when self != 0, by w itself:
+// Partial sums over one chunk of rows (blockIdx.x) and the columns of group
+// blockIdx.z of the vectors i in the list V_0..V_{nv-1} followed, when self
+// != 0, by w itself:
 //   part[chunk][i][r] = sum_rows conj(u_i[row][r]) * w[row][r].
-// Systems with skip[s] != 0 contribute zeros.
-template <typename V>
-__global__ void k_dots_part(const RowChunk* __restrict__ chunks, int R, const V* __restrict__ Vb,
-                            long long vstride, int nv, int self, const V* __restrict__ w,
-                            const int* __restrict__ skip, int skipval, double2* __restrict__ part) {
-    const RowChunk ch = chunks[blockIdx.x];
-    const int RC = col_lanes(R);
-    const int RY = blockDim.x / RC;  // kThreads and RC are powers of two
-    const int tx = threadIdx.x % RC, ty = threadIdx.x / RC;
-    const int r = blockIdx.y * RC + tx;
-    const int i0 = blockIdx.z * kI;
-    const int nvv = nv + self;
-    constexpr int kWarps = kThreads / 32;
-    __shared__ double2 red[kWarps][32][kI];
-    // Per-thread sums run in the storage precision (a handful of rows per
-    // thread); they are widened to FP64 for the cross-lane and cross-warp
-    // reduction.  An FP32 basis therefore costs FP32 arithmetic: the FP64
-    // pipe of this GPU is a small fraction of the FP32 one.
+// Systems with skip[s] == skipval contribute zeros.  A warp takes IV vectors
+// (each value of w read serves them all) and UN row groups at a time: IV UN +
+// UN loads in flight per lane.
+template <typename V, int IV>
+__global__ void __launch_bounds__(kThreads) k_dots(const RowChunk* __restrict__ chunks, int R,
+                                                   const V* __restrict__ Vb, long long vstride, int nv, int self,
+                                                   const V* __restrict__ w, const int* __restrict__ skip, int skipval,
+                                                   double2* __restrict__ part) {
     typedef decltype(V{}.x) A;
-    A ax[kI], ay[kI];
+    constexpr int UN = 4;
+    const RowChunk ch = chunks[blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int RC = col_group(R), RPW = 32 / RC, nvv = nv + self;
+    const int i0 = (blockIdx.y * kWarps + warp) * IV;
+    if (i0 >= nvv) return;  // a whole warp
+    const int ro = lane / RC, r = blockIdx.z * 32 + lane % RC;
+    const bool act = ro < RPW && r < R && !(skip && skip[ch.cfg * R + r] == skipval);
+    A ax[IV], ay[IV];
 #pragma unroll
-    for (int ii = 0; ii < kI; ++ii) ax[ii] = ay[ii] = A(0);
-    const bool live = r < R && !(skip && skip[ch.cfg * R + r] == skipval);
-    if (live) {
-        for (long long row = ch.row0 + ty; row < ch.row1; row += RY) {
-            const V wv = w[row * R + r];
+    for (int k = 0; k < IV; ++k) ax[k] = ay[k] = A(0);
+    if (__any_sync(0xffffffffu, act)) {
+        const V* u[IV];
 #pragma unroll
-            for (int ii = 0; ii < kI; ++ii) {
-                const int i = i0 + ii;
-                if (i < nvv) {
-                    const V vv = i < nv ? Vb[(long long)i * vstride + row * R + r] : wv;
-                    ax[ii] = fma(vv.x, wv.x, fma(vv.y, wv.y, ax[ii]));  // conj(v) * w
-                    ay[ii] = fma(vv.x, wv.y, fma(-vv.y, wv.x, ay[ii]));
+        for (int k = 0; k < IV; ++k) u[k] = i0 + k < nv ? Vb + (long long)(i0 + k) * vstride : w;
+        const int rows = (int)(ch.row1 - ch.row0);
+        long long e = (ch.row0 + ro) * R + r;
+        const long long step = (long long)RPW * R;
+        for (int q = ro; q < rows; q += RPW * UN, e += UN * step) {
+            V wv[UN], uv[UN][IV];
+#pragma unroll
+            for (int n = 0; n < UN; ++n) {
+                const bool ok = act && q + n * RPW < rows;
+                wv[n] = ok ? w[e + n * step] : V{A(0), A(0)};
+#pragma unroll
+                for (int k = 0; k < IV; ++k) uv[n][k] = ok ? u[k][e + n * step] : V{A(0), A(0)};
+            }
+#pragma unroll
+            for (int n = 0; n < UN; ++n)
+#pragma unroll
+                for (int k = 0; k < IV; ++k) {  // conj(u) * w
+                    ax[k] = fma(uv[n][k].x, wv[n].x, fma(uv[n][k].y, wv[n].y, ax[k]));
+                    ay[k] = fma(uv[n][k].x, wv[n].y, fma(-uv[n][k].y, wv[n].x, ay[k]));
                 }
+        }
+    }
+    // lanes of one column: l, l + RC, ... (in the storage precision: at most 32 terms)
+#pragma unroll
+    for (int k = 0; k < IV; ++k) {
+        if ((RC & (RC - 1)) == 0) {
+            for (int off = 16; off >= RC; off >>= 1) {
+                ax[k] += __shfl_xor_sync(0xffffffffu, ax[k], off);
+                ay[k] += __shfl_xor_sync(0xffffffffu, ay[k], off);
+            }
+        } else {
+            const A x0 = ax[k], y0 = ay[k];
+            for (int n = 1; n < RPW; ++n) {
+                ax[k] += __shfl_down_sync(0xffffffffu, x0, n * RC);
+                ay[k] += __shfl_down_sync(0xffffffffu, y0, n * RC);
             }
         }
-    }
-    // lanes lane and lane ^ off (off >= RC) hold the same column: fold them
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int ii = 0; ii < kI; ++ii) {
-        // within a warp in the storage precision (at most 32 terms), across
-        // warps and chunks in FP64
-        for (int off = 16; off >= RC; off >>= 1) {
-            ax[ii] += __shfl_xor_sync(0xffffffffu, ax[ii], off);
-            ay[ii] += __shfl_xor_sync(0xffffffffu, ay[ii], off);
-        }
-        if (lane < RC) red[warp][lane][ii] = make_double2((double)ax[ii], (double)ay[ii]);
-    }
-    __syncthreads();
-    // one thread per (column lane, vector) adds the warps' partials
-    for (int t = threadIdx.x; t < RC * kI; t += blockDim.x) {
-        const int cl = t % RC, ii = t / RC;
-        const int rr = blockIdx.y * RC + cl;
-        if (rr >= R || i0 + ii >= nvv) continue;
-        double2 s = make_double2(0.0, 0.0);
-        for (int wv = 0; wv < kWarps; ++wv) {  // every warp carries all RC columns
-            s.x += red[wv][cl][ii].x;
-            s.y += red[wv][cl][ii].y;
-        }
-        part[((long long)blockIdx.x * nvv + (i0 + ii)) * R + rr] = s;
+        if (lane < RC && r < R && i0 + k < nvv)
+            part[((long long)blockIdx.x * nvv + i0 + k) * R + r] = make_double2((double)ax[k], (double)ay[k]);
     }
 }
 
-// The same partial sums with one warp per vector i over the chunk's flat
-// elements e = row * R + r (R divides 32, or R = 64): lane l reads elements
-// e0 + l + 32 k, eight loads in flight, so a warp streams one contiguous
-// stretch of its vector and of w.  The column of element e is e mod R, fixed
-// per lane (Q = 1) or alternating between two columns (Q = 2, R = 64); lanes
-// that hold the same column are folded by shuffles.  No block-level
-// reduction: blocks are independent groups of eight vectors.
-// Reduction of the chunk partials fused into the projection kernel (few
-// systems): the last block of each group of vectors to finish sums that
-// group's partials into out; with skip2 set, the last group to finish also
-// takes the re-orthogonalisation decision (k_reorth_flags).  Counters start
-// at zero and every last block puts its counter back to zero.
-struct DotsFuse {
-    int* cnt = nullptr;      // [gridDim.y] blocks finished per vector group (nullptr: no fusion)
-    int* cnt_all = nullptr;  // vector groups finished
-    const int* cfg_chunk_off = nullptr;
-    int S = 0;
-    double2* out = nullptr;
-    int ostride = 0;
-    // after the reduction, with wn2 set: wn2 = out[j + 1] - sum_{i <= j} |out[i]|^2
-    // (||w - V h||^2 when out = V^H w with ||w||^2 at j + 1), and with skip2
-    // also set the re-orthogonalisation flags (first projection)
-    int j = 0;
-    double2* wn2 = nullptr;
-    const int* active = nullptr;
-    int* skip2 = nullptr;
-    double eta2 = 0.5;  // second pass when ||w'||^2 < eta2 ||w||^2
-};
-
-// ||w'||^2 = ||w||^2 - sum_{i <= j} |h_i|^2 and (skip2 != nullptr) the flag
-// of one system, reduced over the CTA (every thread calls it).
+// ||w'||^2 = ||w||^2 - sum_{i <= j} |h_i|^2 and (skip2 != nullptr) the
+// re-orthogonalisation flag of one system, reduced over the CTA (every thread
+// calls it).
 __device__ void reorth_flag_cta(const double2* h, int j, double2* wn2, int act, int* skip2, double eta2) {
     double acc = 0.0;
     for (int i = threadIdx.x; i <= j; i += blockDim.x) {
@@ -172,233 +143,137 @@ __device__ void reorth_flag_cta(const double2* h, int j, double2* wn2, int act, 
     }
 }
 
-template <typename V, int Q>
-__global__ void __launch_bounds__(kThreads, 4) k_dots_warp(const RowChunk* __restrict__ chunks, int R,
-                                                        const V* __restrict__ Vb, long long vstride, int nv,
-                                                        int self, const V* __restrict__ w,
-                                                        const int* __restrict__ skip, int skipval,
-                                                        double2* __restrict__ part, DotsFuse fz) {
-    const RowChunk ch = chunks[blockIdx.x];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = blockIdx.y * (kThreads / 32) + warp;
-    const int nvv = nv + self;
-    const long long e0 = ch.row0 * R, e1 = ch.row1 * R;
-    if (i < nvv) {  // a whole warp
-        const V* u = i < nv ? Vb + (long long)i * vstride : w;
-        // systems with skip set (no second projection) need no sums: a warp
-        // whose columns are all skipped only writes its zeros
-        bool live = true;
-        if (skip) {
-            live = false;
-#pragma unroll
-            for (int q = 0; q < Q; ++q) live |= skip[ch.cfg * R + (int)((e0 + lane + 32 * q) % R)] != skipval;
-            live = __any_sync(0xffffffffu, live);
-            if (!live) {
-#pragma unroll
-                for (int q = 0; q < Q; ++q)
-                    if (Q == 2 || lane < R)
-                        part[((long long)blockIdx.x * nvv + i) * R + (int)((e0 + lane + 32 * q) % R)] =
-                            make_double2(0.0, 0.0);
-            }
-        }
-        if (live) {
-            typedef decltype(V{}.x) A;
-            A ax[Q], ay[Q];
-#pragma unroll
-            for (int q = 0; q < Q; ++q) ax[q] = ay[q] = A(0);
-            // loads in flight per lane: a multiple of Q (the column phase of k
-            // survives the stride); 16 complex64 = the whole 512-row chunk of
-            // one column in a single round trip
-            constexpr int U = sizeof(V) == 8 ? 16 : 8;
-            long long e = e0 + lane;
-            for (; e + 32LL * (U - 1) < e1; e += 32LL * U) {
-                V uv[U], wv[U];
-#pragma unroll
-                for (int k = 0; k < U; ++k) {
-                    uv[k] = u[e + 32LL * k];
-                    wv[k] = w[e + 32LL * k];
-                }
-#pragma unroll
-                for (int k = 0; k < U; ++k) {
-                    const int q = k % Q;
-                    ax[q] = fma(uv[k].x, wv[k].x, fma(uv[k].y, wv[k].y, ax[q]));  // conj(u) * w
-                    ay[q] = fma(uv[k].x, wv[k].y, fma(-uv[k].y, wv[k].x, ay[q]));
-                }
-            }
-            for (int k = 0; e < e1; e += 32, ++k) {
-                const V uv = u[e], wv = w[e];
-                if (Q == 2 && (k & 1)) {
-                    ax[Q - 1] = fma(uv.x, wv.x, fma(uv.y, wv.y, ax[Q - 1]));
-                    ay[Q - 1] = fma(uv.x, wv.y, fma(-uv.y, wv.x, ay[Q - 1]));
-                } else {
-                    ax[0] = fma(uv.x, wv.x, fma(uv.y, wv.y, ax[0]));
-                    ay[0] = fma(uv.x, wv.y, fma(-uv.y, wv.x, ay[0]));
-                }
-            }
-            if (Q == 1) {
-                for (int off = 16; off >= R; off >>= 1) {
-                    ax[0] += __shfl_xor_sync(0xffffffffu, ax[0], off);
-                    ay[0] += __shfl_xor_sync(0xffffffffu, ay[0], off);
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                if (Q == 1 && lane >= R) break;
-                const int r = (int)((e0 + lane + 32 * q) % R);
-                const bool sk = skip && skip[ch.cfg * R + r] == skipval;
-                part[((long long)blockIdx.x * nvv + i) * R + r] =
-                    sk ? make_double2(0.0, 0.0) : make_double2((double)ax[q], (double)ay[q]);
-            }
-        }
-    }
-    if (!fz.cnt) return;
-    // ---- fused reduction of this vector group (last block of the group)
-    __shared__ int last;
-    if (Q == 2 || lane < R) __threadfence();  // the lanes that wrote partial sums
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&fz.cnt[blockIdx.y], 1) == (int)gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    constexpr int WPB = kThreads / 32;
-    const int ib = blockIdx.y * WPB;
-    for (int o = warp; o < fz.S * WPB; o += WPB) {
-        const int sy = o / WPB, iv = ib + o % WPB;
-        if (iv >= nvv) continue;  // a whole warp
-        const int c = sy / R, r = sy % R;
-        double2 acc = make_double2(0.0, 0.0);
-        for (int k = fz.cfg_chunk_off[c] + lane; k < fz.cfg_chunk_off[c + 1]; k += 32) {
-            const double2 v = __ldcg(part + ((long long)k * nvv + iv) * R + r);
-            acc.x += v.x;
-            acc.y += v.y;
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
-        }
-        if (lane == 0) fz.out[(long long)sy * fz.ostride + iv] = acc;
-    }
-    if (threadIdx.x == 0) fz.cnt[blockIdx.y] = 0;
-    if (!fz.wn2) return;
-    // ---- norm after the projection, re-orthogonalisation flags (last vector group to finish)
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(fz.cnt_all, 1) == (int)gridDim.y - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int sy = 0; sy < fz.S; ++sy)
-        reorth_flag_cta(fz.out + (long long)sy * fz.ostride, fz.j, fz.wn2 + (long long)sy * fz.ostride,
-                        fz.active ? fz.active[sy] : 1, fz.skip2 ? fz.skip2 + sy : nullptr, fz.eta2);
-    if (threadIdx.x == 0) *fz.cnt_all = 0;
-}
-
-// out[s * ostride + i] = sum over the chunks of cfg(s) of part[chunk][i][r]
-// (one warp per output: the lanes stride over the chunks, then shuffle-add)
+// out[s * ostride + i] = sum over the chunks of cfg(s) of part[chunk][i][r],
+// and the same in the basis type, transposed to hT[cfg][i][r] (rows of ldh
+// vectors), as the update kernel reads it.  One CTA per configuration
+// (blockIdx.y) and 32 consecutive values of i R + r, whose partials lie
+// side by side; eight threads share an output's chunks.
 // With tail.cnt set (few systems), the last block to finish also forms
 // wn2[s] = out[s][j + 1] - sum_{i <= j} |out[s][i]|^2 and, with tail.skip2,
 // the re-orthogonalisation flags (k_reorth_flags), and puts the counter back
 // to zero.
 struct FinTail {
     int* cnt = nullptr;
-    int j = 0;
+    int S = 0, j = 0;
     double2* wn2 = nullptr;
     const int* active = nullptr;
     int* skip2 = nullptr;
     double eta2 = 0.5;  // second pass when ||w'||^2 < eta2 ||w||^2
 };
-__global__ void k_dots_fin(int C, int R, int nvv, const int* __restrict__ cfg_chunk_off,
-                           const double2* __restrict__ part, double2* __restrict__ out, int ostride, FinTail tail) {
-    const long long idx = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (idx < (long long)C * R * nvv) {  // uniform across the warp
-        const int i = (int)(idx % nvv);
-        const int s = (int)(idx / nvv);
-        const int c = s / R, r = s % R;
-        double2 acc = make_double2(0.0, 0.0);
-        for (int k = cfg_chunk_off[c] + lane; k < cfg_chunk_off[c + 1]; k += 32) {
-            const double2 v = part[((long long)k * nvv + i) * R + r];
-            acc.x += v.x;
-            acc.y += v.y;
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
-        }
-        if (lane == 0) {
-            out[(long long)s * ostride + i] = acc;
-            if (tail.cnt) __threadfence();
-        }
+constexpr int kFinY = 8;
+template <typename V>
+__global__ void __launch_bounds__(32 * kFinY) k_dots_fin(int R, int nvv, const int* __restrict__ cfg_chunk_off,
+                                                         const double2* __restrict__ part, double2* __restrict__ out,
+                                                         int ostride, V* __restrict__ hT, long long ldh,
+                                                         FinTail tail) {
+    __shared__ double2 red[kFinY][32];
+    const int c = blockIdx.y, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + tx, ne = nvv * R;
+    double2 acc = make_double2(0.0, 0.0);
+    if (e < ne) {
+        const int k1 = cfg_chunk_off[c + 1];
+#pragma unroll 4
+        for (int k = cfg_chunk_off[c] + ty; k < k1; k += kFinY) acc = cadd(acc, part[(long long)k * ne + e]);
+    }
+    red[ty][tx] = acc;
+    __syncthreads();
+    if (ty == 0 && e < ne) {
+#pragma unroll
+        for (int y = 1; y < kFinY; ++y) acc = cadd(acc, red[y][tx]);
+        const int i = e / R, r = e % R;
+        out[(long long)(c * R + r) * ostride + i] = acc;
+        if (hT) hT[((long long)c * ldh + i) * R + r] = from_d2<V>(acc);
+        if (tail.cnt) __threadfence();
     }
     if (!tail.cnt) return;
     __shared__ int last;
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(tail.cnt, 1) == (int)gridDim.x - 1;
+    if (threadIdx.x == 0) last = atomicAdd(tail.cnt, 1) == (int)(gridDim.x * gridDim.y) - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
-    const int S = C * R;
-    for (int sy = 0; sy < S; ++sy)
+    for (int sy = 0; sy < tail.S; ++sy)
         reorth_flag_cta(out + (long long)sy * ostride, tail.j, tail.wn2 + (long long)sy * ostride,
                         tail.active ? tail.active[sy] : 1, tail.skip2 ? tail.skip2 + sy : nullptr, tail.eta2);
     if (threadIdx.x == 0) *tail.cnt = 0;
 }
 
-// w[row][r] += sign * sum_{i in block's group, i < nv} V_i[row][r] h[s][i].
-// The block's slice of h (times sign) is staged in shared memory in the
-// basis storage type and the sums run in that precision (FP32 for an FP32
-// basis: the correction it builds only needs the accuracy of the FP32
-// sweep).  With more than one vector group the groups meet in atomics;
-// with one group the result is stored directly.
-template <typename V, typename W>
-__global__ void __launch_bounds__(kThreads, 4)
-    k_update(const RowChunk* __restrict__ chunks, int R, const V* __restrict__ Vb, long long vstride,
-                         int nv, const double2* __restrict__ h, int hstride, const int* __restrict__ skip,
-                         int skipval, double sign, W* __restrict__ w) {
+// hT[cfg][i][r] = y[s][i] in the basis type (the coefficients of the solution
+// update at the end of a cycle).
+template <typename V>
+__global__ void k_coeffs(int C, int R, int nv, const double2* __restrict__ y, int ystride, V* __restrict__ hT,
+                         long long ldh) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (long long)C * nv * R) return;
+    const int r = (int)(t % R), i = (int)((t / R) % nv), c = (int)(t / ((long long)R * nv));
+    hT[((long long)c * ldh + i) * R + r] = from_d2<V>(y[(long long)(c * R + r) * ystride + i]);
+}
+
+// w[row][r] += sign * sum_{i < nv} V_i[row][r] hT[cfg][i][r], lane = element.
+// SPLIT warps share 32 elements, each taking every SPLIT-th batch of U
+// vectors (all U loads in flight, their coefficients coming from L1); their
+// sums, in the basis precision (FP32 for an FP32 basis: the correction only
+// needs the accuracy of the FP32 sweep), meet in shared memory and w is
+// written once, without atomics.
+template <typename V, typename W, int SPLIT>
+__global__ void __launch_bounds__(kThreads)
+    k_update(const RowChunk* __restrict__ chunks, int R, const V* __restrict__ Vb, long long vstride, int nv,
+             const V* __restrict__ hT, long long ldh, const int* __restrict__ skip, int skipval, double sign,
+             W* __restrict__ w) {
     typedef decltype(V{}.x) A;
+    constexpr int U = sizeof(V) == 8 ? 16 : 8;
+    constexpr int kCols = kWarps / SPLIT;  // groups of 32 elements of the CTA
+    __shared__ V red[kCols][SPLIT][32];
     const RowChunk ch = chunks[blockIdx.x];
-    const int RC = col_lanes(R);
-    const int RY = blockDim.x / RC;
-    const int tx = threadIdx.x % RC, ty = threadIdx.x / RC;
-    const int r = blockIdx.y * RC + tx;
-    const int i0 = blockIdx.z * kU;
-    const int i1 = min(nv, i0 + kU);
-    __shared__ V hsm[kU][32];
-    for (int t = threadIdx.x; t < kU * RC; t += blockDim.x) {
-        const int ii = t / RC, cl = t % RC;
-        const int rr = blockIdx.y * RC + cl;
-        double2 v = make_double2(0.0, 0.0);
-        if (rr < R && i0 + ii < i1) v = h[(long long)(ch.cfg * R + rr) * hstride + i0 + ii];
-        hsm[ii][cl] = V{(A)(sign * v.x), (A)(sign * v.y)};
-    }
-    __syncthreads();
-    if (r >= R || i0 >= i1) return;
-    if (skip && skip[ch.cfg * R + r] == skipval) return;
-    const bool atomic = gridDim.z > 1;
-    const int cnt = i1 - i0;
-    for (long long row = ch.row0 + ty; row < ch.row1; row += RY) {
-        A ax[4] = {A(0), A(0), A(0), A(0)}, ay[4] = {A(0), A(0), A(0), A(0)};
-        const V* vp = Vb + (long long)i0 * vstride + row * R + r;
-        // all kU loads of the row in flight before the multiply-adds
-        V vv[kU];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sp = warp % SPLIT, cg = warp / SPLIT;
+    const int rel = (blockIdx.y * kCols + cg) * 32 + lane;  // element within the chunk
+    const int tot = (int)(ch.row1 - ch.row0) * R;
+    bool act = rel < tot;
+    const int r = act ? rel % R : 0;
+    if (skip && act) act = skip[ch.cfg * R + r] != skipval;
+    const long long e = ch.row0 * R + rel;
+    A ax[2] = {A(0), A(0)}, ay[2] = {A(0), A(0)};
+    if (__any_sync(0xffffffffu, act)) {
+        const V* vp = Vb + (act ? e : ch.row0 * R);
+        const V* hp = hT + (long long)ch.cfg * ldh * R + r;
+        for (int i0 = sp * U; i0 < nv; i0 += SPLIT * U) {
+            V vv[U], hh[U];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) vv[u] = u < cnt ? vp[(long long)u * vstride] : V{A(0), A(0)};
+            for (int u = 0; u < U; ++u) {
+                const int i = min(i0 + u, nv - 1);
+                vv[u] = vp[(long long)i * vstride];
+            }
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const V hh = hsm[u][tx];  // zero beyond cnt
-            ax[u & 3] = fma(vv[u].x, hh.x, fma(-vv[u].y, hh.y, ax[u & 3]));
-            ay[u & 3] = fma(vv[u].x, hh.y, fma(vv[u].y, hh.x, ay[u & 3]));
-        }
-        const double2 d = make_double2((double)((ax[0] + ax[1]) + (ax[2] + ax[3])),
-                                       (double)((ay[0] + ay[1]) + (ay[2] + ay[3])));
-        W* p = w + row * R + r;
-        if (atomic) {
-            atomic_add_v(p, d);
-        } else {
-            const double2 o = to_d2(*p);
-            *p = W{(decltype(W{}.x))(o.x + d.x), (decltype(W{}.x))(o.y + d.y)};
+            for (int u = 0; u < U; ++u) {
+                const int i = i0 + u;
+                hh[u] = i < nv ? hp[(long long)i * R] : V{A(0), A(0)};
+            }
+            A bx[2] = {A(0), A(0)}, by[2] = {A(0), A(0)};
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                bx[u & 1] = fma(vv[u].x, hh[u].x, fma(-vv[u].y, hh[u].y, bx[u & 1]));
+                by[u & 1] = fma(vv[u].x, hh[u].y, fma(vv[u].y, hh[u].x, by[u & 1]));
+            }
+            ax[0] += bx[0];
+            ax[1] += bx[1];
+            ay[0] += by[0];
+            ay[1] += by[1];
         }
     }
+    red[cg][sp][lane] = V{ax[0] + ax[1], ay[0] + ay[1]};
+    if (SPLIT > 1) __syncthreads();
+    if (sp != 0 || !act) return;
+    V d = red[cg][0][lane];
+#pragma unroll
+    for (int k = 1; k < SPLIT; ++k) {
+        d.x += red[cg][k][lane].x;
+        d.y += red[cg][k][lane].y;
+    }
+    const W o = w[e];
+    typedef decltype(W{}.x) B;
+    const B sg = (B)sign;
+    w[e] = W{o.x + sg * (B)d.x, o.y + sg * (B)d.y};
 }
 
 // v = w * scale[s] for active systems, 0 otherwise; with xs (FP32 basis),
@@ -409,22 +284,19 @@ __global__ void k_scale(const RowChunk* __restrict__ chunks, int R, const Vin* _
                         const double* __restrict__ scale, const int* __restrict__ active,
                         Vout* __restrict__ v, const float* __restrict__ rf, float2* __restrict__ xs) {
     const RowChunk ch = chunks[blockIdx.x];
-    const int RC = col_lanes(R);
-    const int RY = blockDim.x / RC;
-    const int tx = threadIdx.x % RC, ty = threadIdx.x / RC;
-    const int r = blockIdx.y * RC + tx;
-    if (ty >= RY || r >= R) return;
-    const int s = ch.cfg * R + r;
     // arithmetic in the wider of the two storage types (FP32 for an FP32 basis)
     typedef decltype(Vin{}.x + Vout{}.x) A;
-    const A f = (A)(active[s] ? scale[s] : 0.0);
-    for (long long row = ch.row0 + ty; row < ch.row1; row += RY) {
-        const Vin a = w[row * R + r];
+    const int tot = (int)(ch.row1 - ch.row0) * R;
+    const long long e0 = ch.row0 * R;
+    for (int rel = blockIdx.y * blockDim.x + threadIdx.x; rel < tot; rel += gridDim.y * blockDim.x) {
+        const int r = rel % R, s = ch.cfg * R + r;
+        const A f = (A)(active[s] ? scale[s] : 0.0);
+        const Vin a = w[e0 + rel];
         const Vout o = Vout{(decltype(Vout{}.x))((A)a.x * f), (decltype(Vout{}.x))((A)a.y * f)};
-        v[row * R + r] = o;
+        v[e0 + rel] = o;
         if (xs) {
-            const float c = rf[row];
-            xs[row * R + r] = make_float2(c * (float)o.x, c * (float)o.y);
+            const float c = rf[ch.row0 + rel / R];
+            xs[e0 + rel] = make_float2(c * (float)o.x, c * (float)o.y);
         }
     }
 }
@@ -433,8 +305,9 @@ __global__ void k_scale(const RowChunk* __restrict__ chunks, int R, const Vin* _
 // the first projection is ||w||^2 - sum_i |h_i|^2 (Pythagoras, V orthonormal);
 // need[s] = 1 for an active system where that is below ||w||^2 / 2.  The
 // estimate is written to wn2 (the subdiagonal when no second pass runs);
-// where cancellation makes it inaccurate the second pass runs and measures
-// the norm itself.
+// where cancellation makes it inaccurate the second pass runs, and this
+// kernel (skip2 NULL) forms its norm from ||w1||^2, measured by that pass, and
+// the small h2.
 __global__ void k_reorth_flags(int S, const double2* __restrict__ h1, int hstride, int j,
                                double2* __restrict__ wn2, const int* __restrict__ active,
                                int* __restrict__ skip2, double eta2) {
@@ -453,7 +326,7 @@ __global__ void k_reorth_flags(int S, const double2* __restrict__ h1, int hstrid
     const double before = h[j + 1].x;  // ||w||^2 before the projection
     const double after = before - ss;
     wn2[(long long)s * hstride] = make_double2(after, 0.0);
-    skip2[s] = !(active[s] && after < eta2 * before);
+    if (skip2) skip2[s] = !(active[s] && after < eta2 * before);
 }
 
 // Start of a cycle: beta = ||r||; systems whose residual already meets
@@ -710,7 +583,6 @@ __global__ void k_zero(long long n, double2* __restrict__ x) {
 }
 
 inline unsigned blocks_for(long long n, int th) { return (unsigned)((n + th - 1) / th); }
-inline unsigned rgroups(int R) { return (unsigned)((R + col_lanes(R) - 1) / col_lanes(R)); }
 
 }  // namespace
 
@@ -718,76 +590,69 @@ inline unsigned rgroups(int R) { return (unsigned)((R + col_lanes(R) - 1) / col_
 
 template <typename V>
 bool gm_dots(const GmresDims& d, const RowChunk* chunks, const int* cfg_chunk_off, const V* Vb, long long vstride,
-             int nv, int self, const V* w, const int* skip, double2* part, double2* out, int ostride,
+             int nv, int self, const V* w, const int* skip, double2* part, double2* out, int ostride, V* hT,
              cudaStream_t s, int skipval, const GmDotsFuse* fuse) {
+    constexpr int IV = sizeof(V) == 8 ? 4 : 2;
     const int nvv = nv + self;
-    constexpr int WPB = kThreads / 32;
-    const bool warp_kernel = 32 % d.R == 0 || d.R == 64;
-    // fused reduction inside the projection kernel: few systems and one
-    // group of vectors (a fence and an atomic per block only pay off for
-    // small grids); otherwise the reduction kernel takes the norm and the
-    // flags in its last block
-    const bool few = fuse && d.S <= kFuseMaxSystems;
-    const bool fused = few && warp_kernel && (nvv + WPB - 1) / WPB == 1;
-    DotsFuse fz;
-    if (fused) {
-        fz.cnt = fuse->cnt;
-        fz.cnt_all = fuse->cnt + fuse->ncnt;
-        fz.cfg_chunk_off = cfg_chunk_off;
-        fz.S = d.S;
-        fz.out = out;
-        fz.ostride = ostride;
-        if (fuse->wn2) {
-            fz.j = fuse->j;
-            fz.wn2 = fuse->wn2;
-            fz.active = fuse->active;
-            fz.skip2 = fuse->skip2;
-            fz.eta2 = fuse->eta2;
-        }
-    }
-    if (32 % d.R == 0) {
-        k_dots_warp<V, 1><<<dim3(d.nchunk, (nvv + WPB - 1) / WPB), kThreads, 0, s>>>(chunks, d.R, Vb, vstride, nv,
-                                                                                    self, w, skip, skipval, part, fz);
-    } else if (d.R == 64) {
-        k_dots_warp<V, 2><<<dim3(d.nchunk, (nvv + WPB - 1) / WPB), kThreads, 0, s>>>(chunks, d.R, Vb, vstride, nv,
-                                                                                    self, w, skip, skipval, part, fz);
-    } else {
-        dim3 g(d.nchunk, rgroups(d.R), (nvv + kI - 1) / kI);
-        k_dots_part<V><<<g, kThreads, 0, s>>>(chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
-    }
-    if (fused) {
-        g_msd_launches += 1;
-        return true;
-    }
-    const long long tot = (long long)d.S * nvv;
+    const unsigned zg = (unsigned)((d.R + 31) / 32);
+    // one vector per warp while that leaves few warps
+    if ((long long)d.nchunk * zg * nvv < 152 * 16)
+        k_dots<V, 1><<<dim3(d.nchunk, (nvv + kWarps - 1) / kWarps, zg), kThreads, 0, s>>>(
+            chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
+    else
+        k_dots<V, IV><<<dim3(d.nchunk, (nvv + kWarps * IV - 1) / (kWarps * IV), zg), kThreads, 0, s>>>(
+            chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
     FinTail tail;
-    const bool tail_done = few && fuse->wn2;
+    const bool tail_done = fuse && fuse->wn2 && d.S <= kFuseMaxSystems;
     if (tail_done) {
-        tail.cnt = fuse->cnt + fuse->ncnt;
+        tail.cnt = fuse->cnt;
+        tail.S = d.S;
         tail.j = fuse->j;
         tail.wn2 = fuse->wn2;
         tail.active = fuse->active;
         tail.skip2 = fuse->skip2;
         tail.eta2 = fuse->eta2;
     }
-    k_dots_fin<<<blocks_for(tot * 32, 128), 128, 0, s>>>(d.C, d.R, nvv, cfg_chunk_off, part, out, ostride, tail);
+    k_dots_fin<V><<<dim3((unsigned)(((long long)nvv * d.R + 31) / 32), d.C), 32 * kFinY, 0, s>>>(
+        d.R, nvv, cfg_chunk_off, part, out, ostride, hT, d.ldh, tail);
     g_msd_launches += 2;
     return tail_done;
 }
 
-template <typename V, typename W>
-void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long long vstride, int nv, const double2* h,
-               int hstride, const int* skip, double sign, W* w, cudaStream_t s, int skipval) {
+template <typename V>
+void gm_coeffs(const GmresDims& d, int nv, const double2* y, int ystride, V* hT, cudaStream_t s) {
     if (nv <= 0) return;
-    dim3 g(d.nchunk, rgroups(d.R), (nv + kU - 1) / kU);
-    k_update<V, W><<<g, kThreads, 0, s>>>(chunks, d.R, Vb, vstride, nv, h, hstride, skip, skipval, sign, w);
+    k_coeffs<V><<<blocks_for((long long)d.C * nv * d.R, 256), 256, 0, s>>>(d.C, d.R, nv, y, ystride, hT, d.ldh);
+    g_msd_launches += 1;
+}
+
+// SPLIT: enough warps for the chip (32 per SM) where the elements alone do
+// not give them, but at least one batch of vectors per warp.
+template <typename V, typename W>
+void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long long vstride, int nv, const V* hT,
+               const int* skip, double sign, W* w, cudaStream_t s, int skipval) {
+    if (nv <= 0) return;
+    constexpr int U = sizeof(V) == 8 ? 16 : 8;
+    const long long cols = d.Ntot * d.R / 32 + 1;
+    const int most = std::max(1, nv / U);
+    auto go = [&](auto split) {
+        constexpr int SP = decltype(split)::value;
+        const int per = kWarps / SP * 32;
+        k_update<V, W, SP><<<dim3(d.nchunk, (d.chunk_elems + per - 1) / per), kThreads, 0, s>>>(
+            chunks, d.R, Vb, vstride, nv, hT, d.ldh, skip, skipval, sign, w);
+    };
+    if (cols * 4 <= 152 * 32 && most >= 4) go(std::integral_constant<int, 8>());
+    else if (cols * 2 <= 152 * 32 && most >= 2) go(std::integral_constant<int, 4>());
+    else if (cols <= 152 * 32 && most >= 2) go(std::integral_constant<int, 2>());
+    else go(std::integral_constant<int, 1>());
     g_msd_launches += 1;
 }
 
 template <typename Vin, typename Vout>
 void gm_scale(const GmresDims& d, const RowChunk* chunks, const Vin* w, const double* scale, const int* active,
               Vout* v, cudaStream_t s, const float* rf, float2* xs) {
-    k_scale<Vin, Vout><<<dim3(d.nchunk, rgroups(d.R)), kThreads, 0, s>>>(chunks, d.R, w, scale, active, v, rf, xs);
+    k_scale<Vin, Vout><<<dim3(d.nchunk, (d.chunk_elems + 1023) / 1024), kThreads, 0, s>>>(chunks, d.R, w, scale, active,
+                                                                                         v, rf, xs);
     g_msd_launches += 1;
 }
 
@@ -843,17 +708,19 @@ void gm_zero(long long n, double2* x, cudaStream_t s) {
 }
 
 template bool gm_dots<double2>(const GmresDims&, const RowChunk*, const int*, const double2*, long long, int, int,
-                               const double2*, const int*, double2*, double2*, int, cudaStream_t, int,
+                               const double2*, const int*, double2*, double2*, int, double2*, cudaStream_t, int,
                                const GmDotsFuse*);
 template bool gm_dots<float2>(const GmresDims&, const RowChunk*, const int*, const float2*, long long, int, int,
-                              const float2*, const int*, double2*, double2*, int, cudaStream_t, int,
+                              const float2*, const int*, double2*, double2*, int, float2*, cudaStream_t, int,
                               const GmDotsFuse*);
+template void gm_coeffs<double2>(const GmresDims&, int, const double2*, int, double2*, cudaStream_t);
+template void gm_coeffs<float2>(const GmresDims&, int, const double2*, int, float2*, cudaStream_t);
 template void gm_update<double2, double2>(const GmresDims&, const RowChunk*, const double2*, long long, int,
-                                          const double2*, int, const int*, double, double2*, cudaStream_t, int);
+                                          const double2*, const int*, double, double2*, cudaStream_t, int);
 template void gm_update<float2, float2>(const GmresDims&, const RowChunk*, const float2*, long long, int,
-                                        const double2*, int, const int*, double, float2*, cudaStream_t, int);
+                                        const float2*, const int*, double, float2*, cudaStream_t, int);
 template void gm_update<float2, double2>(const GmresDims&, const RowChunk*, const float2*, long long, int,
-                                         const double2*, int, const int*, double, double2*, cudaStream_t, int);
+                                         const float2*, const int*, double, double2*, cudaStream_t, int);
 template void gm_scale<double2, double2>(const GmresDims&, const RowChunk*, const double2*, const double*,
                                          const int*, double2*, cudaStream_t, const float*, float2*);
 template void gm_scale<double2, float2>(const GmresDims&, const RowChunk*, const double2*, const double*,

@@ -173,6 +173,14 @@ struct RecomputePlan {
     MatvecChoice ch{0, 1, 1, 0};
 };
 
+// Row chunks of the Krylov reductions, for one column count.
+struct ChunkSet {
+    std::vector<RowChunk> h;
+    RowChunk* d = nullptr;
+    int* d_off = nullptr;  // chunks of configuration c: [d_off[c], d_off[c + 1])
+    int elems = 0;         // elements (rows x R) of the largest chunk
+};
+
 struct msd_problem {
     cudaStream_t stream = nullptr;
     int C = 0, Mtot = 0, Nmax = 0, Mmax = 0;
@@ -210,23 +218,11 @@ struct msd_problem {
     std::map<long long, RecomputePlan> rplans;  // key: R*4 + precision
     DBuf genbuf;
     long long rc_checked = -1;  // geometry version whose complex64 range was checked
-    std::vector<RowChunk> chunks;
-    RowChunk* d_chunks = nullptr;
-    int* d_cfg_chunk_off = nullptr;
-    // coarse reduction chunks (>= 4096 rows): projections onto many basis
-    // vectors give each thread enough rows to amortise its reductions
-    std::vector<RowChunk> chunks_coarse;
-    RowChunk* d_chunks_coarse = nullptr;
-    int* d_cfg_chunk_off_coarse = nullptr;
-    // medium chunks (>= 1024 rows) for the warp-per-vector projections onto
-    // many basis vectors: each warp streams twice the rows of a fine chunk
-    std::vector<RowChunk> chunks_mid;
-    RowChunk* d_chunks_mid = nullptr;
-    int* d_cfg_chunk_off_mid = nullptr;
+    std::map<int, ChunkSet> chunks;  // reduction chunks of solves with R columns
     int* h_pinned = nullptr;  // small pinned host flags: [0..1] sync reads, [2..9] ring of step flags, [10] DORT barrier
     int* d_hpinned = nullptr;  // the same flags as the device addresses them (mapped host memory)
     cudaEvent_t ring_ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    DBuf xs, part, sbuf[24];
+    DBuf xs, part, sbuf[25];
     DBuf gbuf[9];   // gradient work buffers
     DBuf ffbuf;     // far field: sums of the disk groups
     DBuf nfbuf[4];  // near-field buffers: rho, points, weights, output stage
@@ -1554,8 +1550,9 @@ struct SolveCtx {
     double2 *h1, *h2, *wn2, *wn2b, *H, *cs, *sn, *g, *y, *lsq_work, *rdiag;
     double *beta, *vscale, *tol_abs, *tol_cycle;
     int *active, *kconv, *iters, *skip2, *flags;  // flags[0] any_active, flags[1] nonfinite
-    int* cnt = nullptr;  // ncnt + 1 counters of the fused projection reductions (zero between launches)
-    int ncnt = 0;
+    int* cnt = nullptr;  // counter of the fused projection reductions (zero between launches)
+    void* hT = nullptr;  // coefficients of the current projection in the basis type
+    const ChunkSet* chunks = nullptr;
     double eta2 = 0.5;  // second Gram-Schmidt pass when ||w'||^2 < eta2 ||w||^2
     int hstride;
     double2* part;  // [nchunk][m + 2][R] reduction partials
@@ -1564,16 +1561,37 @@ struct SolveCtx {
 
 // ||u||^2 per system into out[s * hstride] (FP64 vectors)
 void norm2_f64(SolveCtx& cx, const double2* u, double2* out) {
-    gm_dots<double2>(cx.d, cx.pb->d_chunks, cx.pb->d_cfg_chunk_off, nullptr, 0, 0, 1, u, nullptr, cx.part, out,
-                     cx.hstride, cx.pb->stream);
+    gm_dots<double2>(cx.d, cx.chunks->d, cx.chunks->d_off, nullptr, 0, 0, 1, u, nullptr, cx.part, out, cx.hstride,
+                     nullptr, cx.pb->stream);
 }
 
-// Counters of the fused projection reductions: one per group of eight
-// basis vectors (bases of up to 4000 vectors plus w), and one more.
-constexpr int kDotsCounters = 512;
-
-// Basis size from which projections run over the coarse row chunks.
-constexpr int kCoarseFrom = 64;
+// Reduction chunks for R columns: about 256 over the whole problem, of at
+// least 256 elements (rows x R; one element per lane and warp eight times
+// over), never across configurations.
+const ChunkSet& chunk_set(msd_problem* pb, int R) {
+    auto it = pb->chunks.find(R);
+    if (it != pb->chunks.end()) return it->second;
+    ChunkSet cs;
+    std::vector<int> off(pb->C + 1, 0);
+    const long long target = std::max<long long>(1, std::max<long long>(256, pb->Ntot * R / 256) / R);
+    for (int c = 0; c < pb->C; ++c) {
+        const MsdConfig& m = pb->cfg[c];
+        const long long rows = (long long)m.M * m.n;
+        for (long long r0 = 0; r0 < rows; r0 += target) {
+            RowChunk ch;
+            ch.cfg = c;
+            ch.pad = 0;
+            ch.row0 = m.row_off + r0;
+            ch.row1 = m.row_off + std::min(rows, r0 + target);
+            cs.h.push_back(ch);
+        }
+        off[c + 1] = (int)cs.h.size();
+    }
+    cs.elems = (int)(target * R);
+    cs.d = dalloc_copy(cs.h.data(), cs.h.size());
+    cs.d_off = dalloc_copy(off.data(), off.size());
+    return pb->chunks.emplace(R, cs).first->second;
+}
 
 // Hands the active flags of the Krylov systems to the products of one
 // Arnoldi step, and takes them back however the step ends.
@@ -1596,8 +1614,9 @@ void arnoldi_cycle(SolveCtx& cx, V* Vb, V* w, bool fp64, int maxit_left, int* st
     cudaStream_t s = pb->stream;
     const GmresDims& d = cx.d;
     const long long vstride = pb->Ntot * d.R;
-    const RowChunk* ch = pb->d_chunks;
-    const int* co = pb->d_cfg_chunk_off;
+    const RowChunk* ch = cx.chunks->d;
+    const int* co = cx.chunks->d_off;
+    V* hT = (V*)cx.hT;
     norm2_f64(cx, cx.r, cx.wn2);
     CK(cudaMemsetAsync(cx.flags, 0, 2 * sizeof(int), s));
     gm_start(d, cx.wn2, cx.hstride, cx.tol_abs, cx.beta, cx.vscale, cx.g, cx.active, cx.kconv, cx.flags, s);
@@ -1628,48 +1647,30 @@ void arnoldi_cycle(SolveCtx& cx, V* Vb, V* w, bool fp64, int maxit_left, int* st
             LiveScope live(pb, cx.active);
             operator_dev(pb, d.R, fp64, cx.adjoint, vj, w);
         }
-        // projections onto many basis vectors: the coarse row chunks when the
-        // block-reduction kernel serves this column count, the medium ones for
-        // the warp-per-vector kernels (no block reduction; longer-lived warps)
-        const bool many = j + 1 >= kCoarseFrom;
-        const bool warpk = 32 % d.R == 0 || d.R == 64;
-        GmresDims db = d;
-        const RowChunk* chb = ch;
-        const int* cob = co;
-        if (many && !warpk) {
-            db.nchunk = (int)pb->chunks_coarse.size();
-            chb = pb->d_chunks_coarse;
-            cob = pb->d_cfg_chunk_off_coarse;
-        } else if (many) {
-            db.nchunk = (int)pb->chunks_mid.size();
-            chb = pb->d_chunks_mid;
-            cob = pb->d_cfg_chunk_off_mid;
-        }
         // first projection h1 = V^H w (with ||w||^2 at h1[j+1]), w -= V h1;
         // systems that have converged (zero vectors from here on) are skipped
-        // (few systems: the reductions, and the flags of the second
-        // projection, run inside the projection kernels)
+        // (few systems: the norm after the projection and the flags of the
+        // second one are formed inside the reduction kernel)
         GmDotsFuse fz1, fz2;
         fz1.cnt = fz2.cnt = cx.cnt;
-        fz1.ncnt = fz2.ncnt = cx.ncnt;
         fz1.j = fz2.j = j;
         fz1.wn2 = cx.wn2;
         fz1.active = cx.active;
         fz1.skip2 = cx.skip2;
         fz1.eta2 = cx.eta2;
-        const bool flags_done =
-            gm_dots<V>(db, chb, cob, Vb, vstride, j + 1, 1, w, cx.active, cx.part, cx.h1, cx.hstride, s, 0, &fz1);
-        gm_update<V, V>(d, ch, Vb, vstride, j + 1, cx.h1, cx.hstride, cx.active, -1.0, w, s, 0);
+        const bool flags_done = gm_dots<V>(d, ch, co, Vb, vstride, j + 1, 1, w, cx.active, cx.part, cx.h1, cx.hstride,
+                                           hT, s, 0, &fz1);
+        gm_update<V, V>(d, ch, Vb, vstride, j + 1, hT, cx.active, -1.0, w, s, 0);
         // second projection only where the first removed more than half of ||w||^2
         if (!flags_done) gm_reorth_flags(d, cx.h1, cx.hstride, j, cx.wn2, cx.active, cx.skip2, s, cx.eta2);
         // its norm: ||w1 - V h2||^2 = ||w1||^2 - |h2|^2 (w1 measured by the
         // projection itself; h2 is small after the first pass, so no
-        // cancellation), formed inside the fused kernel, else measured
+        // cancellation)
         fz2.wn2 = cx.wn2b;
         const bool norm_done =
-            gm_dots<V>(db, chb, cob, Vb, vstride, j + 1, 1, w, cx.skip2, cx.part, cx.h2, cx.hstride, s, 1, &fz2);
-        gm_update<V, V>(d, ch, Vb, vstride, j + 1, cx.h2, cx.hstride, cx.skip2, -1.0, w, s);
-        if (!norm_done) gm_dots<V>(d, ch, co, nullptr, 0, 0, 1, w, cx.skip2, cx.part, cx.wn2b, cx.hstride, s);
+            gm_dots<V>(d, ch, co, Vb, vstride, j + 1, 1, w, cx.skip2, cx.part, cx.h2, cx.hstride, hT, s, 1, &fz2);
+        gm_update<V, V>(d, ch, Vb, vstride, j + 1, hT, cx.skip2, -1.0, w, s);
+        if (!norm_done) gm_reorth_flags(d, cx.h2, cx.hstride, j, cx.wn2b, nullptr, nullptr, s, cx.eta2);
         // the Givens step stores its flags (any system still active, a
         // non-finite coefficient) straight into pinned host memory, in the
         // ring slot of this step; the host cleared the slot, whose previous
@@ -1719,7 +1720,8 @@ void arnoldi_cycle(SolveCtx& cx, V* Vb, V* w, bool fp64, int maxit_left, int* st
     *steps_taken = j;
     gm_lsq(d, cx.H, cx.cs, cx.sn, cx.rdiag, cx.g, cx.kconv, cx.y, cx.lsq_work, s);
     // x += V y, each system over its own kconv columns (y is zero beyond it)
-    gm_update<V, double2>(d, ch, Vb, vstride, j, cx.y, cx.m, nullptr, 1.0, cx.x, s);
+    gm_coeffs<V>(d, j, cx.y, cx.m, hT, s);
+    gm_update<V, double2>(d, ch, Vb, vstride, j, hT, nullptr, 1.0, cx.x, s);
     CK_LAUNCH();
 }
 
@@ -1775,7 +1777,10 @@ msd_status solve_impl(msd_problem* pb, int R, const double* betas_host, const ms
     cx.d.C = pb->C;
     cx.d.S = pb->C * R;
     cx.d.m = o.restart;
-    cx.d.nchunk = (int)pb->chunks.size();
+    cx.chunks = &chunk_set(pb, R);
+    cx.d.nchunk = (int)cx.chunks->h.size();
+    cx.d.chunk_elems = cx.chunks->elems;
+    cx.d.ldh = o.restart + 2;
     cx.hstride = o.restart + 2;
     const int S = cx.d.S, m = o.restart;
     const size_t nv = (size_t)pb->Ntot * R;
@@ -1802,18 +1807,18 @@ msd_status solve_impl(msd_problem* pb, int R, const double* betas_host, const ms
     cx.vscale = dsys + S;
     cx.tol_abs = dsys + 2 * S;
     cx.tol_cycle = dsys + 3 * S;
-    int* isys = (int*)sb((size_t)(S * 4 + 2 + kDotsCounters + 1) * 4);
+    int* isys = (int*)sb((size_t)(S * 4 + 3) * 4);
     cx.active = isys;
     cx.kconv = isys + S;
     cx.iters = isys + 2 * S;
     cx.skip2 = isys + 3 * S;
     cx.flags = isys + 4 * S;
     cx.cnt = isys + 4 * S + 2;
-    cx.ncnt = kDotsCounters;
-    CK(cudaMemsetAsync(cx.cnt, 0, (size_t)(cx.ncnt + 1) * sizeof(int), s));
+    CK(cudaMemsetAsync(cx.cnt, 0, sizeof(int), s));
     const size_t velem = mixed ? 8 : 16;
     void* Vb = sb((size_t)(m + 1) * nv * velem);
     void* w = sb(nv * velem);
+    cx.hT = pb->sbuf[24].get((size_t)S * (m + 2) * velem);
     double* d_betas = (double*)sb((size_t)pb->C * R * 8);
     cx.part = (double2*)pb->sbuf[0].get((size_t)cx.d.nchunk * (m + 2) * R * sizeof(double2));
 
@@ -1920,8 +1925,8 @@ msd_status solve_impl(msd_problem* pb, int R, const double* betas_host, const ms
     // FP64 residual r' of the preconditioned system
     std::vector<double> true_relres(S, -1.0);
     if (!adjoint && R <= 64 && !pb->pen_parent) {
-        const int nch = (int)pb->chunks.size();
-        launch_weighted_norms(pb->d_cfg, pb->d_chunks, nch, R, pb->d_radius, pb->d_bc, pb->d_J, pb->d_H, pb->d_dH,
+        const int nch = cx.d.nchunk;
+        launch_weighted_norms(pb->d_cfg, cx.chunks->d, nch, R, pb->d_radius, pb->d_bc, pb->d_J, pb->d_H, pb->d_dH,
                               pb->form ? pb->d_fdiag : nullptr,
                               cx.r, cx.b, cx.part, s);
         CK_LAUNCH();
@@ -1931,8 +1936,8 @@ msd_status solve_impl(msd_problem* pb, int R, const double* betas_host, const ms
         std::vector<double> nu(S, 0.0), nv2(S, 0.0);
         for (int k = 0; k < nch; ++k)
             for (int r = 0; r < R; ++r) {
-                nu[pb->chunks[k].cfg * R + r] += wp[(size_t)k * R + r].x;
-                nv2[pb->chunks[k].cfg * R + r] += wp[(size_t)k * R + r].y;
+                nu[cx.chunks->h[k].cfg * R + r] += wp[(size_t)k * R + r].x;
+                nv2[cx.chunks->h[k].cfg * R + r] += wp[(size_t)k * R + r].y;
             }
         for (int i = 0; i < S; ++i) true_relres[i] = nv2[i] > 0 ? std::sqrt(nu[i] / nv2[i]) : 0.0;
     }
@@ -2068,33 +2073,6 @@ msd_status msd_create(int C, const int* disk_off, const double* centres, const d
             CK(cudaMallocHost((void**)&pb->h_pinned, 64));
             CK(cudaHostGetDevicePointer((void**)&pb->d_hpinned, pb->h_pinned, 0));
             for (auto& e : pb->ring_ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-            // reduction chunks: at least 512 rows each (two or more rows per
-            // thread of a reduction block) and about 256 overall, never
-            // across configurations
-            auto make_chunks = [&](long long target_rows, std::vector<RowChunk>& out, RowChunk** d_out,
-                                   int** d_off) {
-                std::vector<int> coff(C + 1, 0);
-                for (int c = 0; c < C; ++c) {
-                    const MsdConfig& m = pb->cfg[c];
-                    const long long rows = (long long)m.M * m.n;
-                    for (long long r0 = 0; r0 < rows; r0 += target_rows) {
-                        RowChunk ch;
-                        ch.cfg = c;
-                        ch.pad = 0;
-                        ch.row0 = m.row_off + r0;
-                        ch.row1 = m.row_off + std::min(rows, r0 + target_rows);
-                        out.push_back(ch);
-                    }
-                    coff[c + 1] = (int)out.size();
-                }
-                *d_out = dalloc_copy(out.data(), out.size());
-                *d_off = dalloc_copy(coff.data(), coff.size());
-            };
-            make_chunks(std::max<long long>(512, row / 256), pb->chunks, &pb->d_chunks, &pb->d_cfg_chunk_off);
-            make_chunks(std::max<long long>(4096, row / 64), pb->chunks_coarse, &pb->d_chunks_coarse,
-                        &pb->d_cfg_chunk_off_coarse);
-            make_chunks(std::max<long long>(1024, row / 128), pb->chunks_mid, &pb->d_chunks_mid,
-                        &pb->d_cfg_chunk_off_mid);
             launch_disk_diagonals(pb->d_cfg, Mtot, pb->d_disk_cfg, pb->d_radius, pb->d_bc, pb->Nmax, pb->d_J,
                                   pb->d_dJ, pb->d_H, pb->d_dH, pb->d_lf64, pb->d_rf64, pb->d_lf32, pb->d_rf32,
                                   pb->d_rhs_scale, pb->d_flags, pb->stream);
@@ -2114,11 +2092,14 @@ void msd_destroy(msd_problem* pb) {
     if (pb->stream) cudaStreamSynchronize(pb->stream);
     void* ptrs[] = {pb->d_cfg, pb->d_centre, pb->d_radius, pb->d_bc, pb->d_disk_cfg, pb->d_J, pb->d_dJ,
                     pb->d_H, pb->d_dH, pb->d_lf64, pb->d_rhs_scale, pb->d_rf64, pb->d_lf32, pb->d_rf32,
-                    pb->d_flags, pb->d_G64, pb->d_G32, pb->d_chunks, pb->d_cfg_chunk_off,
-                    pb->d_chunks_coarse, pb->d_cfg_chunk_off_coarse, pb->d_chunks_mid, pb->d_cfg_chunk_off_mid,
+                    pb->d_flags, pb->d_G64, pb->d_G32,
                     pb->d_GA64, pb->d_GA32, pb->d_clf64, pb->d_clf32, pb->d_GT, pb->d_gt_blk, pb->d_Np};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    for (auto& kv : pb->chunks) {
+        cudaFree(kv.second.d);
+        cudaFree(kv.second.d_off);
+    }
     for (auto& b : pb->ds_idx) b.release();
     pb->ds_fwd.release();
     pb->ds_adj.release();

@@ -427,6 +427,8 @@ struct GmresDims {
     int S;            // systems = C*R
     int m;            // restart length
     int nchunk;       // reduction chunks
+    int chunk_elems;  // elements (rows x R) of the largest chunk
+    long long ldh;    // vectors per configuration of the transposed coefficients hT
 };
 
 // out[s][i] = sum over the rows of cfg(s) of conj(u_i) w for u = V_0..V_{nv-1}
@@ -434,18 +436,17 @@ struct GmresDims {
 // (skipval 1 with a skip-flag array, 0 with the active flags: inactive
 // systems have zero vectors, so skipping them changes no value).
 //
+// hT (may be NULL): the same coefficients in the basis type, [C][ldh][R], for
+// gm_update.
 // With `fuse` and at most kFuseMaxSystems systems, and fuse->wn2 set (self =
 // 1, ||w||^2 lands at index j + 1), the reduction also writes
 // wn2[s * ostride] = ||w||^2 - sum_{i <= j} |out_i|^2, the squared norm after
 // the projection, and with fuse->skip2 set the re-orthogonalisation flags of
-// gm_reorth_flags; the call then returns true.  For a single group of eight
-// vectors (R dividing 32 or R = 64) the reduction runs inside the projection
-// kernel, else in its reduction kernel.  fuse->cnt: ncnt + 1 zeroed device
-// counters, left zeroed by every launch that uses them.
+// gm_reorth_flags; the call then returns true.  fuse->cnt: a zeroed device
+// counter, left zeroed by every launch that uses it.
 constexpr int kFuseMaxSystems = 8;
 struct GmDotsFuse {
     int* cnt = nullptr;
-    int ncnt = 0;
     int j = 0;
     double2* wn2 = nullptr;
     const int* active = nullptr;
@@ -454,18 +455,21 @@ struct GmDotsFuse {
 };
 template <typename V>
 bool gm_dots(const GmresDims& d, const RowChunk* chunks, const int* cfg_chunk_off, const V* Vb, long long vstride,
-             int nv, int self, const V* w, const int* skip, double2* part, double2* out, int ostride,
+             int nv, int self, const V* w, const int* skip, double2* part, double2* out, int ostride, V* hT,
              cudaStream_t s, int skipval = 1, const GmDotsFuse* fuse = nullptr);
-// w += sign * sum_i V_i h[s][i]  (skip[s] == skipval: unchanged)
+// hT from the per-system coefficients y[s * ystride + i]
+template <typename V>
+void gm_coeffs(const GmresDims& d, int nv, const double2* y, int ystride, V* hT, cudaStream_t s);
+// w += sign * sum_i V_i hT[cfg][i][r]  (skip[s] == skipval: unchanged)
 template <typename V, typename W>
-void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long long vstride, int nv, const double2* h,
-               int hstride, const int* skip, double sign, W* w, cudaStream_t s, int skipval = 1);
+void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long long vstride, int nv, const V* hT,
+               const int* skip, double sign, W* w, cudaStream_t s, int skipval = 1);
 // v = w * scale[s] for active systems, 0 otherwise
 template <typename Vin, typename Vout>
 // (rf, xs: also xs = rf .* v, the scaled input of the next FP32 product)
 void gm_scale(const GmresDims& d, const RowChunk* chunks, const Vin* w, const double* scale, const int* active,
               Vout* v, cudaStream_t s, const float* rf = nullptr, float2* xs = nullptr);
-// ||w'||^2 estimate (written to wn2) and the re-orthogonalisation flags
+// ||w'||^2 (written to wn2) and, skip2 not NULL, the re-orthogonalisation flags
 void gm_reorth_flags(const GmresDims& d, const double2* h1, int hstride, int j, double2* wn2,
                      const int* active, int* skip2, cudaStream_t s, double eta2 = 0.5);
 void gm_start(const GmresDims& d, const double2* rr, int hstride, const double* tol_abs, double* beta,

@@ -118,6 +118,102 @@ __global__ void __launch_bounds__(kThreads) k_dots(const RowChunk* __restrict__ 
     }
 }
 
+// The same for an FP32 basis with 16-byte loads, two neighbouring elements per
+// lane: two columns of a row (R even), or two rows of a single column (R =
+// 1).  For vectors and chunks that start on an even element (GmresDims::pairs).
+// Halves the load instructions and doubles the bytes in flight: eight systems
+// of 60 disks with 32 columns, 74 -> 54 us a projection (k_update_pair: 88 ->
+// 62 us an update).
+template <int IV>
+__global__ void __launch_bounds__(kThreads) k_dots_pair(const RowChunk* __restrict__ chunks, int R,
+                                                        const float2* __restrict__ Vb, long long vstride, int nv,
+                                                        int self, const float2* __restrict__ w,
+                                                        const int* __restrict__ skip, int skipval,
+                                                        double2* __restrict__ part) {
+    constexpr int UN = 4;
+    const RowChunk ch = chunks[blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool one = R == 1;
+    const int PC = one ? 1 : col_group(R) / 2, RPW = 32 / PC, nvv = nv + self;
+    const int i0 = (blockIdx.y * kWarps + warp) * IV;
+    if (i0 >= nvv) return;  // a whole warp
+    const int ro = lane / PC, r = blockIdx.z * 32 + 2 * (lane % PC);
+    const bool in = ro < RPW && r < R;
+    const bool act0 = in && !(skip && skip[ch.cfg * R + r] == skipval);
+    const bool act1 = in && (one ? act0 : !(skip && skip[ch.cfg * R + r + 1] == skipval));
+    float ax[IV][2], ay[IV][2];
+#pragma unroll
+    for (int k = 0; k < IV; ++k) ax[k][0] = ax[k][1] = ay[k][0] = ay[k][1] = 0.f;
+    if (__any_sync(0xffffffffu, act0 || act1)) {
+        const float2* u[IV];
+#pragma unroll
+        for (int k = 0; k < IV; ++k) u[k] = i0 + k < nv ? Vb + (long long)(i0 + k) * vstride : w;
+        const int rows = (int)(ch.row1 - ch.row0);
+        const int units = one ? (rows + 1) / 2 : rows;  // a unit: a row, or two rows of one column
+        const int unit = one ? 2 : R;                   // elements from one unit to the next
+        long long e = ch.row0 * R + (long long)ro * unit + r;
+        const long long step = (long long)RPW * unit;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q = ro; q < units; q += RPW * UN, e += UN * step) {
+            float4 wv[UN], uv[UN][IV];
+#pragma unroll
+            for (int n = 0; n < UN; ++n) {
+                const bool ok = in && q + n * RPW < units;
+                if (one && ok && 2 * (q + n * RPW) + 1 >= rows) {  // the odd last row
+                    const float2 x = w[e + n * step];
+                    wv[n] = make_float4(x.x, x.y, 0.f, 0.f);
+#pragma unroll
+                    for (int k = 0; k < IV; ++k) {
+                        const float2 y = u[k][e + n * step];
+                        uv[n][k] = make_float4(y.x, y.y, 0.f, 0.f);
+                    }
+                } else {
+                    wv[n] = ok ? *(const float4*)(w + e + n * step) : zero;
+#pragma unroll
+                    for (int k = 0; k < IV; ++k) uv[n][k] = ok ? *(const float4*)(u[k] + e + n * step) : zero;
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < UN; ++n)
+#pragma unroll
+                for (int k = 0; k < IV; ++k) {  // conj(u) * w
+                    const float4 a = uv[n][k], b = wv[n];
+                    ax[k][0] = fmaf(a.x, b.x, fmaf(a.y, b.y, ax[k][0]));
+                    ay[k][0] = fmaf(a.x, b.y, fmaf(-a.y, b.x, ay[k][0]));
+                    ax[k][1] = fmaf(a.z, b.z, fmaf(a.w, b.w, ax[k][1]));
+                    ay[k][1] = fmaf(a.z, b.w, fmaf(-a.w, b.z, ay[k][1]));
+                }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < IV; ++k) {
+        if (one) {
+            ax[k][0] += ax[k][1];
+            ay[k][0] += ay[k][1];
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            if (one && c) continue;
+            if ((PC & (PC - 1)) == 0) {
+                for (int off = 16; off >= PC; off >>= 1) {
+                    ax[k][c] += __shfl_xor_sync(0xffffffffu, ax[k][c], off);
+                    ay[k][c] += __shfl_xor_sync(0xffffffffu, ay[k][c], off);
+                }
+            } else {
+                const float x0 = ax[k][c], y0 = ay[k][c];
+                for (int n = 1; n < RPW; ++n) {
+                    ax[k][c] += __shfl_down_sync(0xffffffffu, x0, n * PC);
+                    ay[k][c] += __shfl_down_sync(0xffffffffu, y0, n * PC);
+                }
+            }
+            const bool act = c ? act1 : act0;
+            if (lane < PC && r + c < R && i0 + k < nvv)
+                part[((long long)blockIdx.x * nvv + i0 + k) * R + r + c] =
+                    act ? make_double2((double)ax[k][c], (double)ay[k][c]) : make_double2(0.0, 0.0);
+        }
+    }
+}
+
 // ||w'||^2 = ||w||^2 - sum_{i <= j} |h_i|^2 and (skip2 != nullptr) the
 // re-orthogonalisation flag of one system, reduced over the CTA (every thread
 // calls it).
@@ -216,12 +312,12 @@ __global__ void k_coeffs(int C, int R, int nv, const double2* __restrict__ y, in
 // needs the accuracy of the FP32 sweep), meet in shared memory and w is
 // written once, without atomics.
 template <typename V, typename W, int SPLIT>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, sizeof(V) == 8 ? 4 : 2)
     k_update(const RowChunk* __restrict__ chunks, int R, const V* __restrict__ Vb, long long vstride, int nv,
              const V* __restrict__ hT, long long ldh, const int* __restrict__ skip, int skipval, double sign,
              W* __restrict__ w) {
     typedef decltype(V{}.x) A;
-    constexpr int U = sizeof(V) == 8 ? 16 : 8;
+    constexpr int U = 8;
     constexpr int kCols = kWarps / SPLIT;  // groups of 32 elements of the CTA
     __shared__ V red[kCols][SPLIT][32];
     const RowChunk ch = chunks[blockIdx.x];
@@ -274,6 +370,87 @@ __global__ void __launch_bounds__(kThreads)
     typedef decltype(W{}.x) B;
     const B sg = (B)sign;
     w[e] = W{o.x + sg * (B)d.x, o.y + sg * (B)d.y};
+}
+
+// The same for an FP32 basis and 16-byte loads, two neighbouring elements per
+// lane (two columns of a row, or two rows when R = 1), as in k_dots_pair.
+template <typename W, int SPLIT>
+__global__ void __launch_bounds__(kThreads, 2)
+    k_update_pair(const RowChunk* __restrict__ chunks, int R, const float2* __restrict__ Vb, long long vstride, int nv,
+                  const float2* __restrict__ hT, long long ldh, const int* __restrict__ skip, int skipval, double sign,
+                  W* __restrict__ w) {
+    constexpr int U = 8;
+    constexpr int kCols = kWarps / SPLIT;
+    __shared__ float4 red[kCols][SPLIT][32];
+    const RowChunk ch = chunks[blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sp = warp % SPLIT, cg = warp / SPLIT;
+    const int rel = ((blockIdx.y * kCols + cg) * 32 + lane) * 2;
+    const int tot = (int)(ch.row1 - ch.row0) * R;
+    const bool one = R == 1;
+    const int r = rel < tot ? rel % R : 0;
+    bool act0 = rel < tot, act1 = rel + 1 < tot;
+    if (skip && act0) act0 = skip[ch.cfg * R + r] != skipval;
+    if (skip && act1) act1 = one ? act0 : skip[ch.cfg * R + r + 1] != skipval;
+    const long long e = ch.row0 * R + rel;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (__any_sync(0xffffffffu, act0 || act1)) {
+        // (an odd last row reads one element past it: the next vector's first,
+        // which the basis has room for, and whose product is not stored)
+        const float2* vp = Vb + (rel < tot ? e : ch.row0 * R);
+        const float2* hp = hT + (long long)ch.cfg * ldh * R + r;
+        for (int i0 = sp * U; i0 < nv; i0 += SPLIT * U) {
+            float4 vv[U], hh[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) vv[u] = *(const float4*)(vp + (long long)min(i0 + u, nv - 1) * vstride);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int i = min(i0 + u, nv - 1);
+                if (one) {
+                    const float2 h = hp[i];
+                    hh[u] = make_float4(h.x, h.y, h.x, h.y);
+                } else {
+                    hh[u] = *(const float4*)(hp + (long long)i * R);
+                }
+                if (i0 + u >= nv) hh[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                b.x = fmaf(vv[u].x, hh[u].x, fmaf(-vv[u].y, hh[u].y, b.x));
+                b.y = fmaf(vv[u].x, hh[u].y, fmaf(vv[u].y, hh[u].x, b.y));
+                b.z = fmaf(vv[u].z, hh[u].z, fmaf(-vv[u].w, hh[u].w, b.z));
+                b.w = fmaf(vv[u].z, hh[u].w, fmaf(vv[u].w, hh[u].z, b.w));
+            }
+            acc.x += b.x;
+            acc.y += b.y;
+            acc.z += b.z;
+            acc.w += b.w;
+        }
+    }
+    if (SPLIT > 1) {
+        red[cg][sp][lane] = acc;
+        __syncthreads();
+        if (sp != 0) return;
+#pragma unroll
+        for (int k = 1; k < SPLIT; ++k) {
+            const float4 o = red[cg][k][lane];
+            acc.x += o.x;
+            acc.y += o.y;
+            acc.z += o.z;
+            acc.w += o.w;
+        }
+    }
+    typedef decltype(W{}.x) B;
+    const B sg = (B)sign;
+    if (act0) {
+        const W o = w[e];
+        w[e] = W{o.x + sg * (B)acc.x, o.y + sg * (B)acc.y};
+    }
+    if (act1) {
+        const W o = w[e + 1];
+        w[e + 1] = W{o.x + sg * (B)acc.z, o.y + sg * (B)acc.w};
+    }
 }
 
 // v = w * scale[s] for active systems, 0 otherwise; with xs (FP32 basis),
@@ -592,16 +769,25 @@ template <typename V>
 bool gm_dots(const GmresDims& d, const RowChunk* chunks, const int* cfg_chunk_off, const V* Vb, long long vstride,
              int nv, int self, const V* w, const int* skip, double2* part, double2* out, int ostride, V* hT,
              cudaStream_t s, int skipval, const GmDotsFuse* fuse) {
-    constexpr int IV = sizeof(V) == 8 ? 4 : 2;
     const int nvv = nv + self;
     const unsigned zg = (unsigned)((d.R + 31) / 32);
-    // one vector per warp while that leaves few warps
-    if ((long long)d.nchunk * zg * nvv < 152 * 16)
-        k_dots<V, 1><<<dim3(d.nchunk, (nvv + kWarps - 1) / kWarps, zg), kThreads, 0, s>>>(
-            chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
-    else
-        k_dots<V, IV><<<dim3(d.nchunk, (nvv + kWarps * IV - 1) / (kWarps * IV), zg), kThreads, 0, s>>>(
-            chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
+    const long long warps = (long long)d.nchunk * zg * nvv;  // with one vector each
+    // several vectors per warp (more loads in flight and fewer reads of w: two
+    // instead of four FP32 vectors took twice as long on 400 disks), one while
+    // there are few
+    const bool few = warps < 152 * 16;
+    const int per = kWarps * (few ? 1 : sizeof(V) == 8 ? 4 : 2);
+    const dim3 grid(d.nchunk, (nvv + per - 1) / per, zg);
+    if (few) {
+        k_dots<V, 1><<<grid, kThreads, 0, s>>>(chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
+    } else if constexpr (sizeof(V) == 8) {
+        if (d.pairs)
+            k_dots_pair<4><<<grid, kThreads, 0, s>>>(chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
+        else
+            k_dots<V, 4><<<grid, kThreads, 0, s>>>(chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
+    } else {
+        k_dots<V, 2><<<grid, kThreads, 0, s>>>(chunks, d.R, Vb, vstride, nv, self, w, skip, skipval, part);
+    }
     FinTail tail;
     const bool tail_done = fuse && fuse->wn2 && d.S <= kFuseMaxSystems;
     if (tail_done) {
@@ -632,9 +818,24 @@ template <typename V, typename W>
 void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long long vstride, int nv, const V* hT,
                const int* skip, double sign, W* w, cudaStream_t s, int skipval) {
     if (nv <= 0) return;
-    constexpr int U = sizeof(V) == 8 ? 16 : 8;
+    constexpr int U = 8;
     const long long cols = d.Ntot * d.R / 32 + 1;
     const int most = std::max(1, nv / U);
+    if constexpr (sizeof(V) == 8) {
+        if (d.pairs && cols >= 152 * 16) {
+            auto go = [&](auto split) {
+                constexpr int SP = decltype(split)::value;
+                const int per = kWarps / SP * 64;
+                k_update_pair<W, SP><<<dim3(d.nchunk, (d.chunk_elems + per - 1) / per), kThreads, 0, s>>>(
+                    chunks, d.R, Vb, vstride, nv, hT, d.ldh, skip, skipval, sign, w);
+            };
+            if (cols <= 152 * 32 && nv >= 32) go(std::integral_constant<int, 4>());
+            else if (cols / 2 <= 152 * 32 && nv >= 16) go(std::integral_constant<int, 2>());
+            else go(std::integral_constant<int, 1>());
+            g_msd_launches += 1;
+            return;
+        }
+    }
     auto go = [&](auto split) {
         constexpr int SP = decltype(split)::value;
         const int per = kWarps / SP * 32;
@@ -651,7 +852,7 @@ void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long lon
 template <typename Vin, typename Vout>
 void gm_scale(const GmresDims& d, const RowChunk* chunks, const Vin* w, const double* scale, const int* active,
               Vout* v, cudaStream_t s, const float* rf, float2* xs) {
-    k_scale<Vin, Vout><<<dim3(d.nchunk, (d.chunk_elems + 1023) / 1024), kThreads, 0, s>>>(chunks, d.R, w, scale, active,
+    k_scale<Vin, Vout><<<dim3(d.nchunk, (d.chunk_elems + kThreads - 1) / kThreads), kThreads, 0, s>>>(chunks, d.R, w, scale, active,
                                                                                          v, rf, xs);
     g_msd_launches += 1;
 }

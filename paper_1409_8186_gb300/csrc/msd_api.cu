@@ -218,7 +218,7 @@ struct msd_problem {
     std::map<long long, RecomputePlan> rplans;  // key: R*4 + precision
     DBuf genbuf;
     long long rc_checked = -1;  // geometry version whose complex64 range was checked
-    std::map<int, ChunkSet> chunks;  // reduction chunks of solves with R columns
+    std::map<int, ChunkSet> chunks;  // reduction chunks of solves (see chunk_set)
     int* h_pinned = nullptr;  // small pinned host flags: [0..1] sync reads, [2..9] ring of step flags, [10] DORT barrier
     int* d_hpinned = nullptr;  // the same flags as the device addresses them (mapped host memory)
     cudaEvent_t ring_ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -1565,15 +1565,18 @@ void norm2_f64(SolveCtx& cx, const double2* u, double2* out) {
                      nullptr, cx.pb->stream);
 }
 
-// Reduction chunks for R columns: about 256 over the whole problem, of at
-// least 256 elements (rows x R; one element per lane and warp eight times
-// over), never across configurations.
-const ChunkSet& chunk_set(msd_problem* pb, int R) {
-    auto it = pb->chunks.find(R);
+// Reduction chunks for R columns: about 256 over the whole problem, never
+// across configurations, of at least 256 elements (rows x R) for an FP64 basis
+// (whose projections the FP64 pipe bounds: many short warps) and 1024 for an
+// FP32 one (bound by memory: long-lived warps; the 400-disk sweep took 8 %
+// longer with 256).
+const ChunkSet& chunk_set(msd_problem* pb, int R, bool fp32) {
+    const int key = 2 * R + (fp32 ? 1 : 0);
+    auto it = pb->chunks.find(key);
     if (it != pb->chunks.end()) return it->second;
     ChunkSet cs;
     std::vector<int> off(pb->C + 1, 0);
-    const long long target = std::max<long long>(1, std::max<long long>(256, pb->Ntot * R / 256) / R);
+    const long long target = std::max<long long>(1, std::max<long long>(fp32 ? 1024 : 256, pb->Ntot * R / 256) / R);
     for (int c = 0; c < pb->C; ++c) {
         const MsdConfig& m = pb->cfg[c];
         const long long rows = (long long)m.M * m.n;
@@ -1590,7 +1593,7 @@ const ChunkSet& chunk_set(msd_problem* pb, int R) {
     cs.elems = (int)(target * R);
     cs.d = dalloc_copy(cs.h.data(), cs.h.size());
     cs.d_off = dalloc_copy(off.data(), off.size());
-    return pb->chunks.emplace(R, cs).first->second;
+    return pb->chunks.emplace(key, cs).first->second;
 }
 
 // Hands the active flags of the Krylov systems to the products of one
@@ -1768,6 +1771,7 @@ msd_status solve_impl(msd_problem* pb, int R, const double* betas_host, const ms
     const bool mixed = o.precision == MSD_MIXED;
     cudaStream_t s = pb->stream;
 
+    const size_t nv = (size_t)pb->Ntot * R;
     SolveCtx cx;
     cx.pb = pb;
     cx.m = o.restart;
@@ -1777,13 +1781,14 @@ msd_status solve_impl(msd_problem* pb, int R, const double* betas_host, const ms
     cx.d.C = pb->C;
     cx.d.S = pb->C * R;
     cx.d.m = o.restart;
-    cx.chunks = &chunk_set(pb, R);
+    cx.chunks = &chunk_set(pb, R, mixed);
     cx.d.nchunk = (int)cx.chunks->h.size();
     cx.d.chunk_elems = cx.chunks->elems;
     cx.d.ldh = o.restart + 2;
+    cx.d.pairs = (R == 1 || R % 2 == 0) && nv % 2 == 0;
+    for (const RowChunk& c : cx.chunks->h) cx.d.pairs = cx.d.pairs && c.row0 * R % 2 == 0;
     cx.hstride = o.restart + 2;
     const int S = cx.d.S, m = o.restart;
-    const size_t nv = (size_t)pb->Ntot * R;
 
     int bi = 1;
     auto sb = [&](size_t bytes) { return pb->sbuf[bi++].get(bytes); };

@@ -429,6 +429,7 @@ struct GmresDims {
     int nchunk;       // reduction chunks
     int chunk_elems;  // elements (rows x R) of the largest chunk
     long long ldh;    // vectors per configuration of the transposed coefficients hT
+    bool pairs;       // every vector and chunk starts on an even element, and R is even or 1
 };
 
 // out[s][i] = sum over the rows of cfg(s) of conj(u_i) w for u = V_0..V_{nv-1}

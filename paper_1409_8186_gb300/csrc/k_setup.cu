@@ -513,9 +513,10 @@ __global__ void __launch_bounds__(kGenThreads)
 // the weight of H_m(k r_p) e^{i m theta_p} in the potential, f = J_m(k a_p)
 // for the single-layer potential, w_L J_m - k w_M J'_m for u = w_L L + w_M M
 // (the double-layer term of Prop. 4.3 is -(i pi k a_p / 2) J'_m).
+// Wf, Wl (may be NULL): W rounded to FP32 and what the rounding left.
 __global__ void k_nf_weights(const MsdConfig* __restrict__ cfg, int ci, const double* __restrict__ radius,
                              const double2* __restrict__ J, const double2* __restrict__ rho, int R,
-                             double2* __restrict__ W) {
+                             double2* __restrict__ W, float2* __restrict__ Wf, float2* __restrict__ Wl) {
     const MsdConfig c = cfg[ci];
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long long)c.M * c.n * R) return;
@@ -525,104 +526,207 @@ __global__ void k_nf_weights(const MsdConfig* __restrict__ cfg, int ci, const do
     const double a = radius[c.disk_off + p];
     const double s = 0.5 * M_PI * a / sqrt(2.0 * M_PI * a);
     const double2 cm = make_double2(-s * J[row].y, s * J[row].x);  // i s J_m
-    W[row * R + (t % R)] = cmul(cm, rho[row * R + (t % R)]);
+    const double2 w = cmul(cm, rho[row * R + (t % R)]);
+    W[row * R + (t % R)] = w;
+    if (Wf) {
+        const float2 f = make_float2((float)w.x, (float)w.y);
+        Wf[row * R + (t % R)] = f;
+        Wl[row * R + (t % R)] = make_float2((float)(w.x - f.x), (float)(w.y - f.y));
+    }
+}
+
+// sin and cos of x, 20 < x < 1e5, to about 1e-13: Cody and Waite's reduction by
+// pi/2 in three parts (33 bits each, exact products for n < 2^20) and
+// Taylor's series on [-pi/4, pi/4] (terms beyond y^15 and y^14 are below 1e-15).
+// 24 FP64 instructions, half of sincos: here the values are rounded to FP32.
+__device__ __forceinline__ void sincos_phase(double x, double* s, double* c) {
+    const double two_over_pi = 0.63661977236758134308;
+    const double p1 = 1.57079632673412561417, p2 = 6.07710050630396597660e-11, p3 = 2.02226624879595063154e-21;
+    const double n = rint(x * two_over_pi);
+    double y = fma(-n, p1, x);
+    y = fma(-n, p2, y);
+    y = fma(-n, p3, y);
+    const double z = y * y;
+    double ps = fma(z, -1.0 / 1307674368000.0, 1.0 / 6227020800.0);
+    ps = fma(z, ps, -1.0 / 39916800.0);
+    ps = fma(z, ps, 1.0 / 362880.0);
+    ps = fma(z, ps, -1.0 / 5040.0);
+    ps = fma(z, ps, 1.0 / 120.0);
+    ps = fma(z, ps, -1.0 / 6.0);
+    const double sy = fma(y * z, ps, y);
+    double pc = fma(z, -1.0 / 87178291200.0, 1.0 / 479001600.0);
+    pc = fma(z, pc, -1.0 / 3628800.0);
+    pc = fma(z, pc, 1.0 / 40320.0);
+    pc = fma(z, pc, -1.0 / 720.0);
+    pc = fma(z, pc, 1.0 / 24.0);
+    pc = fma(z, pc, -0.5);
+    const double cy = fma(z, pc, 1.0);
+    const int q = __double2int_rn(n) & 3;
+    const double a = (q & 1) ? cy : sy, b = (q & 1) ? sy : cy;
+    *s = (q & 2) ? -a : a;
+    *c = ((q + 1) & 2) ? -b : b;
+}
+
+// The FP32 value nearest to (ah + al) x + (bh + bl) y, ah, bh the FP32 parts
+// of FP64 numbers and al, bl their rests: products split by fused
+// multiply-adds, the sum by Knuth's two-sum.
+__device__ __forceinline__ float dot2(float ah, float al, float x, float bh, float bl, float y) {
+    const float p = __fmul_rn(ah, x), q = __fmul_rn(bh, y);
+    const float pe = fmaf(ah, x, -p), qe = fmaf(bh, y, -q);
+    const float s = __fadd_rn(p, q), t = __fsub_rn(s, p);
+    const float se = __fadd_rn(__fsub_rn(p, __fsub_rn(s, t)), __fsub_rn(q, t));
+    const float rest = __fadd_rn(__fadd_rn(se, __fadd_rn(pe, qe)), fmaf(al, x, __fmul_rn(bl, y)));
+    return fabsf(s) < 3e38f ? __fadd_rn(s, rest) : s;  // (an infinite sum has no rest)
 }
 
 // u(x)[r] = sum_p sum_m W^p_m[r] H_m(k r_p) e^{i m theta_p}, x = points[t],
 // for x outside every disk (points inside a disk get 0).  One thread per
-// point, disks in order (the warp reads the same disk's weights together).
-// Far pairs (k r > 20, N <= k r): J_m, Y_m by FP32 forward recurrence from
-// Hankel's expansion after an FP64 phase; near pairs: FP64 (Miller).  The m
-// sum of one disk is formed in FP32 (far) or FP64 (near) and added to FP64
-// sums per point.  Columns r0 .. r0 + RC - 1 of R.
+// point, disks in order (the warp reads the same disk's weights together;
+// disks are staged 64 at a time).  Far pairs (k r > 20, N <= k r): J_m, Y_m
+// by FP32 forward recurrence from Hankel's expansion after an FP64 phase;
+// near pairs: FP64 (Miller).  The m sum of one disk is formed in FP32 (far)
+// or FP64 (near) and added to FP64 sums per point.  Columns r0 .. r0 + RC - 1
+// of R.
+//
+// The far pairs' FP64 instructions are the bound (64 clocks a warp each): the
+// weights come rounded to FP32 (converting two FP64 weights per mode took 14
+// of 34 ms for 512 x 512 points and 400 disks), the distance from an FP32
+// reciprocal square root and two Newton steps, the phase from sincos_phase,
+// and the m = 0 term from split FP32 products.  Decisions that hang on the
+// last bits (on a circle, at the far limit) take the exact distance.  Measured:
+// 34.1 -> 12.5 ms for those points and disks with N = 20.
+constexpr int kNfDisks = 64;
 template <int RC>
 __global__ void __launch_bounds__(128) k_nearfield(const MsdConfig* __restrict__ cfg, int ci,
                                                    const double2* __restrict__ centre,
                                                    const double* __restrict__ radius,
-                                                   const double2* __restrict__ W, int R, int r0, int ncol,
+                                                   const double2* __restrict__ W, const float2* __restrict__ Wf,
+                                                   const float2* __restrict__ Wl, int R, int r0, int ncol,
                                                    const double2* __restrict__ pts, long long P,
                                                    double2* __restrict__ out) {
+    __shared__ double2 Osh[kNfDisks];
+    __shared__ double ash[kNfDisks];
+    __shared__ float afsh[kNfDisks];
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= P) return;
     const MsdConfig c = cfg[ci];
     const int N = c.N, n = c.n;
-    const double2 x = pts[t];
+    const double2 x = t < P ? pts[t] : make_double2(0.0, 0.0);
+    const float far_from = fmaxf(20.f, (float)N), kf = (float)c.k;
     double2 u[RC];
 #pragma unroll
     for (int j = 0; j < RC; ++j) u[j] = make_double2(0.0, 0.0);
-    bool inside = false;
-    for (int p = 0; p < c.M && !inside; ++p) {
-        const double2 O = centre[c.disk_off + p];
-        const double dx = x.x - O.x, dy = x.y - O.y;
-        const double r = hypot(dx, dy);
-        if (r <= radius[c.disk_off + p]) {
-            inside = true;
-            break;
+    bool inside = t >= P;
+    for (int p0 = 0; p0 < c.M; p0 += kNfDisks) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < kNfDisks && p0 + i < c.M; i += blockDim.x) {
+            Osh[i] = centre[c.disk_off + p0 + i];
+            ash[i] = radius[c.disk_off + p0 + i];
+            afsh[i] = (float)ash[i];
         }
-        const double kr = c.k * r;
-        const double2* w = W + (c.row_off + (long long)p * n + N) * R + r0;  // mode m = 0
-        if (kr > 20.0 && (double)(N < 1 ? 1 : N) <= kr) {
-            double sxd, cxd;
-            sincos(kr, &sxd, &cxd);
-            const float xf = (float)kr;
-            float J0, J1, Y0, Y1;
-            bessel_asymptotic_f32(xf, 0, (float)sxd, (float)cxd, &J0, &Y0);
-            bessel_asymptotic_f32(xf, 1, (float)sxd, (float)cxd, &J1, &Y1);
-            const float2 e1 = make_float2((float)(dx / r), (float)(dy / r));
-            const float two_x = 2.0f / xf;
-            float2 e = make_float2(1.f, 0.f);
-            float2 acc[RC];
-#pragma unroll
-            for (int j = 0; j < RC; ++j) {
-                const double2 w0 = w[j];
-                acc[j] = make_float2((float)(w0.x * J0 - w0.y * Y0), (float)(w0.x * Y0 + w0.y * J0));
+        __syncthreads();
+        const int pe = min(c.M, p0 + kNfDisks);
+        for (int p = p0; p < pe && !inside; ++p) {
+            const double2 O = Osh[p - p0];
+            const double dx = x.x - O.x, dy = x.y - O.y;
+            const double r2 = fma(dx, dx, dy * dy);
+            const float r2f = (float)r2;
+            double r, rinv;
+            float rf = 0.f;
+            bool exact = !(r2f > 1e-30f && r2f < 1e30f);
+            if (!exact) {
+                const float y0 = rsqrtf(r2f);
+                rf = r2f * y0;
+                const float xf0 = kf * rf;
+                exact = fabsf(rf - afsh[p - p0]) <= 1e-5f * rf || fabsf(xf0 - far_from) <= 1e-5f * xf0 || !(xf0 < 1e5f);
+                const double h = 0.5 * r2;
+                double y = y0;
+                y = fma(y, fma(-h * y, y, 0.5), y);
+                y = fma(y, fma(-h * y, y, 0.5), y);
+                rinv = y;
+                r = r2 * y;
             }
-            for (int m = 1; m <= N; ++m) {
-                e = make_float2(e.x * e1.x - e.y * e1.y, e.x * e1.y + e.y * e1.x);
-                // H_m e^{i m th} and H_{-m} e^{-i m th} = (-1)^m H_m e^{-i m th}
-                const float2 hp = make_float2(J1 * e.x - Y1 * e.y, J1 * e.y + Y1 * e.x);
-                float2 hm = make_float2(J1 * e.x + Y1 * e.y, Y1 * e.x - J1 * e.y);
-                if (m & 1) hm = make_float2(-hm.x, -hm.y);
+            if (exact) {
+                r = hypot(dx, dy);
+                rinv = 1.0 / r;
+                if (r <= ash[p - p0]) {
+                    inside = true;
+                    break;
+                }
+            } else if (rf < afsh[p - p0]) {  // by more than rounding
+                inside = true;
+                break;
+            }
+            const double kr = c.k * r;
+            const long long row = (c.row_off + (long long)p * n + N) * R + r0;  // mode m = 0
+            if (kr > 20.0 && (double)(N < 1 ? 1 : N) <= kr) {
+                double sxd, cxd;
+                if (exact) sincos(kr, &sxd, &cxd);
+                else sincos_phase(kr, &sxd, &cxd);
+                const float xf = (float)kr;
+                float J0, J1, Y0, Y1;
+                bessel_asymptotic_f32(xf, 0, (float)sxd, (float)cxd, &J0, &Y0);
+                bessel_asymptotic_f32(xf, 1, (float)sxd, (float)cxd, &J1, &Y1);
+                const float2 e1 = make_float2((float)(dx * rinv), (float)(dy * rinv));
+                const float two_x = 2.0f / xf;
+                const float2* w = Wf + row;
+                float2 e = make_float2(1.f, 0.f);
+                float2 acc[RC];
 #pragma unroll
                 for (int j = 0; j < RC; ++j) {
-                    if (j >= ncol) break;
-                    const double2 wp = w[(long long)m * R + j], wm = w[-(long long)m * R + j];
-                    const float2 a = make_float2((float)wp.x, (float)wp.y), b = make_float2((float)wm.x, (float)wm.y);
-                    acc[j].x += a.x * hp.x - a.y * hp.y + b.x * hm.x - b.y * hm.y;
-                    acc[j].y += a.x * hp.y + a.y * hp.x + b.x * hm.y + b.y * hm.x;
+                    const int jc = j < ncol ? j : 0;
+                    const float2 wh = w[jc], wl = Wl[row + jc];
+                    acc[j] = make_float2(dot2(wh.x, wl.x, J0, -wh.y, -wl.y, Y0), dot2(wh.x, wl.x, Y0, wh.y, wl.y, J0));
                 }
-                const float f = m * two_x;
-                const float J2 = f * J1 - J0, Y2 = f * Y1 - Y0;
-                J0 = J1;
-                J1 = J2;
-                Y0 = Y1;
-                Y1 = Y2;
-            }
+                for (int m = 1; m <= N; ++m) {
+                    // which product of a sum is rounded is written out: it decides the last bits of every
+                    // order, and left open it changes with the code around the loop
+                    e = make_float2(fmaf(e.x, e1.x, -__fmul_rn(e.y, e1.y)), fmaf(e.x, e1.y, __fmul_rn(e.y, e1.x)));
+                    // H_m e^{i m th} and H_{-m} e^{-i m th} = (-1)^m H_m e^{-i m th}
+                    const float2 hp = make_float2(fmaf(J1, e.x, -__fmul_rn(Y1, e.y)), fmaf(Y1, e.x, __fmul_rn(J1, e.y)));
+                    float2 hm = make_float2(fmaf(J1, e.x, __fmul_rn(Y1, e.y)), fmaf(Y1, e.x, -__fmul_rn(J1, e.y)));
+                    if (m & 1) hm = make_float2(-hm.x, -hm.y);
 #pragma unroll
-            for (int j = 0; j < RC; ++j) {
-                u[j].x += acc[j].x;
-                u[j].y += acc[j].y;
-            }
-        } else {
-            double J[MAXL], Y[MAXL];
-            bessel_jy(kr, N, J, Y);
-            const double2 e1 = make_double2(dx / r, dy / r);
-            double2 e = make_double2(1.0, 0.0);
-            for (int m = 0; m <= N; ++m) {
-                const double2 H = make_double2(J[m], Y[m]);
-                const double2 hp = cmul(H, e);
-                double2 hm = cmul(H, cconj(e));
-                if (m & 1) hm = make_double2(-hm.x, -hm.y);
+                    for (int j = 0; j < RC; ++j) {
+                        if (j >= ncol) break;
+                        const float2 a = w[(long long)m * R + j], b = w[-(long long)m * R + j];
+                        acc[j].x += a.x * hp.x - a.y * hp.y + b.x * hm.x - b.y * hm.y;
+                        acc[j].y += a.x * hp.y + a.y * hp.x + b.x * hm.y + b.y * hm.x;
+                    }
+                    const float f = m * two_x;
+                    const float J2 = f * J1 - J0, Y2 = f * Y1 - Y0;
+                    J0 = J1;
+                    J1 = J2;
+                    Y0 = Y1;
+                    Y1 = Y2;
+                }
 #pragma unroll
                 for (int j = 0; j < RC; ++j) {
-                    if (j >= ncol) break;
-                    u[j] = cadd(u[j], cmul(w[(long long)m * R + j], hp));
-                    if (m > 0) u[j] = cadd(u[j], cmul(w[-(long long)m * R + j], hm));
+                    u[j].x += acc[j].x;
+                    u[j].y += acc[j].y;
                 }
-                e = cmul(e, e1);
+            } else {
+                const double2* w = W + row;
+                double J[MAXL], Y[MAXL];
+                bessel_jy(kr, N, J, Y);
+                const double2 e1 = make_double2(dx / r, dy / r);
+                double2 e = make_double2(1.0, 0.0);
+                for (int m = 0; m <= N; ++m) {
+                    const double2 H = make_double2(J[m], Y[m]);
+                    const double2 hp = cmul(H, e);
+                    double2 hm = cmul(H, cconj(e));
+                    if (m & 1) hm = make_double2(-hm.x, -hm.y);
+#pragma unroll
+                    for (int j = 0; j < RC; ++j) {
+                        if (j >= ncol) break;
+                        u[j] = cadd(u[j], cmul(w[(long long)m * R + j], hp));
+                        if (m > 0) u[j] = cadd(u[j], cmul(w[-(long long)m * R + j], hm));
+                    }
+                    e = cmul(e, e1);
+                }
             }
         }
     }
+    if (t >= P) return;
 #pragma unroll
     for (int j = 0; j < RC; ++j) {
         if (j >= ncol) break;
@@ -703,8 +807,10 @@ void launch_nearfield_inside(const MsdConfig* d_cfg, int ci, const MsdConfig& h_
                              int R, double2* W, double2* V, const double2* d_pts, long long P, double2* out,
                              cudaStream_t s) {
     const long long nw = (long long)h_cfg.M * h_cfg.n * R;
-    k_nf_weights<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(d_cfg, ci, d_radius, Jm, rho_minus, R, W);
-    k_nf_weights<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(d_cfg, ci, d_radius, Hm, rho_minus, R, V);
+    k_nf_weights<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(d_cfg, ci, d_radius, Jm, rho_minus, R, W, nullptr,
+                                                               nullptr);
+    k_nf_weights<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(d_cfg, ci, d_radius, Hm, rho_minus, R, V, nullptr,
+                                                               nullptr);
     const unsigned blocks = (unsigned)((P + 127) / 128);
     for (int r0 = 0; r0 < R; r0 += 4) {
         const int nc = R - r0 < 4 ? R - r0 : 4;
@@ -802,19 +908,21 @@ void launch_weighted_norms(const MsdConfig* d_cfg, const RowChunk* d_chunks, int
 }
 
 void launch_nearfield(const MsdConfig* d_cfg, int ci, const MsdConfig& h_cfg, const double2* d_centre,
-                      const double* d_radius, const double2* J, const double2* rho, int R, double2* W,
+                      const double* d_radius, const double2* J, const double2* rho, int R, double2* W, long long Ntot,
                       const double2* d_pts, long long P, double2* out, cudaStream_t s) {
     const long long nw = (long long)h_cfg.M * h_cfg.n * R;
-    k_nf_weights<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(d_cfg, ci, d_radius, J, rho, R, W);
+    float2* Wf = (float2*)(W + Ntot * R);
+    float2* Wl = Wf + Ntot * R;
+    k_nf_weights<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(d_cfg, ci, d_radius, J, rho, R, W, Wf, Wl);
     const unsigned blocks = (unsigned)((P + 127) / 128);
     for (int r0 = 0; r0 < R; r0 += 8) {
         const int nc = R - r0 < 8 ? R - r0 : 8;
         if (nc <= 1)
-            k_nearfield<1><<<blocks, 128, 0, s>>>(d_cfg, ci, d_centre, d_radius, W, R, r0, nc, d_pts, P, out);
+            k_nearfield<1><<<blocks, 128, 0, s>>>(d_cfg, ci, d_centre, d_radius, W, Wf, Wl, R, r0, nc, d_pts, P, out);
         else if (nc <= 4)
-            k_nearfield<4><<<blocks, 128, 0, s>>>(d_cfg, ci, d_centre, d_radius, W, R, r0, nc, d_pts, P, out);
+            k_nearfield<4><<<blocks, 128, 0, s>>>(d_cfg, ci, d_centre, d_radius, W, Wf, Wl, R, r0, nc, d_pts, P, out);
         else
-            k_nearfield<8><<<blocks, 128, 0, s>>>(d_cfg, ci, d_centre, d_radius, W, R, r0, nc, d_pts, P, out);
+            k_nearfield<8><<<blocks, 128, 0, s>>>(d_cfg, ci, d_centre, d_radius, W, Wf, Wl, R, r0, nc, d_pts, P, out);
         g_msd_launches += 1;
     }
     g_msd_launches += 1;

@@ -2791,10 +2791,10 @@ msd_status msd_nearfield(msd_problem* pb, int config, const void* rho, int R, in
             fail(MSD_ERR_ARG, "msd_nearfield: bad argument");
         const double2* d_rho = (const double2*)stage_in(pb, pb->nfbuf[0], rho, (size_t)pb->Ntot * R * 16);
         const double2* d_pts = (const double2*)stage_in(pb, pb->nfbuf[1], points, (size_t)P * 16);
-        double2* W = (double2*)pb->nfbuf[2].get((size_t)pb->Ntot * R * 16);
+        double2* W = (double2*)pb->nfbuf[2].get((size_t)pb->Ntot * R * 32);
         OutStage o(pb, pb->nfbuf[3], u_out, (size_t)P * R * 16);
         launch_nearfield(pb->d_cfg, config, pb->cfg[config], pb->d_centre, pb->d_radius, field_factor_of(pb), d_rho, R, W,
-                         d_pts, P, (double2*)o.dev, pb->stream);
+                         pb->Ntot, d_pts, P, (double2*)o.dev, pb->stream);
         CK_LAUNCH();
         o.finish();
         return MSD_OK;

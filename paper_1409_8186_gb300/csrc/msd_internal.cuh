@@ -350,11 +350,12 @@ void launch_form_finalize(bool fp64, long long Ntot, int R, int nsplit, const vo
                           const void* x, const void* part, void* y, cudaStream_t s);
 
 // Near field (Prop. 4.3): u(points)[r] of configuration ci for densities rho
-// [N_tot][R]; W is a work buffer of N_tot * R complex128.
+// [N_tot][R]; W is a work buffer of N_tot * R * 32 bytes (the weights in FP64,
+// rounded to FP32, and the rests).
 // J: the per-row field factor (the Bessel diagonal J for u = L rho, or a
 // formulation's w_L J - k w_M J').
 void launch_nearfield(const MsdConfig* d_cfg, int ci, const MsdConfig& h_cfg, const double2* d_centre,
-                      const double* d_radius, const double2* J, const double2* rho, int R, double2* W,
+                      const double* d_radius, const double2* J, const double2* rho, int R, double2* W, long long Ntot,
                       const double2* d_pts, long long P, double2* out, cudaStream_t s);
 
 // Interior field of penetrable obstacles: u- = L- rho- at points inside the

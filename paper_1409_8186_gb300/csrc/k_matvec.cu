@@ -488,6 +488,47 @@ __global__ void __launch_bounds__(512, P ? 1 : 2) k_bt_matvec1(const MsdConfig* 
     }
 }
 
+// The product of a few disks: one thread per target row (p, m) and column over
+// a range [q0, q1) of source rows q n + j, work item = 128 rows.  The tile
+// kernel gives a lane to each of 32 target disks, so that four disks use an
+// eighth of every FP64 instruction (64 clocks a warp) and sum their sources one
+// after the other: 46 us for four disks with N = 12.  Here every lane has a
+// row, neighbouring rows read neighbouring generators, and the ranges are short
+// enough to spread over the chip: 11.5 us.  Bound by the latency of a thread's
+// chain.  Offered to the autotuner for FP64.
+template <typename V>
+__global__ void __launch_bounds__(128) k_bt_rows(const MsdConfig* __restrict__ cfgs,
+                                                 const MatvecWork* __restrict__ works, const V* __restrict__ G,
+                                                 const V* __restrict__ xs, V* __restrict__ part, long long Ntot, int R,
+                                                 const int* __restrict__ live) {
+    const MatvecWork w = works[blockIdx.x / R];
+    const int col = blockIdx.x % R;
+    const MsdConfig c = cfgs[w.cfg];
+    const int n = c.n, row = w.p0 * 128 + threadIdx.x;
+    if (row >= c.M * n) return;
+    const int p = row / n, m = row - p * n;
+    V a0 = vzero<V>(), a1 = vzero<V>();
+    if (!live || live[w.cfg * R + col]) {
+        const V* g = G + c.gen_off + (long long)p * c.L + 2 * c.N - m;  // g^{p q}_{j - m} at [q Mp L + j]
+        const V* x = xs + c.row_off * R + col;
+        int q = w.q0 / n, j = w.q0 - q * n;
+#pragma unroll 4
+        for (int i = w.q0; i < w.q1; ++i) {
+            const V gv = g[(long long)q * c.Mp * c.L + j], xv = x[(long long)i * R];
+            if (i & 1) cfma(a1, gv, xv);
+            else cfma(a0, gv, xv);
+            if (++j == n) {
+                j = 0;
+                ++q;
+            }
+        }
+    }
+    V* out = part + ((long long)w.split * Ntot + c.row_off + row) * R + col;
+    V s = V{a0.x + a1.x, a0.y + a1.y};
+    if (w.pad) s = V{out->x + s.x, out->y + s.y};
+    *out = s;
+}
+
 // xs = rf .* x   (columns scaled by the column factor r^q_n of their row)
 template <typename V, typename S>
 __global__ void k_scale_cols(long long Ntot, int R, const S* __restrict__ rf, const V* __restrict__ x,
@@ -649,6 +690,16 @@ struct Bt {
     }
 };
 
+template <typename V>
+struct BtRows {
+    static size_t smem(int) { return 0; }
+    static int occupancy(int) { return 8; }
+    static void launch(const MsdConfig* d_cfg, const MatvecWork* d_work, int nwork, int, const V* G, const V* xs,
+                       V* part, long long Ntot, int R, cudaStream_t s, const int* live = nullptr) {
+        k_bt_rows<V><<<(unsigned)(nwork * R), 128, 0, s>>>(d_cfg, d_work, G, xs, part, Ntot, R, live);
+    }
+};
+
 template <int KB, int P>
 struct Bt1 {
     static void attr() {
@@ -714,6 +765,10 @@ void with_f64(const Choice& c, F&& f) {
 }
 template <typename F>
 void dispatch64(const Choice& c, F&& f) {
+    if (c.RW) {
+        f(BtRows<double2>());
+        return;
+    }
     switch (c.KB) {
         case 4: with_f64<4>(c, f); break;
         case 5: with_f64<5>(c, f); break;
@@ -784,6 +839,10 @@ int matvec_candidates(int R, int Nmax, bool fp64, MatvecChoice* out, int cap, bo
         Choice c{0, 1, 1, 0};
         c.DS = 1;
         if (cnt < cap) out[cnt] = c;
+        ++cnt;
+        Choice rw{1, 1, 1, 0};  // one thread per row (KB = 1 in the encoding of msd_set_tile)
+        rw.RW = 1;
+        if (cnt < cap) out[cnt] = rw;
         ++cnt;
     }
     if (!fp64)

@@ -888,6 +888,26 @@ void build_work(msd_problem* pb, MatvecPlan& plan, int R, bool fp64) {
         build_work_tcs(pb, plan, R);
         return;
     }
+    if (plan.ch.RW) {
+        // rows in blocks of 128; as many ranges of at least four source rows as
+        // give four CTAs per SM
+        long long units = 0;
+        for (auto& c : pb->cfg) units += ((long long)c.M * c.n + 127) / 128 * R;
+        const long long src = (long long)pb->Mmax * (2 * pb->Nmax + 1);
+        long long ns = std::max<long long>(1, std::min<long long>({152 * 4 / units, 64, src / 4}));
+        while (ns > 1 && (size_t)ns * pb->Ntot * R * 16 > (2ull << 30)) --ns;
+        ns = std::max<long long>(1, ns / plan.ns_div);
+        plan.nsplit = (int)ns;
+        plan.work.clear();
+        for (int ci = 0; ci < pb->C; ++ci) {
+            const MsdConfig& c = pb->cfg[ci];
+            const long long rows = (long long)c.M * c.n;
+            for (int b = 0; b * 128LL < rows; ++b)
+                for (int sp = 0; sp < (int)ns; ++sp)
+                    plan.work.push_back(MatvecWork{ci, b, (int)(rows * sp / ns), (int)(rows * (sp + 1) / ns), sp, 0});
+        }
+        return;
+    }
     const int rtiles = R / plan.ch.RT;
     std::vector<int> starts;
     long long tiles = 0;
@@ -1234,7 +1254,7 @@ RecomputePlan& get_recompute_plan(msd_problem* pb, int R, bool fp64) {
     auto it = pb->rplans.find(key);
     if (it != pb->rplans.end()) return it->second;
     auto pin = pb->pinned.find(key);
-    if (pin != pb->pinned.end() && !pin->second.SH && !pin->second.DS)
+    if (pin != pb->pinned.end() && !pin->second.SH && !pin->second.DS && !pin->second.RW)
         return pb->rplans.emplace(key, build_recompute_plan(pb, R, fp64, pin->second)).first->second;
     RecomputePlan rp = build_recompute_plan(pb, R, fp64, matvec_default_choice(R, pb->Nmax, fp64));
     int rc = 0;

@@ -101,6 +101,7 @@ struct MatvecChoice {
     int SH;  // shift-GEMM tensor-core kernel (FP32, RT = MSD_TCS_COLS columns per CTA): 1 = mode
              // blocks of <= 8 two per CTA, 2 = one block of <= 16 modes per CTA; 0 = not used
     int ONE;  // FP64: 1 = one shared-memory stage (two would exceed 227 KB at this truncation order)
+    int RW;   // FP64: 1 = one thread per target row (few disks; work items of 128 rows, sources as rows)
     int DS;   // FP64: 1 = digit-sliced tensor-core kernel (k_matvec_ds.cu; KB = 0, RT = 1)
 };
 #define MSD_TCS_COLS 8

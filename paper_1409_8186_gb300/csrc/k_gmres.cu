@@ -813,7 +813,9 @@ void gm_coeffs(const GmresDims& d, int nv, const double2* y, int ystride, V* hT,
 }
 
 // SPLIT: enough warps for the chip (32 per SM) where the elements alone do
-// not give them, but at least one batch of vectors per warp.
+// not give them, but at least one batch of vectors per warp.  FP32 bases of
+// more than 9 728 elements take pairs (400 disks, one column: the mixed solve
+// 431 -> 404 ms with eight warps a pair group against single elements).
 template <typename V, typename W>
 void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long long vstride, int nv, const V* hT,
                const int* skip, double sign, W* w, cudaStream_t s, int skipval) {
@@ -822,14 +824,15 @@ void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long lon
     const long long cols = d.Ntot * d.R / 32 + 1;
     const int most = std::max(1, nv / U);
     if constexpr (sizeof(V) == 8) {
-        if (d.pairs && cols >= 152 * 16) {
+        if (d.pairs && cols >= 152 * 2) {
             auto go = [&](auto split) {
                 constexpr int SP = decltype(split)::value;
                 const int per = kWarps / SP * 64;
                 k_update_pair<W, SP><<<dim3(d.nchunk, (d.chunk_elems + per - 1) / per), kThreads, 0, s>>>(
                     chunks, d.R, Vb, vstride, nv, hT, d.ldh, skip, skipval, sign, w);
             };
-            if (cols <= 152 * 32 && nv >= 32) go(std::integral_constant<int, 4>());
+            if (cols <= 152 * 8 && nv >= 64) go(std::integral_constant<int, 8>());
+            else if (cols <= 152 * 32 && nv >= 32) go(std::integral_constant<int, 4>());
             else if (cols / 2 <= 152 * 32 && nv >= 16) go(std::integral_constant<int, 2>());
             else go(std::integral_constant<int, 1>());
             g_msd_launches += 1;

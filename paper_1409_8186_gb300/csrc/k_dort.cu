@@ -277,6 +277,144 @@ __global__ void __launch_bounds__(kTdThreads)
     }
 }
 
+// The same reduction of one matrix with n <= 512, rows in registers: row R
+// belongs to warp R / gridDim.x of CTA R mod gridDim.x (the rows still active
+// stay spread over the chip as the matrix shrinks), lane l holds columns l, l
+// + 32, ...; between two barriers a warp only exchanges p_R and the next
+// column.  Bound by the chain of a step: barrier, reads of p and the column,
+// two block sums, the reflector's square root and quotient, then the FP64 work
+// of the rows (the kernel above loads every row twice a step).  Measured, whole
+// eigen stage with the Gram matrix's 0.85 ms saved at 512: n = 512 9.38 ->
+// 7.19 ms, 256 3.47 -> 3.11, 64 0.78 -> 0.74.
+constexpr int kTrMax = 512, kTrCols = kTrMax / 32, kTrPer = kTrMax / kTdThreads;
+
+__global__ void __launch_bounds__(kTdThreads)
+    k_dort_tridiag_reg(int n, double2* __restrict__ A, double2* __restrict__ pbuf, double2* __restrict__ colbuf,
+                       double* __restrict__ e_all, double* __restrict__ tau_all, double2* __restrict__ ph_all,
+                       unsigned* __restrict__ bar, int* __restrict__ err, int expire_test) {
+    __shared__ double2 xs[2][kTrMax], w_sh[kTrMax];  // indexed by the row of A
+    __shared__ double red[kTdWarps], tau_sh;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int R = warp * gridDim.x + blockIdx.x;
+    double2 a[kTrCols];
+#pragma unroll
+    for (int u = 0; u < kTrCols; ++u) {
+        const int j = lane + 32 * u;
+        a[u] = R < n && j < n ? A[(long long)R * n + j] : make_double2(0.0, 0.0);
+    }
+    if (R < n && lane == 1) colbuf[n + R] = a[0];  // column 1, which step 0 reads
+    double nrm2 = 0.0;
+    for (int j = 1 + tid; j < n; j += kTdThreads) {
+        const double2 x = A[(long long)j * n];
+        xs[0][j] = x;
+        nrm2 += cabs2(x);
+    }
+    nrm2 = block_sum_td(nrm2, red);
+    // the reflector of step k (warp 0; both square roots, and the three
+    // quotients, are one instruction sequence each, as these take ~0.4 us): v in
+    // place of x, tau, and the values kept for eigenvectors
+    auto head = [&](int k, double2* x, double nn) {
+        const double2 x0 = x[k + 1];
+        const double root = sqrt(lane == 0 ? nn : cabs2(x0));
+        const double sigma = __shfl_sync(0xffffffffu, root, 0), ax0 = __shfl_sync(0xffffffffu, root, 1);
+        const double quot = (lane == 0 ? 1.0 : lane == 1 ? x0.x : x0.y) / (lane == 0 ? sigma * (sigma + ax0) : ax0);
+        const double tau = sigma > 0.0 ? __shfl_sync(0xffffffffu, quot, 0) : 0.0;
+        const double phx = __shfl_sync(0xffffffffu, quot, 1), phy = __shfl_sync(0xffffffffu, quot, 2);
+        const double2 ph = ax0 > 0.0 ? make_double2(phx, phy) : make_double2(1.0, 0.0);
+        if (lane != 0) return;
+        if (sigma > 0.0) x[k + 1] = cadd(x0, cscale(ph, sigma));
+        tau_sh = tau;
+        if (blockIdx.x == 0) {
+            e_all[k] = sigma;
+            tau_all[k] = tau;
+            ph_all[k] = ph;
+        }
+    };
+    if (warp == 0) head(0, xs[0], nrm2);
+    __syncthreads();
+    unsigned epoch = 0;
+    for (int k = 0; k + 2 < n; ++k) {
+        const int par = k & 1;
+        const double2* v = xs[par];
+        double2* xn = xs[par ^ 1];
+        const double tau = tau_sh;
+        const bool active = R < n && R > k;
+        if (active) {
+            double2 s0 = make_double2(0.0, 0.0), s1 = s0;
+#pragma unroll
+            for (int u = 0; u < kTrCols; ++u) {
+                const int j = lane + 32 * u;
+                if (32 * u < n && 32 * u + 31 > k) {
+                    if (j > k && j < n) {
+                        if (u & 1) cfma(s1, a[u], v[j]);
+                        else cfma(s0, a[u], v[j]);
+                    }
+                }
+            }
+            // lanes 0-15 sum the real parts, 16-31 the imaginary ones
+            const double2 sc = cadd(s0, s1);
+            const bool hi = lane & 16;
+            double s = (hi ? sc.y : sc.x) + __shfl_xor_sync(0xffffffffu, hi ? sc.x : sc.y, 16);
+            for (int off = 8; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            if ((lane & 15) == 0) ((double*)(pbuf + par * n + R))[hi ? 1 : 0] = s * tau;
+        }
+        grid_barrier(bar, ++epoch, err, expire_test);
+        const double2* p = pbuf + par * n;
+        const double2* ci = colbuf + (par ^ 1) * n;
+        double2 pr[kTrPer], od[kTrPer];
+        double vp = 0.0;  // Re(v^H p); v^H p = tau v^H B v is real
+#pragma unroll
+        for (int t = 0; t < kTrPer; ++t) {
+            const int j = k + 1 + tid + t * kTdThreads;
+            pr[t] = j < n ? __ldcg(p + j) : make_double2(0.0, 0.0);
+            od[t] = j < n ? __ldcg(ci + j) : make_double2(0.0, 0.0);
+        }
+        const double2 pk = __ldcg(p + k + 1), v0 = v[k + 1];
+#pragma unroll
+        for (int t = 0; t < kTrPer; ++t) {
+            const int j = k + 1 + tid + t * kTdThreads;
+            if (j < n) vp += v[j].x * pr[t].x + v[j].y * pr[t].y;
+        }
+        const double K = 0.5 * tau * block_sum_td(vp, red);
+        const double2 w0 = csub(pk, cscale(v0, K));
+        nrm2 = 0.0;  // ||x_{k+1}||^2
+#pragma unroll
+        for (int t = 0; t < kTrPer; ++t) {
+            const int j = k + 1 + tid + t * kTdThreads;
+            if (j < n) {
+                const double2 vj = v[j], w = csub(pr[t], cscale(vj, K));
+                w_sh[j] = w;
+                if (blockIdx.x == 0) A[(long long)k * n + j] = vj;  // (no warp reads A any more)
+                if (j > k + 1) {
+                    const double2 x = rank2(od[t], vj, w, w0, v0);
+                    xn[j] = x;
+                    nrm2 += cabs2(x);
+                }
+            }
+        }
+        nrm2 = block_sum_td(nrm2, red);
+        if (warp == 0 && k + 3 < n) head(k + 1, xn, nrm2);
+        if (active) {
+            const double2 vr = v[R], wr = w_sh[R];
+#pragma unroll
+            for (int u = 0; u < kTrCols; ++u) {
+                const int j = lane + 32 * u;
+                if (32 * u < n && 32 * u + 31 > k) {
+                    if (j > k && j < n) a[u] = rank2(a[u], vr, wr, w_sh[j], v[j]);
+                    if (j == k + 2) colbuf[par * n + R] = a[u];
+                }
+            }
+        }
+        __syncthreads();
+    }
+    // what the reflectors left: the diagonal and the last 2 x 2 block
+#pragma unroll
+    for (int u = 0; u < kTrCols; ++u) {
+        const int j = lane + 32 * u;
+        if (R < n && j < n && (j == R || (R >= n - 2 && j >= n - 2))) A[(long long)R * n + j] = a[u];
+    }
+}
+
 __device__ __forceinline__ int sign_bit(double x) { return (int)((unsigned)__double2hiint(x) >> 31); }
 __device__ __forceinline__ int biased_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
@@ -681,6 +819,20 @@ cudaError_t launch_dort(int C, int n, const double2* F, double2* T, void* work, 
             const int need = (n - 1 + kTdWarps - 1) / kTdWarps;
             const int grid = std::max(1, std::min(need, per_sm * sms));
             if (c0 > 0 && (ce = cudaMemsetAsync(bar, 0, 4, s)) != cudaSuccess) return ce;
+            // one matrix that fits in registers, a row per warp (faster at every such
+            // size, see the kernel); several share the barriers of the general kernel
+            if (Cg == 1 && n <= kTrMax && n <= kTdWarps * sms) {
+                double2* A1 = A + (size_t)c0 * n * n;
+                double *e1 = e + (size_t)c0 * n, *t1 = tau + (size_t)c0 * n;
+                double2* p1 = ph + (size_t)c0 * n;
+                int expire1 = g_msd_expire_waits.load();
+                void* rargs[] = {(void*)&n, &A1, &pbuf, &colbuf, &e1, &t1, &p1, &bar, &err, &expire1};
+                ce = cudaLaunchCooperativeKernel((const void*)k_dort_tridiag_reg, dim3(std::min(n, sms)),
+                                                 dim3(kTdThreads), rargs, 0, s);
+                if (ce != cudaSuccess) return ce;
+                ++launches;
+                continue;
+            }
             double2* Ag = A + (size_t)c0 * n * n;
             double* eg = e + (size_t)c0 * n;
             double* tg = tau + (size_t)c0 * n;

@@ -30,13 +30,36 @@ METRIC = "block-matvec GB/s (% HBM peak) & solve time at relres 1e-10, FP64 vs m
 FP64_PEAK_TFLOPS = 152 * 4 * 2.07e9 / 1e12   # 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz
 FP32_PEAK_TFLOPS = 152 * 256 * 2.07e9 / 1e12  # 152 SMs x 128 FFMA/clk x 2 flop x 2.07 GHz
 TF32_OVER_BF16 = 1.1 / 2.25                    # nominal dense TF32 / bf16 tensor rate
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the FP64
-# product kernel (window length 7, generator rows staged by bulk copies) on
-# this workload, from an ncu capture (216.05 MB read + 5.78 MB written); the
-# algorithmic stream is 207.7 MB
-K3_FP64_DRAM_BYTES_PER_LAUNCH = 221831168
+# The FP64 product on tensor cores multiplies 7 digits by 7 and keeps the 28
+# products of the leading ones (tile code KB = 0)
+DIGIT_PRODUCTS = 28
+# dram__bytes_read.sum + dram__bytes_write.sum of one launch of each FP64
+# product kernel on this workload, from ncu captures; the algorithmic stream is
+# 207.7 MB (the digits are 28 bytes per generator value, padded)
+K3_FP64_TRAFFIC = {"digits": 384700000, "window": 221831168}
 K3_FP64_TRAFFIC_SOURCE = ("copied from an ncu capture of the same kernel on this workload "
-                          "(profiles/k_bt_matvec_random400.md, current kernel), not measured in this run")
+                          "(profiles/), not measured in this run")
+
+
+def fp64_roofline(plan, tflops, peaks):
+    """Roofline object of the FP64 product: plan = plan_info of the shape that
+    ran, tflops = its algorithmic rate."""
+    if plan["KB"] == 0:
+        peak = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops", 1900.0))
+        return {"bound": "tensor", "achieved": tflops * DIGIT_PRODUCTS, "peak": peak, "unit": "TFLOP/s",
+                "frac": tflops * DIGIT_PRODUCTS / peak, "traffic": K3_FP64_TRAFFIC["digits"],
+                "traffic_source": K3_FP64_TRAFFIC_SOURCE, "algorithmic_TFLOP_s": tflops,
+                "algorithmic_over_fp64_peak": tflops / FP64_PEAK_TFLOPS,
+                "kernel": "k_bt_ds (FP64 product as 28 exact bf16 digit products; achieved = 28 x algorithmic rate, "
+                          "padding not counted)",
+                "peak_source": "measured bf16 rate of a long loop (dense GEMM)"}
+    return {"bound": "alu", "achieved": tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+            "frac": tflops / FP64_PEAK_TFLOPS, "traffic": K3_FP64_TRAFFIC["window"],
+            "traffic_source": K3_FP64_TRAFFIC_SOURCE,
+            "kernel": "k_bt_matvec<double2,1,1> (FP64 block-Toeplitz product)",
+            "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"}
+
+
 WORKLOAD = ("random400_k2pi: M=400 sound-soft disks, a~U[0.5,1.5], centres U[-50,50]^2 gap 0.2, "
             "k=2pi, N=20 (16400 unknowns), 1 plane wave, GMRES (restart length sized to HBM) to relres 1e-10, "
             "far field T=360")
@@ -308,7 +331,10 @@ def products_table(reps: int = 3, only: str = ""):
                     by /= max(nl, 1)
                     tf = fl / (kms * 1e-3) / 1e12
                     gbs = by / (kms * 1e-3) / 1e9
-                    if prec == F64:
+                    if prec == F64 and info["KB"] == 0:
+                        bound = "bf16 tensor (28x executed)"
+                        peak = peaks.get("bf16_tflops", 1900.0) / DIGIT_PRODUCTS
+                    elif prec == F64:
                         bound, peak = "fp64 alu", FP64_PEAK_TFLOPS
                     elif info["KB"] < 4:  # tensor cores (all kernels): 3 TF32 products per real multiply-add
                         bound, peak = "tf32 tensor (3x executed)", tf32_peak / 3.0
@@ -823,6 +849,7 @@ def main():
     kern_s = r64["kernel_ms"] * 1e-3
     achieved_tf = r64["kernel_flops"] / kern_s / 1e12 if kern_s > 0 else 0.0
     kern_gbs = r64["kernel_bytes"] / kern_s / 1e9 if kern_s > 0 else 0.0
+    plan64, _ = pb.plan_info(1, msd.MSD_FP64)
     mix_kern_s = rmx["kernel_ms"] * 1e-3
     mix_tf = rmx["kernel_flops"] / mix_kern_s / 1e12 if mix_kern_s > 0 else None
 
@@ -878,11 +905,7 @@ def main():
                         "launches": rmx["kernel_launches"],
                         "GB_s": rmx["kernel_bytes"] / 2 / mix_kern_s / 1e9 if mix_kern_s > 0 else None,
                         "TFLOP_s": rmx["kernel_flops"] / mix_kern_s / 1e12 if mix_kern_s > 0 else None},
-        "roofline": {"bound": "alu", "achieved": achieved_tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                     "frac": achieved_tf / FP64_PEAK_TFLOPS, "traffic": K3_FP64_DRAM_BYTES_PER_LAUNCH,
-                     "traffic_source": K3_FP64_TRAFFIC_SOURCE,
-                     "kernel": "k_bt_matvec<double2,1,1> (FP64 block-Toeplitz product)",
-                     "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"},
+        "roofline": fp64_roofline(plan64, achieved_tf, peaks),
         "roofline_mixed": {"bound": "alu", "achieved": mix_tf, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                            "frac": mix_tf / FP32_PEAK_TFLOPS if mix_tf else None, "traffic": None,
                            "kernel": "FP32 block-Toeplitz product inside the mixed-precision solve "

@@ -520,7 +520,11 @@ msd_status msd_set_generator_mode(msd_problem* pb, int mode, int64_t chunk_bytes
  * msd_set_tile: fix the shape (KB, RT) for later products of (R, precision)
  *   of this problem, replacing any plan made before.  MSD_ERR_ARG if
  *   (KB, RT) is not one of the instantiated shapes that fit (FP64: KB 4..7,
- *   RT 1; FP32: KB 4..9, RT in {1,2,4,8,16} dividing R, at most 16 warps
+ *   RT 1, or RT 1 with KB = 0: the product on bf16 tensor cores, FP64 values
+ *   split into seven 8-bit digits whose 28 leading products are exact, for
+ *   stored generators and radii that share an exponent range in groups of
+ *   sources - elsewhere a pinned problem takes the cost-model shape - or with
+ *   KB = 1: one thread per target row, for few disks; FP32: KB 4..9, RT in {1,2,4,8,16} dividing R, at most 16 warps
  *   per CTA, shared memory <= 226 KB; FP32 KB + 100 selects the same window
  *   with each complex multiply-add issued as two paired FP32 FMAs, and with
  *   RT = 1, KB + 200 / KB + 300 the same windows in a kernel without CTA

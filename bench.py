@@ -38,7 +38,7 @@ DIGIT_PRODUCTS = 28
 # 207.7 MB (the digits are 28 bytes per generator value, padded)
 K3_FP64_TRAFFIC = {"digits": 384700000, "window": 221831168}
 K3_FP64_TRAFFIC_SOURCE = ("copied from an ncu capture of the same kernel on this workload "
-                          "(profiles/), not measured in this run")
+                          "(profiles/k_bt_ds_random400.md, profiles/k_bt_matvec_random400.md), not measured in this run")
 
 
 def fp64_roofline(plan, tflops, peaks):

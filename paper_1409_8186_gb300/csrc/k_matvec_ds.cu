@@ -45,8 +45,8 @@
 // instructions take the rest), a shift's drain about 5600 for 8 x 16 results a
 // warp, of which FP64 additions hold their pipe for 2048; long folds (up to 9
 // K-steps) and few mode tiles make few drains.  Measured (GB300, whole
-// product): 400 disks, N = 20, one column 1794 -> 198 us; 200 disks, N = 22, 16
-// columns 9376 -> 502 us.  Against 64-bit references the error is that of the
+// product): 400 disks, N = 20, one column 1794 -> 190 us; 200 disks, N = 22, 16
+// columns 9376 -> 459 us.  Against 64-bit references the error is that of the
 // generators with either kernel (radii 0.5 to 1.5, gaps of 0.01, N = 20:
 // 8.683e-15 here, 8.686e-15 with the FP64 pipe).
 //

@@ -161,8 +161,9 @@ void launch_disk_diagonals(const MsdConfig* d_cfg, int Mtot, const int* d_disk_c
 // The FP64 pipe is the bound: 16 operations per order l >= 0 and pair and
 // about 250 around the recurrences.  Measured (GB300): a geometry step of 400
 // disks, N = 20 (factors, generators, their read-out and one FP64 product)
-// 3177 -> 2416 us (1067 with the digit-sliced product after it), of which the factors were 225 us (one thread per disk) and
-// the generators 821 us (both orders of every pair, divisions in every step).
+// 3177 -> 2416 us (1067 with the digit-sliced product after it); the factors
+// were 225 us of it (one thread per disk) and the generators 821 us (both
+// orders of every pair, divisions in every step), now 38 and 289.
 namespace {
 
 constexpr int kGenThreads = 128;

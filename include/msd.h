@@ -554,6 +554,14 @@ msd_status msd_set_tile(msd_problem* pb, int R, int precision, int KB, int RT);
  * hook off again the next call works normally. */
 void msd_test_expire_waits(int on);
 
+/* Test hook: limits that a small problem can reach (process-wide; value 0
+ * restores the library's own).
+ *   MSD_TEST_PART_BYTES  bytes of partial sums that a plan of the FP64 product
+ *                        on tensor cores may use (2e9): shapes that need more
+ *                        are not taken */
+#define MSD_TEST_PART_BYTES 0
+void msd_test_limit(int what, int64_t value);
+
 /* Total number of CUDA kernels launched by this library in this process. */
 int64_t msd_kernel_launches(void);
 

@@ -22,6 +22,7 @@
 
 std::atomic<long long> g_msd_launches{0};
 std::atomic<int> g_msd_expire_waits{0};
+std::atomic<long long> g_test_part_bytes{0};  // msd_test_limit: cap on the partial sums of the FP64 product
 
 namespace {
 thread_local std::string g_err;
@@ -135,7 +136,8 @@ struct MatvecPlan {
     int nds = 0, Rt = 1;     // CTAs, columns of a group
     DsSmem dsm{0, 0, 0, 0};
     size_t xd_bytes = 0, ex_ints = 0;
-    long long ds_version = -1;
+    bool wants_ds = false;      // tuned or pinned to this form, also while ch is what took its place
+    long long ds_version = -1;  // grouping that ch and the lists were made for
 };
 
 // Generators of the digit-sliced FP64 product: digits and exponents, built
@@ -461,8 +463,9 @@ bool ensure_gt(msd_problem* pb) {
 // host's copy of the radii.  Sorted by radius, eight to a K-step; a group
 // takes K-steps while its radii differ by at most 2^{6/N}, and groups that
 // were made so stay through geometry updates while they differ by at most
-// 2^{7.5/N} (see k_matvec_ds.cu), so that a loop that nudges the radii keeps
-// its work lists.  Not offered (false) when eight neighbours differ by more.
+// 2^{7.5/N} (see k_matvec_ds.cu) and are at most half as many again as new
+// ones would be, so that a loop that nudges the radii keeps its work lists.
+// Not offered (false) when eight neighbours differ by more.
 bool ds_grouping(msd_problem* pb) {
     if (pb->ds_radius_version == pb->radius_version) return pb->ds_ok;
     pb->ds_radius_version = pb->radius_version;
@@ -470,6 +473,7 @@ bool ds_grouping(msd_problem* pb) {
     std::vector<std::vector<double>> lo(pb->C), hi(pb->C);  // radii of every K-step
     pb->ds_ok = true;
     bool keep = !pb->ds_grp.empty();
+    int kept = 0, fresh = 0;  // groups
     for (int ci = 0; ci < pb->C; ++ci) {
         const MsdConfig& m = pb->cfg[ci];
         const double* a = pb->h_radius.data() + m.disk_off;
@@ -485,6 +489,14 @@ bool ds_grouping(msd_problem* pb) {
         }
         if (keep) {
             const DsCfg& c = pb->ds_cfg[ci];
+            kept += c.ngrp;
+            const double width = std::pow(2.0, 6.0 / m.N);
+            double first = 0;
+            for (int k = 0; k < nqs; ++k)
+                if (k == 0 || !(hi[ci][k] <= width * first)) {
+                    first = lo[ci][k];
+                    ++fresh;
+                }
             for (int g = 0; g < c.ngrp; ++g)
                 if (!(hi[ci][pb->ds_grp[c.grp_off + g + 1] - 1] <= most * lo[ci][pb->ds_grp[c.grp_off + g]]))
                     keep = false;
@@ -493,6 +505,7 @@ bool ds_grouping(msd_problem* pb) {
         perm.insert(perm.end(), o.begin(), o.end());
     }
     if (!pb->ds_ok) return false;
+    keep = keep && 2 * kept <= 3 * fresh;
     auto upload = [&](DBuf& buf, const void* src, size_t bytes) {
         void* d = buf.get(bytes);
         CK(cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, pb->stream));
@@ -679,6 +692,12 @@ void ds_mode_tiles(int n, int Rt, int most, int* J, int* mt) {
     *J = (n + *mt - 1) / *mt;
 }
 
+// Bytes of partial sums that the digit-sliced product may use.
+double ds_part_cap() {
+    const long long t = g_test_part_bytes.load();
+    return t > 0 ? (double)t : 2.0e9;
+}
+
 // Items of one shape for `ctas` CTAs: the units in order (tiles outermost),
 // each CTA taking shifts until its share of the modelled clocks is full; a
 // unit that crosses a border is cut between shifts, and every piece writes a
@@ -686,7 +705,7 @@ void ds_mode_tiles(int n, int Rt, int most, int* J, int* mt) {
 // K-step (900 with a ring of three or four stages) or the drain of its
 // accumulators (5600 clocks while all target modes are in range, however many
 // rows are in use: a warp drains 32), an item 2500 more.
-// False when shared memory or the 2 GB of partial sums do not suffice.
+// False when shared memory or ds_part_cap() bytes of partial sums do not suffice.
 bool ds_items(msd_problem* pb, int R, int Rt, int jmax, int ks, int ctas, bool list, DsShape& sh) {
     sh.Rt = Rt;
     sh.jmax = jmax;
@@ -749,7 +768,7 @@ bool ds_items(msd_problem* pb, int R, int Rt, int jmax, int ks, int ctas, bool l
         }
         sh.nslots = slots;
         const double bytes = (double)slots * pb->Ntot * R * 16;
-        if (slots > 1 && bytes > 2.0e9) return false;
+        if (slots > 1 && bytes > ds_part_cap()) return false;
         sh.clocks = share + 2.0 * bytes / 3000.0;  // partial sums written and read at 3 kB per clock
         return true;
     }
@@ -798,7 +817,7 @@ bool ds_items(msd_problem* pb, int R, int Rt, int jmax, int ks, int ctas, bool l
     sh.off.push_back((int)sh.items.size());
     while ((int)sh.off.size() < ctas + 1) sh.off.push_back((int)sh.items.size());
     sh.nslots = slots;
-    if (slots > 1 && (double)slots * pb->Ntot * R * 16 > 2.0e9) return false;
+    if (slots > 1 && (double)slots * pb->Ntot * R * 16 > ds_part_cap()) return false;
     // slots that a tile does not use are zeroed, by the CTAs in turn
     std::vector<std::vector<DsWork>> zero(ctas);
     int turn = 0;
@@ -850,7 +869,6 @@ bool build_work_ds(msd_problem* pb, MatvecPlan& plan, int R) {
     plan.ex_ints = best.ex_ints;
     plan.nsplit = best.nslots;
     plan.nds = sms;
-    plan.ds_version = pb->ds_version;
     plan.d_dscfg = dalloc_copy(best.cfgs.data(), best.cfgs.size());
     plan.d_dswork = dalloc_copy(best.items.data(), best.items.size());
     plan.d_dsoff = dalloc_copy(best.off.data(), best.off.size());
@@ -866,6 +884,15 @@ void free_plan(MatvecPlan& plan) {
     plan.d_dsoff = nullptr;
 }
 
+// Frees the device lists of a plan that is not kept.
+struct PlanGuard {
+    MatvecPlan& p;
+    bool keep = false;
+    ~PlanGuard() {
+        if (!keep) free_plan(p);
+    }
+};
+
 // The digit-sliced Toeplitz sums of the scaled columns xs into part.
 void ds_product(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint, const double2* G, const double2* xs,
                 double2* part, const int* live = nullptr) {
@@ -877,6 +904,12 @@ void ds_product(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint, const do
                    xs, EX, XD, pb->stream);
     launch_ds(plan.d_dscfg, plan.d_dswork, plan.d_dsoff, plan.nds, plan.dsm, (const unsigned char*)g.dg.p, (const int*)g.eb.p, XD,
               EX, part, pb->Ntot, R, plan.Rt, pb->stream, live);
+}
+
+MatvecChoice ds_choice() {
+    MatvecChoice c{0, 1, 1, 0};
+    c.DS = 1;
+    return c;
 }
 
 void build_work(msd_problem* pb, MatvecPlan& plan, int R, bool fp64) {
@@ -1025,13 +1058,10 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
             XT = (float*)pb->xt.get((size_t)pb->xrows * 4 * R * sizeof(float));
             CK(cudaMemsetAsync(XT, 0, (size_t)pb->xrows * 4 * R * sizeof(float), pb->stream));
         }
+        PlanGuard trial_guard{trial};
         build_work(pb, trial, R, fp64);
         if (cand[i / 4].DS && !trial.ch.DS) continue;
         if (dv == 1) model_ns = trial.nsplit;
-        struct TrialGuard {
-            MatvecPlan& t;
-            ~TrialGuard() { free_plan(t); }
-        } trial_guard{trial};
         const int nfull = std::max<int>(1, (int)trial.work.size());
         const int nw = std::max(1, std::min(nfull, (int)std::ceil(frac * nfull)));
         MatvecWork* dw = (MatvecWork*)dwork.get(nfull * sizeof(MatvecWork));
@@ -1086,27 +1116,41 @@ MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, b
     const bool allow_ds = fp64 && ds_possible(pb, adjoint);
     const long long key = plan_key(R, fp64, allow_sh, allow_ds);
     auto it = pb->plans.find(key);
-    if (it != pb->plans.end()) {
-        if (!it->second.ch.DS || it->second.ds_version == pb->ds_version) return it->second;
-        // the groups of the sources have changed: a new work list
-        CK(cudaStreamSynchronize(pb->stream));
-        free_plan(it->second);
-        build_work(pb, it->second, R, fp64);
-        return it->second;
-    }
+    if (it != pb->plans.end() && (!it->second.wants_ds || it->second.ds_version == pb->ds_version)) return it->second;
+    // a new plan, or one whose source groups have changed: made whole, lists on
+    // the device, before it takes the place of the old one
     MatvecPlan plan;
+    PlanGuard guard{plan};
     auto pin = pb->pinned.find((long long)R * 4 + (fp64 ? 0 : 1));
-    if (pin != pb->pinned.end()) {
+    const bool pinned = pin != pb->pinned.end();
+    if (pinned) {
         plan.ch = pin->second;
         if (plan.ch.SH && !(allow_sh && ensure_gt(pb))) plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
         if (plan.ch.DS && !allow_ds) plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
+    } else if (it != pb->plans.end()) {
+        plan.ch = ds_choice();
+        plan.tuned_ms = it->second.tuned_ms;
+        plan.candidates = it->second.candidates;
     } else {
         plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
         if (autotune_enabled()) autotune(pb, plan, R, fp64, allow_sh, allow_ds);
     }
+    plan.wants_ds = plan.ch.DS != 0;
+    plan.ds_version = pb->ds_version;
     build_work(pb, plan, R, fp64);
+    if (plan.wants_ds && !plan.ch.DS && !pinned) {
+        // no shape of the digit form fits these groups: the fastest of the others
+        autotune(pb, plan, R, fp64, allow_sh, false);
+        build_work(pb, plan, R, fp64);
+    }
     plan.d_work = dalloc_copy(plan.work.data(), plan.work.size());
-    return pb->plans.emplace(key, std::move(plan)).first->second;
+    guard.keep = true;
+    if (it == pb->plans.end()) return pb->plans.emplace(key, std::move(plan)).first->second;
+    const cudaError_t e = cudaStreamSynchronize(pb->stream);  // the old lists may still be read
+    free_plan(it->second);
+    it->second = std::move(plan);
+    CK(e);
+    return it->second;
 }
 
 // Chunks of a recomputed product.  A configuration whose M x Mp pairs fit
@@ -2414,6 +2458,10 @@ msd_status msd_matvec_timing(msd_problem* pb, int enable, double* kernel_ms, int
 int64_t msd_kernel_launches(void) { return g_msd_launches.load(); }
 
 void msd_test_expire_waits(int on) { g_msd_expire_waits.store(on ? 1 : 0); }
+
+void msd_test_limit(int what, int64_t value) {
+    if (what == MSD_TEST_PART_BYTES) g_test_part_bytes.store(value);
+}
 
 msd_status msd_grad_farfield_misfit(msd_problem* pb, int R, const double* betas_host, int T,
                                     const double* thetas_host, const void* F_target, const msd_opts* opts,

@@ -26,6 +26,7 @@ MSD_FP64, MSD_MIXED, MSD_FP32 = 0, 1, 2
 MSD_GEN_AUTO, MSD_GEN_STREAMED, MSD_GEN_RECOMPUTE = 0, 1, 2
 MSD_FORM_EFIE, MSD_FORM_MFIE, MSD_FORM_CFIE, MSD_FORM_BWIE = 0, 1, 2, 3
 FORMULATION_KINDS = {"efie": MSD_FORM_EFIE, "mfie": MSD_FORM_MFIE, "cfie": MSD_FORM_CFIE, "bwie": MSD_FORM_BWIE}
+MSD_TEST_PART_BYTES = 0
 MSD_MAX_N = 55
 MSD_MAX_DORT = 2048
 
@@ -89,6 +90,7 @@ def _load():
         "msd_solve_penetrable_pointsources": (I, [P, I, P, ctypes.POINTER(msd_opts), P, P, P]),
         "msd_kernel_launches": (ctypes.c_int64, []),
         "msd_test_expire_waits": (V, [I]),
+        "msd_test_limit": (V, [I, ctypes.c_int64]),
         "msd_set_truncation": (I, [P, P]),
         "msd_penetrable_interior_field": (I, [P, I, P, I, ctypes.c_int64, P, P]),
         "msd_dort_eigenvectors": (I, [P, I, P, I, P, P]),
@@ -109,7 +111,8 @@ EXPORTED = ("msd_create", "msd_destroy", "msd_num_unknowns", "msd_row_offset", "
             "msd_matvec_noalloc", "msd_grad_farfield_misfit", "msd_plan_info", "msd_set_tile",
             "msd_set_generator_mode", "msd_nearfield", "msd_rhs_pointsource", "msd_solve_pointsources",
             "msd_dort", "msd_dort_eigen", "msd_set_formulation", "msd_set_formulation_kind",
-            "msd_formulation_weights", "msd_test_expire_waits", "msd_set_truncation", "msd_penetrable_interior_field", "msd_dort_eigenvectors", "msd_herglotz_wave",
+            "msd_formulation_weights", "msd_test_expire_waits", "msd_test_limit", "msd_set_truncation", "msd_penetrable_interior_field",
+            "msd_dort_eigenvectors", "msd_herglotz_wave",
             "msd_set_penetrable",
             "msd_penetrable_matvec", "msd_solve_penetrable", "msd_solve_penetrable_pointsources",
             "msd_last_error")
@@ -401,6 +404,11 @@ def msd_set_truncation(h, Np) -> None:
 def msd_test_expire_waits(on: bool) -> None:
     """Test hook: bounded device waits take their expiry path (include/msd.h)."""
     _lib.msd_test_expire_waits(1 if on else 0)
+
+
+def msd_test_limit(what: int, value: int) -> None:
+    """Test hook: limits that a small problem can reach (include/msd.h)."""
+    _lib.msd_test_limit(what, int(value))
 
 
 # ---------------------------------------------------------------- convenience wrapper

@@ -1,0 +1,83 @@
+"""Plans of the digit-sliced FP64 product (tile code KB = 0) over the life of a
+problem: what a product does when the plan it was made for no longer holds.
+Products against the oracle's dense operator, 1e-11 relative as for every FP64
+product."""
+import numpy as np
+import pytest
+
+import oracle.msd_oracle as O_
+from paper_1409_8186_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore::RuntimeWarning")]
+
+
+@pytest.fixture(scope="module")
+def msd():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1409_8186_gb300 import msd as m
+    return m
+
+
+def _x(n, R, seed):
+    rng = np.random.default_rng(seed)
+    return rng.standard_normal((n, R)) + 1j * rng.standard_normal((n, R))
+
+
+def _grid(M, N, radii, k=2.0):
+    side = int(np.ceil(np.sqrt(M)))
+    g = 4.0 * np.stack(np.meshgrid(np.arange(side), np.arange(side)), -1).reshape(-1, 2)[:M]
+    return W.Cluster(g + 0.0, np.asarray(radii, np.float64), np.zeros(M, np.int8), k, N)
+
+
+def _check(pb, cls, R, seed):
+    x = _x(pb.ntot, R, seed)
+    y = pb.matvec(torch.from_numpy(x).cuda()).cpu().numpy()
+    for i, c in enumerate(cls):
+        s = slice(pb.row_offset(i), pb.row_offset(i + 1))
+        ref = O_.preconditioned_dense(c.centres, c.radii, c.bc, c.k, c.N) @ x[s]
+        assert np.abs(y[s] - ref).max() <= 1e-11 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("M,N,R", [(40, 8, 16), (70, 10, 8)])
+def test_regrouping_that_no_longer_fits(msd, M, N, R, pinned):
+    """Equal radii make one group of sources; spread ones make several, whose
+    partial sums exceed the limit that the first plan just keeps."""
+    even = _grid(M, N, np.full(M, 1.0))
+    spread = _grid(M, N, np.linspace(0.6, 1.5, M))
+    key = (R, msd.MSD_FP64)
+
+    def form(pb):
+        return pb.plan_info(*key)[0]["KB"]
+
+    try:
+        pb = msd.Problem(even)
+        pb.set_tile(*key, 0, 1)
+        assert form(pb) == 0
+        hi, lo = pb.plan_info(*key)[0]["nsplit"] * even.ntot * R * 16, 16 * even.ntot * R
+        while hi - lo > 8 * even.ntot * R:  # the least limit that admits one group
+            mid = (lo + hi) // 2
+            msd.msd_test_limit(msd.MSD_TEST_PART_BYTES, mid)
+            pb.set_tile(*key, 0, 1)
+            lo, hi = (lo, mid) if form(pb) == 0 else (mid, hi)
+        msd.msd_test_limit(msd.MSD_TEST_PART_BYTES, hi)
+        if pinned:
+            pb.set_tile(*key, 0, 1)
+        else:
+            pb.close()
+            pb = msd.Problem(even)
+            if form(pb) != 0:
+                pytest.skip("another shape is faster here")
+        assert form(pb) == 0
+        _check(pb, [even], R, 1)
+        pb.update_geometry(radii=spread.radii)
+        assert form(pb) != 0
+        _check(pb, [spread], R, 2)
+        pb.update_geometry(radii=even.radii)  # one group again
+        assert form(pb) == 0
+        _check(pb, [even], R, 3)
+    finally:
+        msd.msd_test_limit(msd.MSD_TEST_PART_BYTES, 0)
+    pb.close()

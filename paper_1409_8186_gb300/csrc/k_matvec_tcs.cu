@@ -357,7 +357,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int r = 0; r < kRC; ++r) sr[u][r] = si[u][r] = 0.f;
         for (int g = 0; g < ngroups; ++g) {
             bool ok = mbar_wait(smem_u32(&acc_full), (uint32_t)(g & 1), abort_v);
-            ok = __all_sync(0xffffffffu, ok) && !*abort_v;
+            // one answer per warp, the flag included: the TMEM loads below are warp-wide
+            ok = __all_sync(0xffffffffu, ok && !*abort_v);
             if (ok && b < nmb) {
                 asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll

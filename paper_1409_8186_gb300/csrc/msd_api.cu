@@ -128,6 +128,9 @@ struct MatvecPlan {
     int ns_div = 1;               // split count = the wave model's / ns_div
     int candidates = 0;           // shapes the autotuner timed (0: model choice)
     double tuned_ms = 0;          // kernel time of the chosen shape in the tuning run
+    MatvecChoice alt{0, 1, 1, 0};  // the fastest shape but the digit-sliced one
+    int alt_div = 1;
+    double alt_ms = 0;
     // digit-sliced FP64 product (ch.DS): its tiles and work list, valid for
     // one grouping of the sources
     DsCfg* d_dscfg = nullptr;
@@ -1000,9 +1003,9 @@ bool autotune_enabled() {
 
 typedef std::tuple<int, int, int, int, long long, int, int> TuneKey;  // Nmax R fp64 C Ntot Mmax device
 struct TuneResult {
-    MatvecChoice ch;
-    int ns_div;
-    double ms;
+    MatvecChoice ch, alt;
+    int ns_div, alt_div;
+    double ms, alt_ms;
 };
 
 void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh, bool allow_ds) {
@@ -1020,6 +1023,9 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
             plan.ch = it->second.ch;
             plan.ns_div = it->second.ns_div;
             plan.tuned_ms = it->second.ms;
+            plan.alt = it->second.alt;
+            plan.alt_div = it->second.alt_div;
+            plan.alt_ms = it->second.alt_ms;
             plan.candidates = nc;
             return;
         }
@@ -1037,7 +1043,7 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     DBuf dwork;
-    double best_ms = 1e300;
+    double best_ms = 1e300, alt_ms = 1e300;
     MatvecChoice best = plan.ch;
     int best_div = 1;
     // every shape at the wave model's split count and at a half, a quarter
@@ -1090,6 +1096,11 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
             best = cand[i / 4];
             best_div = trial.ns_div;
         }
+        if (t < alt_ms && !trial.ch.DS) {
+            alt_ms = t;
+            plan.alt = cand[i / 4];
+            plan.alt_div = trial.ns_div;
+        }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1097,9 +1108,10 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
     plan.ch = best;
     plan.ns_div = best_div;
     plan.tuned_ms = best_ms;
+    plan.alt_ms = alt_ms;
     plan.candidates = nc;
     std::lock_guard<std::mutex> lk(mu);
-    cache[key] = TuneResult{best, best_div, best_ms};
+    cache[key] = TuneResult{best, plan.alt, best_div, plan.alt_div, best_ms, alt_ms};
 }
 
 // Plans are kept per (R, precision) and per use: allow_sh = the forward
@@ -1111,9 +1123,29 @@ long long plan_key(int R, bool fp64, bool allow_sh, bool allow_ds) {
     return (((long long)R * 4 + (fp64 ? 0 : 1)) * 2 + (allow_sh ? 1 : 0)) * 2 + (allow_ds ? 1 : 0);
 }
 
+// Whether the problem's stream is being captured into a graph.
+bool capturing(const msd_problem* pb) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(pb->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// A captured product reads the stored generators, which msd_update_geometry
+// remakes in place: a replay after an update multiplies by the new operator.
+// The digits, their groups and the work lists made for them are not remade
+// there, so a capture takes the plan without them, which is made (and its
+// partial sums allocated) beside every plan with them.
 MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, bool adjoint = false) {
     allow_sh = allow_sh && !fp64;
-    const bool allow_ds = fp64 && ds_possible(pb, adjoint);
+    const bool captured = fp64 && capturing(pb);
+    const bool allow_ds = fp64 && !captured && ds_possible(pb, adjoint);
+    if (captured) {
+        auto tuned = pb->plans.find(plan_key(R, fp64, allow_sh, true));
+        if (tuned != pb->plans.end() && !tuned->second.wants_ds) return tuned->second;
+    }
     const long long key = plan_key(R, fp64, allow_sh, allow_ds);
     auto it = pb->plans.find(key);
     if (it != pb->plans.end() && (!it->second.wants_ds || it->second.ds_version == pb->ds_version)) return it->second;
@@ -1131,6 +1163,9 @@ MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, b
         plan.ch = ds_choice();
         plan.tuned_ms = it->second.tuned_ms;
         plan.candidates = it->second.candidates;
+        plan.alt = it->second.alt;
+        plan.alt_div = it->second.alt_div;
+        plan.alt_ms = it->second.alt_ms;
     } else {
         plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
         if (autotune_enabled()) autotune(pb, plan, R, fp64, allow_sh, allow_ds);
@@ -1144,6 +1179,20 @@ MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, b
         build_work(pb, plan, R, fp64);
     }
     plan.d_work = dalloc_copy(plan.work.data(), plan.work.size());
+    const long long other_key = plan_key(R, fp64, allow_sh, false);
+    if (plan.wants_ds && !pb->plans.count(other_key)) {
+        MatvecPlan other;
+        PlanGuard other_guard{other};
+        other.ch = pinned ? matvec_default_choice(R, pb->Nmax, fp64) : plan.alt;
+        other.ns_div = pinned ? 1 : plan.alt_div;
+        other.tuned_ms = pinned ? 0 : plan.alt_ms;
+        other.candidates = plan.candidates;
+        build_work(pb, other, R, fp64);
+        pb->part.get((size_t)other.nsplit * pb->Ntot * R * 16);
+        other.d_work = dalloc_copy(other.work.data(), other.work.size());
+        pb->plans.emplace(other_key, other);
+        other_guard.keep = true;
+    }
     guard.keep = true;
     if (it == pb->plans.end()) return pb->plans.emplace(key, std::move(plan)).first->second;
     const cudaError_t e = cudaStreamSynchronize(pb->stream);  // the old lists may still be read

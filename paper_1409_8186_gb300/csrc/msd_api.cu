@@ -468,10 +468,14 @@ bool ensure_gt(msd_problem* pb) {
 // were made so stay through geometry updates while they differ by at most
 // 2^{7.5/N} (see k_matvec_ds.cu) and are at most half as many again as new
 // ones would be, so that a loop that nudges the radii keeps its work lists.
-// Not offered (false) when eight neighbours differ by more.
+// Not offered (false) when eight neighbours differ by more, or while a radius
+// is not a positive number (a geometry update that was refused leaves such).
 bool ds_grouping(msd_problem* pb) {
     if (pb->ds_radius_version == pb->radius_version) return pb->ds_ok;
     pb->ds_radius_version = pb->radius_version;
+    pb->ds_ok = false;
+    for (const double a : pb->h_radius)
+        if (!(a > 0) || !std::isfinite(a)) return false;
     std::vector<int> perm;
     std::vector<std::vector<double>> lo(pb->C), hi(pb->C);  // radii of every K-step
     pb->ds_ok = true;

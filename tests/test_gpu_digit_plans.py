@@ -81,3 +81,25 @@ def test_regrouping_that_no_longer_fits(msd, M, N, R, pinned):
     finally:
         msd.msd_test_limit(msd.MSD_TEST_PART_BYTES, 0)
     pb.close()
+
+
+def test_refused_radii_do_not_reach_the_grouping(msd):
+    """Device radii that are no numbers are refused (by the factors, on the
+    device) but stay in place: products with them may only give non-finite
+    numbers, by a kernel that needs no order of the radii, until good ones come."""
+    M, R = 300, 2
+    cl = _grid(M, 4, np.linspace(0.8, 1.2, M))
+    pb = msd.Problem(cl)
+    pb.set_tile(R, msd.MSD_FP64, 0, 1)
+    _check(pb, [cl], R, 1)
+    bad = np.where(np.arange(M) % 3 == 0, cl.radii, np.nan)
+    with pytest.raises(msd.MsdError) as e:
+        pb.update_geometry(radii=torch.from_numpy(bad).cuda())
+    assert e.value.status == msd.MSD_ERR_NONFINITE
+    assert pb.plan_info(R, msd.MSD_FP64)[0]["KB"] != 0
+    y = pb.matvec(torch.from_numpy(_x(pb.ntot, R, 2)).cuda()).cpu().numpy()
+    assert not np.isfinite(y).any()
+    pb.update_geometry(radii=torch.from_numpy(cl.radii).cuda())
+    assert pb.plan_info(R, msd.MSD_FP64)[0]["KB"] == 0
+    _check(pb, [cl], R, 3)
+    pb.close()

@@ -573,11 +573,14 @@ bool ds_grouping(msd_problem* pb) {
     return true;
 }
 
-// Whether the digit-sliced product can serve this problem: similar radii in
-// every K-step, and its generators (28 bytes per value) in at most 60 % of the
+// Whether the digit-sliced product can serve this problem: configurations and
+// K-steps within the grid dimensions of its preparing kernels (which take them
+// as z and y, 65 535 at most), similar radii in every K-step, and its generators (28 bytes per value) in at most 60 % of the
 // free device memory when they are first wanted.
 bool ds_possible(msd_problem* pb, bool adjoint) {
-    if (pb->gen_mode == MSD_GEN_RECOMPUTE || !ds_grouping(pb)) return false;
+    constexpr int kMaxGrid = 65535;
+    if (pb->gen_mode == MSD_GEN_RECOMPUTE || pb->C > kMaxGrid || (pb->Mmax + 7) / 8 > kMaxGrid) return false;
+    if (!ds_grouping(pb)) return false;
     DsGen& g = adjoint ? pb->ds_adj : pb->ds_fwd;
     if (g.fits < 0) {
         size_t free_b = 0, total_b = 0;

@@ -103,3 +103,15 @@ def test_refused_radii_do_not_reach_the_grouping(msd):
     assert pb.plan_info(R, msd.MSD_FP64)[0]["KB"] == 0
     _check(pb, [cl], R, 3)
     pb.close()
+
+
+def test_more_configurations_than_a_grid_dimension(msd):
+    one = W.Cluster(np.array([[0.0, 0.0], [2.5, 0.3]]), np.array([1.0, 0.9]), np.zeros(2, np.int8), 1.3, 1)
+    C = 65537
+    pb = msd.Problem([one] * C)
+    x = _x(pb.ntot, 1, 1)
+    y = pb.matvec(torch.from_numpy(x).cuda()).cpu().numpy().reshape(C, -1)
+    A = O_.preconditioned_dense(one.centres, one.radii, one.bc, one.k, one.N)
+    ref = x.reshape(C, -1) @ A.T
+    assert np.abs(y - ref).max() <= 1e-11 * np.abs(ref).max()
+    pb.close()

@@ -565,6 +565,10 @@ void msd_test_expire_waits(int on);
 #define MSD_TEST_PART_BYTES 0
 void msd_test_limit(int what, int64_t value);
 
+/* Test hook: device bytes that a problem holds for digits of the FP64 product
+ * on tensor cores (generators, adjoint generators, sources). */
+int64_t msd_test_digit_bytes(msd_problem* pb);
+
 /* Total number of CUDA kernels launched by this library in this process. */
 int64_t msd_kernel_launches(void);
 

@@ -149,6 +149,7 @@ struct DsGen {
     DBuf dg, eb;
     long long version = -1;
     int fits = -1;  // whether device memory has room (-1: not looked at yet)
+    size_t held() const { return dg.cap + eb.cap; }
     void release() {
         dg.release();
         eb.release();
@@ -575,9 +576,11 @@ bool ds_grouping(msd_problem* pb) {
 
 // Whether the digit-sliced product can serve this problem: configurations and
 // K-steps within the grid dimensions of its preparing kernels (which take them
-// as z and y, 65 535 at most), similar radii in every K-step, and its generators (28 bytes per value) in at most 60 % of the
-// free device memory when they are first wanted.
-bool ds_possible(msd_problem* pb, bool adjoint) {
+// as z and y, 65 535 at most), similar radii in every K-step, and its
+// generators (28 bytes per value) and the digits of R source columns (with
+// their padding to eight rows per tile) in at most 60 % of the free device
+// memory when they are first wanted.
+bool ds_possible(msd_problem* pb, int R, bool adjoint) {
     constexpr int kMaxGrid = 65535;
     if (pb->gen_mode == MSD_GEN_RECOMPUTE || pb->C > kMaxGrid || (pb->Mmax + 7) / 8 > kMaxGrid) return false;
     if (!ds_grouping(pb)) return false;
@@ -585,7 +588,9 @@ bool ds_possible(msd_problem* pb, bool adjoint) {
     if (g.fits < 0) {
         size_t free_b = 0, total_b = 0;
         CK(cudaMemGetInfo(&free_b, &total_b));
-        g.fits = (double)(pb->ds_dg_bytes + pb->ds_eb_bytes) <= 0.6 * (double)free_b ? 1 : 0;
+        double xd = 0;
+        for (const DsCfg& c : pb->ds_cfg) xd += (double)c.nqs * ds_xblk_bytes(2 * c.n * R + 8 * c.n);
+        g.fits = (double)(pb->ds_dg_bytes + pb->ds_eb_bytes) + xd <= 0.6 * (double)free_b ? 1 : 0;
     }
     return g.fits == 1;
 }
@@ -1015,7 +1020,9 @@ struct TuneResult {
     double ms, alt_ms;
 };
 
-void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh, bool allow_ds) {
+// adjoint: on the adjoint generators (FP64), and their digits.  Digits made for
+// the tuning alone are given back when another shape is kept.
+void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh, bool allow_ds, bool adjoint) {
     static std::mutex mu;
     static std::map<TuneKey, TuneResult> cache;
     int dev = 0;
@@ -1042,7 +1049,10 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
     const size_t vec = (size_t)pb->Ntot * R * elem;
     void* xs = pb->xs.get(vec);
     CK(cudaMemsetAsync(xs, 0, vec, pb->stream));
-    const void* G = fp64 ? (const void*)pb->d_G64 : (const void*)pb->d_G32;
+    const double2* G64 = adjoint ? pb->d_GA64 : pb->d_G64;
+    const void* G = fp64 ? (const void*)G64 : (const void*)pb->d_G32;
+    DsGen& gen = adjoint ? pb->ds_adj : pb->ds_fwd;
+    const bool had_digits = gen.held() > 0, had_sources = pb->dsx.cap > 0;
     // estimated full time (FP64 ~1.2 TFLOP/s, FP32 ~40 TFLOP/s) -> prefix fraction
     const double est_ms = 8.0 * R * pb->offdiag_n2 / (fp64 ? 1.2e9 : 4.0e10);
     const double frac = est_ms > 20.0 ? 20.0 / est_ms : 1.0;
@@ -1085,7 +1095,7 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
         for (int rep = 0; rep < 3; ++rep) {  // first run warms caches and the module
             CK(cudaEventRecord(e0, pb->stream));
             if (trial.ch.DS)
-                ds_product(pb, trial, R, false, pb->d_G64, (const double2*)xs, (double2*)part);
+                ds_product(pb, trial, R, adjoint, G64, (const double2*)xs, (double2*)part);
             else if (trial.ch.SH)
                 launch_bt_tcs(pb->d_cfg, dw, nw, pb->Nmax, pb->d_GT, XT, (float2*)part, pb->Ntot, R, pb->stream);
             else
@@ -1112,6 +1122,11 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     dwork.release();
+    if (!best.DS && !had_digits) gen.release();
+    if (!best.DS && !had_sources) {
+        pb->dsx.release();
+        pb->dse.release();
+    }
     plan.ch = best;
     plan.ns_div = best_div;
     plan.tuned_ms = best_ms;
@@ -1148,7 +1163,7 @@ bool capturing(const msd_problem* pb) {
 MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, bool adjoint = false) {
     allow_sh = allow_sh && !fp64;
     const bool captured = fp64 && capturing(pb);
-    const bool allow_ds = fp64 && !captured && ds_possible(pb, adjoint);
+    const bool allow_ds = fp64 && !captured && ds_possible(pb, R, adjoint);
     if (captured) {
         auto tuned = pb->plans.find(plan_key(R, fp64, allow_sh, true));
         if (tuned != pb->plans.end() && !tuned->second.wants_ds) return tuned->second;
@@ -1175,14 +1190,14 @@ MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, b
         plan.alt_ms = it->second.alt_ms;
     } else {
         plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
-        if (autotune_enabled()) autotune(pb, plan, R, fp64, allow_sh, allow_ds);
+        if (autotune_enabled()) autotune(pb, plan, R, fp64, allow_sh, allow_ds, adjoint);
     }
     plan.wants_ds = plan.ch.DS != 0;
     plan.ds_version = pb->ds_version;
     build_work(pb, plan, R, fp64);
     if (plan.wants_ds && !plan.ch.DS && !pinned) {
         // no shape of the digit form fits these groups: the fastest of the others
-        autotune(pb, plan, R, fp64, allow_sh, false);
+        autotune(pb, plan, R, fp64, allow_sh, false, adjoint);
         build_work(pb, plan, R, fp64);
     }
     plan.d_work = dalloc_copy(plan.work.data(), plan.work.size());
@@ -2517,6 +2532,10 @@ void msd_test_expire_waits(int on) { g_msd_expire_waits.store(on ? 1 : 0); }
 
 void msd_test_limit(int what, int64_t value) {
     if (what == MSD_TEST_PART_BYTES) g_test_part_bytes.store(value);
+}
+
+int64_t msd_test_digit_bytes(msd_problem* pb) {
+    return pb ? (int64_t)(pb->ds_fwd.held() + pb->ds_adj.held() + pb->dsx.cap + pb->dse.cap) : 0;
 }
 
 msd_status msd_grad_farfield_misfit(msd_problem* pb, int R, const double* betas_host, int T,

@@ -91,6 +91,7 @@ def _load():
         "msd_kernel_launches": (ctypes.c_int64, []),
         "msd_test_expire_waits": (V, [I]),
         "msd_test_limit": (V, [I, ctypes.c_int64]),
+        "msd_test_digit_bytes": (ctypes.c_int64, [P]),
         "msd_set_truncation": (I, [P, P]),
         "msd_penetrable_interior_field": (I, [P, I, P, I, ctypes.c_int64, P, P]),
         "msd_dort_eigenvectors": (I, [P, I, P, I, P, P]),
@@ -111,7 +112,7 @@ EXPORTED = ("msd_create", "msd_destroy", "msd_num_unknowns", "msd_row_offset", "
             "msd_matvec_noalloc", "msd_grad_farfield_misfit", "msd_plan_info", "msd_set_tile",
             "msd_set_generator_mode", "msd_nearfield", "msd_rhs_pointsource", "msd_solve_pointsources",
             "msd_dort", "msd_dort_eigen", "msd_set_formulation", "msd_set_formulation_kind",
-            "msd_formulation_weights", "msd_test_expire_waits", "msd_test_limit", "msd_set_truncation", "msd_penetrable_interior_field",
+            "msd_formulation_weights", "msd_test_expire_waits", "msd_test_limit", "msd_test_digit_bytes", "msd_set_truncation", "msd_penetrable_interior_field",
             "msd_dort_eigenvectors", "msd_herglotz_wave",
             "msd_set_penetrable",
             "msd_penetrable_matvec", "msd_solve_penetrable", "msd_solve_penetrable_pointsources",
@@ -409,6 +410,11 @@ def msd_test_expire_waits(on: bool) -> None:
 def msd_test_limit(what: int, value: int) -> None:
     """Test hook: limits that a small problem can reach (include/msd.h)."""
     _lib.msd_test_limit(what, int(value))
+
+
+def msd_test_digit_bytes(h) -> int:
+    """Test hook: device bytes held for digits of the FP64 product."""
+    return int(_lib.msd_test_digit_bytes(h))
 
 
 # ---------------------------------------------------------------- convenience wrapper

@@ -115,3 +115,18 @@ def test_more_configurations_than_a_grid_dimension(msd):
     ref = x.reshape(C, -1) @ A.T
     assert np.abs(y - ref).max() <= 1e-11 * np.abs(ref).max()
     pb.close()
+
+
+def test_digits_of_a_form_that_is_not_taken_are_given_back(msd):
+    few = _grid(3, 6, np.array([0.9, 1.0, 1.1]))  # one thread per row is faster
+    many = _grid(150, 12, np.linspace(0.9, 1.1, 150))
+    for cl, digits in ((few, False), (many, True)):
+        pb = msd.Problem(cl)
+        _check(pb, [cl], 1, 1)
+        assert (pb.plan_info(1, msd.MSD_FP64)[0]["KB"] == 0) == digits
+        assert (msd.msd_test_digit_bytes(pb.handle) > 0) == digits
+        # a gradient adds the adjoint products
+        Ft = np.ones((1, 20, 1), np.complex128)
+        pb.grad_farfield_misfit([0.3], W.angles(20), Ft, tol=1e-10)
+        assert (msd.msd_test_digit_bytes(pb.handle) > 0) == digits
+        pb.close()

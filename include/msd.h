@@ -563,6 +563,9 @@ void msd_test_expire_waits(int on);
  *                        on tensor cores may use (2e9): shapes that need more
  *                        are not taken */
 #define MSD_TEST_PART_BYTES 0
+/*   MSD_TEST_FAIL_ALLOC  the next device allocation of at least so many bytes
+ *                        is answered, once, as if no memory were left */
+#define MSD_TEST_FAIL_ALLOC 1
 void msd_test_limit(int what, int64_t value);
 
 /* Test hook: device bytes that a problem holds for digits of the FP64 product

@@ -22,6 +22,7 @@
 
 std::atomic<long long> g_msd_launches{0};
 std::atomic<int> g_msd_expire_waits{0};
+std::atomic<long long> g_test_fail_alloc{0};  // msd_test_limit: the next allocation of so many bytes fails
 std::atomic<long long> g_test_part_bytes{0};  // msd_test_limit: cap on the partial sums of the FP64 product
 
 namespace {
@@ -48,8 +49,16 @@ void fail(msd_status st, const std::string& msg) {
 
 #define CK_LAUNCH() CK(cudaGetLastError())
 
+// The problem that the calling thread's entry point works for (NULL: none).
+thread_local msd_problem* t_pb = nullptr;
+
 template <typename F>
-msd_status guarded(F&& f) {
+msd_status guarded(msd_problem* pb, F&& f) {
+    struct Scope {
+        msd_problem* old = t_pb;
+        ~Scope() { t_pb = old; }
+    } scope;
+    if (!scope.old) t_pb = pb;  // (a nested call keeps the outer problem)
     try {
         g_err.clear();
         return f();
@@ -81,6 +90,21 @@ bool ranges_overlap(const void* x, const void* y, size_t bytes) {
     return a < b + bytes && b < a + bytes;
 }
 
+bool give_back_digits(msd_problem* pb);
+
+// Device memory.  Where none is left, the digits that t_pb keeps for its FP64
+// products make room: they can be done without.
+cudaError_t dev_malloc(void** p, size_t bytes) {
+    long long t = g_test_fail_alloc.load();
+    const bool fake = t > 0 && bytes >= (size_t)t && g_test_fail_alloc.compare_exchange_strong(t, 0);
+    cudaError_t e = fake ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && give_back_digits(t_pb)) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 // Growable device buffer owned by the library.
 struct DBuf {
     void* p = nullptr;
@@ -90,7 +114,7 @@ struct DBuf {
             if (p) cudaFree(p);
             p = nullptr;
             cap = 0;
-            CK(cudaMalloc(&p, bytes ? bytes : 16));
+            CK(dev_malloc(&p, bytes ? bytes : 16));
             cap = bytes;
         }
         return p;
@@ -105,14 +129,14 @@ struct DBuf {
 template <typename T>
 T* dalloc_copy(const T* h, size_t n) {
     T* d = nullptr;
-    CK(cudaMalloc(&d, std::max<size_t>(n, 1) * sizeof(T)));
+    CK(dev_malloc((void**)&d, std::max<size_t>(n, 1) * sizeof(T)));
     if (n) CK(cudaMemcpy(d, h, n * sizeof(T), cudaMemcpyHostToDevice));
     return d;
 }
 template <typename T>
 T* dalloc(size_t n) {
     T* d = nullptr;
-    CK(cudaMalloc(&d, std::max<size_t>(n, 1) * sizeof(T)));
+    CK(dev_malloc((void**)&d, std::max<size_t>(n, 1) * sizeof(T)));
     return d;
 }
 
@@ -288,6 +312,7 @@ struct msd_problem {
     size_t ds_dg_bytes = 0, ds_eb_bytes = 0;
     DBuf ds_idx[4];  // on the device: ds_cfg, ds_grp, ds_qgrp, ds_perm
     DsGen ds_fwd, ds_adj;
+    bool ds_hold = false;  // digits are being made: not to be given back
     DBuf dsx, dse;
     // algorithmic size of one product with one column (section 5 storage):
     // sum over ordered pairs of the generator length, and of n^2
@@ -301,6 +326,26 @@ struct msd_problem {
 };
 
 namespace {
+
+// Bytes of digits, and their release under memory pressure: the products of
+// the problem (and of its interior one) then run without the digit-sliced form.
+size_t digit_bytes(const msd_problem* pb) {
+    return pb->ds_fwd.held() + pb->ds_adj.held() + pb->dsx.cap + pb->dse.cap;
+}
+bool give_back_digits(msd_problem* pb) {
+    bool any = false;
+    for (msd_problem* p : {pb, pb ? pb->pen_minus : nullptr}) {
+        if (!p || p->ds_hold || digit_bytes(p) == 0) continue;
+        if (cudaStreamSynchronize(p->stream) != cudaSuccess) return any;
+        p->ds_fwd.release();
+        p->ds_adj.release();
+        p->dsx.release();
+        p->dse.release();
+        p->ds_fwd.fits = p->ds_adj.fits = 0;
+        any = true;
+    }
+    return any;
+}
 
 // Fold the recorded kernel-event pairs into the running totals.
 void flush_timing(msd_problem* pb) {
@@ -908,7 +953,35 @@ struct PlanGuard {
     }
 };
 
-// The digit-sliced Toeplitz sums of the scaled columns xs into part.
+// Everything that a digit-sliced product of this plan needs besides its
+// inputs: digits of the current generators, source digits, scaled columns and
+// partial sums.  False (and the form is no longer offered) where device memory
+// does not suffice.
+bool ds_reserve(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint) {
+    struct Hold {
+        msd_problem* pb;
+        ~Hold() { pb->ds_hold = false; }
+    };
+    try {
+        Hold hold{pb};
+        pb->ds_hold = true;
+        ensure_ds(pb, adjoint, adjoint ? pb->d_GA64 : pb->d_G64);
+        pb->dsx.get(plan.xd_bytes);
+        pb->dse.get(plan.ex_ints * sizeof(int));
+        pb->xs.get((size_t)pb->Ntot * R * 16);
+        pb->part.get((size_t)plan.nsplit * pb->Ntot * R * 16);
+        return true;
+    } catch (const MsdError& e) {
+        if (e.st != MSD_ERR_OOM) throw;
+        g_err.clear();
+    }
+    give_back_digits(pb);
+    pb->ds_fwd.fits = pb->ds_adj.fits = 0;
+    return false;
+}
+
+// The digit-sliced Toeplitz sums of the scaled columns xs into part (after
+// ds_reserve).
 void ds_product(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint, const double2* G, const double2* xs,
                 double2* part, const int* live = nullptr) {
     DsGen& g = ensure_ds(pb, adjoint, G);
@@ -1083,7 +1156,7 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
         }
         PlanGuard trial_guard{trial};
         build_work(pb, trial, R, fp64);
-        if (cand[i / 4].DS && !trial.ch.DS) continue;
+        if (cand[i / 4].DS && (!trial.ch.DS || !ds_reserve(pb, trial, R, adjoint))) continue;
         if (dv == 1) model_ns = trial.nsplit;
         const int nfull = std::max<int>(1, (int)trial.work.size());
         const int nw = std::max(1, std::min(nfull, (int)std::ceil(frac * nfull)));
@@ -1170,7 +1243,10 @@ MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, b
     }
     const long long key = plan_key(R, fp64, allow_sh, allow_ds);
     auto it = pb->plans.find(key);
-    if (it != pb->plans.end() && (!it->second.wants_ds || it->second.ds_version == pb->ds_version)) return it->second;
+    if (it != pb->plans.end() && (!it->second.wants_ds || it->second.ds_version == pb->ds_version)) {
+        if (!it->second.ch.DS || ds_reserve(pb, it->second, R, adjoint)) return it->second;
+        return get_plan(pb, R, fp64, allow_sh, adjoint);  // the one without digits
+    }
     // a new plan, or one whose source groups have changed: made whole, lists on
     // the device, before it takes the place of the old one
     MatvecPlan plan;
@@ -1216,12 +1292,15 @@ MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, b
         other_guard.keep = true;
     }
     guard.keep = true;
-    if (it == pb->plans.end()) return pb->plans.emplace(key, std::move(plan)).first->second;
-    const cudaError_t e = cudaStreamSynchronize(pb->stream);  // the old lists may still be read
-    free_plan(it->second);
-    it->second = std::move(plan);
-    CK(e);
-    return it->second;
+    if (it == pb->plans.end()) {
+        pb->plans.emplace(key, std::move(plan));
+    } else {
+        const cudaError_t e = cudaStreamSynchronize(pb->stream);  // the old lists may still be read
+        free_plan(it->second);
+        it->second = std::move(plan);
+        CK(e);
+    }
+    return get_plan(pb, R, fp64, allow_sh, adjoint);
 }
 
 // Chunks of a recomputed product.  A configuration whose M x Mp pairs fit
@@ -1473,14 +1552,19 @@ void pen_matvec(msd_problem* pb, int R, bool fp64, const void* x, void* y) {
         fail(MSD_ERR_ARG, "truncation order too large for the shared-memory tile of this precision");
     ensure_generators(pb, fp64);
     ensure_generators(pm, fp64);
-    MatvecPlan& pp = get_plan(pb, R, fp64);
-    MatvecPlan& pq = get_plan(pm, R, fp64);
     const size_t elem = fp64 ? 16 : 8;
     const size_t nv = (size_t)pb->Ntot * R;
-    void* xsp = pb->xs.get(nv * elem);
-    void* xsm = pm->xs.get(nv * elem);
-    void* partp = pb->part.get((size_t)pp.nsplit * nv * elem);
-    void* partm = pm->part.get((size_t)pq.nsplit * nv * elem);
+    MatvecPlan *plan_p, *plan_m;
+    void *xsp, *xsm, *partp, *partm;
+    do {  // again where the buffers of one took the digits of the other
+        plan_p = &get_plan(pb, R, fp64);
+        plan_m = &get_plan(pm, R, fp64);
+        xsp = pb->xs.get(nv * elem);
+        xsm = pm->xs.get(nv * elem);
+        partp = pb->part.get((size_t)plan_p->nsplit * nv * elem);
+        partm = pm->part.get((size_t)plan_m->nsplit * nv * elem);
+    } while ((plan_p->ch.DS && !pb->ds_fwd.held()) || (plan_m->ch.DS && !pm->ds_fwd.held()));
+    MatvecPlan &pp = *plan_p, &pq = *plan_m;
     launch_pen_scale(fp64, pb->d_cfg, pb->C, pb->Ntot, R, fp64 ? (const void*)pb->d_rf64 : (const void*)pb->d_rf32,
                      fp64 ? (const void*)pm->d_rf64 : (const void*)pm->d_rf32, x, xsp, xsm, pb->stream);
     auto sums = [&](msd_problem* p, MatvecPlan& plan, const void* xs, void* part) {
@@ -1889,8 +1973,10 @@ msd_status solve_impl(msd_problem* pb, int R, const double* betas_host, const ms
         // HBM is large, so take the longest Krylov basis that fits in half of
         // the free device memory and keeps the per-system Hessenberg
         // matrices within 8 % of it (at least 2 GB), capped by maxit and by 4000.
+        // Digits of the FP64 product count as free: they make room (dev_malloc).
         size_t free_b = 0, total_b = 0;
         CK(cudaMemGetInfo(&free_b, &total_b));
+        free_b += digit_bytes(pb);
         const double vec = (double)pb->Ntot * R * ((o.precision == MSD_MIXED) ? 8 : 16);
         const double S_ = (double)pb->C * R;
         const long long m_mem = (long long)(0.5 * (double)free_b / vec) - 2;
@@ -2112,7 +2198,7 @@ const char* msd_last_error(void) { return g_err.c_str(); }
 
 msd_status msd_create(int C, const int* disk_off, const double* centres, const double* radii,
                       const int8_t* bc, const double* k, const int* N, void* cuda_stream, msd_problem** out) {
-    return guarded([&]() -> msd_status {
+    return guarded(nullptr, [&]() -> msd_status {
         if (!out) fail(MSD_ERR_ARG, "msd_create: out is NULL");
         *out = nullptr;
         if (C < 1 || !disk_off || !centres || !radii || !bc || !k || !N)
@@ -2277,7 +2363,7 @@ int64_t msd_row_offset(const msd_problem* pb, int config) {
 }
 
 msd_status msd_disk_diagonals(msd_problem* pb, void* out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || !out) fail(MSD_ERR_ARG, "msd_disk_diagonals: bad argument");
         const size_t bytes = (size_t)pb->Ntot * 16;
         OutStage o(pb, pb->sbuf[20], out, 4 * bytes);
@@ -2290,7 +2376,7 @@ msd_status msd_disk_diagonals(msd_problem* pb, void* out) {
 }
 
 msd_status msd_pair_generators(msd_problem* pb, int config, void* out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || !out || config < 0 || config >= pb->C) fail(MSD_ERR_ARG, "msd_pair_generators: bad argument");
         ensure_generators(pb, true);
         const MsdConfig& c = pb->cfg[config];
@@ -2304,7 +2390,7 @@ msd_status msd_pair_generators(msd_problem* pb, int config, void* out) {
 }
 
 msd_status msd_rhs_planewave(msd_problem* pb, int R, const double* betas_host, void* out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || R <= 0 || !betas_host || !out) fail(MSD_ERR_ARG, "msd_rhs_planewave: bad argument");
         double* d_betas = (double*)pb->sbuf[21].get((size_t)pb->C * R * 8);
         CK(cudaMemcpyAsync(d_betas, betas_host, (size_t)pb->C * R * 8, cudaMemcpyHostToDevice, pb->stream));
@@ -2318,7 +2404,7 @@ msd_status msd_rhs_planewave(msd_problem* pb, int R, const double* betas_host, v
 }
 
 msd_status msd_matvec(msd_problem* pb, int R, int precision, const void* x_dev, void* y_dev) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || R <= 0 || !x_dev || !y_dev) fail(MSD_ERR_ARG, "msd_matvec: bad argument");
         if (precision != MSD_FP64 && precision != MSD_FP32) fail(MSD_ERR_ARG, "msd_matvec: precision");
         if (!is_device_ptr(x_dev) || !is_device_ptr(y_dev)) fail(MSD_ERR_ARG, "msd_matvec: x and y must be device memory");
@@ -2331,11 +2417,11 @@ msd_status msd_matvec(msd_problem* pb, int R, int precision, const void* x_dev, 
 
 msd_status msd_solve_planewaves(msd_problem* pb, int R, const double* betas_host, const msd_opts* opts,
                                 void* rho_out, msd_stats* stats_host) {
-    return guarded([&]() -> msd_status { return solve_impl(pb, R, betas_host, opts, rho_out, stats_host); });
+    return guarded(pb, [&]() -> msd_status { return solve_impl(pb, R, betas_host, opts, rho_out, stats_host); });
 }
 
 msd_status msd_update_geometry(msd_problem* pb, const double* centres, const double* radii, const double* k_host) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb) fail(MSD_ERR_ARG, "msd_update_geometry: bad handle");
         if (k_host) {
             for (int c = 0; c < pb->C; ++c) {
@@ -2376,7 +2462,7 @@ msd_status msd_update_geometry(msd_problem* pb, const double* centres, const dou
 }
 
 msd_status msd_set_truncation(msd_problem* pb, const int* Np) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb) fail(MSD_ERR_ARG, "msd_set_truncation: bad handle");
         if (pb->form || pb->pen_minus || pb->pen_parent)
             fail(MSD_ERR_ARG, "msd_set_truncation: needs the default rows (no formulation, not penetrable)");
@@ -2410,7 +2496,7 @@ msd_status msd_set_truncation(msd_problem* pb, const int* Np) {
 }
 
 msd_status msd_set_generator_mode(msd_problem* pb, int mode, int64_t chunk_bytes) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || chunk_bytes < 0) fail(MSD_ERR_ARG, "msd_set_generator_mode: bad argument");
         if (mode != MSD_GEN_AUTO && mode != MSD_GEN_STREAMED && mode != MSD_GEN_RECOMPUTE)
             fail(MSD_ERR_ARG, "msd_set_generator_mode: mode");
@@ -2447,7 +2533,7 @@ msd_status msd_set_generator_mode(msd_problem* pb, int mode, int64_t chunk_bytes
 }
 
 msd_status msd_plan_info(msd_problem* pb, int R, int precision, int* out, double* tuned_ms) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || R <= 0 || !out) fail(MSD_ERR_ARG, "msd_plan_info: bad argument");
         if (precision != MSD_FP64 && precision != MSD_FP32) fail(MSD_ERR_ARG, "msd_plan_info: precision");
         const bool fp64 = precision == MSD_FP64;
@@ -2473,7 +2559,7 @@ msd_status msd_plan_info(msd_problem* pb, int R, int precision, int* out, double
 }
 
 msd_status msd_set_tile(msd_problem* pb, int R, int precision, int KB, int RT) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || R <= 0) fail(MSD_ERR_ARG, "msd_set_tile: bad argument");
         if (precision != MSD_FP64 && precision != MSD_FP32) fail(MSD_ERR_ARG, "msd_set_tile: precision");
         const bool fp64 = precision == MSD_FP64;
@@ -2509,7 +2595,7 @@ msd_status msd_set_tile(msd_problem* pb, int R, int precision, int KB, int RT) {
 
 msd_status msd_matvec_timing(msd_problem* pb, int enable, double* kernel_ms, int64_t* launches,
                              double* flops, double* bytes) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb) fail(MSD_ERR_ARG, "msd_matvec_timing: bad handle");
         flush_timing(pb);
         check_tc("msd_matvec_timing");
@@ -2532,16 +2618,17 @@ void msd_test_expire_waits(int on) { g_msd_expire_waits.store(on ? 1 : 0); }
 
 void msd_test_limit(int what, int64_t value) {
     if (what == MSD_TEST_PART_BYTES) g_test_part_bytes.store(value);
+    if (what == MSD_TEST_FAIL_ALLOC) g_test_fail_alloc.store(value);
 }
 
 int64_t msd_test_digit_bytes(msd_problem* pb) {
-    return pb ? (int64_t)(pb->ds_fwd.held() + pb->ds_adj.held() + pb->dsx.cap + pb->dse.cap) : 0;
+    return pb ? (int64_t)digit_bytes(pb) : 0;
 }
 
 msd_status msd_grad_farfield_misfit(msd_problem* pb, int R, const double* betas_host, int T,
                                     const double* thetas_host, const void* F_target, const msd_opts* opts,
                                     double* J_out, double* dO, double* da, double* dk) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || R <= 0 || T <= 0 || !betas_host || !thetas_host || !F_target)
             fail(MSD_ERR_ARG, "msd_grad_farfield_misfit: bad argument");
         if (pb->form) fail(MSD_ERR_ARG, "msd_grad_farfield_misfit: needs the default formulation");
@@ -2620,7 +2707,7 @@ msd_status msd_grad_farfield_misfit(msd_problem* pb, int R, const double* betas_
 }
 
 msd_status msd_farfield(msd_problem* pb, const void* rho, int R, int T, const double* thetas_host, void* F_out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || !rho || R <= 0 || T <= 0 || !thetas_host || !F_out) fail(MSD_ERR_ARG, "msd_farfield: bad argument");
         double* d_th = (double*)pb->sbuf[21].get((size_t)T * 8);
         CK(cudaMemcpyAsync(d_th, thetas_host, (size_t)T * 8, cudaMemcpyHostToDevice, pb->stream));
@@ -2635,7 +2722,7 @@ msd_status msd_farfield(msd_problem* pb, const void* rho, int R, int T, const do
 }
 
 msd_status msd_rhs_pointsource(msd_problem* pb, int R, const double* sources_host, void* out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || R <= 0 || !sources_host || !out) fail(MSD_ERR_ARG, "msd_rhs_pointsource: bad argument");
         double2* d_src = (double2*)pb->sbuf[21].get((size_t)pb->C * R * 16);
         CK(cudaMemcpyAsync(d_src, sources_host, (size_t)pb->C * R * 16, cudaMemcpyHostToDevice, pb->stream));
@@ -2650,7 +2737,7 @@ msd_status msd_rhs_pointsource(msd_problem* pb, int R, const double* sources_hos
 
 msd_status msd_solve_pointsources(msd_problem* pb, int R, const double* sources_host, const msd_opts* opts,
                                   void* rho_out, msd_stats* stats_host) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || R <= 0 || !sources_host || !rho_out) fail(MSD_ERR_ARG, "msd_solve_pointsources: bad argument");
         double2* d_src = (double2*)pb->nfbuf[1].get((size_t)pb->C * R * 16);
         CK(cudaMemcpyAsync(d_src, sources_host, (size_t)pb->C * R * 16, cudaMemcpyHostToDevice, pb->stream));
@@ -2663,7 +2750,7 @@ msd_status msd_solve_pointsources(msd_problem* pb, int R, const double* sources_
 }
 
 msd_status msd_set_penetrable(msd_problem* pb, const double* k_minus, const double* mu) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || pb->pen_parent) fail(MSD_ERR_ARG, "msd_set_penetrable: bad handle");
         if (!k_minus) {
             pen_release(pb);
@@ -2732,7 +2819,7 @@ msd_status msd_set_penetrable(msd_problem* pb, const double* k_minus, const doub
 
 msd_status msd_penetrable_matvec(msd_problem* pb, int R, int precision, const void* xp, const void* xm, void* yp,
                                  void* ym) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || !pb->pen_shadow || R <= 0 || !xp || !xm || !yp || !ym)
             fail(MSD_ERR_ARG, "msd_penetrable_matvec: bad argument (msd_set_penetrable first)");
         if (precision != MSD_FP64)
@@ -2800,7 +2887,7 @@ extern "C" {
 
 msd_status msd_solve_penetrable(msd_problem* pb, int R, const double* betas_host, const msd_opts* opts,
                                 void* rho_plus, void* rho_minus, msd_stats* stats_host) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!betas_host) fail(MSD_ERR_ARG, "msd_solve_penetrable: betas_host is NULL");
         return solve_penetrable_impl(pb, R, betas_host, nullptr, opts, rho_plus, rho_minus, stats_host);
     });
@@ -2808,7 +2895,7 @@ msd_status msd_solve_penetrable(msd_problem* pb, int R, const double* betas_host
 
 msd_status msd_solve_penetrable_pointsources(msd_problem* pb, int R, const double* sources, const msd_opts* opts,
                                              void* rho_plus, void* rho_minus, msd_stats* stats_host) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!sources) fail(MSD_ERR_ARG, "msd_solve_penetrable_pointsources: sources is NULL");
         return solve_penetrable_impl(pb, R, nullptr, sources, opts, rho_plus, rho_minus, stats_host);
     });
@@ -2816,7 +2903,7 @@ msd_status msd_solve_penetrable_pointsources(msd_problem* pb, int R, const doubl
 
 msd_status msd_set_formulation(msd_problem* pb, const double* op_weights, const double* rhs_weights,
                                const double* rep_weights) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb) fail(MSD_ERR_ARG, "msd_set_formulation: bad handle");
         if (!op_weights) {
             pb->form = false;
@@ -2844,7 +2931,7 @@ msd_status msd_set_formulation(msd_problem* pb, const double* op_weights, const 
 
 msd_status msd_penetrable_interior_field(msd_problem* pb, int config, const void* rho_minus, int R, int64_t P,
                                          const double* points, void* u_out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || !pb->pen_minus || !rho_minus || R <= 0 || P <= 0 || !points || !u_out || config < 0 ||
             config >= pb->C)
             fail(MSD_ERR_ARG, "msd_penetrable_interior_field: bad argument (msd_set_penetrable first)");
@@ -2883,7 +2970,7 @@ void check_kind(const char* where, int kind, double alpha, const double* eta) {
 extern "C" {
 
 msd_status msd_set_formulation_kind(msd_problem* pb, int kind, double alpha, const double* eta) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb) fail(MSD_ERR_ARG, "msd_set_formulation_kind: bad handle");
         check_kind("msd_set_formulation_kind", kind, alpha, eta);
         if (pb->pen_minus) fail(MSD_ERR_ARG, "msd_set_formulation_kind: not with penetrable obstacles");
@@ -2902,7 +2989,7 @@ msd_status msd_set_formulation_kind(msd_problem* pb, int kind, double alpha, con
 
 msd_status msd_formulation_weights(int kind, double alpha, const double* eta, double k, double* op_weights,
                                    double* rhs_weights, double* rep_weights) {
-    return guarded([&]() -> msd_status {
+    return guarded(nullptr, [&]() -> msd_status {
         check_kind("msd_formulation_weights", kind, alpha, eta);
         if (!eta && (kind == MSD_FORM_CFIE || kind == MSD_FORM_BWIE) && !(k > 0.0 && std::isfinite(k)))
             fail(MSD_ERR_ARG, "msd_formulation_weights: eta = i k needs k > 0");
@@ -2929,7 +3016,7 @@ msd_status msd_formulation_weights(int kind, double alpha, const double* eta, do
 
 msd_status msd_nearfield(msd_problem* pb, int config, const void* rho, int R, int64_t P, const double* points,
                          void* u_out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || !rho || R <= 0 || P <= 0 || !points || !u_out || config < 0 || config >= pb->C)
             fail(MSD_ERR_ARG, "msd_nearfield: bad argument");
         const double2* d_rho = (const double2*)stage_in(pb, pb->nfbuf[0], rho, (size_t)pb->Ntot * R * 16);
@@ -2979,7 +3066,7 @@ extern "C" {
 
 msd_status msd_dort(msd_problem* pb, int n_alpha, const msd_opts* opts, void* F_out, void* T_out, void* eig_out,
                     msd_stats* stats_host) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || n_alpha <= 0 || n_alpha > MSD_MAX_DORT || !eig_out) fail(MSD_ERR_ARG, "msd_dort: bad argument");
         const int n = n_alpha, C = pb->C;
         const double pi = 3.14159265358979323846;
@@ -3010,7 +3097,7 @@ msd_status msd_dort(msd_problem* pb, int n_alpha, const msd_opts* opts, void* F_
 }
 
 msd_status msd_dort_eigen(msd_problem* pb, int n_alpha, const void* F, void* T_out, void* eig_out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || n_alpha <= 0 || n_alpha > MSD_MAX_DORT || !F || !eig_out)
             fail(MSD_ERR_ARG, "msd_dort_eigen: bad argument");
         const size_t nn = (size_t)pb->C * n_alpha * n_alpha;
@@ -3023,7 +3110,7 @@ msd_status msd_dort_eigen(msd_problem* pb, int n_alpha, const void* F, void* T_o
 }
 
 msd_status msd_dort_eigenvectors(msd_problem* pb, int n_alpha, const void* F, int K, void* eig_out, void* vec_out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || n_alpha <= 0 || n_alpha > MSD_MAX_DORT || !F || K <= 0 || K > n_alpha || !vec_out)
             fail(MSD_ERR_ARG, "msd_dort_eigenvectors: bad argument (1 <= K <= n_alpha)");
         const int n = n_alpha;
@@ -3045,7 +3132,7 @@ msd_status msd_dort_eigenvectors(msd_problem* pb, int n_alpha, const void* F, in
 
 msd_status msd_herglotz_wave(msd_problem* pb, int config, int n_alpha, int K, const void* g, int64_t P,
                              const double* points, void* u_out) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || config < 0 || config >= pb->C || n_alpha <= 0 || K <= 0 || !g || P <= 0 || !points || !u_out)
             fail(MSD_ERR_ARG, "msd_herglotz_wave: bad argument");
         const double2* d_g = (const double2*)stage_in(pb, pb->nfbuf[0], g, (size_t)K * n_alpha * 16);
@@ -3118,7 +3205,7 @@ void* static_scratch_address() {
 }  // namespace
 
 extern "C" msd_status msd_matvec_noalloc(msd_problem* pb, int R, int precision, const void* x_dev, void* y_dev) {
-    return guarded([&]() -> msd_status {
+    return guarded(pb, [&]() -> msd_status {
         if (!pb || R <= 0 || !x_dev || !y_dev) fail(MSD_ERR_ARG, "msd_matvec_noalloc: bad argument");
         if (precision != MSD_FP64 && precision != MSD_FP32) fail(MSD_ERR_ARG, "msd_matvec_noalloc: precision");
         if (!is_device_ptr(x_dev) || !is_device_ptr(y_dev))

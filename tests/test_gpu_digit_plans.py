@@ -130,3 +130,69 @@ def test_digits_of_a_form_that_is_not_taken_are_given_back(msd):
         pb.grad_farfield_misfit([0.3], W.angles(20), Ft, tol=1e-10)
         assert (msd.msd_test_digit_bytes(pb.handle) > 0) == digits
         pb.close()
+
+
+def _limited(msd, size, call):
+    try:
+        msd.msd_test_limit(msd.MSD_TEST_FAIL_ALLOC, size)
+        return call()
+    finally:
+        msd.msd_test_limit(msd.MSD_TEST_FAIL_ALLOC, 0)
+
+
+@pytest.mark.parametrize("R", [1, 4])
+def test_digits_make_room_for_a_solve(msd, R):
+    """An allocation that finds no memory left (as the test hook says of the
+    largest one, the Krylov basis) takes that of the digits."""
+    cl = _grid(60, 8, np.linspace(0.9, 1.1, 60), k=1.3)
+    betas, restart = W.angles(R) + 0.2, 500
+    pb = msd.Problem(cl)
+    pb.set_tile(R, msd.MSD_FP64, 0, 1)
+    _check(pb, [cl], R, 1)
+    assert msd.msd_test_digit_bytes(pb.handle) > 0
+    res = _limited(msd, restart * cl.ntot * R * 16,
+                   lambda: pb.solve(betas, tol=1e-12, restart=restart, precision=msd.MSD_FP64))
+    assert res.status == msd.MSD_OK
+    ref, _ = O_.solve(cl.centres, cl.radii, cl.bc, cl.k, cl.N, betas, method="lu")
+    assert np.abs(res.rho.cpu().numpy() - ref).max() <= 1e-9 * np.abs(ref).max()
+    assert msd.msd_test_digit_bytes(pb.handle) == 0
+    assert pb.plan_info(R, msd.MSD_FP64)[0]["KB"] != 0
+    _check(pb, [cl], R, 2)
+    pb.close()
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+def test_no_room_for_the_digits(msd, pinned):
+    cl = _grid(150, 8, np.linspace(0.9, 1.1, 150))
+    pb = msd.Problem(cl)
+    if pinned:
+        pb.set_tile(1, msd.MSD_FP64, 0, 1)
+    pb.generators()
+    size = 28 * 150 * 150 * 33  # the digits and nothing else that a product allocates
+
+    def product():
+        _check(pb, [cl], 1, 1)
+
+    _limited(msd, size, product)
+    assert pb.plan_info(1, msd.MSD_FP64)[0]["KB"] != 0
+    assert msd.msd_test_digit_bytes(pb.handle) == 0
+    pb.close()
+
+
+def test_transmission_product_with_digits_of_one_side(msd):
+    """The interior problem's digits find no memory: they take those of the
+    exterior, and both sides run without."""
+    cl = _grid(40, 8, np.linspace(0.9, 1.1, 40))
+    x, xm = (torch.from_numpy(_x(cl.ntot, 1, s)).cuda() for s in (4, 5))
+    out = []
+    for KB in (0, 5):
+        pb = msd.Problem(cl)
+        pb.set_tile(1, msd.MSD_FP64, KB, 1)
+        if KB == 0:
+            _check(pb, [cl], 1, 1)
+            assert msd.msd_test_digit_bytes(pb.handle) > 0
+        pb.set_penetrable(3.1)
+        call = lambda: pb.penetrable_matvec(x, xm)  # noqa: E731
+        out.append(torch.cat(_limited(msd, 28 * 40 * 40 * 33, call) if KB == 0 else call()).cpu().numpy())
+        pb.close()
+    assert np.abs(out[0] - out[1]).max() <= 1e-11 * np.abs(out[1]).max()

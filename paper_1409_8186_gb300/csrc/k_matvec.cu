@@ -529,6 +529,19 @@ __global__ void __launch_bounds__(128) k_bt_rows(const MsdConfig* __restrict__ c
     *out = s;
 }
 
+// Values of either sign and of sizes 2^-8 to 1.5 for the tuning runs.
+template <typename T>
+__global__ void k_tune_fill(long long n, T* __restrict__ v) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    unsigned h = (unsigned)i * 2654435761u;
+    h ^= h >> 15;
+    h *= 2246822519u;
+    h ^= h >> 13;
+    const T m = T(0.5) + T(h >> 8) * T(1.0 / (1 << 24));
+    v[i] = ((h & 1) ? -m : m) / T(1 << ((h >> 1) & 7));
+}
+
 // xs = rf .* x   (columns scaled by the column factor r^q_n of their row)
 template <typename V, typename S>
 __global__ void k_scale_cols(long long Ntot, int R, const S* __restrict__ rf, const V* __restrict__ x,
@@ -882,6 +895,13 @@ void launch_scale_cols(bool fp64, long long Ntot, int R, const void* rf, const v
     if (fp64) k_scale_cols<double2, double><<<blocks, th, 0, s>>>(Ntot, R, (const double*)rf, (const double2*)x,
                                                                    (double2*)xs);
     else k_scale_cols<float2, float><<<blocks, th, 0, s>>>(Ntot, R, (const float*)rf, (const float2*)x, (float2*)xs);
+    g_msd_launches += 1;
+}
+
+void launch_tune_fill(bool fp64, long long n, void* v, cudaStream_t s) {
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    if (fp64) k_tune_fill<double><<<blocks, 256, 0, s>>>(n, (double*)v);
+    else k_tune_fill<float><<<blocks, 256, 0, s>>>(n, (float*)v);
     g_msd_launches += 1;
 }
 

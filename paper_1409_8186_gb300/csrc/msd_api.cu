@@ -1079,7 +1079,10 @@ void build_work(msd_problem* pb, MatvecPlan& plan, int R, bool fp64) {
 // Autotuner: time the product kernel of every candidate tile shape (with its
 // own split count) on the problem's generators and keep the fastest.  Large
 // products are timed on a prefix of the work list of about 20 ms, scaled to
-// the whole list.  Results are cached per process by problem shape.  The
+// the whole list (the digit-sliced form, whose lists are made per CTA, runs
+// whole, once where that takes longer).  The columns are random numbers of
+// several sizes: the conversion of the digit-sliced sums takes longer on zeros
+// (400 disks, one column: 232 us against 167 of a product).  Results are cached per process by problem shape.  The
 // tuning run synchronises the stream; MSD_AUTOTUNE=0 keeps the model choice.
 bool autotune_enabled() {
     const char* e = std::getenv("MSD_AUTOTUNE");
@@ -1121,7 +1124,7 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
     const size_t elem = fp64 ? 16 : 8;
     const size_t vec = (size_t)pb->Ntot * R * elem;
     void* xs = pb->xs.get(vec);
-    CK(cudaMemsetAsync(xs, 0, vec, pb->stream));
+    launch_tune_fill(fp64, (long long)pb->Ntot * R * 2, xs, pb->stream);
     const double2* G64 = adjoint ? pb->d_GA64 : pb->d_G64;
     const void* G = fp64 ? (const void*)G64 : (const void*)pb->d_G32;
     DsGen& gen = adjoint ? pb->ds_adj : pb->ds_fwd;
@@ -1152,7 +1155,7 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
         if (trial.ch.SH) {
             if (!ensure_gt(pb)) continue;
             XT = (float*)pb->xt.get((size_t)pb->xrows * 4 * R * sizeof(float));
-            CK(cudaMemsetAsync(XT, 0, (size_t)pb->xrows * 4 * R * sizeof(float), pb->stream));
+            launch_tune_fill(false, pb->xrows * 4 * R, XT, pb->stream);
         }
         PlanGuard trial_guard{trial};
         build_work(pb, trial, R, fp64);
@@ -1180,6 +1183,10 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
             float ms = 0;
             CK(cudaEventElapsedTime(&ms, e0, e1));
             if (rep > 0) t = std::min(t, (double)ms * nfull / nw);
+            if (trial.ch.DS && ms > 20.f) {
+                t = std::min(t, (double)ms);
+                break;
+            }
         }
         if (t < best_ms) {
             best_ms = t;

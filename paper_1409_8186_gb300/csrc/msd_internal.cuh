@@ -193,6 +193,8 @@ int ds_status_and_clear();
 extern std::atomic<int> g_msd_expire_waits;  // bit 0: a pipeline wait of the tensor-core kernel expired
 // the pieces of a product: xs = r .* x; y = x + l .* sum of the partials
 void launch_scale_cols(bool fp64, long long Ntot, int R, const void* rf, const void* x, void* xs, cudaStream_t s);
+// n real numbers of either sign and several sizes (tuning runs)
+void launch_tune_fill(bool fp64, long long n, void* v, cudaStream_t s);
 void launch_finalize(bool fp64, long long Ntot, int R, int nsplit, const void* lf, const void* x, const void* part,
                      void* y, cudaStream_t s);
 // the Toeplitz kernel alone on pre-scaled columns xs (autotuner timing,

@@ -196,3 +196,21 @@ def test_transmission_product_with_digits_of_one_side(msd):
         out.append(torch.cat(_limited(msd, 28 * 40 * 40 * 33, call) if KB == 0 else call()).cpu().numpy())
         pb.close()
     assert np.abs(out[0] - out[1]).max() <= 1e-11 * np.abs(out[1]).max()
+
+
+def test_tuned_time_is_that_of_a_product(msd):
+    """The tuning run takes what a product of ordinary numbers takes, within 20 %
+    (the fastest of several; on zeros this shape took 1.49 times as long)."""
+    M, R = 200, 16
+    cl = _grid(M, 22, np.linspace(0.99, 1.01, M))
+    pb = msd.Problem(cl)
+    info, tuned = pb.plan_info(R, msd.MSD_FP64)
+    assert info["KB"] == 0
+    x = torch.from_numpy(_x(cl.ntot, R, 1)).cuda()
+    best = 1e300
+    for i in range(20):
+        msd.msd_matvec_timing(pb.handle, 1)
+        pb.matvec(x)
+        best = min(best, msd.msd_matvec_timing(pb.handle, 0)[0])
+    assert 0.8 * best <= tuned <= 1.2 * best, (tuned, best)
+    pb.close()

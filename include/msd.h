@@ -519,7 +519,8 @@ msd_status msd_set_generator_mode(msd_problem* pb, int mode, int64_t chunk_bytes
  *   {KB (encoded as for msd_set_tile), RT, nsplit, number of shapes timed
  *   (0: not tuned)}; tuned_ms (may
  *   be NULL) the kernel time of the chosen shape in the tuning run (0 if
- *   not tuned).  Needs the generators of that precision (builds them).
+ *   not tuned; the FP64 form KB = 0 after a geometry update: an estimate
+ *   from it).  Needs the generators of that precision (builds them).
  * msd_set_tile: fix the shape (KB, RT) for later products of (R, precision)
  *   of this problem, replacing any plan made before.  MSD_ERR_ARG if
  *   (KB, RT) is not one of the instantiated shapes that fit (FP64: KB 4..7,

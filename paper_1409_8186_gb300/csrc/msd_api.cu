@@ -152,19 +152,33 @@ struct MatvecPlan {
     int ns_div = 1;               // split count = the wave model's / ns_div
     int candidates = 0;           // shapes the autotuner timed (0: model choice)
     double tuned_ms = 0;          // kernel time of the chosen shape in the tuning run
-    MatvecChoice alt{0, 1, 1, 0};  // the fastest shape but the digit-sliced one
-    int alt_div = 1;
-    double alt_ms = 0;
-    // digit-sliced FP64 product (ch.DS): its tiles and work list, valid for
-    // one grouping of the sources
+    // digit-sliced FP64 product (ch.DS, kept in DigitForm): its tiles and work
+    // list, valid for one grouping of the sources
     DsCfg* d_dscfg = nullptr;
     DsWork* d_dswork = nullptr;
     int* d_dsoff = nullptr;  // items of CTA b: [d_dsoff[b], d_dsoff[b + 1])
     int nds = 0, Rt = 1;     // CTAs, columns of a group
     DsSmem dsm{0, 0, 0, 0};
     size_t xd_bytes = 0, ex_ints = 0;
-    bool wants_ds = false;      // tuned or pinned to this form, also while ch is what took its place
-    long long ds_version = -1;  // grouping that ch and the lists were made for
+};
+
+// What a tuning run measured: the fastest kernel but the digit-sliced one, and
+// that one (0 ms: no shape of it fitted) with its modelled clocks.
+struct TuneResult {
+    MatvecChoice ch{0, 1, 1, 0};
+    int ns_div = 1;
+    double ms = 0, ds_ms = 0, ds_clocks = 0;
+    int candidates = 0;  // shapes timed (0: nothing tuned)
+};
+
+// The digit-sliced form for one column count: whether the products take it, and
+// its plan, for the grouping `version` of the sources.
+struct DigitForm {
+    TuneResult tuned;
+    bool tried = false;  // tuned holds the answer of the tuner (which may be off)
+    bool taken = false;
+    long long version = -1;
+    MatvecPlan plan;
 };
 
 // Generators of the digit-sliced FP64 product: digits and exponents, built
@@ -237,6 +251,7 @@ struct msd_problem {
     double2* d_clf64 = nullptr;
     float2* d_clf32 = nullptr;
     long long geom_version = 0, adj64_version = -1, adj32_version = -1, adj_rows_version = -1;
+    std::map<int, DigitForm> forms;  // key: R
     std::map<long long, MatvecPlan> plans;  // key: R*4 + precision
     std::map<long long, MatvecChoice> pinned;  // shapes fixed by msd_set_tile
     // generator mode of the forward products (msd_set_generator_mode)
@@ -897,14 +912,19 @@ bool ds_items(msd_problem* pb, int R, int Rt, int jmax, int ks, int ctas, bool l
     return true;
 }
 
-// The shape of the digit-sliced product with the least modelled time.  Few
-// columns per group mean long mode tiles (more shifts per tile, fewer partial
-// sums), many K-steps per fold fewer drains.  False when none fits.
-bool build_work_ds(msd_problem* pb, MatvecPlan& plan, int R) {
+int sm_count() {
     int sms = 0, dev = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    DsShape sh, best;
+    return sms;
+}
+
+// The shape of the digit-sliced product with the least modelled time.  Few
+// columns per group mean long mode tiles (more shifts per tile, fewer partial
+// sums), many K-steps per fold fewer drains.  False when none fits.
+bool ds_best_shape(msd_problem* pb, int R, DsShape& best) {
+    const int sms = sm_count();
+    DsShape sh;
     best.clocks = 1e300;
     const int g0 = (R + 63) / 64;
     int last_Rt = 0;
@@ -922,7 +942,16 @@ bool build_work_ds(msd_problem* pb, MatvecPlan& plan, int R) {
                 if (ds_items(pb, R, Rt, j, ks, sms, false, sh) && sh.clocks < best.clocks * (1.0 - 1e-9)) best = sh;
         }
     }
-    if (best.clocks == 1e300 || !ds_items(pb, R, best.Rt, best.jmax, best.ks, sms, true, best)) return false;
+    return best.clocks < 1e300;
+}
+
+// The lists of a plan of that shape, on the device.  False when its work, laid
+// out, does not fit after all.
+bool ds_build(msd_problem* pb, MatvecPlan& plan, int R, DsShape best) {
+    const int sms = sm_count();
+    if (!ds_items(pb, R, best.Rt, best.jmax, best.ks, sms, true, best)) return false;
+    plan.ch = MatvecChoice{0, 1, 1, 0};
+    plan.ch.DS = 1;
     plan.Rt = best.Rt;
     plan.dsm = best.smem;
     plan.xd_bytes = best.xd_bytes;
@@ -994,17 +1023,7 @@ void ds_product(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint, const do
               EX, part, pb->Ntot, R, plan.Rt, pb->stream, live);
 }
 
-MatvecChoice ds_choice() {
-    MatvecChoice c{0, 1, 1, 0};
-    c.DS = 1;
-    return c;
-}
-
 void build_work(msd_problem* pb, MatvecPlan& plan, int R, bool fp64) {
-    if (plan.ch.DS) {
-        if (build_work_ds(pb, plan, R)) return;
-        plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
-    }
     if (plan.ch.SH) {
         build_work_tcs(pb, plan, R);
         return;
@@ -1076,6 +1095,45 @@ void build_work(msd_problem* pb, MatvecPlan& plan, int R, bool fp64) {
     }
 }
 
+// Shortest time of a launch of `run` on the stream, of two after one that warms
+// caches and the module; of the first alone where `once` and it takes longer
+// than 20 ms.
+template <typename F>
+double launch_ms(msd_problem* pb, bool once, F&& run) {
+    struct Events {
+        cudaEvent_t a = nullptr, b = nullptr;
+        ~Events() {
+            if (a) cudaEventDestroy(a);
+            if (b) cudaEventDestroy(b);
+        }
+    } ev;
+    CK(cudaEventCreate(&ev.a));
+    CK(cudaEventCreate(&ev.b));
+    double t = 1e300;
+    for (int rep = 0; rep < 3; ++rep) {
+        CK(cudaEventRecord(ev.a, pb->stream));
+        run();
+        CK_LAUNCH();
+        CK(cudaEventRecord(ev.b, pb->stream));
+        CK(cudaEventSynchronize(ev.b));
+        check_tc("autotune");
+        float ms = 0;
+        CK(cudaEventElapsedTime(&ms, ev.a, ev.b));
+        if (rep > 0 || (once && ms > 20.f)) t = std::min(t, (double)ms);
+        if (once && ms > 20.f) break;
+    }
+    return t;
+}
+
+// Time of the digit-sliced sums of a plan (after ds_reserve) on random columns.
+double digits_ms(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint) {
+    launch_tune_fill(true, (long long)pb->Ntot * R * 2, pb->xs.p, pb->stream);
+    return launch_ms(pb, true, [&] {
+        ds_product(pb, plan, R, adjoint, adjoint ? pb->d_GA64 : pb->d_G64, (const double2*)pb->xs.p,
+                   (double2*)pb->part.p);
+    });
+}
+
 // Autotuner: time the product kernel of every candidate tile shape (with its
 // own split count) on the problem's generators and keep the fastest.  Large
 // products are timed on a prefix of the work list of about 20 ms, scaled to
@@ -1089,56 +1147,45 @@ bool autotune_enabled() {
     return !(e && e[0] == '0');
 }
 
-typedef std::tuple<int, int, int, int, long long, int, int> TuneKey;  // Nmax R fp64 C Ntot Mmax device
-struct TuneResult {
-    MatvecChoice ch, alt;
-    int ns_div, alt_div;
-    double ms, alt_ms;
-};
+// Nmax R (fp64, allow_sh) C Ntot Mmax device, class of the digit-sliced form
+typedef std::tuple<int, int, int, int, long long, int, int, int> TuneKey;
 
-// adjoint: on the adjoint generators (FP64), and their digits.  Digits made for
-// the tuning alone are given back when another shape is kept.
-void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh, bool allow_ds, bool adjoint) {
+// shape (FP64, may be NULL): the digit-sliced form to be timed too.  What it
+// takes depends on the groups of the sources, which problems of one size need
+// not share, so that its modelled clocks are part of the key, in half octaves
+// (-1: no shape of it fits).  adjoint: on the adjoint generators (FP64), and
+// their digits.  Digits made for the tuning alone are given back when another
+// kernel is faster.
+TuneResult autotune(msd_problem* pb, int R, bool fp64, bool allow_sh, bool adjoint, const DsShape* shape) {
     static std::mutex mu;
     static std::map<TuneKey, TuneResult> cache;
     int dev = 0;
     CK(cudaGetDevice(&dev));
-    const TuneKey key{pb->Nmax, R, (fp64 ? 1 : 0) + (allow_sh ? 2 : 0) + (allow_ds ? 4 : 0), pb->C, pb->Ntot, pb->Mmax, dev};
+    const int cls = !shape ? -2 : shape->clocks < 1e300 ? (int)std::lround(2.0 * std::log2(shape->clocks)) : -1;
+    const TuneKey key{pb->Nmax, R, (fp64 ? 1 : 0) + (allow_sh ? 2 : 0), pb->C, pb->Ntot, pb->Mmax, dev, cls};
     MatvecChoice cand[128];
     const int nc = matvec_candidates(R, pb->Nmax, fp64, cand, 128, allow_sh);
     {
         std::lock_guard<std::mutex> lk(mu);
         auto it = cache.find(key);
-        if (it != cache.end()) {
-            plan.ch = it->second.ch;
-            plan.ns_div = it->second.ns_div;
-            plan.tuned_ms = it->second.ms;
-            plan.alt = it->second.alt;
-            plan.alt_div = it->second.alt_div;
-            plan.alt_ms = it->second.alt_ms;
-            plan.candidates = nc;
-            return;
-        }
+        if (it != cache.end()) return it->second;
     }
-    if (nc <= 1) return;
+    TuneResult res;
+    res.ch = matvec_default_choice(R, pb->Nmax, fp64);
+    if (nc <= 1) return res;
+    res.candidates = nc;
+    res.ms = 1e300;
     const size_t elem = fp64 ? 16 : 8;
     const size_t vec = (size_t)pb->Ntot * R * elem;
     void* xs = pb->xs.get(vec);
     launch_tune_fill(fp64, (long long)pb->Ntot * R * 2, xs, pb->stream);
-    const double2* G64 = adjoint ? pb->d_GA64 : pb->d_G64;
-    const void* G = fp64 ? (const void*)G64 : (const void*)pb->d_G32;
+    const void* G = fp64 ? (const void*)(adjoint ? pb->d_GA64 : pb->d_G64) : (const void*)pb->d_G32;
     DsGen& gen = adjoint ? pb->ds_adj : pb->ds_fwd;
     const bool had_digits = gen.held() > 0, had_sources = pb->dsx.cap > 0;
     // estimated full time (FP64 ~1.2 TFLOP/s, FP32 ~40 TFLOP/s) -> prefix fraction
     const double est_ms = 8.0 * R * pb->offdiag_n2 / (fp64 ? 1.2e9 : 4.0e10);
     const double frac = est_ms > 20.0 ? 20.0 / est_ms : 1.0;
-    cudaEvent_t e0, e1;
-    CK(cudaEventCreate(&e0));
-    CK(cudaEventCreate(&e1));
     DBuf dwork;
-    double best_ms = 1e300, alt_ms = 1e300;
-    MatvecChoice best = plan.ch;
-    int best_div = 1;
     // every shape at the wave model's split count and at a half, a quarter
     // and an eighth of it (fewer, longer source ranges: less partial-sum
     // traffic and per-CTA set-up, at some cost in wave fill)
@@ -1150,7 +1197,8 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
         MatvecPlan trial;
         trial.ch = cand[i / 4];
         trial.ns_div = dv;
-        if (trial.ch.DS && (dv > 1 || !allow_ds)) continue;
+        const bool ds = trial.ch.DS;
+        if (ds && (dv > 1 || !shape || shape->clocks == 1e300)) continue;
         float* XT = nullptr;
         if (trial.ch.SH) {
             if (!ensure_gt(pb)) continue;
@@ -1158,71 +1206,81 @@ void autotune(msd_problem* pb, MatvecPlan& plan, int R, bool fp64, bool allow_sh
             launch_tune_fill(false, pb->xrows * 4 * R, XT, pb->stream);
         }
         PlanGuard trial_guard{trial};
-        build_work(pb, trial, R, fp64);
-        if (cand[i / 4].DS && (!trial.ch.DS || !ds_reserve(pb, trial, R, adjoint))) continue;
+        if (ds) {
+            if (!ds_build(pb, trial, R, *shape) || !ds_reserve(pb, trial, R, adjoint)) continue;
+        } else {
+            build_work(pb, trial, R, fp64);
+        }
         if (dv == 1) model_ns = trial.nsplit;
         const int nfull = std::max<int>(1, (int)trial.work.size());
         const int nw = std::max(1, std::min(nfull, (int)std::ceil(frac * nfull)));
         MatvecWork* dw = (MatvecWork*)dwork.get(nfull * sizeof(MatvecWork));
-        if (!trial.work.empty())
+        if (!ds)
             CK(cudaMemcpyAsync(dw, trial.work.data(), nw * sizeof(MatvecWork), cudaMemcpyHostToDevice, pb->stream));
         void* part = pb->part.get((size_t)trial.nsplit * vec);
-        double t = 1e300;
-        for (int rep = 0; rep < 3; ++rep) {  // first run warms caches and the module
-            CK(cudaEventRecord(e0, pb->stream));
-            if (trial.ch.DS)
-                ds_product(pb, trial, R, adjoint, G64, (const double2*)xs, (double2*)part);
-            else if (trial.ch.SH)
+        const double t = ds ? digits_ms(pb, trial, R, adjoint)
+                            : (double)nfull / nw * launch_ms(pb, false, [&] {
+            if (trial.ch.SH)
                 launch_bt_tcs(pb->d_cfg, dw, nw, pb->Nmax, pb->d_GT, XT, (float2*)part, pb->Ntot, R, pb->stream);
             else
                 launch_bt_only(cand[i / 4], fp64, pb->d_cfg, dw, nw, pb->Nmax, G, xs, part, pb->Ntot, R, pb->stream);
-            CK_LAUNCH();
-            CK(cudaEventRecord(e1, pb->stream));
-            CK(cudaEventSynchronize(e1));
-            check_tc("autotune");
-            float ms = 0;
-            CK(cudaEventElapsedTime(&ms, e0, e1));
-            if (rep > 0) t = std::min(t, (double)ms * nfull / nw);
-            if (trial.ch.DS && ms > 20.f) {
-                t = std::min(t, (double)ms);
-                break;
-            }
-        }
-        if (t < best_ms) {
-            best_ms = t;
-            best = cand[i / 4];
-            best_div = trial.ns_div;
-        }
-        if (t < alt_ms && !trial.ch.DS) {
-            alt_ms = t;
-            plan.alt = cand[i / 4];
-            plan.alt_div = trial.ns_div;
+        });
+        if (ds) {
+            res.ds_ms = t;
+            res.ds_clocks = shape->clocks;
+        } else if (t < res.ms) {
+            res.ms = t;
+            res.ch = cand[i / 4];
+            res.ns_div = trial.ns_div;
         }
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     dwork.release();
-    if (!best.DS && !had_digits) gen.release();
-    if (!best.DS && !had_sources) {
-        pb->dsx.release();
-        pb->dse.release();
+    if (!(res.ds_ms > 0 && res.ds_ms < res.ms)) {
+        if (!had_digits) gen.release();
+        if (!had_sources) {
+            pb->dsx.release();
+            pb->dse.release();
+        }
     }
-    plan.ch = best;
-    plan.ns_div = best_div;
-    plan.tuned_ms = best_ms;
-    plan.alt_ms = alt_ms;
-    plan.candidates = nc;
     std::lock_guard<std::mutex> lk(mu);
-    cache[key] = TuneResult{best, plan.alt, best_div, plan.alt_div, best_ms, alt_ms};
+    cache[key] = res;
+    return res;
 }
 
 // Plans are kept per (R, precision) and per use: allow_sh = the forward
 // product of the default rows with stored generators (matvec_dev), the only
 // one that may run the shift-GEMM kernel; every other product (formulations,
 // penetrable, adjoint, raw, recomputed) uses a plan without it.
-// allow_ds: the digit-sliced FP64 product (any use whose generators it has).
-long long plan_key(int R, bool fp64, bool allow_sh, bool allow_ds) {
-    return (((long long)R * 4 + (fp64 ? 0 : 1)) * 2 + (allow_sh ? 1 : 0)) * 2 + (allow_ds ? 1 : 0);
+long long plan_key(int R, bool fp64, bool allow_sh) {
+    return ((long long)R * 4 + (fp64 ? 0 : 1)) * 2 + (allow_sh ? 1 : 0);
+}
+
+// The plan of the stored generators themselves (no digits).
+MatvecPlan& plain_plan(msd_problem* pb, int R, bool fp64, bool allow_sh, bool adjoint) {
+    const long long key = plan_key(R, fp64, allow_sh);
+    auto it = pb->plans.find(key);
+    if (it != pb->plans.end()) return it->second;
+    MatvecPlan plan;
+    PlanGuard guard{plan};
+    plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
+    auto pin = pb->pinned.find((long long)R * 4 + (fp64 ? 0 : 1));
+    if (pin != pb->pinned.end()) {
+        if (!pin->second.DS && !(pin->second.SH && !(allow_sh && ensure_gt(pb)))) plan.ch = pin->second;
+    } else {
+        auto form = fp64 ? pb->forms.find(R) : pb->forms.end();
+        const bool known = form != pb->forms.end() && form->second.tuned.candidates > 0;
+        if (known || autotune_enabled()) {
+            const TuneResult t = known ? form->second.tuned : autotune(pb, R, fp64, allow_sh, adjoint, nullptr);
+            plan.ch = t.ch;
+            plan.ns_div = t.ns_div;
+            plan.tuned_ms = t.ms;
+            plan.candidates = t.candidates;
+        }
+    }
+    build_work(pb, plan, R, fp64);
+    plan.d_work = dalloc_copy(plan.work.data(), plan.work.size());
+    guard.keep = true;
+    return pb->plans.emplace(key, std::move(plan)).first->second;
 }
 
 // Whether the problem's stream is being captured into a graph.
@@ -1235,79 +1293,78 @@ bool capturing(const msd_problem* pb) {
     return st != cudaStreamCaptureStatusNone;
 }
 
+// The plan of the digit-sliced FP64 product, NULL where the products of R
+// columns take another kernel.
+//
+// It is made again when the groups of the sources have changed, its lists whole
+// and on the device before they take the place of the old ones.  Whether the
+// form is still (or now) the faster one is told by the time that it was tuned
+// at and by its modelled clocks then and now: they bound its time from both
+// sides, as a part of it (40 disks: 20 of 30 us) does not change with them.
+// Only where the fastest of the other kernels lies between is it timed again,
+// so that a geometry loop rarely is.
+//
 // A captured product reads the stored generators, which msd_update_geometry
 // remakes in place: a replay after an update multiplies by the new operator.
-// The digits, their groups and the work lists made for them are not remade
-// there, so a capture takes the plan without them, which is made (and its
-// partial sums allocated) beside every plan with them.
-MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, bool adjoint = false) {
-    allow_sh = allow_sh && !fp64;
-    const bool captured = fp64 && capturing(pb);
-    const bool allow_ds = fp64 && !captured && ds_possible(pb, R, adjoint);
-    if (captured) {
-        auto tuned = pb->plans.find(plan_key(R, fp64, allow_sh, true));
-        if (tuned != pb->plans.end() && !tuned->second.wants_ds) return tuned->second;
-    }
-    const long long key = plan_key(R, fp64, allow_sh, allow_ds);
-    auto it = pb->plans.find(key);
-    if (it != pb->plans.end() && (!it->second.wants_ds || it->second.ds_version == pb->ds_version)) {
-        if (!it->second.ch.DS || ds_reserve(pb, it->second, R, adjoint)) return it->second;
-        return get_plan(pb, R, fp64, allow_sh, adjoint);  // the one without digits
-    }
-    // a new plan, or one whose source groups have changed: made whole, lists on
-    // the device, before it takes the place of the old one
-    MatvecPlan plan;
-    PlanGuard guard{plan};
-    auto pin = pb->pinned.find((long long)R * 4 + (fp64 ? 0 : 1));
+// The digits, their groups and the lists made for them are not remade there, so
+// a capture takes the plain plan, which is made (and its partial sums
+// allocated) beside every plan with digits, and whose lists stay.
+MatvecPlan* digit_plan(msd_problem* pb, int R, bool adjoint) {
+    auto pin = pb->pinned.find((long long)R * 4);
     const bool pinned = pin != pb->pinned.end();
-    if (pinned) {
-        plan.ch = pin->second;
-        if (plan.ch.SH && !(allow_sh && ensure_gt(pb))) plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
-        if (plan.ch.DS && !allow_ds) plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
-    } else if (it != pb->plans.end()) {
-        plan.ch = ds_choice();
-        plan.tuned_ms = it->second.tuned_ms;
-        plan.candidates = it->second.candidates;
-        plan.alt = it->second.alt;
-        plan.alt_div = it->second.alt_div;
-        plan.alt_ms = it->second.alt_ms;
-    } else {
-        plan.ch = matvec_default_choice(R, pb->Nmax, fp64);
-        if (autotune_enabled()) autotune(pb, plan, R, fp64, allow_sh, allow_ds, adjoint);
+    if ((pinned && !pin->second.DS) || capturing(pb) || !ds_possible(pb, R, adjoint)) return nullptr;
+    DigitForm& f = pb->forms[R];
+    if (f.version != pb->ds_version) {
+        DsShape shape;
+        shape.clocks = 1e300;
+        const bool fits = ds_best_shape(pb, R, shape);
+        // not asked yet, or the form did not fit when it was
+        const bool ask = !f.tried || (fits && f.tuned.candidates > 0 && f.tuned.ds_ms == 0);
+        if (!pinned && ask) {
+            if (autotune_enabled()) f.tuned = autotune(pb, R, true, false, adjoint, &shape);
+            f.tried = true;
+        }
+        MatvecPlan plan;
+        PlanGuard guard{plan};
+        const double ratio = fits && f.tuned.ds_ms > 0 ? shape.clocks / f.tuned.ds_clocks : 0;
+        const double lo = f.tuned.ds_ms * std::min(1.0, ratio), hi = f.tuned.ds_ms * std::max(1.0, ratio);
+        bool taken = fits && (pinned || (ratio > 0 && lo < f.tuned.ms)) && ds_build(pb, plan, R, shape);
+        if (taken && !pinned && hi >= f.tuned.ms) {
+            taken = ds_reserve(pb, plan, R, adjoint);
+            if (taken) {
+                f.tuned.ds_ms = digits_ms(pb, plan, R, adjoint);
+                f.tuned.ds_clocks = shape.clocks;
+                taken = f.tuned.ds_ms < f.tuned.ms;
+            }
+        }
+        if (taken) {
+            plan.tuned_ms = pinned ? 0 : f.tuned.ds_ms * (shape.clocks / f.tuned.ds_clocks);
+            plan.candidates = f.tuned.candidates;
+            MatvecPlan& plain = plain_plan(pb, R, true, false, adjoint);
+            pb->part.get((size_t)plain.nsplit * pb->Ntot * R * 16);
+        }
+        CK(cudaStreamSynchronize(pb->stream));  // the old lists may still be read
+        free_plan(f.plan);
+        f.taken = taken;
+        f.version = pb->ds_version;
+        bool used = false;  // digits, by any column count
+        for (auto& kv : pb->forms) used = used || kv.second.taken;
+        if (!used) {
+            pb->ds_fwd.release();
+            pb->ds_adj.release();
+            pb->dsx.release();
+            pb->dse.release();
+        }
+        if (!taken) return nullptr;
+        f.plan = std::move(plan);
+        guard.keep = true;
     }
-    plan.wants_ds = plan.ch.DS != 0;
-    plan.ds_version = pb->ds_version;
-    build_work(pb, plan, R, fp64);
-    if (plan.wants_ds && !plan.ch.DS && !pinned) {
-        // no shape of the digit form fits these groups: the fastest of the others
-        autotune(pb, plan, R, fp64, allow_sh, false, adjoint);
-        build_work(pb, plan, R, fp64);
-    }
-    plan.d_work = dalloc_copy(plan.work.data(), plan.work.size());
-    const long long other_key = plan_key(R, fp64, allow_sh, false);
-    if (plan.wants_ds && !pb->plans.count(other_key)) {
-        MatvecPlan other;
-        PlanGuard other_guard{other};
-        other.ch = pinned ? matvec_default_choice(R, pb->Nmax, fp64) : plan.alt;
-        other.ns_div = pinned ? 1 : plan.alt_div;
-        other.tuned_ms = pinned ? 0 : plan.alt_ms;
-        other.candidates = plan.candidates;
-        build_work(pb, other, R, fp64);
-        pb->part.get((size_t)other.nsplit * pb->Ntot * R * 16);
-        other.d_work = dalloc_copy(other.work.data(), other.work.size());
-        pb->plans.emplace(other_key, other);
-        other_guard.keep = true;
-    }
-    guard.keep = true;
-    if (it == pb->plans.end()) {
-        pb->plans.emplace(key, std::move(plan));
-    } else {
-        const cudaError_t e = cudaStreamSynchronize(pb->stream);  // the old lists may still be read
-        free_plan(it->second);
-        it->second = std::move(plan);
-        CK(e);
-    }
-    return get_plan(pb, R, fp64, allow_sh, adjoint);
+    return f.taken && ds_reserve(pb, f.plan, R, adjoint) ? &f.plan : nullptr;
+}
+
+MatvecPlan& get_plan(msd_problem* pb, int R, bool fp64, bool allow_sh = false, bool adjoint = false) {
+    MatvecPlan* digits = fp64 ? digit_plan(pb, R, adjoint) : nullptr;
+    return digits ? *digits : plain_plan(pb, R, fp64, allow_sh && !fp64, adjoint);
 }
 
 // Chunks of a recomputed product.  A configuration whose M x Mp pairs fit
@@ -2339,6 +2396,7 @@ void msd_destroy(msd_problem* pb) {
     pb->dsx.release();
     pb->dse.release();
     for (auto& kv : pb->plans) free_plan(kv.second);
+    for (auto& kv : pb->forms) free_plan(kv.second.plan);
     free_recompute_plans(pb);
     if (pb->d_gen_full) cudaFree(pb->d_gen_full);
     pb->genbuf.release();
@@ -2577,13 +2635,18 @@ msd_status msd_set_tile(msd_problem* pb, int R, int precision, int KB, int RT) {
             if (cand[i].KB + 100 * cand[i].P2 == KB && cand[i].RT == RT) hit = i;
         if (hit < 0) fail(MSD_ERR_ARG, "msd_set_tile: (KB, RT) is not an instantiated shape that fits");
         const long long key = (long long)R * 4 + (fp64 ? 0 : 1);
-        for (int use = 0; use < 4; ++use) {
-            auto it = pb->plans.find(plan_key(R, fp64, (use & 1) != 0, (use & 2) != 0));
+        CK(cudaStreamSynchronize(pb->stream));  // the old work lists may still be read
+        for (int sh = 0; sh < 2; ++sh) {
+            auto it = pb->plans.find(plan_key(R, fp64, sh != 0));
             if (it != pb->plans.end()) {
-                CK(cudaStreamSynchronize(pb->stream));  // the old work list may still be read
                 free_plan(it->second);
                 pb->plans.erase(it);
             }
+        }
+        auto form = pb->forms.find(R);
+        if (fp64 && form != pb->forms.end()) {
+            free_plan(form->second.plan);
+            pb->forms.erase(form);
         }
         auto rit = pb->rplans.find(key);
         if (rit != pb->rplans.end()) {

@@ -214,3 +214,36 @@ def test_tuned_time_is_that_of_a_product(msd):
         best = min(best, msd.msd_matvec_timing(pb.handle, 0)[0])
     assert 0.8 * best <= tuned <= 1.2 * best, (tuned, best)
     pb.close()
+
+
+@pytest.mark.parametrize("M,N,R", [(40, 16, 1), (60, 16, 1), (32, 12, 1), (200, 16, 1)])
+def test_groups_of_the_sources_decide_too(msd, M, N, R):
+    """Problems of one size whose radii make one group or several, tuned one
+    after the other or reached by an update: the kernel that is taken is at most
+    a quarter slower than the faster of the digit form and one thread per row or
+    tile (both pinned; fastest of 30 products each)."""
+    def best(pb):
+        x = torch.from_numpy(_x(pb.ntot, R, 1)).cuda()
+        t = 1e300
+        for _ in range(30):
+            msd.msd_matvec_timing(pb.handle, 1)
+            pb.matvec(x)
+            t = min(t, msd.msd_matvec_timing(pb.handle, 0)[0])
+        return t
+
+    even, spread = _grid(M, N, np.full(M, 1.0)), _grid(M, N, np.linspace(0.6, 1.5, M))
+    for first, then in ((even, spread), (spread, even)):
+        pb = msd.Problem(first)
+        for cl in (first, then):
+            if cl is then:
+                pb.update_geometry(radii=then.radii)
+            _check(pb, [cl], R, 1)
+            free = best(pb)
+            other = []
+            for KB in (0, 1, 5, 7):
+                q = msd.Problem(cl)
+                q.set_tile(R, msd.MSD_FP64, KB, 1)
+                other.append(best(q))
+                q.close()
+            assert free <= 1.25 * min(other), (free, other)
+        pb.close()

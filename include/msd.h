@@ -573,6 +573,14 @@ void msd_test_limit(int what, int64_t value);
  * on tensor cores (generators, adjoint generators, sources). */
 int64_t msd_test_digit_bytes(msd_problem* pb);
 
+/* Test hook: one piece of a solve on given vectors (device memory; S = systems =
+ * configurations x R, system c R + r; synchronises the stream).
+ *   MSD_TEST_SOLUTION_UPDATE  x += sum_i V_i y_i, as at the end of a mixed cycle:
+ *     V complex64 [nv][N_tot][R], y complex128 [S][nv], w = x complex128
+ *     [N_tot][R] */
+#define MSD_TEST_SOLUTION_UPDATE 0
+msd_status msd_test_krylov(msd_problem* pb, int op, int R, int nv, const void* V, const void* y, void* w);
+
 /* Total number of CUDA kernels launched by this library in this process. */
 int64_t msd_kernel_launches(void);
 

@@ -12,7 +12,8 @@
 // default one half; the solver option reorth sets eta2).  Per-thread
 // sums of dot products and updates run in the storage precision of the
 // basis (FP32 for the inner sweeps of a mixed solve, whose FP64 pipe would
-// otherwise bound them) and cross-chunk reductions in FP64.  Vectors are
+// otherwise bound them), cross-chunk reductions and the batches of the solution
+// update in FP64.  Vectors are
 // [rows][R] with R innermost; reductions run over row chunks that never
 // straddle two configurations, of a size that follows the number of elements
 // (rows x R) and not of rows alone, so that a few thousand rows with many
@@ -307,19 +308,21 @@ __global__ void k_coeffs(int C, int R, int nv, const double2* __restrict__ y, in
 
 // w[row][r] += sign * sum_{i < nv} V_i[row][r] hT[cfg][i][r], lane = element.
 // SPLIT warps share 32 elements, each taking every SPLIT-th batch of U
-// vectors (all U loads in flight, their coefficients coming from L1); their
-// sums, in the basis precision (FP32 for an FP32 basis: the correction only
-// needs the accuracy of the FP32 sweep), meet in shared memory and w is
-// written once, without atomics.
+// vectors (all U loads in flight, their coefficients coming from L1); a batch is
+// summed in the basis precision and the batches in that of w (FP64 for the
+// solution of a mixed solve, whose basis of up to 4000 FP32 vectors would lose
+// the small terms otherwise; FP32 for a vector of its sweep).  The warps' sums
+// meet in shared memory and w is written once, without atomics.
 template <typename V, typename W, int SPLIT>
 __global__ void __launch_bounds__(kThreads, sizeof(V) == 8 ? 4 : 2)
     k_update(const RowChunk* __restrict__ chunks, int R, const V* __restrict__ Vb, long long vstride, int nv,
              const V* __restrict__ hT, long long ldh, const int* __restrict__ skip, int skipval, double sign,
              W* __restrict__ w) {
     typedef decltype(V{}.x) A;
+    typedef decltype(W{}.x) B;
     constexpr int U = 8;
     constexpr int kCols = kWarps / SPLIT;  // groups of 32 elements of the CTA
-    __shared__ V red[kCols][SPLIT][32];
+    __shared__ W red[kCols][SPLIT][32];
     const RowChunk ch = chunks[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sp = warp % SPLIT, cg = warp / SPLIT;
@@ -329,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(V) == 8 ? 4 : 2)
     const int r = act ? rel % R : 0;
     if (skip && act) act = skip[ch.cfg * R + r] != skipval;
     const long long e = ch.row0 * R + rel;
-    A ax[2] = {A(0), A(0)}, ay[2] = {A(0), A(0)};
+    B ax[2] = {B(0), B(0)}, ay[2] = {B(0), B(0)};
     if (__any_sync(0xffffffffu, act)) {
         const V* vp = Vb + (act ? e : ch.row0 * R);
         const V* hp = hT + (long long)ch.cfg * ldh * R + r;
@@ -351,25 +354,24 @@ __global__ void __launch_bounds__(kThreads, sizeof(V) == 8 ? 4 : 2)
                 bx[u & 1] = fma(vv[u].x, hh[u].x, fma(-vv[u].y, hh[u].y, bx[u & 1]));
                 by[u & 1] = fma(vv[u].x, hh[u].y, fma(vv[u].y, hh[u].x, by[u & 1]));
             }
-            ax[0] += bx[0];
-            ax[1] += bx[1];
-            ay[0] += by[0];
-            ay[1] += by[1];
+            ax[0] += (B)bx[0];
+            ax[1] += (B)bx[1];
+            ay[0] += (B)by[0];
+            ay[1] += (B)by[1];
         }
     }
-    red[cg][sp][lane] = V{ax[0] + ax[1], ay[0] + ay[1]};
+    red[cg][sp][lane] = W{ax[0] + ax[1], ay[0] + ay[1]};
     if (SPLIT > 1) __syncthreads();
     if (sp != 0 || !act) return;
-    V d = red[cg][0][lane];
+    W d = red[cg][0][lane];
 #pragma unroll
     for (int k = 1; k < SPLIT; ++k) {
         d.x += red[cg][k][lane].x;
         d.y += red[cg][k][lane].y;
     }
     const W o = w[e];
-    typedef decltype(W{}.x) B;
     const B sg = (B)sign;
-    w[e] = W{o.x + sg * (B)d.x, o.y + sg * (B)d.y};
+    w[e] = W{o.x + sg * d.x, o.y + sg * d.y};
 }
 
 // The same for an FP32 basis and 16-byte loads, two neighbouring elements per
@@ -379,9 +381,13 @@ __global__ void __launch_bounds__(kThreads, 2)
     k_update_pair(const RowChunk* __restrict__ chunks, int R, const float2* __restrict__ Vb, long long vstride, int nv,
                   const float2* __restrict__ hT, long long ldh, const int* __restrict__ skip, int skipval, double sign,
                   W* __restrict__ w) {
+    typedef decltype(W{}.x) B;
+    struct Pair {
+        B x, y, z, w;
+    };
     constexpr int U = 8;
     constexpr int kCols = kWarps / SPLIT;
-    __shared__ float4 red[kCols][SPLIT][32];
+    __shared__ Pair red[kCols][SPLIT][32];
     const RowChunk ch = chunks[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sp = warp % SPLIT, cg = warp / SPLIT;
@@ -393,7 +399,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (skip && act0) act0 = skip[ch.cfg * R + r] != skipval;
     if (skip && act1) act1 = one ? act0 : skip[ch.cfg * R + r + 1] != skipval;
     const long long e = ch.row0 * R + rel;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    Pair acc{B(0), B(0), B(0), B(0)};
     if (__any_sync(0xffffffffu, act0 || act1)) {
         // (an odd last row reads one element past it: the next vector's first,
         // which the basis has room for, and whose product is not stored)
@@ -422,10 +428,10 @@ __global__ void __launch_bounds__(kThreads, 2)
                 b.z = fmaf(vv[u].z, hh[u].z, fmaf(-vv[u].w, hh[u].w, b.z));
                 b.w = fmaf(vv[u].z, hh[u].w, fmaf(vv[u].w, hh[u].z, b.w));
             }
-            acc.x += b.x;
-            acc.y += b.y;
-            acc.z += b.z;
-            acc.w += b.w;
+            acc.x += (B)b.x;
+            acc.y += (B)b.y;
+            acc.z += (B)b.z;
+            acc.w += (B)b.w;
         }
     }
     if (SPLIT > 1) {
@@ -434,22 +440,21 @@ __global__ void __launch_bounds__(kThreads, 2)
         if (sp != 0) return;
 #pragma unroll
         for (int k = 1; k < SPLIT; ++k) {
-            const float4 o = red[cg][k][lane];
+            const Pair o = red[cg][k][lane];
             acc.x += o.x;
             acc.y += o.y;
             acc.z += o.z;
             acc.w += o.w;
         }
     }
-    typedef decltype(W{}.x) B;
     const B sg = (B)sign;
     if (act0) {
         const W o = w[e];
-        w[e] = W{o.x + sg * (B)acc.x, o.y + sg * (B)acc.y};
+        w[e] = W{o.x + sg * acc.x, o.y + sg * acc.y};
     }
     if (act1) {
         const W o = w[e + 1];
-        w[e + 1] = W{o.x + sg * (B)acc.z, o.y + sg * (B)acc.w};
+        w[e + 1] = W{o.x + sg * acc.z, o.y + sg * acc.w};
     }
 }
 

@@ -1879,6 +1879,32 @@ const ChunkSet& chunk_set(msd_problem* pb, int R, bool fp32) {
     return pb->chunks.emplace(key, cs).first->second;
 }
 
+// Shapes of the vectors and projections of R columns, bases of m + 1 vectors.
+void krylov_dims(SolveCtx& cx, int R, bool fp32, int m) {
+    const msd_problem* pb = cx.pb;
+    cx.m = m;
+    cx.hstride = m + 2;
+    cx.chunks = &chunk_set(cx.pb, R, fp32);
+    cx.d.Ntot = pb->Ntot;
+    cx.d.R = R;
+    cx.d.C = pb->C;
+    cx.d.S = pb->C * R;
+    cx.d.m = m;
+    cx.d.nchunk = (int)cx.chunks->h.size();
+    cx.d.chunk_elems = cx.chunks->elems;
+    cx.d.ldh = m + 2;
+    cx.d.pairs = (R == 1 || R % 2 == 0) && pb->Ntot * R % 2 == 0;
+    for (const RowChunk& c : cx.chunks->h) cx.d.pairs = cx.d.pairs && c.row0 * R % 2 == 0;
+}
+
+// x += V y from the coefficients y [S][stride] of nv basis vectors.
+template <typename V>
+void update_solution(SolveCtx& cx, const V* Vb, int nv, const double2* y, int stride) {
+    cudaStream_t s = cx.pb->stream;
+    gm_coeffs<V>(cx.d, nv, y, stride, (V*)cx.hT, s);
+    gm_update<V, double2>(cx.d, cx.chunks->d, Vb, cx.pb->Ntot * cx.d.R, nv, (V*)cx.hT, nullptr, 1.0, cx.x, s);
+}
+
 // Hands the active flags of the Krylov systems to the products of one
 // Arnoldi step, and takes them back however the step ends.
 struct LiveScope {
@@ -2006,8 +2032,7 @@ void arnoldi_cycle(SolveCtx& cx, V* Vb, V* w, bool fp64, int maxit_left, int* st
     *steps_taken = j;
     gm_lsq(d, cx.H, cx.cs, cx.sn, cx.rdiag, cx.g, cx.kconv, cx.y, cx.lsq_work, s);
     // x += V y, each system over its own kconv columns (y is zero beyond it)
-    gm_coeffs<V>(d, j, cx.y, cx.m, hT, s);
-    gm_update<V, double2>(d, ch, Vb, vstride, j, hT, nullptr, 1.0, cx.x, s);
+    update_solution<V>(cx, Vb, j, cx.y, cx.m);
     CK_LAUNCH();
 }
 
@@ -2059,20 +2084,8 @@ msd_status solve_impl(msd_problem* pb, int R, const double* betas_host, const ms
     const size_t nv = (size_t)pb->Ntot * R;
     SolveCtx cx;
     cx.pb = pb;
-    cx.m = o.restart;
     cx.eta2 = o.reorth;
-    cx.d.Ntot = pb->Ntot;
-    cx.d.R = R;
-    cx.d.C = pb->C;
-    cx.d.S = pb->C * R;
-    cx.d.m = o.restart;
-    cx.chunks = &chunk_set(pb, R, mixed);
-    cx.d.nchunk = (int)cx.chunks->h.size();
-    cx.d.chunk_elems = cx.chunks->elems;
-    cx.d.ldh = o.restart + 2;
-    cx.d.pairs = (R == 1 || R % 2 == 0) && nv % 2 == 0;
-    for (const RowChunk& c : cx.chunks->h) cx.d.pairs = cx.d.pairs && c.row0 * R % 2 == 0;
-    cx.hstride = o.restart + 2;
+    krylov_dims(cx, R, mixed, o.restart);
     const int S = cx.d.S, m = o.restart;
 
     int bi = 1;
@@ -2693,6 +2706,21 @@ void msd_test_limit(int what, int64_t value) {
 
 int64_t msd_test_digit_bytes(msd_problem* pb) {
     return pb ? (int64_t)digit_bytes(pb) : 0;
+}
+
+msd_status msd_test_krylov(msd_problem* pb, int op, int R, int nv, const void* V, const void* y, void* w) {
+    return guarded(pb, [&]() -> msd_status {
+        if (!pb || R <= 0 || nv <= 0 || op != MSD_TEST_SOLUTION_UPDATE) fail(MSD_ERR_ARG, "msd_test_krylov: bad argument");
+        SolveCtx cx;
+        cx.pb = pb;
+        krylov_dims(cx, R, true, nv);
+        cx.hT = pb->sbuf[24].get((size_t)cx.d.S * (nv + 2) * 8);
+        cx.x = (double2*)w;
+        update_solution<float2>(cx, (const float2*)V, nv, (const double2*)y, nv);
+        CK_LAUNCH();
+        CK(cudaStreamSynchronize(pb->stream));
+        return MSD_OK;
+    });
 }
 
 msd_status msd_grad_farfield_misfit(msd_problem* pb, int R, const double* betas_host, int T,

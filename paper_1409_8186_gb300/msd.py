@@ -27,6 +27,7 @@ MSD_GEN_AUTO, MSD_GEN_STREAMED, MSD_GEN_RECOMPUTE = 0, 1, 2
 MSD_FORM_EFIE, MSD_FORM_MFIE, MSD_FORM_CFIE, MSD_FORM_BWIE = 0, 1, 2, 3
 FORMULATION_KINDS = {"efie": MSD_FORM_EFIE, "mfie": MSD_FORM_MFIE, "cfie": MSD_FORM_CFIE, "bwie": MSD_FORM_BWIE}
 MSD_TEST_PART_BYTES, MSD_TEST_FAIL_ALLOC = 0, 1
+MSD_TEST_SOLUTION_UPDATE = 0
 MSD_MAX_N = 55
 MSD_MAX_DORT = 2048
 
@@ -92,6 +93,7 @@ def _load():
         "msd_test_expire_waits": (V, [I]),
         "msd_test_limit": (V, [I, ctypes.c_int64]),
         "msd_test_digit_bytes": (ctypes.c_int64, [P]),
+        "msd_test_krylov": (I, [P, I, I, I, P, P, P]),
         "msd_set_truncation": (I, [P, P]),
         "msd_penetrable_interior_field": (I, [P, I, P, I, ctypes.c_int64, P, P]),
         "msd_dort_eigenvectors": (I, [P, I, P, I, P, P]),
@@ -112,7 +114,7 @@ EXPORTED = ("msd_create", "msd_destroy", "msd_num_unknowns", "msd_row_offset", "
             "msd_matvec_noalloc", "msd_grad_farfield_misfit", "msd_plan_info", "msd_set_tile",
             "msd_set_generator_mode", "msd_nearfield", "msd_rhs_pointsource", "msd_solve_pointsources",
             "msd_dort", "msd_dort_eigen", "msd_set_formulation", "msd_set_formulation_kind",
-            "msd_formulation_weights", "msd_test_expire_waits", "msd_test_limit", "msd_test_digit_bytes", "msd_set_truncation", "msd_penetrable_interior_field",
+            "msd_formulation_weights", "msd_test_expire_waits", "msd_test_limit", "msd_test_digit_bytes", "msd_test_krylov", "msd_set_truncation", "msd_penetrable_interior_field",
             "msd_dort_eigenvectors", "msd_herglotz_wave",
             "msd_set_penetrable",
             "msd_penetrable_matvec", "msd_solve_penetrable", "msd_solve_penetrable_pointsources",
@@ -415,6 +417,11 @@ def msd_test_limit(what: int, value: int) -> None:
 def msd_test_digit_bytes(h) -> int:
     """Test hook: device bytes held for digits of the FP64 product."""
     return int(_lib.msd_test_digit_bytes(h))
+
+
+def msd_test_krylov(h, op: int, R: int, nv: int, V, y, w) -> None:
+    """Test hook: one piece of a solve on given device vectors (include/msd.h)."""
+    _check(_lib.msd_test_krylov(h, op, R, nv, _ptr(V), _ptr(y) if y is not None else None, _ptr(w)))
 
 
 # ---------------------------------------------------------------- convenience wrapper

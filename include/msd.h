@@ -577,9 +577,14 @@ int64_t msd_test_digit_bytes(msd_problem* pb);
  * configurations x R, system c R + r; synchronises the stream).
  *   MSD_TEST_SOLUTION_UPDATE  x += sum_i V_i y_i, as at the end of a mixed cycle:
  *     V complex64 [nv][N_tot][R], y complex128 [S][nv], w = x complex128
- *     [N_tot][R] */
+ *     [N_tot][R]
+ *   MSD_TEST_SECOND_PROJECTION  w -= V (V^H w), as the second projection of an
+ *     FP64 step: V complex128 [nv][N_tot][R], w complex128 [N_tot][R]; norm2
+ *     (host double [S]) receives the ||w||^2 that the step goes on with */
 #define MSD_TEST_SOLUTION_UPDATE 0
-msd_status msd_test_krylov(msd_problem* pb, int op, int R, int nv, const void* V, const void* y, void* w);
+#define MSD_TEST_SECOND_PROJECTION 1
+msd_status msd_test_krylov(msd_problem* pb, int op, int R, int nv, const void* V, const void* y, void* w,
+                           double* norm2);
 
 /* Total number of CUDA kernels launched by this library in this process. */
 int64_t msd_kernel_launches(void);

@@ -487,9 +487,8 @@ __global__ void k_scale(const RowChunk* __restrict__ chunks, int R, const Vin* _
 // the first projection is ||w||^2 - sum_i |h_i|^2 (Pythagoras, V orthonormal);
 // need[s] = 1 for an active system where that is below ||w||^2 / 2.  The
 // estimate is written to wn2 (the subdiagonal when no second pass runs);
-// where cancellation makes it inaccurate the second pass runs, and this
-// kernel (skip2 NULL) forms its norm from ||w1||^2, measured by that pass, and
-// the small h2.
+// where cancellation makes it inaccurate the second pass runs and measures
+// the norm itself.
 __global__ void k_reorth_flags(int S, const double2* __restrict__ h1, int hstride, int j,
                                double2* __restrict__ wn2, const int* __restrict__ active,
                                int* __restrict__ skip2, double eta2) {
@@ -508,7 +507,7 @@ __global__ void k_reorth_flags(int S, const double2* __restrict__ h1, int hstrid
     const double before = h[j + 1].x;  // ||w||^2 before the projection
     const double after = before - ss;
     wn2[(long long)s * hstride] = make_double2(after, 0.0);
-    if (skip2) skip2[s] = !(active[s] && after < eta2 * before);
+    skip2[s] = !(active[s] && after < eta2 * before);
 }
 
 // Start of a cycle: beta = ||r||; systems whose residual already meets

@@ -1897,6 +1897,29 @@ void krylov_dims(SolveCtx& cx, int R, bool fp32, int m) {
     for (const RowChunk& c : cx.chunks->h) cx.d.pairs = cx.d.pairs && c.row0 * R % 2 == 0;
 }
 
+// Second projection h2 = V^H w, w -= V h2 on the first j + 1 basis vectors, of
+// the systems with skip2 == 0, and the squared norm of w after it in wn2b.  Few
+// systems: ||w1||^2 - |h2|^2, formed inside the reduction (w1 measured by the
+// projection itself; h2 is small after the first pass).  A batch of systems:
+// measured on w, as one of many is where the difference cancels (near a
+// breakdown it could fall to 0 or below, which ends a system early).
+template <typename V>
+void second_projection(SolveCtx& cx, const V* Vb, V* w, int j) {
+    cudaStream_t s = cx.pb->stream;
+    const GmresDims& d = cx.d;
+    const long long vstride = cx.pb->Ntot * d.R;
+    GmDotsFuse fz;
+    fz.cnt = cx.cnt;
+    fz.j = j;
+    fz.wn2 = cx.wn2b;
+    const bool norm_done = gm_dots<V>(d, cx.chunks->d, cx.chunks->d_off, Vb, vstride, j + 1, 1, w, cx.skip2, cx.part,
+                                      cx.h2, cx.hstride, (V*)cx.hT, s, 1, &fz);
+    gm_update<V, V>(d, cx.chunks->d, Vb, vstride, j + 1, (V*)cx.hT, cx.skip2, -1.0, w, s);
+    if (!norm_done)
+        gm_dots<V>(d, cx.chunks->d, cx.chunks->d_off, nullptr, 0, 0, 1, w, cx.skip2, cx.part, cx.wn2b, cx.hstride,
+                   nullptr, s);
+}
+
 // x += V y from the coefficients y [S][stride] of nv basis vectors.
 template <typename V>
 void update_solution(SolveCtx& cx, const V* Vb, int nv, const double2* y, int stride) {
@@ -1963,9 +1986,9 @@ void arnoldi_cycle(SolveCtx& cx, V* Vb, V* w, bool fp64, int maxit_left, int* st
         // systems that have converged (zero vectors from here on) are skipped
         // (few systems: the norm after the projection and the flags of the
         // second one are formed inside the reduction kernel)
-        GmDotsFuse fz1, fz2;
-        fz1.cnt = fz2.cnt = cx.cnt;
-        fz1.j = fz2.j = j;
+        GmDotsFuse fz1;
+        fz1.cnt = cx.cnt;
+        fz1.j = j;
         fz1.wn2 = cx.wn2;
         fz1.active = cx.active;
         fz1.skip2 = cx.skip2;
@@ -1975,14 +1998,7 @@ void arnoldi_cycle(SolveCtx& cx, V* Vb, V* w, bool fp64, int maxit_left, int* st
         gm_update<V, V>(d, ch, Vb, vstride, j + 1, hT, cx.active, -1.0, w, s, 0);
         // second projection only where the first removed more than half of ||w||^2
         if (!flags_done) gm_reorth_flags(d, cx.h1, cx.hstride, j, cx.wn2, cx.active, cx.skip2, s, cx.eta2);
-        // its norm: ||w1 - V h2||^2 = ||w1||^2 - |h2|^2 (w1 measured by the
-        // projection itself; h2 is small after the first pass, so no
-        // cancellation)
-        fz2.wn2 = cx.wn2b;
-        const bool norm_done =
-            gm_dots<V>(d, ch, co, Vb, vstride, j + 1, 1, w, cx.skip2, cx.part, cx.h2, cx.hstride, hT, s, 1, &fz2);
-        gm_update<V, V>(d, ch, Vb, vstride, j + 1, hT, cx.skip2, -1.0, w, s);
-        if (!norm_done) gm_reorth_flags(d, cx.h2, cx.hstride, j, cx.wn2b, nullptr, nullptr, s, cx.eta2);
+        second_projection<V>(cx, Vb, w, j);
         // the Givens step stores its flags (any system still active, a
         // non-finite coefficient) straight into pinned host memory, in the
         // ring slot of this step; the host cleared the slot, whose previous
@@ -2708,13 +2724,32 @@ int64_t msd_test_digit_bytes(msd_problem* pb) {
     return pb ? (int64_t)digit_bytes(pb) : 0;
 }
 
-msd_status msd_test_krylov(msd_problem* pb, int op, int R, int nv, const void* V, const void* y, void* w) {
+msd_status msd_test_krylov(msd_problem* pb, int op, int R, int nv, const void* V, const void* y, void* w,
+                           double* norm2) {
     return guarded(pb, [&]() -> msd_status {
-        if (!pb || R <= 0 || nv <= 0 || op != MSD_TEST_SOLUTION_UPDATE) fail(MSD_ERR_ARG, "msd_test_krylov: bad argument");
+        const bool second = op == MSD_TEST_SECOND_PROJECTION;
+        if (!pb || R <= 0 || nv <= 0 || (!second && op != MSD_TEST_SOLUTION_UPDATE) || (second && !norm2))
+            fail(MSD_ERR_ARG, "msd_test_krylov: bad argument");
         SolveCtx cx;
         cx.pb = pb;
-        krylov_dims(cx, R, true, nv);
-        cx.hT = pb->sbuf[24].get((size_t)cx.d.S * (nv + 2) * 8);
+        krylov_dims(cx, R, !second, nv);
+        cx.hT = pb->sbuf[24].get((size_t)cx.d.S * (nv + 2) * (second ? 16 : 8));
+        if (second) {
+            const size_t S = cx.d.S;
+            cx.h2 = (double2*)pb->sbuf[1].get(S * cx.hstride * 16);
+            cx.wn2b = (double2*)pb->sbuf[2].get(S * cx.hstride * 16);
+            cx.skip2 = (int*)pb->sbuf[3].get((S + 1) * sizeof(int));
+            cx.cnt = cx.skip2 + S;
+            cx.part = (double2*)pb->sbuf[0].get((size_t)cx.d.nchunk * (nv + 2) * R * 16);
+            CK(cudaMemsetAsync(cx.skip2, 0, (S + 1) * sizeof(int), pb->stream));
+            second_projection<double2>(cx, (const double2*)V, (double2*)w, nv - 1);
+            CK_LAUNCH();
+            std::vector<double2> h(S * cx.hstride);
+            CK(cudaMemcpyAsync(h.data(), cx.wn2b, h.size() * 16, cudaMemcpyDeviceToHost, pb->stream));
+            CK(cudaStreamSynchronize(pb->stream));
+            for (size_t i = 0; i < S; ++i) norm2[i] = h[i * cx.hstride].x;
+            return MSD_OK;
+        }
         cx.x = (double2*)w;
         update_solution<float2>(cx, (const float2*)V, nv, (const double2*)y, nv);
         CK_LAUNCH();

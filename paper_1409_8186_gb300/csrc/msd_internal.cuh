@@ -474,7 +474,7 @@ template <typename Vin, typename Vout>
 // (rf, xs: also xs = rf .* v, the scaled input of the next FP32 product)
 void gm_scale(const GmresDims& d, const RowChunk* chunks, const Vin* w, const double* scale, const int* active,
               Vout* v, cudaStream_t s, const float* rf = nullptr, float2* xs = nullptr);
-// ||w'||^2 (written to wn2) and, skip2 not NULL, the re-orthogonalisation flags
+// ||w'||^2 estimate (written to wn2) and the re-orthogonalisation flags
 void gm_reorth_flags(const GmresDims& d, const double2* h1, int hstride, int j, double2* wn2,
                      const int* active, int* skip2, cudaStream_t s, double eta2 = 0.5);
 void gm_start(const GmresDims& d, const double2* rr, int hstride, const double* tol_abs, double* beta,

@@ -27,7 +27,7 @@ MSD_GEN_AUTO, MSD_GEN_STREAMED, MSD_GEN_RECOMPUTE = 0, 1, 2
 MSD_FORM_EFIE, MSD_FORM_MFIE, MSD_FORM_CFIE, MSD_FORM_BWIE = 0, 1, 2, 3
 FORMULATION_KINDS = {"efie": MSD_FORM_EFIE, "mfie": MSD_FORM_MFIE, "cfie": MSD_FORM_CFIE, "bwie": MSD_FORM_BWIE}
 MSD_TEST_PART_BYTES, MSD_TEST_FAIL_ALLOC = 0, 1
-MSD_TEST_SOLUTION_UPDATE = 0
+MSD_TEST_SOLUTION_UPDATE, MSD_TEST_SECOND_PROJECTION = 0, 1
 MSD_MAX_N = 55
 MSD_MAX_DORT = 2048
 
@@ -93,7 +93,7 @@ def _load():
         "msd_test_expire_waits": (V, [I]),
         "msd_test_limit": (V, [I, ctypes.c_int64]),
         "msd_test_digit_bytes": (ctypes.c_int64, [P]),
-        "msd_test_krylov": (I, [P, I, I, I, P, P, P]),
+        "msd_test_krylov": (I, [P, I, I, I, P, P, P, P]),
         "msd_set_truncation": (I, [P, P]),
         "msd_penetrable_interior_field": (I, [P, I, P, I, ctypes.c_int64, P, P]),
         "msd_dort_eigenvectors": (I, [P, I, P, I, P, P]),
@@ -419,9 +419,10 @@ def msd_test_digit_bytes(h) -> int:
     return int(_lib.msd_test_digit_bytes(h))
 
 
-def msd_test_krylov(h, op: int, R: int, nv: int, V, y, w) -> None:
+def msd_test_krylov(h, op: int, R: int, nv: int, V, y, w, norm2=None) -> None:
     """Test hook: one piece of a solve on given device vectors (include/msd.h)."""
-    _check(_lib.msd_test_krylov(h, op, R, nv, _ptr(V), _ptr(y) if y is not None else None, _ptr(w)))
+    p = lambda a: _ptr(a) if a is not None else None  # noqa: E731
+    _check(_lib.msd_test_krylov(h, op, R, nv, _ptr(V), p(y), _ptr(w), p(norm2)))
 
 
 # ---------------------------------------------------------------- convenience wrapper

@@ -67,3 +67,32 @@ def test_small_terms_after_a_large_one(msd, Ms, N, R):
     # the first batch: eight additions next to 2^24, whose FP32 spacing is 2
     assert (x - ref).abs().max().item() <= 8.0 + 12 * 2.0 ** -24 * (nv - 1) * 0.1
     pb.close()
+
+
+@pytest.mark.parametrize("Ms,N,R", [((40, 30), 4, 16), ((12,) * 9, 3, 1), ((50,), 3, 33)])
+@pytest.mark.parametrize("eps", [1e-3, 1e-6, 1e-9])
+def test_norm_after_a_second_projection_of_a_batch(msd, Ms, N, R, eps):
+    """w = V c + t with |c| = 1 and a remainder |t| = eps across V, for more than
+    eight systems: the norm that the step goes on with is that of what is left,
+    t and the rounding of the projection (64 x 2^-53 and of V's orthonormality,
+    which is formed in FP64), and not what a difference of squares near 1 leaves
+    (1e-16, so that eps below 1e-8 would be lost)."""
+    nv = 5
+    pb = _problem(msd, Ms, N)
+    assert pb.C * R > 8
+    g = torch.Generator(device="cuda").manual_seed(7)
+    B = torch.randn(nv + 1, pb.ntot, R, dtype=torch.complex128, device="cuda", generator=g)
+    c = torch.randn(nv, pb.C, R, dtype=torch.complex128, device="cuda", generator=g)
+    c = c / c.abs().square().sum(0).sqrt()
+    w = torch.empty(pb.ntot, R, dtype=torch.complex128, device="cuda")
+    for k in range(pb.C):
+        s = slice(pb.row_offset(k), pb.row_offset(k + 1))
+        Q = torch.linalg.qr(B[:, s].permute(2, 1, 0))[0].permute(2, 1, 0)  # [nv + 1, rows, R]
+        B[:, s] = Q
+        w[s] = torch.einsum("inr,ir->nr", Q[:nv], c[:, k]) + eps * Q[nv]
+    norm2 = np.zeros(pb.C * R)
+    msd.msd_test_krylov(pb.handle, msd.MSD_TEST_SECOND_PROJECTION, R, nv, B[:nv].contiguous(), None, w, norm2)
+    left = torch.stack([w[pb.row_offset(k):pb.row_offset(k + 1)].abs().square().sum(0) for k in range(pb.C)])
+    assert np.abs(norm2 - left.cpu().numpy().reshape(-1)).max() <= 1e-13 * eps ** 2
+    assert np.abs(np.sqrt(norm2) - eps).max() <= 64 * 2.0 ** -53
+    pb.close()

@@ -586,6 +586,10 @@ int64_t msd_test_digit_bytes(msd_problem* pb);
 msd_status msd_test_krylov(msd_problem* pb, int op, int R, int nv, const void* V, const void* y, void* w,
                            double* norm2);
 
+/* Test hook: whether the FP32 Krylov kernels of R columns load 16-byte pairs (1,
+ * 0; -1: bad argument). */
+int msd_test_pairs(msd_problem* pb, int R);
+
 /* Total number of CUDA kernels launched by this library in this process. */
 int64_t msd_kernel_launches(void);
 

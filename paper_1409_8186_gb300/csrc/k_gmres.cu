@@ -121,7 +121,8 @@ __global__ void __launch_bounds__(kThreads) k_dots(const RowChunk* __restrict__ 
 
 // The same for an FP32 basis with 16-byte loads, two neighbouring elements per
 // lane: two columns of a row (R even), or two rows of a single column (R =
-// 1).  For vectors and chunks that start on an even element (GmresDims::pairs).
+// 1).  For vectors and chunks that start on an even element (GmresDims::pairs),
+// so that a chunk of a single column has an even number of rows.
 // Halves the load instructions and doubles the bytes in flight: eight systems
 // of 60 disks with 32 columns, 74 -> 54 us a projection (k_update_pair: 88 ->
 // 62 us an update).
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(kThreads) k_dots_pair(const RowChunk* __restri
 #pragma unroll
         for (int k = 0; k < IV; ++k) u[k] = i0 + k < nv ? Vb + (long long)(i0 + k) * vstride : w;
         const int rows = (int)(ch.row1 - ch.row0);
-        const int units = one ? (rows + 1) / 2 : rows;  // a unit: a row, or two rows of one column
+        const int units = one ? rows / 2 : rows;        // a unit: a row, or two rows of one column
         const int unit = one ? 2 : R;                   // elements from one unit to the next
         long long e = ch.row0 * R + (long long)ro * unit + r;
         const long long step = (long long)RPW * unit;
@@ -160,19 +161,9 @@ __global__ void __launch_bounds__(kThreads) k_dots_pair(const RowChunk* __restri
 #pragma unroll
             for (int n = 0; n < UN; ++n) {
                 const bool ok = in && q + n * RPW < units;
-                if (one && ok && 2 * (q + n * RPW) + 1 >= rows) {  // the odd last row
-                    const float2 x = w[e + n * step];
-                    wv[n] = make_float4(x.x, x.y, 0.f, 0.f);
+                wv[n] = ok ? *(const float4*)(w + e + n * step) : zero;
 #pragma unroll
-                    for (int k = 0; k < IV; ++k) {
-                        const float2 y = u[k][e + n * step];
-                        uv[n][k] = make_float4(y.x, y.y, 0.f, 0.f);
-                    }
-                } else {
-                    wv[n] = ok ? *(const float4*)(w + e + n * step) : zero;
-#pragma unroll
-                    for (int k = 0; k < IV; ++k) uv[n][k] = ok ? *(const float4*)(u[k] + e + n * step) : zero;
-                }
+                for (int k = 0; k < IV; ++k) uv[n][k] = ok ? *(const float4*)(u[k] + e + n * step) : zero;
             }
 #pragma unroll
             for (int n = 0; n < UN; ++n)
@@ -401,8 +392,6 @@ __global__ void __launch_bounds__(kThreads, 2)
     const long long e = ch.row0 * R + rel;
     Pair acc{B(0), B(0), B(0), B(0)};
     if (__any_sync(0xffffffffu, act0 || act1)) {
-        // (an odd last row reads one element past it: the next vector's first,
-        // which the basis has room for, and whose product is not stored)
         const float2* vp = Vb + (rel < tot ? e : ch.row0 * R);
         const float2* hp = hT + (long long)ch.cfg * ldh * R + r;
         for (int i0 = sp * U; i0 < nv; i0 += SPLIT * U) {

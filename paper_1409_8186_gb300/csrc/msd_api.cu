@@ -1852,14 +1852,17 @@ void norm2_f64(SolveCtx& cx, const double2* u, double2* out) {
 // across configurations, of at least 256 elements (rows x R) for an FP64 basis
 // (whose projections the FP64 pipe bounds: many short warps) and 1024 for an
 // FP32 one (bound by memory: long-lived warps; the 400-disk sweep took 8 %
-// longer with 256).
+// longer with 256), and of an even number of rows for a single column (an odd
+// one would start every second chunk off a 16-byte boundary, where the pair
+// kernels cannot serve: k_dots_pair).
 const ChunkSet& chunk_set(msd_problem* pb, int R, bool fp32) {
     const int key = 2 * R + (fp32 ? 1 : 0);
     auto it = pb->chunks.find(key);
     if (it != pb->chunks.end()) return it->second;
     ChunkSet cs;
     std::vector<int> off(pb->C + 1, 0);
-    const long long target = std::max<long long>(1, std::max<long long>(fp32 ? 1024 : 256, pb->Ntot * R / 256) / R);
+    long long target = std::max<long long>(1, std::max<long long>(fp32 ? 1024 : 256, pb->Ntot * R / 256) / R);
+    if (R == 1) target += target & 1;
     for (int c = 0; c < pb->C; ++c) {
         const MsdConfig& m = pb->cfg[c];
         const long long rows = (long long)m.M * m.n;
@@ -2722,6 +2725,19 @@ void msd_test_limit(int what, int64_t value) {
 
 int64_t msd_test_digit_bytes(msd_problem* pb) {
     return pb ? (int64_t)digit_bytes(pb) : 0;
+}
+
+int msd_test_pairs(msd_problem* pb, int R) {
+    int pairs = -1;
+    guarded(pb, [&]() -> msd_status {
+        if (!pb || R <= 0) fail(MSD_ERR_ARG, "msd_test_pairs: bad argument");
+        SolveCtx cx;
+        cx.pb = pb;
+        krylov_dims(cx, R, true, 1);
+        pairs = cx.d.pairs ? 1 : 0;
+        return MSD_OK;
+    });
+    return pairs;
 }
 
 msd_status msd_test_krylov(msd_problem* pb, int op, int R, int nv, const void* V, const void* y, void* w,

@@ -93,6 +93,7 @@ def _load():
         "msd_test_expire_waits": (V, [I]),
         "msd_test_limit": (V, [I, ctypes.c_int64]),
         "msd_test_digit_bytes": (ctypes.c_int64, [P]),
+        "msd_test_pairs": (I, [P, I]),
         "msd_test_krylov": (I, [P, I, I, I, P, P, P, P]),
         "msd_set_truncation": (I, [P, P]),
         "msd_penetrable_interior_field": (I, [P, I, P, I, ctypes.c_int64, P, P]),
@@ -114,7 +115,8 @@ EXPORTED = ("msd_create", "msd_destroy", "msd_num_unknowns", "msd_row_offset", "
             "msd_matvec_noalloc", "msd_grad_farfield_misfit", "msd_plan_info", "msd_set_tile",
             "msd_set_generator_mode", "msd_nearfield", "msd_rhs_pointsource", "msd_solve_pointsources",
             "msd_dort", "msd_dort_eigen", "msd_set_formulation", "msd_set_formulation_kind",
-            "msd_formulation_weights", "msd_test_expire_waits", "msd_test_limit", "msd_test_digit_bytes", "msd_test_krylov", "msd_set_truncation", "msd_penetrable_interior_field",
+            "msd_formulation_weights", "msd_test_expire_waits", "msd_test_limit", "msd_test_digit_bytes", "msd_test_krylov", "msd_test_pairs", "msd_set_truncation",
+            "msd_penetrable_interior_field",
             "msd_dort_eigenvectors", "msd_herglotz_wave",
             "msd_set_penetrable",
             "msd_penetrable_matvec", "msd_solve_penetrable", "msd_solve_penetrable_pointsources",
@@ -417,6 +419,11 @@ def msd_test_limit(what: int, value: int) -> None:
 def msd_test_digit_bytes(h) -> int:
     """Test hook: device bytes held for digits of the FP64 product."""
     return int(_lib.msd_test_digit_bytes(h))
+
+
+def msd_test_pairs(h, R: int) -> int:
+    """Test hook: whether the FP32 Krylov kernels of R columns load 16-byte pairs."""
+    return int(_lib.msd_test_pairs(h, R))
 
 
 def msd_test_krylov(h, op: int, R: int, nv: int, V, y, w, norm2=None) -> None:

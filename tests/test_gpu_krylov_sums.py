@@ -96,3 +96,27 @@ def test_norm_after_a_second_projection_of_a_batch(msd, Ms, N, R, eps):
     assert np.abs(norm2 - left.cpu().numpy().reshape(-1)).max() <= 1e-13 * eps ** 2
     assert np.abs(np.sqrt(norm2) - eps).max() <= 64 * 2.0 ** -53
     pb.close()
+
+
+@pytest.mark.parametrize("M,R,pairs", [(4, 1, 1), (5, 1, 0), (87468, 1, 1), (87467, 1, 0), (5, 2, 1), (5, 3, 0),
+                                       (87468, 2, 1), (40000, 1, 1)])
+def test_single_columns_keep_their_pairs(msd, M, R, pairs):
+    """16-byte loads wherever the vectors start on even elements: also where a
+    256th of a single column is an odd number of rows (262404 / 256 = 1025)."""
+    pb = _problem(msd, (M,), 1)
+    assert msd.msd_test_pairs(pb.handle, R) == pairs
+    pb.close()
+
+
+def test_long_single_column(msd):
+    """262404 rows in chunks of 1026, the last one shorter."""
+    pb = _problem(msd, (87468,), 1)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    V = torch.randn(9, pb.ntot, 1, dtype=torch.complex64, device="cuda", generator=g)
+    y = torch.randn(1, 1, 9, dtype=torch.complex128, device="cuda", generator=g)
+    x = torch.zeros(pb.ntot, 1, dtype=torch.complex128, device="cuda")
+    msd.msd_test_krylov(pb.handle, msd.MSD_TEST_SOLUTION_UPDATE, 1, 9, V, y, x)
+    ref = torch.einsum("inr,i->nr", V.to(torch.complex128), y[0, 0])
+    size = torch.einsum("inr,i->nr", V.abs().double(), y[0, 0].abs())
+    assert ((x - ref).abs() <= 12 * 2.0 ** -24 * size).all()
+    pb.close()

@@ -528,7 +528,11 @@ msd_status msd_set_generator_mode(msd_problem* pb, int mode, int64_t chunk_bytes
  *   split into seven 8-bit digits whose 28 leading products are exact, for
  *   stored generators and radii that share an exponent range in groups of
  *   sources - elsewhere a pinned problem takes the cost-model shape - or with
- *   KB = 1: one thread per target row, for few disks; FP32: KB 4..9, RT in {1,2,4,8,16} dividing R, at most 16 warps
+ *   KB = 1: one thread per target row, for few disks.  The errors of KB = 0 are
+ *   FP64 roundings of the largest terms of a column, not of the terms of each
+ *   row: rows far below the others, as of disks whose part of the column is
+ *   10^-6 of the rest, keep fewer of their own digits; KB = 4..7 and 1 keep
+ *   them.  FP32: KB 4..9, RT in {1,2,4,8,16} dividing R, at most 16 warps
  *   per CTA, shared memory <= 226 KB; FP32 KB + 100 selects the same window
  *   with each complex multiply-add issued as two paired FP32 FMAs, and with
  *   RT = 1, KB + 200 / KB + 300 the same windows in a kernel without CTA

@@ -12,9 +12,12 @@
 // 9 K-steps of 16 are integers below 2^24 and so exact in the FP32
 // accumulators of tcgen05.mma, and the sums of equal weight i + j are put
 // together in 64-bit integers before they meet FP64.  The 28 digit products
-// with i + j <= 8 are kept; what is dropped, and what the digits cut off, is
-// below 2^-55 of (largest generator) x (largest source value), the size of an
-// FP64 rounding error.
+// with i + j <= 8 are kept.  Per real product, what the digits cut off is below
+// 2^-53 and what is dropped below 2^-51.4 of (largest generator) x (largest
+// source value) of the group: six digit products of 2^14 at 2^{2 - 72}, for
+// values just above half their power of two with every lower digit -128; with
+// digits of either sign about 2^-55.  Folding a sum of up to 72 sources into
+// 64 bits adds 2^-52 of that product once (tests/test_digit_mirror.py).
 //
 // With d = n - m (see k_matvec_tcs.cu) the sum over the sources q at fixed d
 // is a GEMM whose K index runs over (q, {Re g, Im g}):
@@ -36,9 +39,19 @@
 // product of the two maxima, which belong to different sources; l_m g r_n is
 // bounded by powers of (a_p + a_q)/b <= 1, and stays so with the largest a_q
 // of the group in place of the source's own while the radii in a group differ
-// by less than 2^{7.5/N}.  Sources are sorted by radius and grouped so; where
-// eight neighbours in that order already differ by more, the form is not
-// offered (ds_grouping).
+// by less than 2^{7.5/N} (which can put a source's terms 2^7.5 below the
+// group's).  Sources are sorted by radius and grouped so; where eight neighbours
+// in that order already differ by more, the form is not offered (ds_grouping).
+//
+// So the error of a row is one of the group's largest terms, which are the
+// row's own where the columns are of similar size on all disks: at most 25
+// roundings (2^-53) of |x| + sum |l g r x| of its row, 0.4 on average (radii
+// 0.5 to 1.5, gaps of 0.01, N = 20, columns that fall off with the mode number
+// or not).  Where a column is much larger on some disks than on others, rows
+// that only see the small ones are less exact than with the FP64 pipe: disks
+// of sizes spread over six decades, up to 2e4 roundings of such a row, 15 of
+// the largest result.  msd_set_tile (KB = 4..7) keeps the row-wise accuracy.
+//
 //
 // What bounds it: the drain of the accumulators.  A K-step of MMAs takes about
 // 650 clocks (448 at the tensor pipe's peak; small N and the issue of short

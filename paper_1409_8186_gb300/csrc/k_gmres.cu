@@ -499,6 +499,41 @@ __global__ void k_reorth_flags(int S, const double2* __restrict__ h1, int hstrid
     skip2[s] = !(active[s] && after < eta2 * before);
 }
 
+// ||w'||^2 after the second projection of every system with skip2 == 0, one CTA
+// each: ||w1||^2 - |h2|^2 from the sums of that projection (h2[j + 1] holds
+// ||w1||^2) while at least half is left, where the difference is as exact as the
+// norm itself; else, as near a breakdown, measured on w.
+template <typename V>
+__global__ void __launch_bounds__(128) k_second_norm(const RowChunk* __restrict__ chunks,
+                                                     const int* __restrict__ cfg_chunk_off, int R,
+                                                     const double2* __restrict__ h2, int hstride, int j,
+                                                     const int* __restrict__ skip2, const V* __restrict__ w,
+                                                     double2* __restrict__ wn2) {
+    __shared__ double red[4];
+    const int s = blockIdx.x, c = s / R, r = s % R;
+    if (skip2[s]) return;
+    auto cta_sum = [&](double v) {
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+        __syncthreads();
+        return red[0] + red[1] + red[2] + red[3];
+    };
+    const double2* h = h2 + (long long)s * hstride;
+    double acc = 0.0;
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) acc += cabs2(h[i]);
+    const double before = h[j + 1].x;
+    double after = before - cta_sum(acc);
+    if (!(after >= 0.5 * before)) {
+        acc = 0.0;
+        const long long r1 = chunks[cfg_chunk_off[c + 1] - 1].row1;
+        for (long long row = chunks[cfg_chunk_off[c]].row0 + threadIdx.x; row < r1; row += blockDim.x)
+            acc += cabs2(to_d2(w[row * R + r]));
+        after = cta_sum(acc);
+    }
+    if (threadIdx.x == 0) wn2[(long long)s * hstride] = make_double2(after, 0.0);
+}
+
 // Start of a cycle: beta = ||r||; systems whose residual already meets
 // tol_abs are done.  g = [beta, 0, ...], scale = 1/beta.
 __global__ void k_start(int S, int m, const double2* __restrict__ rr, int hstride,
@@ -853,6 +888,13 @@ void gm_scale(const GmresDims& d, const RowChunk* chunks, const Vin* w, const do
     g_msd_launches += 1;
 }
 
+template <typename V>
+void gm_second_norm(const GmresDims& d, const RowChunk* chunks, const int* cfg_chunk_off, const double2* h2,
+                    int hstride, int j, const int* skip2, const V* w, double2* wn2, cudaStream_t s) {
+    k_second_norm<V><<<d.S, 128, 0, s>>>(chunks, cfg_chunk_off, d.R, h2, hstride, j, skip2, w, wn2);
+    g_msd_launches += 1;
+}
+
 void gm_reorth_flags(const GmresDims& d, const double2* h1, int hstride, int j, double2* wn2,
                      const int* active, int* skip2, cudaStream_t s, double eta2) {
     k_reorth_flags<<<d.S, 128, 0, s>>>(d.S, h1, hstride, j, wn2, active, skip2, eta2);
@@ -910,6 +952,10 @@ template bool gm_dots<double2>(const GmresDims&, const RowChunk*, const int*, co
 template bool gm_dots<float2>(const GmresDims&, const RowChunk*, const int*, const float2*, long long, int, int,
                               const float2*, const int*, double2*, double2*, int, float2*, cudaStream_t, int,
                               const GmDotsFuse*);
+template void gm_second_norm<double2>(const GmresDims&, const RowChunk*, const int*, const double2*, int, int,
+                                      const int*, const double2*, double2*, cudaStream_t);
+template void gm_second_norm<float2>(const GmresDims&, const RowChunk*, const int*, const double2*, int, int,
+                                     const int*, const float2*, double2*, cudaStream_t);
 template void gm_coeffs<double2>(const GmresDims&, int, const double2*, int, double2*, cudaStream_t);
 template void gm_coeffs<float2>(const GmresDims&, int, const double2*, int, float2*, cudaStream_t);
 template void gm_update<double2, double2>(const GmresDims&, const RowChunk*, const double2*, long long, int,

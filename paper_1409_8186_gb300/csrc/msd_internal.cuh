@@ -477,6 +477,10 @@ void gm_scale(const GmresDims& d, const RowChunk* chunks, const Vin* w, const do
 // ||w'||^2 estimate (written to wn2) and the re-orthogonalisation flags
 void gm_reorth_flags(const GmresDims& d, const double2* h1, int hstride, int j, double2* wn2,
                      const int* active, int* skip2, cudaStream_t s, double eta2 = 0.5);
+// ||w'||^2 after the second projection (h2 with ||w1||^2 at j + 1) of the systems with skip2 == 0
+template <typename V>
+void gm_second_norm(const GmresDims& d, const RowChunk* chunks, const int* cfg_chunk_off, const double2* h2,
+                    int hstride, int j, const int* skip2, const V* w, double2* wn2, cudaStream_t s);
 void gm_start(const GmresDims& d, const double2* rr, int hstride, const double* tol_abs, double* beta,
               double* vscale, double2* g, int* active, int* kconv, int* any_active, cudaStream_t s);
 void gm_givens(const GmresDims& d, int j, const double2* h1, const double2* h2, int hstride, const double2* wn2a,

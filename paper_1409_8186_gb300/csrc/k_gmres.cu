@@ -161,9 +161,16 @@ __global__ void __launch_bounds__(kThreads) k_dots_pair(const RowChunk* __restri
 #pragma unroll
             for (int n = 0; n < UN; ++n) {
                 const bool ok = in && q + n * RPW < units;
-                wv[n] = ok ? *(const float4*)(w + e + n * step) : zero;
+                // (a branch: as conditional loads they are compiled to 64 registers with spills, 74 us for 67)
+                if (ok) {
+                    wv[n] = *(const float4*)(w + e + n * step);
 #pragma unroll
-                for (int k = 0; k < IV; ++k) uv[n][k] = ok ? *(const float4*)(u[k] + e + n * step) : zero;
+                    for (int k = 0; k < IV; ++k) uv[n][k] = *(const float4*)(u[k] + e + n * step);
+                } else {
+                    wv[n] = zero;
+#pragma unroll
+                    for (int k = 0; k < IV; ++k) uv[n][k] = zero;
+                }
             }
 #pragma unroll
             for (int n = 0; n < UN; ++n)

@@ -154,7 +154,7 @@ struct MatvecPlan {
     double tuned_ms = 0;          // kernel time of the chosen shape in the tuning run
     // digit-sliced FP64 product (ch.DS, kept in DigitForm): its tiles and work
     // list, valid for one grouping of the sources
-    DsCfg* d_dscfg = nullptr;
+    DsCfg* d_dscfg = nullptr;  // (one allocation with the two that follow)
     DsWork* d_dswork = nullptr;
     int* d_dsoff = nullptr;  // items of CTA b: [d_dsoff[b], d_dsoff[b + 1])
     int nds = 0, Rt = 1;     // CTAs, columns of a group
@@ -958,14 +958,21 @@ bool ds_build(msd_problem* pb, MatvecPlan& plan, int R, DsShape best) {
     plan.ex_ints = best.ex_ints;
     plan.nsplit = best.nslots;
     plan.nds = sms;
-    plan.d_dscfg = dalloc_copy(best.cfgs.data(), best.cfgs.size());
-    plan.d_dswork = dalloc_copy(best.items.data(), best.items.size());
-    plan.d_dsoff = dalloc_copy(best.off.data(), best.off.size());
+    // one allocation: configurations, items, offsets (8-, 4- and 4-byte values)
+    const size_t cb = best.cfgs.size() * sizeof(DsCfg), wb = best.items.size() * sizeof(DsWork);
+    std::vector<char> all(cb + wb + best.off.size() * sizeof(int));
+    memcpy(all.data(), best.cfgs.data(), cb);
+    if (wb) memcpy(all.data() + cb, best.items.data(), wb);
+    memcpy(all.data() + cb + wb, best.off.data(), best.off.size() * sizeof(int));
+    char* d = dalloc_copy(all.data(), all.size());
+    plan.d_dscfg = (DsCfg*)d;
+    plan.d_dswork = (DsWork*)(d + cb);
+    plan.d_dsoff = (int*)(d + cb + wb);
     return true;
 }
 
 void free_plan(MatvecPlan& plan) {
-    for (void* p : {(void*)plan.d_work, (void*)plan.d_dscfg, (void*)plan.d_dswork, (void*)plan.d_dsoff})
+    for (void* p : {(void*)plan.d_work, (void*)plan.d_dscfg})
         if (p) cudaFree(p);
     plan.d_work = nullptr;
     plan.d_dscfg = nullptr;

@@ -1144,32 +1144,27 @@ double digits_ms(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint) {
 // Autotuner: time the product kernel of every candidate tile shape (with its
 // own split count) on the problem's generators and keep the fastest.  Large
 // products are timed on a prefix of the work list of about 20 ms, scaled to
-// the whole list (the digit-sliced form, whose lists are made per CTA, runs
-// whole, once where that takes longer).  The columns are random numbers of
-// several sizes: the conversion of the digit-sliced sums takes longer on zeros
-// (400 disks, one column: 232 us against 167 of a product).  Results are cached per process by problem shape.  The
-// tuning run synchronises the stream; MSD_AUTOTUNE=0 keeps the model choice.
+// the whole list.  The columns are random numbers of several sizes.  Results are
+// cached per process by problem shape.  The tuning run synchronises the stream;
+// MSD_AUTOTUNE=0 keeps the model choice.
 bool autotune_enabled() {
     const char* e = std::getenv("MSD_AUTOTUNE");
     return !(e && e[0] == '0');
 }
 
-// Nmax R (fp64, allow_sh) C Ntot Mmax device, class of the digit-sliced form
-typedef std::tuple<int, int, int, int, long long, int, int, int> TuneKey;
-
-// shape (FP64, may be NULL): the digit-sliced form to be timed too.  What it
-// takes depends on the groups of the sources, which problems of one size need
-// not share, so that its modelled clocks are part of the key, in half octaves
-// (-1: no shape of it fits).  adjoint: on the adjoint generators (FP64), and
-// their digits.  Digits made for the tuning alone are given back when another
-// kernel is faster.
-TuneResult autotune(msd_problem* pb, int R, bool fp64, bool allow_sh, bool adjoint, const DsShape* shape) {
-    static std::mutex mu;
-    static std::map<TuneKey, TuneResult> cache;
+// Nmax R (fp64, allow_sh) C Ntot Mmax device
+typedef std::tuple<int, int, int, int, long long, int, int> TuneKey;
+TuneKey tune_key(const msd_problem* pb, int R, bool fp64, bool allow_sh) {
     int dev = 0;
     CK(cudaGetDevice(&dev));
-    const int cls = !shape ? -2 : shape->clocks < 1e300 ? (int)std::lround(2.0 * std::log2(shape->clocks)) : -1;
-    const TuneKey key{pb->Nmax, R, (fp64 ? 1 : 0) + (allow_sh ? 2 : 0), pb->C, pb->Ntot, pb->Mmax, dev, cls};
+    return TuneKey{pb->Nmax, R, (fp64 ? 1 : 0) + (allow_sh ? 2 : 0), pb->C, pb->Ntot, pb->Mmax, dev};
+}
+
+// Every kernel but the digit-sliced one; adjoint: on the adjoint generators (FP64).
+TuneResult autotune(msd_problem* pb, int R, bool fp64, bool allow_sh, bool adjoint) {
+    static std::mutex mu;
+    static std::map<TuneKey, TuneResult> cache;
+    const TuneKey key = tune_key(pb, R, fp64, allow_sh);
     MatvecChoice cand[128];
     const int nc = matvec_candidates(R, pb->Nmax, fp64, cand, 128, allow_sh);
     {
@@ -1187,8 +1182,6 @@ TuneResult autotune(msd_problem* pb, int R, bool fp64, bool allow_sh, bool adjoi
     void* xs = pb->xs.get(vec);
     launch_tune_fill(fp64, (long long)pb->Ntot * R * 2, xs, pb->stream);
     const void* G = fp64 ? (const void*)(adjoint ? pb->d_GA64 : pb->d_G64) : (const void*)pb->d_G32;
-    DsGen& gen = adjoint ? pb->ds_adj : pb->ds_fwd;
-    const bool had_digits = gen.held() > 0, had_sources = pb->dsx.cap > 0;
     // estimated full time (FP64 ~1.2 TFLOP/s, FP32 ~40 TFLOP/s) -> prefix fraction
     const double est_ms = 8.0 * R * pb->offdiag_n2 / (fp64 ? 1.2e9 : 4.0e10);
     const double frac = est_ms > 20.0 ? 20.0 / est_ms : 1.0;
@@ -1204,8 +1197,7 @@ TuneResult autotune(msd_problem* pb, int R, bool fp64, bool allow_sh, bool adjoi
         MatvecPlan trial;
         trial.ch = cand[i / 4];
         trial.ns_div = dv;
-        const bool ds = trial.ch.DS;
-        if (ds && (dv > 1 || !shape || shape->clocks == 1e300)) continue;
+        if (trial.ch.DS) continue;
         float* XT = nullptr;
         if (trial.ch.SH) {
             if (!ensure_gt(pb)) continue;
@@ -1213,45 +1205,61 @@ TuneResult autotune(msd_problem* pb, int R, bool fp64, bool allow_sh, bool adjoi
             launch_tune_fill(false, pb->xrows * 4 * R, XT, pb->stream);
         }
         PlanGuard trial_guard{trial};
-        if (ds) {
-            if (!ds_build(pb, trial, R, *shape) || !ds_reserve(pb, trial, R, adjoint)) continue;
-        } else {
-            build_work(pb, trial, R, fp64);
-        }
+        build_work(pb, trial, R, fp64);
         if (dv == 1) model_ns = trial.nsplit;
-        const int nfull = std::max<int>(1, (int)trial.work.size());
+        const int nfull = (int)trial.work.size();
         const int nw = std::max(1, std::min(nfull, (int)std::ceil(frac * nfull)));
         MatvecWork* dw = (MatvecWork*)dwork.get(nfull * sizeof(MatvecWork));
-        if (!ds)
-            CK(cudaMemcpyAsync(dw, trial.work.data(), nw * sizeof(MatvecWork), cudaMemcpyHostToDevice, pb->stream));
+        CK(cudaMemcpyAsync(dw, trial.work.data(), nw * sizeof(MatvecWork), cudaMemcpyHostToDevice, pb->stream));
         void* part = pb->part.get((size_t)trial.nsplit * vec);
-        const double t = ds ? digits_ms(pb, trial, R, adjoint)
-                            : (double)nfull / nw * launch_ms(pb, false, [&] {
+        const double t = (double)nfull / nw * launch_ms(pb, false, [&] {
             if (trial.ch.SH)
                 launch_bt_tcs(pb->d_cfg, dw, nw, pb->Nmax, pb->d_GT, XT, (float2*)part, pb->Ntot, R, pb->stream);
             else
                 launch_bt_only(cand[i / 4], fp64, pb->d_cfg, dw, nw, pb->Nmax, G, xs, part, pb->Ntot, R, pb->stream);
         });
-        if (ds) {
-            res.ds_ms = t;
-            res.ds_clocks = shape->clocks;
-        } else if (t < res.ms) {
+        if (t < res.ms) {
             res.ms = t;
             res.ch = cand[i / 4];
             res.ns_div = trial.ns_div;
         }
     }
     dwork.release();
-    if (!(res.ds_ms > 0 && res.ds_ms < res.ms)) {
-        if (!had_digits) gen.release();
-        if (!had_sources) {
-            pb->dsx.release();
-            pb->dse.release();
-        }
-    }
     std::lock_guard<std::mutex> lk(mu);
     cache[key] = res;
     return res;
+}
+
+// The time of the digit-sliced form of that shape into res (0: it cannot be
+// laid out).  It depends on the groups of the sources, which problems of one
+// size need not share: its modelled clocks are part of the key, in half octaves.
+// The form's lists are made per CTA, so that it runs whole.  Generator digits
+// made for the tuning alone are given back where another kernel is faster.  Random
+// columns matter here: the conversion of its sums takes longer on zeros (400
+// disks, one column: 232 us against 167 of a product).
+void tune_digits(msd_problem* pb, int R, bool adjoint, const DsShape& shape, TuneResult& res) {
+    static std::mutex mu;
+    static std::map<std::pair<TuneKey, int>, std::pair<double, double>> cache;  // ms, clocks
+    const std::pair<TuneKey, int> key{tune_key(pb, R, true, false), (int)std::lround(2.0 * std::log2(shape.clocks))};
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = cache.find(key);
+        if (it != cache.end()) {
+            std::tie(res.ds_ms, res.ds_clocks) = it->second;
+            return;
+        }
+    }
+    res.ds_ms = 0;
+    DsGen& gen = adjoint ? pb->ds_adj : pb->ds_fwd;
+    const bool had = gen.held() > 0;
+    MatvecPlan trial;
+    PlanGuard guard{trial};
+    if (!ds_build(pb, trial, R, shape) || !ds_reserve(pb, trial, R, adjoint)) return;
+    res.ds_ms = digits_ms(pb, trial, R, adjoint);
+    res.ds_clocks = shape.clocks;
+    if (!had && !(res.ds_ms < res.ms)) gen.release();
+    std::lock_guard<std::mutex> lk(mu);
+    cache[key] = {res.ds_ms, res.ds_clocks};
 }
 
 // Plans are kept per (R, precision) and per use: allow_sh = the forward
@@ -1277,7 +1285,7 @@ MatvecPlan& plain_plan(msd_problem* pb, int R, bool fp64, bool allow_sh, bool ad
         auto form = fp64 ? pb->forms.find(R) : pb->forms.end();
         const bool known = form != pb->forms.end() && form->second.tuned.candidates > 0;
         if (known || autotune_enabled()) {
-            const TuneResult t = known ? form->second.tuned : autotune(pb, R, fp64, allow_sh, adjoint, nullptr);
+            const TuneResult t = known ? form->second.tuned : autotune(pb, R, fp64, allow_sh, adjoint);
             plan.ch = t.ch;
             plan.ns_div = t.ns_div;
             plan.tuned_ms = t.ms;
@@ -1328,7 +1336,10 @@ MatvecPlan* digit_plan(msd_problem* pb, int R, bool adjoint) {
         // not asked yet, or the form did not fit when it was
         const bool ask = !f.tried || (fits && f.tuned.candidates > 0 && f.tuned.ds_ms == 0);
         if (!pinned && ask) {
-            if (autotune_enabled()) f.tuned = autotune(pb, R, true, false, adjoint, &shape);
+            if (autotune_enabled()) {
+                f.tuned = autotune(pb, R, true, false, adjoint);
+                if (fits) tune_digits(pb, R, adjoint, shape, f.tuned);
+            }
             f.tried = true;
         }
         MatvecPlan plan;

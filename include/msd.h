@@ -512,7 +512,8 @@ msd_status msd_set_generator_mode(msd_problem* pb, int mode, int64_t chunk_bytes
  * MSD_AUTOTUNE=0 (cost-model choice) or msd_set_tile fixed one.  A captured
  * FP64 product takes the fastest shape but the one on bf16 tensor cores
  * (KB = 0): the graph then stays valid when msd_update_geometry remakes the
- * generators.
+ * generators.  (A captured FP32 product on the shift-GEMM kernel reads a copy of
+ * them that the next uncaptured product remakes.)
  *
  * msd_plan_info: the shape used for (R, precision), precision MSD_FP64 or
  *   MSD_FP32, creating the plan (and tuning) if needed.  out[4] receives

@@ -850,7 +850,9 @@ void gm_coeffs(const GmresDims& d, int nv, const double2* y, int ystride, V* hT,
 // SPLIT: enough warps for the chip (32 per SM) where the elements alone do
 // not give them, but at least one batch of vectors per warp.  FP32 bases of
 // more than 9 728 elements take pairs (400 disks, one column: the mixed solve
-// 431 -> 404 ms with eight warps a pair group against single elements).
+// 431 -> 404 ms with eight warps a pair group against single elements).  That
+// first step of the pairs' ladder is measured; its later ones, and the ladder of
+// single elements, follow the count of warps alone.
 template <typename V, typename W>
 void gm_update(const GmresDims& d, const RowChunk* chunks, const V* Vb, long long vstride, int nv, const V* hT,
                const int* skip, double sign, W* w, cudaStream_t s, int skipval) {

@@ -329,6 +329,7 @@ struct msd_problem {
     DsGen ds_fwd, ds_adj;
     bool ds_hold = false;  // digits are being made: not to be given back
     DBuf dsx, dse;
+    DBuf dspart;  // its partial sums: `part` may be held by a captured product, and their number follows the groups
     // algorithmic size of one product with one column (section 5 storage):
     // sum over ordered pairs of the generator length, and of n^2
     double offdiag_L = 0, offdiag_n2 = 0;
@@ -345,7 +346,7 @@ namespace {
 // Bytes of digits, and their release under memory pressure: the products of
 // the problem (and of its interior one) then run without the digit-sliced form.
 size_t digit_bytes(const msd_problem* pb) {
-    return pb->ds_fwd.held() + pb->ds_adj.held() + pb->dsx.cap + pb->dse.cap;
+    return pb->ds_fwd.held() + pb->ds_adj.held() + pb->dsx.cap + pb->dse.cap + pb->dspart.cap;
 }
 bool give_back_digits(msd_problem* pb) {
     bool any = false;
@@ -356,6 +357,7 @@ bool give_back_digits(msd_problem* pb) {
         p->ds_adj.release();
         p->dsx.release();
         p->dse.release();
+        p->dspart.release();
         p->ds_fwd.fits = p->ds_adj.fits = 0;
         any = true;
     }
@@ -1005,7 +1007,7 @@ bool ds_reserve(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint) {
         pb->dsx.get(plan.xd_bytes);
         pb->dse.get(plan.ex_ints * sizeof(int));
         pb->xs.get((size_t)pb->Ntot * R * 16);
-        pb->part.get((size_t)plan.nsplit * pb->Ntot * R * 16);
+        pb->dspart.get((size_t)plan.nsplit * pb->Ntot * R * 16);
         return true;
     } catch (const MsdError& e) {
         if (e.st != MSD_ERR_OOM) throw;
@@ -1014,6 +1016,11 @@ bool ds_reserve(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint) {
     give_back_digits(pb);
     pb->ds_fwd.fits = pb->ds_adj.fits = 0;
     return false;
+}
+
+// Partial sums of a product by that plan.
+void* part_of(msd_problem* pb, const MatvecPlan& plan, size_t bytes) {
+    return (plan.ch.DS ? pb->dspart : pb->part).get(bytes);
 }
 
 // The digit-sliced Toeplitz sums of the scaled columns xs into part (after
@@ -1137,7 +1144,7 @@ double digits_ms(msd_problem* pb, MatvecPlan& plan, int R, bool adjoint) {
     launch_tune_fill(true, (long long)pb->Ntot * R * 2, pb->xs.p, pb->stream);
     return launch_ms(pb, true, [&] {
         ds_product(pb, plan, R, adjoint, adjoint ? pb->d_GA64 : pb->d_G64, (const double2*)pb->xs.p,
-                   (double2*)pb->part.p);
+                   (double2*)pb->dspart.p);
     });
 }
 
@@ -1372,6 +1379,7 @@ MatvecPlan* digit_plan(msd_problem* pb, int R, bool adjoint) {
             pb->ds_adj.release();
             pb->dsx.release();
             pb->dse.release();
+            pb->dspart.release();
         }
         if (!taken) return nullptr;
         f.plan = std::move(plan);
@@ -1611,7 +1619,7 @@ void matvec_form_dev(msd_problem* pb, int R, bool fp64, const void* x, void* y) 
     MatvecPlan& plan = get_plan(pb, 2 * R, fp64);
     const size_t elem = fp64 ? 16 : 8;
     void* xs = pb->xs.get((size_t)pb->Ntot * 2 * R * elem);
-    void* part = pb->part.get((size_t)plan.nsplit * pb->Ntot * 2 * R * elem);
+    void* part = part_of(pb, plan, (size_t)plan.nsplit * pb->Ntot * 2 * R * elem);
     launch_form_scale(fp64, pb->Ntot, R, fp64 ? (const void*)pb->d_rf64 : (const void*)pb->d_rf32,
                       fp64 ? (const void*)pb->d_frf2_64 : (const void*)pb->d_frf2_32, x, xs, pb->stream);
     if (plan.ch.DS)
@@ -1643,8 +1651,8 @@ void pen_matvec(msd_problem* pb, int R, bool fp64, const void* x, void* y) {
         plan_m = &get_plan(pm, R, fp64);
         xsp = pb->xs.get(nv * elem);
         xsm = pm->xs.get(nv * elem);
-        partp = pb->part.get((size_t)plan_p->nsplit * nv * elem);
-        partm = pm->part.get((size_t)plan_m->nsplit * nv * elem);
+        partp = part_of(pb, *plan_p, (size_t)plan_p->nsplit * nv * elem);
+        partm = part_of(pm, *plan_m, (size_t)plan_m->nsplit * nv * elem);
     } while ((plan_p->ch.DS && !pb->ds_fwd.held()) || (plan_m->ch.DS && !pm->ds_fwd.held()));
     MatvecPlan &pp = *plan_p, &pq = *plan_m;
     launch_pen_scale(fp64, pb->d_cfg, pb->C, pb->Ntot, R, fp64 ? (const void*)pb->d_rf64 : (const void*)pb->d_rf32,
@@ -1686,7 +1694,7 @@ void matvec_dev(msd_problem* pb, int R, bool fp64, const void* x, void* y) {
     void* xs = plan.ch.SH ? nullptr : pb->xs.get((size_t)pb->Ntot * R * elem);
     const bool xs_ready = !fp64 && !plan.ch.SH && x == pb->xs_src;
     pb->xs_src = nullptr;
-    void* part = pb->part.get((size_t)plan.nsplit * pb->Ntot * R * elem);
+    void* part = part_of(pb, plan, (size_t)plan.nsplit * pb->Ntot * R * elem);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (pb->timing) {
         // events bracket the block-Toeplitz kernel alone (not the scaling or
@@ -1772,7 +1780,7 @@ void product_dev(msd_problem* pb, int R, bool fp64, bool adjoint, bool raw, cons
     MatvecPlan& plan = get_plan(pb, R, fp64, false, adjoint);
     const size_t elem = fp64 ? 16 : 8;
     void* xs = pb->xs.get((size_t)pb->Ntot * R * elem);
-    void* part = pb->part.get((size_t)plan.nsplit * pb->Ntot * R * elem);
+    void* part = part_of(pb, plan, (size_t)plan.nsplit * pb->Ntot * R * elem);
     const int nwork = (int)plan.work.size();
     if (fp64) {
         const double2* G = adjoint ? pb->d_GA64 : pb->d_G64;
@@ -2446,6 +2454,7 @@ void msd_destroy(msd_problem* pb) {
     pb->ds_adj.release();
     pb->dsx.release();
     pb->dse.release();
+    pb->dspart.release();
     for (auto& kv : pb->plans) free_plan(kv.second);
     for (auto& kv : pb->forms) free_plan(kv.second.plan);
     free_recompute_plans(pb);
@@ -2640,6 +2649,7 @@ msd_status msd_set_generator_mode(msd_problem* pb, int mode, int64_t chunk_bytes
             pb->ds_adj.release();
             pb->dsx.release();
             pb->dse.release();
+            pb->dspart.release();
         } else {
             free_recompute_plans(pb);
             pb->genbuf.release();

@@ -58,6 +58,9 @@ def test_replay_after_update(M, N, R, form, pinned):
             graph.replay()  # before any other product of the new geometry
             assert close(y, ref(new, x))
             assert close(pb.matvec(x), ref(new, x))
+            y.zero_()
+            graph.replay()  # nothing that it uses was moved by a product of other groups
+            assert close(y, ref(new, x))
         pb.update_geometry(cl.centres, cl.radii)
         unused = torch.cuda.CUDAGraph()
         with torch.cuda.graph(unused, stream=s):

@@ -377,13 +377,15 @@ void flush_timing(msd_problem* pb) {
     pb->ev_used = 0;
 }
 
-// A pipeline wait of the tensor-core product expired (results invalid).
+// A pipeline wait of a product kernel expired (results invalid).  Every record
+// is read, and so cleared, before any is reported: a call in which waits of two
+// kernels expire leaves nothing for the next one to fail on.
 void check_tc(const char* where) {
-    const int t = tc_status_and_clear();
-    const int u = tcs_status_and_clear();
-    if (t > 0 || u > 0) fail(MSD_ERR_CUDA, std::string(where) + ": a tensor-core pipeline wait expired");
-    if (ds_status_and_clear() > 0) fail(MSD_ERR_CUDA, std::string(where) + ": a pipeline wait of the FP64 product expired");
-    if (bt_status_and_clear() > 0) fail(MSD_ERR_CUDA, std::string(where) + ": a generator bulk-copy wait expired");
+    const bool tensor = tc_status_and_clear() > 0, shift = tcs_status_and_clear() > 0;
+    const bool digits = ds_status_and_clear() > 0, bulk = bt_status_and_clear() > 0;
+    if (tensor || shift) fail(MSD_ERR_CUDA, std::string(where) + ": a tensor-core pipeline wait expired");
+    if (digits) fail(MSD_ERR_CUDA, std::string(where) + ": a pipeline wait of the FP64 product expired");
+    if (bulk) fail(MSD_ERR_CUDA, std::string(where) + ": a generator bulk-copy wait expired");
 }
 
 void check_flags(msd_problem* pb, const char* where) {
